@@ -521,20 +521,39 @@ cem_status cem_mesh_create(const cem_mesh_desc *desc, cem_handle **out) {
     for (int k0 = 0; k0 < 4; ++k0) {
       double DX = (XN[(k0 + 1) % 4] - XN[k0]) * (0.5 * desc->hx);
       double DY = (EN[(k0 + 1) % 4] - EN[k0]) * (0.5 * desc->hy);
+      d.g.DX[k0] = DX;
+      d.g.DY[k0] = DY;
+      d.g.ref2[k0] = DX * DX + DY * DY;
+      const double x0 = (XG[k0] + 1.0) * (0.5 * desc->hx), y0 = (EG[k0] + 1.0) * (0.5 * desc->hy);
       d.g.DXf[k0] = (float)DX;
       d.g.DYf[k0] = (float)DY;
       for (int k = 0; k < 4; ++k) {
-        if (k == k0) { d.g.nxf[k0][k] = d.g.nyf[k0][k] = 0.f; continue; }
+        if (k == k0) {
+          d.g.nxf[k0][k] = d.g.nyf[k0][k] = 0.f;
+          d.g.cnx[k0][k] = d.g.cny[k0][k] = 0.0;
+          continue;
+        }
         double sx = (XG[k] - XG[k0]) * (0.5 * desc->hx), sy = (EG[k] - EG[k0]) * (0.5 * desc->hy);
         double rx = -sy, ry = sx;
         if (rx * DX + ry * DY < 0.0) { rx = -rx; ry = -ry; }
         double len = sqrt(sx * sx + sy * sy);
         d.g.nxf[k0][k] = (float)(rx / len);
         d.g.nyf[k0][k] = (float)(ry / len);
+        // FP64: the edge midpoints' own coordinates subtracted, as the definition has them
+        const double xk = (XG[k] + 1.0) * (0.5 * desc->hx), yk = (EG[k] + 1.0) * (0.5 * desc->hy);
+        sx = xk - x0;
+        sy = yk - y0;
+        rx = -sy;
+        ry = sx;
+        if (rx * DX + ry * DY < 0.0) { rx = -rx; ry = -ry; }
+        len = sqrt(sx * sx + sy * sy);
+        d.g.cnx[k0][k] = rx / len;
+        d.g.cny[k0][k] = ry / len;
       }
     }
   }
   d.precision = desc->precision;
+  tile64_shape(desc->nx, desc->ny, d.t64x, d.t64y);
   d.ph_cap = desc->phantom_capacity > 0 ? desc->phantom_capacity : (int)(ne / 4 + 4096);
   d.ck_cap = desc->crack_capacity > 0 ? desc->crack_capacity : (int)(ne / 4 + 4096);
   long rim = 0;
@@ -1599,7 +1618,8 @@ cem_status batch_upload(cem_handle *b) {
       for (int q = 0; q < ng; ++q) wm.push_back(make_int4(s, q, 0, ng));
       tiles = tiles_fp32(d, p->tile_rows);
     } else {
-      const int gx = (d.g.nx + 1 + 31) / 32, gy = tiles_fp64(d) / gx;
+      int gx, gy;
+      grid_main64(d, gx, gy);
       for (int y = 0; y < gy; ++y)
         for (int x = 0; x < gx; ++x) wm.push_back(make_int4(s, x, y, gx | (gy << 16)));
       tiles = gx * gy;
@@ -1609,8 +1629,9 @@ cem_status batch_upload(cem_handle *b) {
     // (its counts, not its capacities, set the work: 78.9 against 102.1 us
     // per step of the 64-specimen batch).  FP64 keeps a solo run's grids, so
     // that its energy partials are grouped, and rounded, as when stepped alone.
-    int gph = grid_phantoms(d), gp = grid_pieces(d);
-    if (p->precision == CEM_FP32_MIXED) {
+    const bool mixed = p->precision == CEM_FP32_MIXED;
+    int gph = grid_phantoms(d), gp = mixed ? grid_pieces(d) : grid_pieces64(d);
+    if (mixed) {
       gph = std::min(gph, 8);
       gp = std::min(gp, 8);
     }
@@ -1618,7 +1639,7 @@ cem_status batch_upload(cem_handle *b) {
     for (int q = 0; q < gph; ++q) wph.push_back(make_int4(s, q, tiles + gp, gph));
     // the evaluation has no energy partials: a few virtual blocks per member
     // walk its list (its length, not its capacity, sets the work)
-    const int ge = std::min(grid_eval(d), 8);
+    const int ge = mixed ? std::min(grid_eval(d), 8) : std::min(grid_eval64(d), 32);
     for (int q = 0; q < ge; ++q) we.push_back(make_int4(s, q, 0, ge));
     // FP32 phantom blocks write one energy partial per warp
     nparts[s] = tiles + gp + (p->precision == CEM_FP32_MIXED ? kPhWarps : 1) * gph;

@@ -49,6 +49,8 @@ struct Geo {
   float rxf, ryf, qAf;     // 1/hx, 1/hy, A/4
   float DXf[4], DYf[4];    // reference vector X_N2 - X_N1 of local edge k
   float nxf[4][4], nyf[4][4];  // unit normal of candidate path k0 -> k
+  // FP64: the same vectors and normals, and |X_N2 - X_N1|^2
+  double DX[4], DY[4], ref2[4], cnx[4][4], cny[4][4];
 };
 
 struct Mat {
@@ -64,6 +66,7 @@ struct DevState {
   int precision;
   int ph_cap, ck_cap, list_cap, prop_cap, ncap;
   int lam_cap;
+  int t64x, t64y;  // tile of the FP64 node update (tile64_shape)
   // batched stepping (cem_batch_create): the member takes no step at or
   // after step_end (INT_MAX when stepped alone), and its current
   // displacement buffer at batch step n is (n & 1) ^ cur_xor
@@ -320,6 +323,10 @@ int energy_parts_step(const DevState &d);    // partials one step writes (alone)
 int tiles_fp32(const DevState &d, int tile_rows);   // energy partials of the node update
 int groups_fp32(const DevState &d, int tile_rows);  // its CTAs (four warp tiles each)
 int tiles_fp64(const DevState &d);
+void tile64_shape(int nx, int ny, int &tx, int &ty);
+void grid_main64(const DevState &d, int &gx, int &gy);
+int grid_pieces64(const DevState &d);
+int grid_eval64(const DevState &d);
 int grid_pieces(const DevState &d);
 int grid_phantoms(const DevState &d);
 int grid_eval(const DevState &d);

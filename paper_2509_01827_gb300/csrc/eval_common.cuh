@@ -68,47 +68,33 @@ __device__ __forceinline__ bool is_tip_edge(const DevState &d, int e, int k0) {
   return (info & 3) == kf || ((info >> 2) & 3) == kf;
 }
 
-// Reference vector X_N2 - X_N1 of local edge k0 and the unit normal of the
-// candidate segment from edge point k0 to edge point k, oriented along it.
-__device__ __forceinline__ void candidate_normal(const Geo &g, int k0, int k, double &nx,
-                                                 double &ny) {
-  double DX = (xi_n((k0 + 1) & 3) - xi_n(k0)) * (0.5 * g.hx);
-  double DY = (eta_n((k0 + 1) & 3) - eta_n(k0)) * (0.5 * g.hy);
-  double x0 = (xi_g(k0) + 1.0) * (0.5 * g.hx), y0 = (eta_g(k0) + 1.0) * (0.5 * g.hy);
-  double xk = (xi_g(k) + 1.0) * (0.5 * g.hx), yk = (eta_g(k) + 1.0) * (0.5 * g.hy);
-  double sx = xk - x0, sy = yk - y0;
-  double rx = -sy, ry = sx;
-  if (rx * DX + ry * DY < 0.0) { rx = -rx; ry = -ry; }
-  double len = sqrt(sx * sx + sy * sy);
-  nx = rx / len;
-  ny = ry / len;
-}
-
 // G of the three candidate paths of surface point (e, k0); G[k0] = -1.
 // delta_d = (u_N2 - u_N1) H(|x_N2 - x_N1| > |X_N2 - X_N1|), G = delta_d.(sigma n)/2.
+// eval_G64_k: the candidate of local edge k alone (-1 for k = k0).  The
+// reference vectors and unit normals are the mesh's (Geo: formed once, their
+// square root and divisions with it).
 template <class UA>
-__device__ void eval_G64(const DevState &d, const UA &U, int e, int k0, double G[4]) {
+__device__ __forceinline__ double eval_G64_k(const DevState &d, const UA &U, int e, int k0, int k) {
   const Geo &g = d.g;
+  if (k == k0) return -1.0;
   int N1 = elem_node(g, e, k0), N2 = elem_node(g, e, (k0 + 1) & 3);
-  double DX = (xi_n((k0 + 1) & 3) - xi_n(k0)) * (0.5 * g.hx);
-  double DY = (eta_n((k0 + 1) & 3) - eta_n(k0)) * (0.5 * g.hy);
   double dux = U.ux(N2) - U.ux(N1);
   double duy = U.uy(N2) - U.uy(N1);
-  double dx = DX + dux, dy = DY + duy;
+  double dx = g.DX[k0] + dux, dy = g.DY[k0] + duy;
   double cur2 = dx * dx + dy * dy;
-  double ref2 = DX * DX + DY * DY;
-  double H = cur2 > ref2 ? 1.0 : 0.0;
+  double H = cur2 > g.ref2[k0] ? 1.0 : 0.0;
   double ddx = dux * H, ddy = duy * H;
-  for (int k = 0; k < 4; ++k) {
-    if (k == k0) { G[k] = -1.0; continue; }
-    double nx, ny;
-    candidate_normal(g, k0, k, nx, ny);
-    double s[3];
-    used_stress(d, U, e, k, s);
-    double tx = s[0] * nx + s[2] * ny;
-    double ty = s[2] * nx + s[1] * ny;
-    G[k] = 0.5 * (ddx * tx + ddy * ty);
-  }
+  double s[3];
+  used_stress(d, U, e, k, s);
+  const double nx = g.cnx[k0][k], ny = g.cny[k0][k];
+  double tx = s[0] * nx + s[2] * ny;
+  double ty = s[2] * nx + s[1] * ny;
+  return 0.5 * (ddx * tx + ddy * ty);
+}
+
+template <class UA>
+__device__ void eval_G64(const DevState &d, const UA &U, int e, int k0, double G[4]) {
+  for (int k = 0; k < 4; ++k) G[k] = eval_G64_k(d, U, e, k0, k);
 }
 
 // Q4 cracking conditions with the split ratio gamma (Sec. 2.2).

@@ -3,7 +3,7 @@
 // One step of the explicit MCT-2D-CEM (see include/cem.h):
 //   k_pieces64   internal force of every split-element piece (Eq. 6 with the
 //                piece area), own strain at each edge point (smoothing off);
-//   k_main64     one CTA per 32x8 tile of real nodes: ES-FEM edge strains
+//   k_main64     one CTA per tile of real nodes: ES-FEM edge strains
 //                (Eqs. 1, 2, 4) of the intact elements around the tile,
 //                stresses, the node gather of intact and piece forces in
 //                increasing element id, and the central-difference update
@@ -24,11 +24,7 @@ namespace cem {
 
 namespace {
 
-constexpr int TX = 32, TY = 8, NT = TX * TY;
-constexpr int UXn = TX + 4, UYn = TY + 4;  // nodes [i0-2, i0+TX+1] x [j0-2, j0+TY+1]
-constexpr int EXn = TX + 3, EYn = TY + 3;  // elements [i0-2, i0+TX] x [j0-2, j0+TY]
-constexpr int HXn = TX + 1, HYn = TY + 2;  // horizontal edges [i0-1, i0+TX) x [j0-1, j0+TY]
-constexpr int VXn = TX + 2, VYn = TY + 1;  // vertical edges [i0-1, i0+TX] x [j0-1, j0+TY)
+constexpr int NT = 256;  // threads of a node-update CTA (its tile shape: tile64_shape)
 
 __device__ __forceinline__ double dot3(const double e[3], const double s[3]) {
   return e[0] * s[0] + e[1] * s[1] + e[2] * s[2];
@@ -55,53 +51,62 @@ __device__ void block_sum2(double a, double b, double *out) {
   }
 }
 
-// Central-difference update of one node (real or phantom); mirrors the
-// oracle's expression order exactly.
-struct NodeOut {
-  double ke;
-};
-
-__device__ __forceinline__ double update_node(const DevState &d, int N, int cur, bool first,
-                                              double fintx, double finty, uint8_t nf,
-                                              double lamN, double lamD) {
-  const double dt = d.mat.dt;
-  const double dtv = first ? 0.5 * dt : dt;
-  bool loaded = (nf & NF_LOADED) != 0;
-  double fex = loaded ? lamN * d.Fx[N] : 0.0;
-  double fey = loaded ? lamN * d.Fy[N] : 0.0;
-  double minv = d.minv[N];
-  double ax = (fex - fintx) * minv;
-  double ay = (fey - finty) * minv;
-  double vxo = d.vx[N], vyo = d.vy[N];
-  double vxn = vxo + dtv * ax;
-  double vyn = vyo + dtv * ay;
-  if (nf & NF_DIRX) vxn = lamD * d.Vx[N];
-  if (nf & NF_DIRY) vyn = lamD * d.Vy[N];
-  double vbx = first ? vxo : 0.5 * (vxo + vxn);
-  double vby = first ? vyo : 0.5 * (vyo + vyn);
-  if (loaded) d.Wn[N] = d.Wn[N] + dt * (fex * vbx + fey * vby);
-  if (nf & (NF_DIRX | NF_DIRY)) {
-    double m = d.m[N];
-    double Rx = m * ((vxn - vxo) / dtv) - (fex - fintx);
-    double Ry = m * ((vyn - vyo) / dtv) - (fey - finty);
-    double w = 0.0;
-    if (nf & NF_DIRX) w = w + Rx * vbx;
-    if (nf & NF_DIRY) w = w + Ry * vby;
-    d.Wd[N] = d.Wd[N] + dt * w;
-  }
-  d.vx[N] = vxn;
-  d.vy[N] = vyn;
-  // a non-finite velocity (NaN or Inf) is reported through the status word
-  if (!(fabs(vxn) <= DBL_MAX) || !(fabs(vyn) <= DBL_MAX)) atomicOr(&d.cnt->status, STAT_NONFINITE);
-  d.ux[cur ^ 1][N] = d.ux[cur][N] + dt * vxn;
-  d.uy[cur ^ 1][N] = d.uy[cur][N] + dt * vyn;
-  return 0.5 * (d.m[N] * (vbx * vbx + vby * vby));
+__device__ __forceinline__ bool finite64(double x) {
+  return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;  // an integer test: FP64 compares share the FP64 pipe
 }
 
 __device__ __forceinline__ void load_factors(const DevState &d, double &lamN, double &lamD) {
   int idx = d.cnt->step - d.cnt->lam_base;
   lamN = d.lamN[idx];
   lamD = d.lamD[idx];
+}
+
+// Central-difference update of one node (real or phantom); mirrors the
+// oracle's expression order exactly.  Returns its kinetic energy on record
+// steps; the mean velocity that needs is formed only there and at nodes with
+// a load or a prescribed velocity.
+__device__ __forceinline__ double update_node(const DevState &d, int N, int cur, bool first,
+                                              double fintx, double finty, uint8_t nf, bool energy) {
+  const double dt = d.mat.dt;
+  const double dtv = first ? 0.5 * dt : dt;
+  double fex = 0.0, fey = 0.0, lamN = 0.0, lamD = 0.0;
+  if (nf) load_factors(d, lamN, lamD);
+  const bool loaded = (nf & NF_LOADED) != 0;
+  if (loaded) {
+    fex = lamN * d.Fx[N];
+    fey = lamN * d.Fy[N];
+  }
+  double minv = d.minv[N];
+  double ax = (loaded ? fex - fintx : -fintx) * minv;
+  double ay = (loaded ? fey - finty : -finty) * minv;
+  double vxo = d.vx[N], vyo = d.vy[N];
+  double vxn = vxo + dtv * ax;
+  double vyn = vyo + dtv * ay;
+  if (nf & NF_DIRX) vxn = lamD * d.Vx[N];
+  if (nf & NF_DIRY) vyn = lamD * d.Vy[N];
+  double ke = 0.0;
+  if (nf || energy) {
+    double vbx = first ? vxo : 0.5 * (vxo + vxn);
+    double vby = first ? vyo : 0.5 * (vyo + vyn);
+    if (loaded) d.Wn[N] = d.Wn[N] + dt * (fex * vbx + fey * vby);
+    if (nf & (NF_DIRX | NF_DIRY)) {
+      double m = d.m[N];
+      double Rx = m * ((vxn - vxo) / dtv) - (fex - fintx);
+      double Ry = m * ((vyn - vyo) / dtv) - (fey - finty);
+      double w = 0.0;
+      if (nf & NF_DIRX) w = w + Rx * vbx;
+      if (nf & NF_DIRY) w = w + Ry * vby;
+      d.Wd[N] = d.Wd[N] + dt * w;
+    }
+    if (energy) ke = 0.5 * (d.m[N] * (vbx * vbx + vby * vby));
+  }
+  d.vx[N] = vxn;
+  d.vy[N] = vyn;
+  // a non-finite velocity (NaN or Inf) is reported through the status word
+  if (!finite64(vxn) || !finite64(vyn)) atomicOr(&d.cnt->status, STAT_NONFINITE);
+  d.ux[cur ^ 1][N] = d.ux[cur][N] + dt * vxn;
+  d.uy[cur ^ 1][N] = d.uy[cur][N] + dt * vyn;
+  return ke;
 }
 
 // ------------------------------------------------------------------ pieces
@@ -146,158 +151,266 @@ __global__ void k_pieces64(DevState d, int cur, int energy, int part_off) {
 }
 
 // -------------------------------------------------------------- main tile
-__device__ __forceinline__ void main64_tile(const DevState &d, VBlk vb, int cur, int first,
-                                            int energy) {
-  __shared__ double sux[UYn][UXn], suy[UYn][UXn];
-  __shared__ uint8_t sst[EYn][EXn];
-  // stress (3) and eps.sigma (1) used by the element below/left (lo) and
-  // above/right (hi) of each edge
-  __shared__ double hlo[HYn][HXn][4], hhi[HYn][HXn][4];
-  __shared__ double vlo[VYn][VXn][4], vhi[VYn][VXn][4];
+// The node update is bound by the FP64 pipe (about 0.5 T instructions/s on
+// the whole GPU, 1/74 of FP32), so it is built to issue as few FP64
+// instructions as the definition allows while keeping every rounding:
+//   - each node's products with 1/h are formed once and every difference and
+//     sum that two edges, two sides or two elements share is formed once;
+//   - with both sides of an edge intact the tangential derivative is the same
+//     on both sides, and 0.5 a + 0.5 b is formed as 0.5 (a + b), the halving
+//     and the doubling 1/(2h) -> 1/h by an exponent step in integer
+//     registers.  These are exact unless a value is subnormal or close to
+//     overflow: a CTA whose products leave [2^-800, 2^800] (other than zero)
+//     takes the plain formulas instead (a CTA-wide vote);
+//   - the bracketed pairs of Eq. 6's sum are formed per edge, up to a sign,
+//     not per element and node.
+// About 120 instead of 309 FP64 instructions per node: 2683 -> 1156 us on the
+// 2048 x 2048 plate, 58 -> 26 us on 400 x 160, 36 -> 10 us on 100 x 40.
+// The tile shape follows the mesh (tile64_shape): a small mesh is cut finer so
+// that every SM gets a share.
+struct Tile64 {
+  int tx, ty;    // nodes [i0, i0+tx) x [j0, j0+ty)
+  int nw, nh;    // nodes [i0-2, i0+tx+1] x [j0-2, j0+ty+1]
+  int ew, eh;    // elements [i0-2, i0+tx] x [j0-2, j0+ty]
+  int hw, hh;    // horizontal edges [i0-1, i0+tx) x [j0-1, j0+ty]
+  int vw, vh;    // vertical edges [i0-1, i0+tx] x [j0-1, j0+ty)
+  __host__ __device__ Tile64(int tx_, int ty_)
+      : tx(tx_), ty(ty_), nw(tx_ + 4), nh(ty_ + 4), ew(tx_ + 3), eh(ty_ + 3), hw(tx_ + 1),
+        hh(ty_ + 2), vw(tx_ + 2), vh(ty_ + 1) {}
+  __host__ __device__ int nodes() const { return nw * nh; }
+  __host__ __device__ int elems() const { return ew * eh; }
+  __host__ __device__ int hedges() const { return hw * hh; }
+  __host__ __device__ int vedges() const { return vw * vh; }
+  // node products (4), element sums (4), edge terms (6) and, on record steps,
+  // eps.sigma; then the element states
+  __host__ __device__ size_t bytes(bool energy) const {
+    return 8 * (4 * (size_t)nodes() + 4 * (size_t)elems() +
+                (energy ? 7 : 6) * (size_t)(hedges() + vedges())) + elems();
+  }
+};
 
+// FP64 instructions of one tile, in warp instructions
+inline double tile64_cost(const Tile64 &t) {
+  auto w = [](int n) { return (double)((n + 31) / 32); };
+  return 4 * w(t.nodes()) + 12 * w(t.elems()) + 21 * w(t.hedges() + t.vedges()) +
+         52 * w(t.tx * t.ty);
+}
+
+// x / 2 and 2 x of a normal number or zero, by its exponent field
+__device__ __forceinline__ double half64(double x) {
+  const int h = __double2hiint(x);
+  return __hiloint2double(h - ((h & 0x7ff00000) ? 0x00100000 : 0), __double2loint(x));
+}
+__device__ __forceinline__ double twice64(double x) {
+  const int h = __double2hiint(x);
+  return __hiloint2double(h + ((h & 0x7ff00000) ? 0x00100000 : 0), __double2loint(x));
+}
+// zero, or within [2^-800, 2^800]
+__device__ __forceinline__ bool mid_range64(double x) {
+  const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7ff;
+  return e - (1023u - 800u) <= 1600u || (e == 0 && ((__double2hiint(x) << 1) | __double2loint(x)) == 0);
+}
+
+__device__ __forceinline__ void main64_tile(const DevState &d, VBlk vb, int cur, int first,
+                                            int energy, double *sm) {
   const Geo &g = d.g;
-  const int i0 = vb.x * TX, j0 = vb.y * TY;
+  const Tile64 T(d.t64x, d.t64y);
+  const int i0 = vb.x * T.tx, j0 = vb.y * T.ty;
   const int tid = threadIdx.x;
   const double *uxc = d.ux[cur], *uyc = d.uy[cur];
+  const int nn = T.nodes(), ne = T.elems(), nhe = T.hedges(), nve = T.vedges();
+  // node products u/(2hx), v/(2hx), u/(2hy), v/(2hy) (u, v themselves on the plain path)
+  double *pa = sm, *pb = pa + nn;
+  const bool square = g.rxh == g.ryh;
+  double *pc = square ? pa : pb + nn, *pd = square ? pb : pc + nn;
+  // element sums: half the normal derivatives that enter exx (vertical edges)
+  // and eyy (horizontal edges), and the whole ones that enter gxy
+  double *eX = sm + 4 * nn, *eN = eX + ne, *eXv = eN + ne, *eNu = eXv + ne;
+  // edge terms, planes of nhe (nve) values: see edge_terms
+  const int planes = energy ? 7 : 6;
+  double *H = eNu + ne, *V = H + planes * nhe;
+  uint8_t *sst = reinterpret_cast<uint8_t *>(V + planes * nve);
 
-  for (int q = tid; q < UXn * UYn; q += NT) {
-    int li = q % UXn, lj = q / UXn, i = i0 - 2 + li, j = j0 - 2 + lj;
+  int ok = 1;
+  for (int q = tid; q < nn; q += NT) {
+    const int li = q % T.nw, lj = q / T.nw, i = i0 - 2 + li, j = j0 - 2 + lj;
     double a = 0.0, b = 0.0;
     if (i >= 0 && j >= 0 && i <= g.nx && j <= g.ny) {
-      int N = j * (g.nx + 1) + i;
+      const int N = j * (g.nx + 1) + i;
       a = uxc[N];
       b = uyc[N];
     }
-    sux[lj][li] = a;
-    suy[lj][li] = b;
+    const double a1 = g.rxh * a, b1 = g.rxh * b;
+    pa[q] = a1;
+    pb[q] = b1;
+    ok &= (int)(mid_range64(a1) && mid_range64(b1));
+    if (!square) {
+      const double a2 = g.ryh * a, b2 = g.ryh * b;
+      pc[q] = a2;
+      pd[q] = b2;
+      ok &= (int)(mid_range64(a2) && mid_range64(b2));
+    }
   }
-  for (int q = tid; q < EXn * EYn; q += NT) {
-    int li = q % EXn, lj = q / EXn, i = i0 - 2 + li, j = j0 - 2 + lj;
+  for (int q = tid; q < ne; q += NT) {
+    const int li = q % T.ew, lj = q / T.ew, i = i0 - 2 + li, j = j0 - 2 + lj;
     uint8_t s = ST_OUT;
     if (i >= 0 && j >= 0 && i < g.nx && j < g.ny) s = d.estate[j * g.nx + i];
-    sst[lj][li] = s;
+    sst[q] = s;
   }
-  __syncthreads();
+  ok = __syncthreads_and(ok);
 
-  // element (ei, ej) -> its four nodes' displacements from shared memory
-  auto gather = [&](int ei, int ej, double u[4], double v[4]) {
-    int li = ei - (i0 - 2), lj = ej - (j0 - 2);
-    u[0] = sux[lj][li];         v[0] = suy[lj][li];
-    u[1] = sux[lj][li + 1];     v[1] = suy[lj][li + 1];
-    u[2] = sux[lj + 1][li + 1]; v[2] = suy[lj + 1][li + 1];
-    u[3] = sux[lj + 1][li];     v[3] = suy[lj + 1][li];
-  };
-  auto est = [&](int ei, int ej) -> int { return sst[ej - (j0 - 2)][ei - (i0 - 2)]; };
-
-  // horizontal edges: below element (i, j-1) at its edge 2, above (i, j) at edge 0
-  for (int q = tid; q < HXn * HYn; q += NT) {
-    int li = q % HXn, lj = q / HXn, i = i0 - 1 + li, j = j0 - 1 + lj;
-    int sb = est(i, j - 1), sa = est(i, j);
-    double eb[3], ea[3], u[4], v[4];
-    if (sb == ST_INTACT) { gather(i, j - 1, u, v); strain64<2>(g, u, v, eb); }
-    if (sa == ST_INTACT) { gather(i, j, u, v); strain64<0>(g, u, v, ea); }
-    if (sb == ST_INTACT && sa == ST_INTACT) {
-      double e[3], s[3];
-      for (int c = 0; c < 3; ++c) e[c] = 0.5 * eb[c] + 0.5 * ea[c];
-      stress64(d.mat, e, s);
-      double dd = dot3(e, s);
-      for (int c = 0; c < 3; ++c) { hlo[lj][li][c] = s[c]; hhi[lj][li][c] = s[c]; }
-      hlo[lj][li][3] = dd;
-      hhi[lj][li][3] = dd;
-    } else {
-      if (sb == ST_INTACT) {
-        double s[3];
-        stress64(d.mat, eb, s);
-        for (int c = 0; c < 3; ++c) hlo[lj][li][c] = s[c];
-        hlo[lj][li][3] = dot3(eb, s);
-      }
-      if (sa == ST_INTACT) {
-        double s[3];
-        stress64(d.mat, ea, s);
-        for (int c = 0; c < 3; ++c) hhi[lj][li][c] = s[c];
-        hhi[lj][li][3] = dot3(ea, s);
-      }
+  if (ok) {
+    for (int q = tid; q < ne; q += NT) {
+      if (sst[q] != ST_INTACT) continue;
+      const int li = q % T.ew, lj = q / T.ew;
+      const int n0 = lj * T.nw + li, n1 = n0 + 1, n3 = n0 + T.nw, n2 = n3 + 1;
+      eX[q] = half64(((pa[n1] - pa[n0]) + pa[n2]) - pa[n3]);
+      eXv[q] = ((pb[n1] - pb[n0]) + pb[n2]) - pb[n3];
+      eN[q] = half64((pd[n2] - (pd[n0] + pd[n1])) + pd[n3]);
+      eNu[q] = (pc[n2] - (pc[n0] + pc[n1])) + pc[n3];
     }
-  }
-  // vertical edges: left element (i-1, j) at its edge 1, right (i, j) at edge 3
-  for (int q = tid; q < VXn * VYn; q += NT) {
-    int li = q % VXn, lj = q / VXn, i = i0 - 1 + li, j = j0 - 1 + lj;
-    int sl = est(i - 1, j), sr = est(i, j);
-    double el[3], er[3], u[4], v[4];
-    if (sl == ST_INTACT) { gather(i - 1, j, u, v); strain64<1>(g, u, v, el); }
-    if (sr == ST_INTACT) { gather(i, j, u, v); strain64<3>(g, u, v, er); }
-    if (sl == ST_INTACT && sr == ST_INTACT) {
-      double e[3], s[3];
-      for (int c = 0; c < 3; ++c) e[c] = 0.5 * el[c] + 0.5 * er[c];
-      stress64(d.mat, e, s);
-      double dd = dot3(e, s);
-      for (int c = 0; c < 3; ++c) { vlo[lj][li][c] = s[c]; vhi[lj][li][c] = s[c]; }
-      vlo[lj][li][3] = dd;
-      vhi[lj][li][3] = dd;
-    } else {
-      if (sl == ST_INTACT) {
-        double s[3];
-        stress64(d.mat, el, s);
-        for (int c = 0; c < 3; ++c) vlo[lj][li][c] = s[c];
-        vlo[lj][li][3] = dot3(el, s);
-      }
-      if (sr == ST_INTACT) {
-        double s[3];
-        stress64(d.mat, er, s);
-        for (int c = 0; c < 3; ++c) vhi[lj][li][c] = s[c];
-        vhi[lj][li][3] = dot3(er, s);
-      }
+  } else {
+    // plain path: the displacements themselves
+    pc = pa;
+    pd = pb;
+    for (int q = tid; q < nn; q += NT) {
+      const int li = q % T.nw, lj = q / T.nw, i = i0 - 2 + li, j = j0 - 2 + lj;
+      const bool in = i >= 0 && j >= 0 && i <= g.nx && j <= g.ny;
+      const int N = j * (g.nx + 1) + i;
+      pa[q] = in ? uxc[N] : 0.0;
+      pb[q] = in ? uyc[N] : 0.0;
     }
   }
   __syncthreads();
 
-  // stresses used by intact element (ei, ej) at its edges 0..3
-  auto elem_sig = [&](int ei, int ej, double s[4][3]) {
-    int hi_ = ei - (i0 - 1), hj = ej - (j0 - 1);
-    for (int c = 0; c < 3; ++c) {
-      s[0][c] = hhi[hj][hi_][c];      // bottom edge h(ei, ej): element above it
-      s[1][c] = vlo[hj][hi_ + 1][c];  // right edge v(ei+1, ej): element left of it
-      s[2][c] = hlo[hj + 1][hi_][c];  // top edge h(ei, ej+1): element below it
-      s[3][c] = vhi[hj][hi_][c];      // left edge v(ei, ej): element right of it
+  // every edge of the tile: the strain its intact sides use (with both intact
+  // the average of theirs), the stress, and the terms the node sums take
+  // from it.  Both sides take the same terms, so one set per edge is kept.
+  for (int q = tid; q < nhe + nve; q += NT) {
+    const bool hor = q < nhe;
+    const int p = hor ? q : q - nhe, w = hor ? T.hw : T.vw;
+    const int li = p % w, lj = p / w;
+    // the elements below and above (left and right) of the edge, the node at its start
+    const int eb = hor ? lj * T.ew + li + 1 : (lj + 1) * T.ew + li;
+    const int ea = hor ? eb + T.ew : eb + 1;
+    const int n0 = (lj + 1) * T.nw + li + 1;
+    const bool ib = sst[eb] == ST_INTACT, ia = sst[ea] == ST_INTACT;
+    if (!ib && !ia) continue;
+    double e[3];
+    if (ok) {
+      const int es = ib ? eb : ea;  // the (or one) intact side
+      if (hor) {
+        e[0] = twice64(pa[n0 + 1] - pa[n0]);
+        const double t = twice64(pb[n0 + 1] - pb[n0]);
+        if (ib && ia) {
+          e[1] = eN[eb] + eN[ea];
+          e[2] = half64((eNu[eb] + t) + (eNu[ea] + t));
+        } else {
+          e[1] = twice64(eN[es]);
+          e[2] = eNu[es] + t;
+        }
+      } else {
+        e[1] = twice64(pd[n0 + T.nw] - pd[n0]);
+        const double t = twice64(pc[n0 + T.nw] - pc[n0]);
+        if (ib && ia) {
+          e[0] = eX[eb] + eX[ea];
+          e[2] = half64((t + eXv[eb]) + (t + eXv[ea]));
+        } else {
+          e[0] = twice64(eX[es]);
+          e[2] = t + eXv[es];
+        }
+      }
+    } else {
+      double eB[3], eA[3], u[4], v[4];
+      auto gather = [&](int el) {
+        const int m0 = (el / T.ew) * T.nw + el % T.ew;
+        u[0] = pa[m0];            v[0] = pb[m0];
+        u[1] = pa[m0 + 1];        v[1] = pb[m0 + 1];
+        u[2] = pa[m0 + T.nw + 1]; v[2] = pb[m0 + T.nw + 1];
+        u[3] = pa[m0 + T.nw];     v[3] = pb[m0 + T.nw];
+      };
+      if (ib) {
+        gather(eb);
+        if (hor) strain64<2>(g, u, v, eB); else strain64<1>(g, u, v, eB);
+      }
+      if (ia) {
+        gather(ea);
+        if (hor) strain64<0>(g, u, v, eA); else strain64<3>(g, u, v, eA);
+      }
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        e[c] = ib && ia ? 0.5 * eB[c] + 0.5 * eA[c] : ib ? eB[c] : eA[c];
     }
-  };
+    double s[3];
+    stress64(d.mat, e, s);
+    // horizontal: x sum 1/hx sxx (k), 1/(2hy) sxy (m); y sum 1/(2hy) syy (l), 1/hx sxy (n)
+    // vertical:   x sum 1/(2hx) sxx (k), 1/hy sxy (m); y sum 1/hy syy (l), 1/(2hx) sxy (n)
+    double *o = hor ? H + q : V + p;
+    const int st = hor ? nhe : nve;
+    const double rk = hor ? g.rx : g.rxh, rm = hor ? g.ryh : g.ry;
+    const double k = rk * s[0], m = rm * s[2], l = rm * s[1], n = rk * s[2];
+    o[0] = k + m;
+    o[st] = k - m;
+    o[2 * st] = l + n;
+    o[3 * st] = n - l;
+    o[4 * st] = hor ? m : k;
+    o[5 * st] = hor ? l : n;
+    if (energy) o[6 * st] = dot3(e, s);
+  }
+  __syncthreads();
 
-  const int tx = tid % TX, ty = tid / TX;
-  const int i = i0 + tx, j = j0 + ty;
   double ke = 0.0, se = 0.0;
-  if (i <= g.nx && j <= g.ny) {
+  const double qA = g.A * 0.25;
+  for (int q = tid; q < T.tx * T.ty; q += NT) {
+    const int tx = q % T.tx, ty = q / T.tx;
+    const int i = i0 + tx, j = j0 + ty;
+    if (i > g.nx || j > g.ny) continue;
     const int N = j * (g.nx + 1) + i;
-    const double qA = g.A * 0.25;
     double fx = 0.0, fy = 0.0;
     // adjacent elements in increasing id: (i-1,j-1) a=2, (i,j-1) a=3, (i-1,j) a=1, (i,j) a=0
-    const int ei[4] = {i - 1, i, i - 1, i}, ej[4] = {j - 1, j - 1, j, j}, la[4] = {2, 3, 1, 0};
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      int s = est(ei[q], ej[q]);
-      if (s == ST_INTACT) {
-        double sg[4][3], ax, ay;
-        elem_sig(ei[q], ej[q], sg);
-        node_force64_rt(g, la[q], sg, qA, ax, ay);
-        fx = fx + ax;
-        fy = fy + ay;
-      } else if (s == ST_CRACKED) {
-        int e = ej[q] * g.nx + ei[q];
-        int c = d.crack_of[e];
-        int side = (d.ck_info[c] >> (4 + la[q])) & 1;
-        fx = fx + d.pf[c * 16 + side * 8 + 2 * la[q]];
-        fy = fy + d.pf[c * 16 + side * 8 + 2 * la[q] + 1];
+    for (int r = 0; r < 4; ++r) {
+      const int di = (r & 1) - 1, dj = (r >> 1) - 1;
+      constexpr int kLocal[4] = {2, 3, 1, 0};
+      const int a = kLocal[r];
+      const int st = sst[(ty + 2 + dj) * T.ew + tx + 2 + di];
+      if (st == ST_INTACT) {
+        // bottom, top, left and right edge of the element
+        const double *hb = H + (ty + 1 + dj) * T.hw + tx + 1 + di, *ht = hb + T.hw;
+        const double *vl = V + (ty + 1 + dj) * T.vw + tx + 1 + di, *vr = vl + 1;
+        double sx, sy;
+        if (a == 2) {
+          sx = ((hb[4 * nhe] + vr[0]) + ht[0]) + vl[4 * nve];
+          sy = ((hb[5 * nhe] + vr[2 * nve]) + ht[2 * nhe]) + vl[5 * nve];
+        } else if (a == 3) {
+          sx = ((hb[4 * nhe] - vr[4 * nve]) - ht[nhe]) - vl[nve];
+          sy = ((hb[5 * nhe] - vr[5 * nve]) - ht[3 * nhe]) - vl[3 * nve];
+        } else if (a == 1) {
+          sx = ((hb[nhe] + vr[nve]) - ht[4 * nhe]) + vl[4 * nve];
+          sy = ((hb[3 * nhe] + vr[3 * nve]) - ht[5 * nhe]) + vl[5 * nve];
+        } else {
+          sx = -(((hb[0] + vr[4 * nve]) + ht[4 * nhe]) + vl[0]);
+          sy = -(((hb[2 * nhe] + vr[5 * nve]) + ht[5 * nhe]) + vl[2 * nve]);
+        }
+        fx = fx + sx * qA;
+        fy = fy + sy * qA;
+      } else if (st == ST_CRACKED) {
+        const int e = (j + dj) * g.nx + i + di;
+        const int c = d.crack_of[e];
+        const int side = (d.ck_info[c] >> (4 + a)) & 1;
+        fx = fx + d.pf[c * 16 + side * 8 + 2 * a];
+        fy = fy + d.pf[c * 16 + side * 8 + 2 * a + 1];
       }
     }
-    double lamN, lamD;
-    load_factors(d, lamN, lamD);
-    ke = update_node(d, N, cur, first != 0, fx, fy, d.nflag[N], lamN, lamD);
-    if (energy && i < g.nx && j < g.ny && est(i, j) == ST_INTACT) {
-      int hi_ = i - (i0 - 1), hj = j - (j0 - 1);
-      double dk[4] = {hhi[hj][hi_][3], vlo[hj][hi_ + 1][3], hlo[hj + 1][hi_][3], vhi[hj][hi_][3]};
+    ke += update_node(d, N, cur, first != 0, fx, fy, d.nflag[N], energy != 0);
+    if (energy && i < g.nx && j < g.ny && sst[(ty + 2) * T.ew + tx + 2] == ST_INTACT) {
+      const double *hb = H + 6 * nhe + (ty + 1) * T.hw + tx + 1, *ht = hb + T.hw;
+      const double *vl = V + 6 * nve + (ty + 1) * T.vw + tx + 1, *vr = vl + 1;
+      const double dk[4] = {*hb, *vr, *ht, *vl};
       double acc = 0.0;
 #pragma unroll
       for (int k = 0; k < 4; ++k) acc = acc + 0.5 * (qA * dk[k]);
-      se = acc;
+      se += acc;
     }
   }
   if (energy) {
@@ -307,7 +420,8 @@ __device__ __forceinline__ void main64_tile(const DevState &d, VBlk vb, int cur,
 }
 
 __global__ void __launch_bounds__(NT) k_main64(DevState d, int cur, int first, int energy) {
-  main64_tile(d, hw_vblk(), cur, first, energy);
+  extern __shared__ double sm64[];
+  main64_tile(d, hw_vblk(), cur, first, energy, sm64);
 }
 
 // ---------------------------------------------------------------- phantoms
@@ -315,8 +429,6 @@ __device__ __forceinline__ void phantom64(const DevState &d, VBlk vb, int cur, i
                                           int energy, int part_off) {
   const int n = d.cnt->n_ph;
   double ke = 0.0;
-  double lamN, lamD;
-  load_factors(d, lamN, lamD);
   for (int t = vb.x * blockDim.x + threadIdx.x; t < n; t += vb.gx * blockDim.x) {
     int N = d.g.nn + t;
     // users' piece-force indices in increasing element id, -1 unused
@@ -329,7 +441,7 @@ __device__ __forceinline__ void phantom64(const DevState &d, VBlk vb, int cur, i
       fx = fx + d.pf[us[q]];
       fy = fy + d.pf[us[q] + 1];
     }
-    ke += update_node(d, N, cur, first != 0, fx, fy, 0, lamN, lamD);
+    ke += update_node(d, N, cur, first != 0, fx, fy, 0, energy != 0);
   }
   if (energy) block_sum2(ke, 0.0, d.e_part + 2 * (part_off + vb.x));
 }
@@ -338,42 +450,56 @@ __global__ void k_phantom64(DevState d, int cur, int first, int energy, int part
   phantom64(d, hw_vblk(), cur, first, energy, part_off);
 }
 
+// Surface evaluation, 32 points per block of four warps: warp k forms the
+// candidate of local edge k (every lane of a warp then runs the same
+// formulas), warp 0 applies the rule.  Bound by the FP64 pipe of the SMs that
+// hold points, so few points per SM: a block of 256 threads, one point each,
+// took 36 us for 380 points (two SMs busy) on the 100 x 40 plate, this 7 us;
+// 43 and 13 us for the 9,008 points of the 2048 x 2048 plate.
+constexpr int kEvalPts = 32, kEvalTB = 4 * kEvalPts;
+
 __device__ __forceinline__ void eval64(const DevState &d, VBlk vb, int cur) {
+  __shared__ double sG[4][kEvalPts];
   const int n = d.cnt->n_S;
+  const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
   const U64 U{d.ux[cur], d.uy[cur]};
-  // whole warps iterate together so that the ballot sees every lane
-  for (int base = vb.x * blockDim.x; base < n; base += vb.gx * blockDim.x) {
-    int i = base + threadIdx.x;
-    bool has = false;
-    int key = 0, edge = 0, kk = -1;
-    double Gk = 0.0;
-    if (i < n) {
-      edge = d.S[i];
-      if (edge >= 0) {
-        key = d.S_info[i];
-        int e = key >> 2, k0 = key & 3;
-        if (d.mat.scope != 2 || is_tip_edge(d, e, k0)) {
-          double G[4];
-          eval_G64(d, U, e, k0, G);
-          double gm = -1.0;
-          for (int k = 0; k < 4; ++k) gm = fmax(gm, G[k]);
-          d.S_G[i] = gm;
-          kk = q4_rule(d, e, k0, G);
-          if (kk >= 0) { has = true; Gk = G[kk]; }
-        }
-      }
+  for (int base = vb.x * kEvalPts; base < n; base += vb.gx * kEvalPts) {
+    const int i = base + lane;
+    int key = 0, edge = -1;
+    if (i < n) edge = d.S[i];
+    bool live = edge >= 0;
+    if (live) {
+      key = d.S_info[i];
+      live = d.mat.scope != 2 || is_tip_edge(d, key >> 2, key & 3);
     }
-    append_proposal(d, has, key, edge, kk, Gk);
+    if (live) sG[k][lane] = eval_G64_k(d, U, key >> 2, key & 3, k);
+    __syncthreads();
+    if (k == 0) {
+      bool has = false;
+      int kk = -1;
+      double Gk = 0.0;
+      if (live) {
+        const double G[4] = {sG[0][lane], sG[1][lane], sG[2][lane], sG[3][lane]};
+        double gm = -1.0;
+        for (int c = 0; c < 4; ++c) gm = fmax(gm, G[c]);
+        d.S_G[i] = gm;
+        kk = q4_rule(d, key >> 2, key & 3, G);
+        if (kk >= 0) { has = true; Gk = G[kk]; }
+      }
+      append_proposal(d, has, key, edge, kk, Gk);
+    }
+    __syncthreads();
   }
 }
 
-__global__ void k_eval64(DevState d, int cur) { eval64(d, hw_vblk(), cur); }
+__global__ void __launch_bounds__(kEvalTB) k_eval64(DevState d, int cur) { eval64(d, hw_vblk(), cur); }
 
 // ---------------------------------------------------------------- batched
 // One launch per kernel kind for every member of a batch (persistent grids
 // walking the work lists; 1-D items are (member, block, energy-partial
 // offset, member's grid size)).
 __global__ void __launch_bounds__(NT) k_main64_batch(BatchDev b, int first, int energy) {
+  extern __shared__ double sm64[];
   __shared__ DevState sd;
   int held = -1, w0, w1;
   const int n = *b.bstep;
@@ -382,7 +508,7 @@ __global__ void __launch_bounds__(NT) k_main64_batch(BatchDev b, int first, int 
     const int4 it = b.w_main[w];
     stage_member(b.ds, it.x, sd, held);
     if (!member_active(sd, n)) continue;
-    main64_tile(sd, item_vblk(it), member_cur(sd, n), first, energy);
+    main64_tile(sd, item_vblk(it), member_cur(sd, n), first, energy, sm64);
     __syncthreads();
   }
 }
@@ -415,7 +541,7 @@ __global__ void k_phantom64_batch(BatchDev b, int first, int energy) {
   }
 }
 
-__global__ void k_eval64_batch(BatchDev b) {
+__global__ void __launch_bounds__(kEvalTB) k_eval64_batch(BatchDev b) {
   __shared__ DevState sd;
   int held = -1, w0, w1;
   const int n = *b.bstep;
@@ -455,9 +581,71 @@ int grid_for(int n, int block, int maxb) {
 
 int energy_parts_fp32(const DevState &d);
 
-int tiles_fp64(const DevState &d) {
-  return ((d.g.nx + 1 + TX - 1) / TX) * ((d.g.ny + 1 + TY - 1) / TY);
+// Tile shape of a mesh's FP64 node update: of the shapes below, the one with
+// the fewest FP64 instructions on the busiest SM, tiles being dealt evenly to
+// the 152 SMs, plus a constant for a tile's load and barrier latency (about
+// 60 warp instructions' time; it matters for small meshes only).  On the 100 x
+// 40 plate that is 16 x 2 nodes (10 us; 32 x 8 takes 36), on 400 x 160 32 x 8,
+// on large meshes 32 x 12, of which two CTAs share an SM.
+void tile64_shape(int nx, int ny, int &tx, int &ty) {
+  constexpr int kTx[] = {32, 16}, kTy[] = {12, 8, 6, 4, 3, 2, 1}, kSms = 152;
+  double best = 0.0;
+  tx = 0;
+  for (int x : kTx)
+    for (int y : kTy) {
+      const long n = (long)((nx + 1 + x - 1) / x) * ((ny + 1 + y - 1) / y);
+      const double c = (double)((n + kSms - 1) / kSms) * (tile64_cost(Tile64(x, y)) + 60.0);
+      if (tx == 0 || c < best) {
+        best = c;
+        tx = x;
+        ty = y;
+      }
+    }
 }
+
+void grid_main64(const DevState &d, int &gx, int &gy) {
+  gx = (d.g.nx + 1 + d.t64x - 1) / d.t64x;
+  gy = (d.g.ny + 1 + d.t64y - 1) / d.t64y;
+}
+
+int tiles_fp64(const DevState &d) {
+  int gx, gy;
+  grid_main64(d, gx, gy);
+  return gx * gy;
+}
+
+// piece blocks of kPieceTB threads (one per piece): small blocks, so that
+// the pieces of a small crack set spread over the SMs' FP64 pipes (100 x 40
+// plate, 5,700 pieces: 15 -> 8 us against blocks of 256)
+constexpr int kPieceTB = 64;
+int grid_pieces64(const DevState &d) { return grid_for(2 * d.ck_cap, kPieceTB, 608); }
+
+// evaluation blocks: 32 surface points each
+int grid_eval64(const DevState &d) { return grid_for(d.list_cap, kEvalPts, 608); }
+
+namespace {
+// The FP64 step's kernels ask for one shared-memory split (see
+// match_tile_carveout), so that the surface evaluation's blocks do not keep
+// the node update off their SMs.
+cudaError_t fp64_attrs() {
+  static bool done = false;
+  if (done) return cudaSuccess;
+  const int most = (int)Tile64(32, 12).bytes(true);
+  cudaError_t e = cudaFuncSetAttribute(k_main64, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_main64_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess) e = match_tile_carveout(k_main64);
+  if (e == cudaSuccess) e = match_tile_carveout(k_main64_batch);
+  if (e == cudaSuccess) e = match_tile_carveout(k_pieces64);
+  if (e == cudaSuccess) e = match_tile_carveout(k_pieces64_batch);
+  if (e == cudaSuccess) e = match_tile_carveout(k_phantom64);
+  if (e == cudaSuccess) e = match_tile_carveout(k_phantom64_batch);
+  if (e == cudaSuccess) e = match_tile_carveout(k_eval64);
+  if (e == cudaSuccess) e = match_tile_carveout(k_eval64_batch);
+  done = e == cudaSuccess;
+  return e;
+}
+}  // namespace
 
 int energy_parts_needed(const DevState &d) {
   if (d.precision == 1) return energy_parts_fp32(d);
@@ -469,7 +657,7 @@ int march_rows_solo(const DevState &d);
 
 int energy_parts_step(const DevState &d) {
   if (d.precision == 1) return energy_parts_step_fp32(d, march_rows_solo(d));
-  return tiles_fp64(d) + grid_pieces(d) + grid_phantoms(d);
+  return tiles_fp64(d) + grid_pieces64(d) + grid_phantoms(d);
 }
 
 cudaError_t launch_init_masses(const DevState &d, cudaStream_t st) {
@@ -479,31 +667,36 @@ cudaError_t launch_init_masses(const DevState &d, cudaStream_t st) {
 
 cudaError_t launch_step_fp64(const DevState &d, int cur, bool first, bool energy,
                              const StepStreams &ss, cudaEvent_t *marks) {
-  dim3 grid((d.g.nx + 1 + TX - 1) / TX, (d.g.ny + 1 + TY - 1) / TY);
-  int tiles = grid.x * grid.y;
-  int gp = grid_pieces(d);
+  cudaError_t e = fp64_attrs();
+  if (e != cudaSuccess) return e;
+  int gx, gy;
+  grid_main64(d, gx, gy);
+  const dim3 grid(gx, gy);
+  const size_t smem = Tile64(d.t64x, d.t64y).bytes(energy);
+  int tiles = gx * gy;
+  int gp = grid_pieces64(d);
   int gph = grid_phantoms(d);
-  const int ge = grid_eval(d);
+  const int ge = grid_eval64(d);
   cudaStream_t st = ss.main;
   if (marks) {
-    k_pieces64<<<gp, 256, 0, st>>>(d, cur, energy ? 1 : 0, tiles);
+    k_pieces64<<<gp, kPieceTB, 0, st>>>(d, cur, energy ? 1 : 0, tiles);
     cudaEventRecord(marks[0], st);
-    k_main64<<<grid, NT, 0, st>>>(d, cur, first ? 1 : 0, energy ? 1 : 0);
+    k_main64<<<grid, NT, smem, st>>>(d, cur, first ? 1 : 0, energy ? 1 : 0);
     cudaEventRecord(marks[1], st);
     k_phantom64<<<gph, 256, 0, st>>>(d, cur, first ? 1 : 0, energy ? 1 : 0, tiles + gp);
     cudaEventRecord(marks[2], st);
-    k_eval64<<<ge, 256, 0, st>>>(d, cur);
+    k_eval64<<<ge, kEvalTB, 0, st>>>(d, cur);
     return cudaGetLastError();
   }
   cudaEventRecord(ss.fork, st);
   cudaStreamWaitEvent(ss.aux2, ss.fork, 0);
-  k_eval64<<<ge, 256, 0, ss.aux2>>>(d, cur);
+  k_eval64<<<ge, kEvalTB, 0, ss.aux2>>>(d, cur);
   launch_select(d, TRACK_STEP, ss.aux2);
-  k_pieces64<<<gp, 256, 0, st>>>(d, cur, energy ? 1 : 0, tiles);
+  k_pieces64<<<gp, kPieceTB, 0, st>>>(d, cur, energy ? 1 : 0, tiles);
   cudaEventRecord(ss.fork, st);
   cudaStreamWaitEvent(ss.aux1, ss.fork, 0);
   k_phantom64<<<gph, 256, 0, ss.aux1>>>(d, cur, first ? 1 : 0, energy ? 1 : 0, tiles + gp);
-  k_main64<<<grid, NT, 0, st>>>(d, cur, first ? 1 : 0, energy ? 1 : 0);
+  k_main64<<<grid, NT, smem, st>>>(d, cur, first ? 1 : 0, energy ? 1 : 0);
   cudaEventRecord(ss.join1, ss.aux1);
   cudaEventRecord(ss.join2, ss.aux2);
   cudaStreamWaitEvent(st, ss.join1, 0);
@@ -515,20 +708,22 @@ cudaError_t launch_step_fp64(const DevState &d, int cur, bool first, bool energy
 // members of the batch.
 cudaError_t launch_step_fp64_batch(const BatchDev &b, bool first, bool energy, int grid_main,
                                    const StepStreams &ss) {
+  cudaError_t e = fp64_attrs();
+  if (e != cudaSuccess) return e;
   const int gm = grid_main < 1 ? 1 : grid_main;
   const int gp = grid_for(b.n_pieces, 1, 1216), gph = grid_for(b.n_ph, 1, 1216);
   const int ge = grid_for(b.n_eval, 1, 1216);
   cudaStream_t st = ss.main;
   cudaEventRecord(ss.fork, st);
   cudaStreamWaitEvent(ss.aux2, ss.fork, 0);
-  k_eval64_batch<<<ge, 256, 0, ss.aux2>>>(b);
-  cudaError_t e = launch_select_batch(b, ss.aux2);
+  k_eval64_batch<<<ge, kEvalTB, 0, ss.aux2>>>(b);
+  e = launch_select_batch(b, ss.aux2);
   if (e != cudaSuccess) return e;
-  k_pieces64_batch<<<gp, 256, 0, st>>>(b, energy ? 1 : 0);
+  k_pieces64_batch<<<gp, kPieceTB, 0, st>>>(b, energy ? 1 : 0);
   cudaEventRecord(ss.fork, st);
   cudaStreamWaitEvent(ss.aux1, ss.fork, 0);
   k_phantom64_batch<<<gph, 256, 0, ss.aux1>>>(b, first ? 1 : 0, energy ? 1 : 0);
-  k_main64_batch<<<gm, NT, 0, st>>>(b, first ? 1 : 0, energy ? 1 : 0);
+  k_main64_batch<<<gm, NT, Tile64(32, 12).bytes(energy), st>>>(b, first ? 1 : 0, energy ? 1 : 0);
   cudaEventRecord(ss.join1, ss.aux1);
   cudaEventRecord(ss.join2, ss.aux2);
   cudaStreamWaitEvent(st, ss.join1, 0);
