@@ -6,16 +6,21 @@
 // kept in FP32 (master copy, Adam state) and mirrored in BF16 for the
 // tensor-core GEMMs.  The 3x3 convolution is an implicit GEMM
 //   y[p, n] = sum_k A[p, k] W[n, k],  p = pixel, k = (ky, kx, c)
-// whose A rows are gathered from the input on the fly (zero outside the
-// image) with 16-byte cp.async copies into a 3-stage shared-memory ring,
-// fed to mma.sync m16n8k16 BF16 through ldmatrix.  The data gradient is the
-// same kernel applied to the output gradient with the weights transposed and
+// on the 5th-generation tensor cores: k_conv3x3_halo keeps a tile's input in
+// shared memory and reads the nine taps as shifted views; k_conv3x3_tc gathers
+// its A rows from the input on the fly (the deepest layers, odd channel
+// counts); k_conv3x3 does so for mma.sync m16n8k16 (cem_sg_set_gemm_path 0).
+// The data gradient is the same kernel applied to the output gradient with the weights transposed and
 // flipped (written by the Adam kernel); the weight gradient is a second
 // implicit GEMM over pixels, split along the pixels into fixed chunks whose
 // FP32 partial sums are added in chunk order (deterministic).
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
+
+#include <atomic>
 
 #include "../../include/cem_surrogate.h"
 
@@ -474,6 +479,751 @@ cudaError_t launch_conv_tc(const ConvArgs &a, cudaStream_t st) {
   dim3 grid((a.P + TCM - 1) / TCM, (a.N + BN - 1) / BN);
   k_conv3x3_tc<BN><<<grid, 128, tc_smem_bytes<BN>(), st>>>(a);
   return cudaGetLastError();
+}
+
+// ------------------------------------------- conv 3x3, resident input tile
+// The implicit GEMM again, with each input pixel fetched about 1.4 times
+// instead of nine: a CTA fetches the halo of an output tile once and forms the
+// nine taps' A operands as shifted views of it.  The gathers of k_conv3x3_tc
+// (a 16-byte copy per pixel, tap and 8 channels) bound the layers of few
+// channels: 32 -> 32 channels on 64 images of 160 x 400 took 467 us there.
+//
+// Layout.  A stage holds the tile's input as planes of 64 (32, 16; 8 when
+// there are 8) channels, one 128- (64-, 32-, 16-) byte row per pixel slot,
+// swizzled by shared-memory address as TMA writes it and the MMA reads it.  A tap is a start address
+// shifted by whole slots, the next 8 rows of the tile are one slot row
+// further (SBO).  Three tilings:
+//   whole  tiles 8 wide x 16 tall inside an image, halo 10 x 18 slots, one TMA box
+//          (zero fill outside the image);
+//   tall   the same tiles on all images stacked with a row of zeros between
+//          two, one TMA box per slot row: images whose height is far from a
+//          multiple of 16 leave no ragged rows (20 rows: 1.31 tiles an image
+//          instead of 2);
+//   flat   narrow images (W <= 30) as one long row with a zero after each
+//          image row, 128 consecutive pixels to a tile, one TMA box per image
+//          row and plane: 25 x 10 images fill 87% of the rows instead of 71%.
+// The weights stay in shared memory for the whole (persistent) CTA when they
+// fit, else they stream by TMA through a ring, each block serving MT tiles.
+//
+// Order.  Steps of 16 of k = (ky, kx, c) are accumulated in increasing k, as
+// k_conv3x3_tc does: the same sums, bit for bit.
+//
+// Roles: warps 0-3 and 4-7 the epilogues of the two accumulator sets (TMEM
+// lanes 32 (w & 3) ..), warp 8 issues the MMAs, warp 9 fetches weights, warp
+// 10 input tiles.  Every wait is bounded; one that gives up raises `fail`,
+// which ends the others.
+//
+// Measured (64 images; before with k_conv3x3_tc):
+//   32 -> 32, 160 x 400   467 -> 129 us, 4.1 TB/s; bound by the MMAs' reads of A from
+//                         shared memory (64 clocks a step, however few the channels)
+//   32 -> 96, 160 x 400   967 -> 194 us, 5.4 TB/s of HBM
+//   64 -> 64, 80 x 200    219 -> 68 us
+//   128 -> 384, 40 x 100  450 -> 131 us, 1725 TFLOP/s (0.91 of cuBLAS)
+//   256 -> 256, 20 x 50   106 -> 52 us, 1460 TFLOP/s
+// One image, 256 -> 256, 20 x 50: 47 -> 12 us.
+constexpr int HB_THREADS = 352, HB_MAXW = 48, HB_MAXA = 8;
+
+enum : int { TILE_WHOLE = 0, TILE_TALL = 1, TILE_FLAT = 2 };
+
+struct HaloArgs {
+  const float *bias;
+  bf16_t *y;
+  const bf16_t *mask;
+  int B, H, W, N, relu, ldy, yoff, ldm;
+  int mode;             // TILE_*
+  int planes;           // of a stage
+  int ky_st, ps, sbo;   // strides of a tap row, a plane and 8 tile rows (bytes)
+  int a_bytes, a_tx;    // a stage's size; the bytes its copies bring in
+  int nrows;            // flat: image rows a stage holds
+  int tiles_x, tiles_y, tiles;  // sub-tiles of 128 pixels (whole: tiles_y per image)
+  uint32_t inv_h, inv_w, inv_x, inv_y;  // ceil(2^32 / (H+1), / (W+1), / tiles_x, / tiles_y)
+  int nblk, nb, nbp;    // output-channel blocks, channels of one (its TMEM columns)
+  int kblocks;          // 64-wide steps of k
+  int na, nw;           // input stages, weight stages
+  int nacc;             // accumulator sets
+  int cols;             // TMEM columns allocated
+  int vec;              // bytes of a row access to y and mask: 32, 16 or 4
+  int off_ctl;          // shared-memory offset of HaloCtl
+};
+
+struct HaloCtl {
+  float bias[256];
+  uint64_t a_full[HB_MAXA], a_empty[HB_MAXA], w_full[HB_MAXW], w_empty[HB_MAXW], acc_full[2], acc_empty[2];
+  uint64_t drain;
+  uint32_t tmem;
+  int fail;
+};
+
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint64_t *bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)),
+               "r"(bytes)
+               : "memory");
+}
+// one lane of a converged warp
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+// Bounded wait (about a second) that also ends when another role has failed;
+// the waiting warp is suspended between tries, so that it takes no issue slots
+// from the others.
+constexpr int ROLE_TRIES = 1 << 20;
+__device__ __forceinline__ bool mbar_try(uint64_t *bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n"
+      " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity), "r"(1000u)
+      : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ bool thread_wait(uint64_t *bar, uint32_t parity, int *fail) {
+  for (int i = 0; i < ROLE_TRIES; ++i) {
+    if (mbar_try(bar, parity)) return true;
+    if (*(volatile int *)fail) return false;
+  }
+  *(volatile int *)fail = 1;
+  return false;
+}
+__device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, int *fail) {
+  for (int i = 0; i < ROLE_TRIES; ++i) {
+    if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+    if (__any_sync(0xffffffffu, *(volatile int *)fail)) return false;
+  }
+  *(volatile int *)fail = 1;
+  return false;
+}
+// one MMA of 128 x N x 16 (a single thread issues it); acc = 0 overwrites
+__device__ __forceinline__ void tc_mma(uint32_t tmem, uint32_t alo, uint32_t ahi, uint32_t blo,
+                                       uint32_t bhi, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n .reg .b64 da, db;\n setp.ne.b32 p, %6, 0;\n"
+      " mov.b64 da, {%1, %2};\n mov.b64 db, {%3, %4};\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n}\n" ::"r"(tmem),
+      "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc)
+      : "memory");
+}
+__device__ __forceinline__ void tc_commit(uint64_t *bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                   smem_u32(bar))
+               : "memory");
+}
+__device__ __forceinline__ void tmem_ld32(uint32_t addr, uint32_t r[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
+      "%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]),
+        "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
+        "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(addr));
+}
+__device__ __forceinline__ void ld_row32(const void *p, uint32_t r[8]) {
+  asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+                 "=r"(r[7])
+               : "l"(p));
+}
+__device__ __forceinline__ void st_row32(void *p, const uint32_t r[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n" ::"l"(p), "r"(r[0]), "r"(r[1]),
+               "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
+}
+// a pair of BF16 outputs set to zero where its mask values are not positive
+__device__ __forceinline__ uint32_t mask_pair(uint32_t v, uint32_t mk) {
+  if (!(bf2f((bf16_t)(mk & 0xffff)) > 0.f)) v &= 0xffff0000u;
+  if (!(bf2f((bf16_t)(mk >> 16)) > 0.f)) v &= 0x0000ffffu;
+  return v;
+}
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t *>(&h);
+}
+__device__ __forceinline__ void tma_load5(uint32_t dst, const CUtensorMap *map, int c0, int c1, int c2,
+                                          int c3, int c4, uint64_t *bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], "
+      "[%1, {%2, %3, %4, %5, %6}], [%7];\n" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4),
+      "r"(smem_u32(bar))
+      : "memory");
+}
+
+// n / d by its reciprocal ceil(2^32 / d): exact while n d < 2^32 (the host checks)
+__device__ __forceinline__ int div_by(int n, uint32_t inv) { return (int)__umulhi((uint32_t)n, inv); }
+
+// output pixel of row m of a sub-tile, or -1 outside the images
+__device__ __forceinline__ int halo_pixel(const HaloArgs &a, int tile, int m) {
+  int b, h, c;
+  if (a.mode == TILE_FLAT) {
+    const int q = a.W + 1 + tile * 128 + m, T = div_by(q, a.inv_w);
+    c = q - T * (a.W + 1);
+    b = div_by(T, a.inv_h);
+    h = T - b * (a.H + 1) - 1;
+  } else {
+    const int ty = a.tiles_x == 1 ? tile : div_by(tile, a.inv_x);
+    c = (tile - ty * a.tiles_x) * 8 + (m & 7);
+    if (a.mode == TILE_WHOLE) {
+      b = a.tiles_y == 1 ? ty : div_by(ty, a.inv_y);
+      h = (ty - b * a.tiles_y) * 16 + (m >> 3);
+    } else {
+      const int T = 1 + ty * 16 + (m >> 3);
+      b = div_by(T, a.inv_h);
+      h = T - b * (a.H + 1) - 1;
+    }
+  }
+  return h >= 0 && h < a.H && b < a.B && c < a.W ? (b * a.H + h) * a.W + c : -1;
+}
+// flat: position of the halo's first slot in the stage (the stage starts with a whole image row)
+__device__ __forceinline__ int flat_first(const HaloArgs &a, int tile, int &row) {
+  const int q = tile * 128 - 1;
+  row = q < 0 ? -1 : div_by(q, a.inv_w);
+  return q - row * (a.W + 1);
+}
+
+// RB: bytes of a slot's row in a plane
+template <int RB, int MT, bool RES>
+__global__ void __launch_bounds__(HB_THREADS, 1)
+    k_conv3x3_halo(const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap xmap,
+                   const HaloArgs a) {
+  extern __shared__ uint8_t hb_raw[];
+  uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(hb_raw) + 1023) &
+                                              ~(uintptr_t)1023);
+  HaloCtl &C = *reinterpret_cast<HaloCtl *>(base + a.off_ctl);
+  // weight blocks first, then the input stages (both 1024-byte aligned)
+  uint8_t *sw = base, *sa = base + (size_t)a.nw * a.nb * 128;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const int nbi = blockIdx.x % a.nblk, n0 = nbi * a.nb;
+  const int step = gridDim.x / a.nblk, g0 = blockIdx.x / a.nblk;
+  const int groups = (a.tiles + MT - 1) / MT;  // a group: MT sub-tiles
+
+  if (tid == 0) {
+    for (int s = 0; s < a.na; ++s) {
+      mbar_init(&C.a_full[s], 1);
+      mbar_init(&C.a_empty[s], 1);
+    }
+    for (int s = 0; s < a.nw; ++s) {
+      mbar_init(&C.w_full[s], 1);
+      mbar_init(&C.w_empty[s], 1);
+    }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&C.acc_full[s], 1);
+      mbar_init(&C.acc_empty[s], 128);
+    }
+    mbar_init(&C.drain, 1);
+    C.fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  if (warp == 8) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                     smem_u32(&C.tmem)),
+                 "r"(a.cols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
+  }
+  if (a.bias)
+    for (int q = tid; q < a.nb; q += HB_THREADS) C.bias[q] = n0 + q < a.N ? a.bias[n0 + q] : 0.f;
+  if (RB == 16) {  // the zero half of the last step: a second plane that no copy writes
+    for (int q = tid; q < a.na * MT * 180; q += HB_THREADS)
+      *reinterpret_cast<uint4 *>(sa + (size_t)(q / 180) * a.a_bytes + a.ps + (q % 180) * 16) =
+          make_uint4(0, 0, 0, 0);
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+  const uint32_t tmem = __shfl_sync(0xffffffffu, C.tmem, 0);
+
+  if (warp == 10) {
+    // ---- input tiles
+    if (elect_one()) {
+      int s = 0, ph = 1, it = 0;
+      for (int g = g0; g < groups; g += step, ++it) {
+        if (!thread_wait(&C.a_empty[s], ph, &C.fail)) break;
+        mbar_expect(&C.a_full[s], (uint32_t)(MT * a.a_tx));
+        for (int m = 0; m < MT; ++m) {
+          const int tile = g * MT + m;  // one past the last: rows outside the images, all zeros
+          const uint32_t dst = smem_u32(sa) + (uint32_t)((s * MT + m) * a.a_bytes);
+          if (a.mode == TILE_FLAT) {
+            int row;
+            flat_first(a, tile, row);
+            for (int r = 0; r < a.nrows; ++r) {
+              const int T = row + r, b = T < 0 ? 0 : div_by(T, a.inv_h);
+              const int h = T < 0 ? -1 : T - b * (a.H + 1) - 1;
+              for (int p = 0; p < a.planes; ++p)
+                tma_load5(dst + p * a.ps + r * (a.W + 1) * RB, &xmap, 0, 0, h, b, p, &C.a_full[s]);
+            }
+          } else {
+            const int ty = a.tiles_x == 1 ? tile : div_by(tile, a.inv_x);
+            const int c = (tile - ty * a.tiles_x) * 8 - 1;
+            if (a.mode == TILE_WHOLE) {
+              const int b = a.tiles_y == 1 ? ty : div_by(ty, a.inv_y);
+              tma_load5(dst, &xmap, 0, c, (ty - b * a.tiles_y) * 16 - 1, b, 0, &C.a_full[s]);
+            } else {
+              for (int r = 0; r < 18; ++r) {
+                const int T = ty * 16 + r, b = div_by(T, a.inv_h);
+                tma_load5(dst + r * a.ky_st, &xmap, 0, c, T - b * (a.H + 1) - 1, b, 0, &C.a_full[s]);
+              }
+            }
+          }
+        }
+        if (++s == a.na) {
+          s = 0;
+          ph ^= 1;
+        }
+      }
+      // no copy outlives the CTA: wait for those of the last na tiles (bounded)
+      for (int q = max(0, it - a.na); q < it; ++q) mbar_wait(&C.a_full[q % a.na], (q / a.na) & 1);
+    }
+  } else if (warp == 9) {
+    // ---- weights
+    if (elect_one()) {
+      const uint32_t bytes = (uint32_t)a.nb * 128;
+      const int mine = g0 < groups ? (groups - 1 - g0) / step + 1 : 0;
+      const int total = RES ? (mine ? a.kblocks : 0) : mine * a.kblocks;
+      int s = 0, ph = 1, kb = 0, q = 0;
+      for (; q < total; ++q) {
+        if (!RES && !thread_wait(&C.w_empty[s], ph, &C.fail)) break;
+        mbar_expect(&C.w_full[s], bytes);
+        asm volatile(
+            "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], "
+            "[%1, {%2, %3}], [%4];\n" ::"r"(smem_u32(sw) + (uint32_t)s * bytes),
+            "l"(reinterpret_cast<uint64_t>(&wmap)), "r"(kb * 64), "r"(n0), "r"(smem_u32(&C.w_full[s]))
+            : "memory");
+        if (++kb == a.kblocks) kb = 0;
+        if (++s == a.nw) {
+          s = 0;
+          ph ^= 1;
+        }
+      }
+      for (int p = max(0, q - a.nw); p < q; ++p) mbar_wait(&C.w_full[p % a.nw], (p / a.nw) & 1);
+    }
+  } else if (warp == 8) {
+    // ---- MMAs, issued by one elected lane; a weight block's four steps are
+    // straight-line code, or their issue would cost several times the MMA
+    if (elect_one()) {
+      const uint32_t idesc = tc_idesc(128, a.nb);
+      // SBO, descriptor version, swizzle of 128-, 64- or 32-byte rows (none of 16-byte rows)
+      const uint32_t ahi = (uint32_t)(a.sbo >> 4) | (1u << 14) |
+                           ((RB == 128 ? 2u : RB == 64 ? 4u : RB == 32 ? 6u : 0u) << 29);
+      const uint32_t whi = (uint32_t)(sw128_desc(0) >> 32), wlo0 = (uint32_t)sw128_desc(smem_u32(sw));
+      const uint32_t sa0 = (smem_u32(sa) >> 4) | (RB == 16 ? 0u : 1u << 16), stage = (uint32_t)a.a_bytes >> 4;
+      const uint32_t ps = (uint32_t)a.ps >> 4, wst = (uint32_t)a.nb * 8;  // in units of 16 bytes
+      constexpr int ROWS = RB == 16 ? 4 : 128 / RB;  // rows of a weight block
+      constexpr int PER = RB == 16 ? 1 : RB / 32;    // steps of a row
+      const uint32_t ky_next = (uint32_t)((a.ky_st - 2 * RB) >> 4);  // from tap kx = 2 to the next row's 0
+      int s = 0, sph = 0, ab = 0, abph = 1, ws = 0, wph = 0;
+      bool first = true;
+      for (int g = g0; g < groups; g += step) {
+        if (!thread_wait(&C.a_full[s], sph, &C.fail)) break;
+        if (!thread_wait(&C.acc_empty[ab], abph, &C.fail)) break;
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        uint32_t tap[MT], row[MT];
+#pragma unroll
+        for (int m = 0; m < MT; ++m) {
+          tap[m] = sa0 + (uint32_t)(s * MT + m) * stage;
+          if (a.mode == TILE_FLAT) {
+            int r;
+            tap[m] += (uint32_t)(flat_first(a, g * MT + m, r) * (RB / 16));
+          }
+          row[m] = tap[m];
+        }
+        const uint32_t d0 = tmem + (uint32_t)(ab * MT * a.nbp);
+        int pl = 0, kx = 0, left = RB == 16 ? 5 : 9 * a.planes;
+        bool ok = true;
+        for (int kb = 0; kb < a.kblocks; ++kb) {
+          if (RES) {
+            if (first && !(ok = thread_wait(&C.w_full[kb], 0, &C.fail))) break;
+          } else if (!(ok = thread_wait(&C.w_full[ws], wph, &C.fail))) {
+            break;
+          }
+          const uint32_t wd = wlo0 + (uint32_t)(RES ? kb : ws) * wst;
+#pragma unroll
+          for (int r = 0; r < ROWS; ++r) {
+            if constexpr (RB == 16) {
+              // 8 channels: taps 2 q and 2 q + 1 are the halves of step q (LBO apart), the
+              // zero plane the second half of the last
+              const int q = 4 * kb + r, t0 = 2 * q, t1 = t0 + 1;
+              if (q >= 5) continue;
+              const uint32_t o0 = (uint32_t)((t0 / 3) * 10 + t0 % 3);
+              const uint32_t o1 = t1 < 9 ? (uint32_t)((t1 / 3) * 10 + t1 % 3) : ps;
+#pragma unroll
+              for (int m = 0; m < MT; ++m)
+                tc_mma(d0 + m * a.nbp, (tap[m] + o0) | ((o1 - o0) << 16), ahi, wd + 2 * r, whi, idesc,
+                       r ? 1u : (uint32_t)(kb > 0));
+            } else if (ROWS == 1 || left > 0) {
+#pragma unroll
+              for (int i = 0; i < PER; ++i)
+#pragma unroll
+                for (int m = 0; m < MT; ++m)
+                  tc_mma(d0 + m * a.nbp, row[m] + 2 * i, ahi, wd + 2 * (r * PER + i), whi, idesc,
+                         (r || i) ? 1u : (uint32_t)(kb > 0));
+              --left;
+              uint32_t adv = ps;
+              if (++pl == a.planes) {
+                pl = 0;
+                uint32_t t = RB / 16;
+                if (++kx == 3) {
+                  kx = 0;
+                  t = ky_next;
+                }
+#pragma unroll
+                for (int m = 0; m < MT; ++m) row[m] = tap[m] = tap[m] + t;
+                adv = 0;
+              }
+#pragma unroll
+              for (int m = 0; m < MT; ++m) row[m] += adv;
+            }
+          }
+          if (!RES) {
+            tc_commit(&C.w_empty[ws]);
+            if (++ws == a.nw) {
+              ws = 0;
+              wph ^= 1;
+            }
+          }
+        }
+        if (!ok) break;
+        first = false;
+        tc_commit(&C.a_empty[s]);
+        tc_commit(&C.acc_full[ab]);
+        if (++s == a.na) {
+          s = 0;
+          sph ^= 1;
+        }
+        if (++ab == a.nacc) {
+          ab = 0;
+          abph ^= 1;
+        }
+      }
+      // every MMA issued has completed before the CTA's memory is given back
+      tc_commit(&C.drain);
+      if (!mbar_wait(&C.drain, 0)) *(volatile int *)&C.fail = 2;
+    }
+  } else {
+    // ---- epilogue: bias, ReLU, mask, BF16; each group of four warps has its own
+    // accumulator set and takes every second tile group (all, with one set)
+    const int e = warp >> 2, w4 = warp & 3;
+    const int mrow = w4 * 32 + lane;
+    uint32_t ph = 0;
+    if (e < a.nacc)
+      for (int g = g0 + e * step; g < groups; g += a.nacc * step, ph ^= 1) {
+        int pix[MT];
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+          pix[m] = g * MT + m < a.tiles ? halo_pixel(a, g * MT + m, mrow) : -1;
+        if (!warp_wait(&C.acc_full[e], ph, &C.fail)) break;
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+#pragma unroll
+        for (int m = 0; m < MT; ++m) {
+          const int p = pix[m];
+#pragma unroll 1
+          for (int cb = 0; cb < a.nb; cb += 32) {
+            uint32_t r[32], o[16];
+            __syncwarp();
+            tmem_ld32(tmem + ((uint32_t)(w4 * 32) << 16) + (uint32_t)((e * MT + m) * a.nbp + cb), r);
+            asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+            if (m == MT - 1 && cb + 32 >= a.nb) {
+              asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+              mbar_arrive(&C.acc_empty[e]);
+            }
+            if (p < 0) continue;
+            if (a.bias) {
+              const float4 *bp = reinterpret_cast<const float4 *>(C.bias + cb);
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                const float4 b4 = bp[j];
+                r[4 * j] = __float_as_uint(__uint_as_float(r[4 * j]) + b4.x);
+                r[4 * j + 1] = __float_as_uint(__uint_as_float(r[4 * j + 1]) + b4.y);
+                r[4 * j + 2] = __float_as_uint(__uint_as_float(r[4 * j + 2]) + b4.z);
+                r[4 * j + 3] = __float_as_uint(__uint_as_float(r[4 * j + 3]) + b4.w);
+              }
+            }
+            if (a.relu) {
+#pragma unroll
+              for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(fmaxf(__uint_as_float(r[j]), 0.f));
+            }
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+              o[j] = pack_bf16(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
+            bf16_t *yp = a.y + (size_t)p * a.ldy + a.yoff + n0 + cb;
+            const bf16_t *mp = a.mask + (size_t)p * a.ldm + n0 + cb;
+            // channels of this block left from here
+            const int left = min(min(a.nb, a.N - n0) - cb, 32);
+            if (a.vec == 32) {
+#pragma unroll
+              for (int q = 0; q < 2; ++q) {
+                if (16 * q >= left) continue;
+                if (a.mask) {
+                  uint32_t mk[8];
+                  ld_row32(mp + 16 * q, mk);
+#pragma unroll
+                  for (int t = 0; t < 8; ++t) o[8 * q + t] = mask_pair(o[8 * q + t], mk[t]);
+                }
+                st_row32(yp + 16 * q, o + 8 * q);
+              }
+            } else if (a.vec == 16) {
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                if (8 * q >= left) continue;
+                uint4 v = make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+                if (a.mask) {
+                  const uint4 mk = *reinterpret_cast<const uint4 *>(mp + 8 * q);
+                  v = make_uint4(mask_pair(v.x, mk.x), mask_pair(v.y, mk.y), mask_pair(v.z, mk.z),
+                                 mask_pair(v.w, mk.w));
+                }
+                *reinterpret_cast<uint4 *>(yp + 8 * q) = v;
+              }
+            } else {
+#pragma unroll
+              for (int q = 0; q < 16; ++q) {
+                if (2 * q >= left) continue;
+                uint32_t v = o[q];
+                if (a.mask) v = mask_pair(v, *reinterpret_cast<const uint32_t *>(mp + 2 * q));
+                *reinterpret_cast<uint32_t *>(yp + 2 * q) = v;
+              }
+            }
+          }
+        }
+      }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+  __syncthreads();
+  if (tid == 0 && C.fail) atomicAdd(&g_tc_timeouts, 1);
+  // TMEM is freed unless MMAs may still be in flight (the drain gave up)
+  if (warp == 8 && C.fail != 2)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(a.cols));
+}
+
+// ---- plan of one call
+constexpr int kSms = 152;
+constexpr size_t kSmemMax = 232448;  // 227 KB a CTA
+
+struct HaloPlan {
+  HaloArgs a;
+  int rb, mt, res, grid, box_w, box_h, box_p;
+  size_t smem;
+};
+
+// Chooses the tiling, the channel blocks (nblk), the tiles per weight block
+// (mt), the input stages (na) and whether the weights stay (res), by an
+// estimate in clocks: an MMA of 128 x nb x 16 takes nb / 2 of them, or 58 + nb / 5
+// (measured: reading its operands), a tile group 350 besides; an SM draws
+// about 45 bytes per clock from L2, a ring no more than it holds in 2000 clocks
+// (the latency under load).  Few tiles (a single image's deep levels) come out with
+// many narrow channel blocks, so that the K loop runs on more SMs.  False when
+// no plan fits (an input stage of more than about 560 channels, channels that
+// are neither 8 nor a multiple of 16): k_conv3x3_tc takes those.
+bool halo_plan(const ConvArgs &v, HaloPlan &best) {
+  if ((v.Cin & 15) && v.Cin != 8) return false;
+  const int rb = !(v.Cin & 63) ? 128 : !(v.Cin & 31) ? 64 : !(v.Cin & 15) ? 32 : 16;
+  auto up = [](long n, long d) { return (n + d - 1) / d; };
+  auto inv = [](long d) { return (uint32_t)(((1ull << 32) + d - 1) / d); };
+  const long rows = (long)v.B * (v.H + 1) - 1;  // of the tall image
+  const int kblocks = (v.K + 63) / 64;
+  const size_t fixed = 1024 + 128 + sizeof(HaloCtl);
+  double best_c = 0.0;
+  bool found = false;
+  for (int mode : {TILE_WHOLE, TILE_TALL, TILE_FLAT}) {
+    HaloArgs a{};
+    a.mode = mode;
+    a.planes = v.Cin * 2 / rb;
+    a.kblocks = kblocks;
+    a.tiles_x = (int)up(v.W, 8);
+    a.tiles_y = (int)up(v.H, 16);
+    long tiles;
+    if (mode == TILE_FLAT) {
+      if (v.W > 30 || rb != 128) continue;
+      a.tiles_x = 1;
+      tiles = up(rows * (v.W + 1), 128);
+      a.nrows = (v.W + 128 + 2 * (v.W + 2) - 1) / (v.W + 1) + 1;
+      a.ky_st = (v.W + 1) * rb;
+      a.ps = a.nrows * a.ky_st;
+      a.sbo = 8 * rb;
+      a.a_tx = a.planes * a.ps;
+    } else {
+      if (mode == TILE_TALL && (a.planes * 10 * rb) % 128) continue;  // TMA rows start on 128 bytes
+      tiles = (mode == TILE_WHOLE ? (long)v.B * a.tiles_y : up(rows, 16)) * a.tiles_x;
+      a.ps = (mode == TILE_WHOLE ? 180 : 10) * rb;
+      a.ky_st = a.sbo = mode == TILE_WHOLE ? 10 * rb : a.planes * a.ps;
+      a.a_tx = 180 * a.planes * rb;
+    }
+    a.a_bytes = ((rb == 16 ? 2 * a.a_tx : a.a_tx) + 1023) & ~1023;
+    a.tiles = (int)tiles;
+    // limits of the kernel's divisions by reciprocals
+    if ((rows + 40) * (v.W + 1) + 256 >= (1L << 32) / (v.W + 1) || (rows + 40) * (v.H + 1) >= (1L << 32) ||
+        (tiles + 2) * a.tiles_x >= (1L << 32) || (tiles + 2) * a.tiles_y >= (1L << 32) || tiles > (1L << 30))
+      continue;
+    a.inv_h = inv(v.H + 1);
+    a.inv_w = inv(v.W + 1);
+    a.inv_x = inv(a.tiles_x);  // tiles_x, tiles_y of 1 are not divided by
+    a.inv_y = inv(a.tiles_y);
+    for (int nblk : {1, 2, 3, 4, 6, 8, 12, 16}) {
+      const int nb = ((v.N + nblk - 1) / nblk + 15) & ~15;
+      if (nb > 256 || (nblk - 1) * nb >= v.N) continue;
+      const int nbp = (nb + 31) & ~31;
+      const size_t wst = (size_t)nb * 128;
+      for (int mt = 1; mt <= 2; ++mt) {
+        if (mt * nbp > 512) continue;
+        const int nacc = 2 * mt * nbp <= 512 ? 2 : 1;
+        const size_t ast = (size_t)mt * a.a_bytes;
+        for (int res = 1; res >= 0; --res) {
+          if (res && kblocks > HB_MAXW) continue;
+          int na = HB_MAXA;
+          while (na && fixed + (res ? kblocks : 2) * wst + na * ast > kSmemMax) --na;
+          if (!na) continue;
+          const int groups = (a.tiles + mt - 1) / mt;
+          int per = kSms / nblk;
+          if (per > groups) per = groups;
+          const double mma = ((v.K + 15) / 16) * mt * fmax(0.53 * nb, 58.0 + 0.2 * nb) + 350.0;
+          const double la = mt * (double)a.a_tx / 45.0;
+          const double epi = mt * (nbp / 32) * 300.0;
+          // with a ring: one or two input stages, the rest of the memory for the ring
+          for (int ns = res ? na : na < 2 ? na : 2; ns; ns = res ? 0 : ns - 1) {
+            int nw = kblocks;
+            if (!res) {
+              nw = 2;
+              while (nw < 12 && nw < kblocks && fixed + (nw + 1) * wst + ns * ast <= kSmemMax) ++nw;
+            }
+            const double lw = kblocks * (double)wst / (res ? 45.0 : fmin(45.0, nw * (double)wst / 2000.0));
+            double t = fmax(mma, fmax(la + (res ? 0.0 : lw), epi));
+            if (ns == 1) t += la + 1000.0;
+            if (nacc == 1) t += epi;
+            const double c = ((groups + per - 1) / per) * t + la + 2500.0 + (res ? lw : 0.0);
+            if (found && c >= best_c) continue;
+            found = true;
+            best_c = c;
+            best.a = a;
+            best.a.nblk = nblk;
+            best.a.nb = nb;
+            best.a.nbp = nbp;
+            best.a.nacc = nacc;
+            best.a.na = ns;
+            best.a.nw = nw;
+            best.mt = mt;
+            best.res = res;
+            best.grid = per * nblk;
+            int cols = 32;
+            while (cols < nacc * mt * nbp) cols <<= 1;
+            best.a.cols = cols;
+            best.a.off_ctl = (int)(((size_t)nw * wst + ns * ast + 127) & ~(size_t)127);
+            best.smem = 1024 + best.a.off_ctl + sizeof(HaloCtl);
+          }
+          break;  // resident weights, when they fit, beat the ring of the same blocks
+        }
+      }
+    }
+  }
+  // k_conv3x3_tc keeps calls it does faster: 256-channel blocks of deep layers
+  // (1700 clocks per tile and 64 of k), where too little memory is left
+  // beside the input stage for a weight ring (512 -> 512 channels, 64 images
+  // of 10 x 25: 94 us there, 113 here)
+  const double old_c = (double)up((long)v.B * v.H * v.W, 128) * up(v.N, 256) / kSms * kblocks * 1700.0;
+  if (!found || (v.N > 128 && v.B * (long)v.H * v.W >= 128L * kSms / 2 && best_c > old_c)) return false;
+  best.rb = rb;
+  best.box_w = best.a.mode == TILE_FLAT ? v.W + 1 : 10;
+  best.box_h = best.a.mode == TILE_WHOLE ? 18 : 1;
+  best.box_p = best.a.mode == TILE_FLAT ? 1 : best.a.planes;
+  return true;
+}
+
+typedef CUresult (*EncodeTiled)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
+                                const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
+                                const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+EncodeTiled encode_tiled() {
+  static const EncodeTiled fn = [] {
+    void *p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) !=
+            cudaSuccess || q != cudaDriverEntryPointSuccess)
+      p = nullptr;
+    return (EncodeTiled)p;
+  }();
+  return fn;
+}
+// BF16 tensor of dims[0] contiguous values; st: byte strides of the others
+bool encode_bf16(CUtensorMap *map, int rank, const void *p, const cuuint64_t *dims, const cuuint64_t *st,
+                 const cuuint32_t *box, CUtensorMapSwizzle swizzle) {
+  const EncodeTiled enc = encode_tiled();
+  const cuuint32_t es[5] = {1, 1, 1, 1, 1};
+  return enc && enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void *>(p), dims, st,
+                    box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+// NHWC images as (channel in plane, w, h, image, plane) of planes of rb bytes
+bool encode_image(CUtensorMap *map, const void *x, int B, int H, int W, int ld, int planes, int rb,
+                  int box_w, int box_h, int box_p) {
+  const cuuint64_t px = (cuuint64_t)ld * 2;
+  const cuuint64_t dims[5] = {(cuuint64_t)rb / 2, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B,
+                              (cuuint64_t)planes};
+  const cuuint64_t st[4] = {px, px * W, px * W * H, (cuuint64_t)rb};
+  const cuuint32_t box[5] = {(cuuint32_t)rb / 2, (cuuint32_t)box_w, (cuuint32_t)box_h, 1, (cuuint32_t)box_p};
+  return encode_bf16(map, 5, x, dims, st, box,
+                     rb == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
+                     : rb == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
+                     : rb == 32 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_NONE);
+}
+
+// raises a kernel's dynamic shared-memory limit, once per device
+template <class K>
+cudaError_t allow_smem(K *kernel, std::atomic<unsigned long long> &done) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (done.load() & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+  if (e == cudaSuccess) done.fetch_or(bit);
+  return e;
+}
+
+template <int RB, int MT, bool RES>
+cudaError_t launch_halo(const HaloPlan &p, const CUtensorMap &wm, const CUtensorMap &xm, cudaStream_t st) {
+  static std::atomic<unsigned long long> done{0};
+  cudaError_t e = allow_smem(k_conv3x3_halo<RB, MT, RES>, done);
+  if (e != cudaSuccess) return e;
+  k_conv3x3_halo<RB, MT, RES><<<p.grid, HB_THREADS, p.smem, st>>>(wm, xm, p.a);
+  return cudaGetLastError();
+}
+template <int RB>
+cudaError_t launch_halo_rb(const HaloPlan &p, const CUtensorMap &wm, const CUtensorMap &xm, cudaStream_t st) {
+  if (p.res)
+    return p.mt == 2 ? launch_halo<RB, 2, true>(p, wm, xm, st) : launch_halo<RB, 1, true>(p, wm, xm, st);
+  return p.mt == 2 ? launch_halo<RB, 2, false>(p, wm, xm, st) : launch_halo<RB, 1, false>(p, wm, xm, st);
+}
+
+// true when the call was launched here (rc its status); false: not this kernel's
+bool conv_halo(const ConvArgs &v, cudaStream_t st, cudaError_t &rc) {
+  HaloPlan p;
+  if (!halo_plan(v, p)) return false;
+  HaloArgs &a = p.a;
+  a.bias = v.bias; a.y = v.y; a.mask = v.mask;
+  a.B = v.B; a.H = v.H; a.W = v.W; a.N = v.N; a.relu = v.relu;
+  a.ldy = v.ldy; a.yoff = v.yoff; a.ldm = v.ldm;
+  // widest row access that y, its offset and stride, and the mask allow
+  auto fits = [&](int c) {
+    const uintptr_t b = (uintptr_t)c * 2 - 1;
+    return !(v.N % c) && !(v.ldy % c) && !(v.yoff % c) && !((uintptr_t)v.y & b) &&
+           (!v.mask || (!(v.ldm % c) && !((uintptr_t)v.mask & b)));
+  };
+  a.vec = fits(16) ? 32 : fits(8) ? 16 : 4;
+  CUtensorMap wm, xm;
+  const cuuint64_t wd[2] = {(cuuint64_t)v.K, (cuuint64_t)v.N}, ws[1] = {(cuuint64_t)v.K * 2};
+  const cuuint32_t wb[2] = {64, (cuuint32_t)a.nb};
+  if (!encode_bf16(&wm, 2, v.w, wd, ws, wb, CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !encode_image(&xm, v.x, v.B, v.H, v.W, v.ldx, a.planes, p.rb, p.box_w, p.box_h, p.box_p))
+    return false;
+  rc = p.rb == 128 ? launch_halo_rb<128>(p, wm, xm, st)
+     : p.rb == 64 ? launch_halo_rb<64>(p, wm, xm, st)
+     : p.rb == 32 ? launch_halo_rb<32>(p, wm, xm, st) : launch_halo_rb<16>(p, wm, xm, st);
+  return true;
 }
 
 int g_use_tc = 1;  // cem_sg_set_gemm_path
@@ -1238,7 +1988,9 @@ int cem_sg_conv3x3(const void *x, int B, int H, int W, int Cin, int ldx, const v
   a.ldm = ldmask;
   cudaStream_t st = (cudaStream_t)stream;
   if (g_use_tc) {
-    cudaError_t e = Cout > 128 ? launch_conv_tc<256>(a, st)
+    cudaError_t e;
+    if (!conv_halo(a, st, e))
+      e = Cout > 128 ? launch_conv_tc<256>(a, st)
                   : Cout > 64 ? launch_conv_tc<128>(a, st)
                   : Cout > 32 ? launch_conv_tc<64>(a, st) : launch_conv_tc<32>(a, st);
     return e == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;

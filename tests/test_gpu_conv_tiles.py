@@ -1,0 +1,65 @@
+"""The tensor-core convolution over its tilings, channel layouts, output
+slices and masks, against a 64-bit convolution (needs a GPU)."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def conv64(x, w):
+    """3x3 convolution, zero padding, NHWC, float64; w [N, 3, 3, C]."""
+    import torch
+    B, H, W, C = x.shape
+    p = torch.zeros(B, H + 2, W + 2, C, dtype=torch.float64, device=x.device)
+    p[:, 1:-1, 1:-1] = x
+    y = torch.zeros(B, H, W, w.shape[0], dtype=torch.float64, device=x.device)
+    for ky in range(3):
+        for kx in range(3):
+            y += p[:, ky:ky + H, kx:kx + W] @ w[:, ky, kx].T
+    return y
+
+
+# images of whole tiles, one row or column around a tile's edge, stacked images
+# whose tiles span two of them, narrow images as one row, single pixels
+@pytest.mark.parametrize("B,H,W", [(1, 16, 8), (2, 17, 33), (3, 15, 7), (5, 20, 50), (7, 10, 25), (4, 5, 30),
+                                   (9, 3, 31), (3, 1, 1), (2, 1, 64), (2, 64, 1), (70, 16, 40)])
+# one to many channel planes of every width; channel blocks of odd sizes
+@pytest.mark.parametrize("cin,cout", [(8, 32), (16, 2), (32, 96), (48, 24), (64, 10), (96, 40), (192, 64),
+                                      (128, 264), (512, 48)])
+def test_conv_tilings(B, H, W, cin, cout):
+    import torch
+    from paper_2509_01827_gb300 import build, surrogate
+    build.build()
+    L = surrogate.sg()
+    dev = "cuda"
+    g = torch.Generator(device=dev).manual_seed(B * 1000 + cin)
+    P, ld, off = B * H * W, cin + 8, 8
+    xw = torch.randn(P, ld, device=dev, generator=g).bfloat16()
+    x = xw[:, off:]  # a channel slice of a wider tensor
+    w = (torch.randn(cout, 3, 3, cin, device=dev, generator=g) / (3 * cin ** 0.5)).bfloat16()
+    b = torch.randn(cout, device=dev, generator=g)
+    mk = torch.randn(P, cout, device=dev, generator=g).bfloat16()
+    st = torch.cuda.current_stream().cuda_stream
+    t0 = surrogate.timeouts()
+    x64, w64 = x.double().view(B, H, W, cin), w.double()
+    ref = conv64(x64, w64).view(P, cout)
+    # rounding to BF16 (2^-9 relative) and of the FP32 sums (9 cin terms, each
+    # at most 2^-22 of the sum of magnitudes off, truncation included)
+    tol = 2.0 ** -8 * ref.abs() + 9 * cin * 2.0 ** -22 * conv64(x64.abs(), w64.abs()).view(P, cout) + 1e-30
+    for pad, bias, relu, mask in ((0, b, 1, None), (6, None, 0, mk), (16, b, 0, mk)):
+        y = torch.full((P, cout + 2 * pad), 7.0, device=dev).bfloat16()
+        rc = L.cem_sg_conv3x3(x.data_ptr(), B, H, W, cin, ld, w.data_ptr(),
+                              None if bias is None else bias.data_ptr(), cout, relu,
+                              None if mask is None else mask.data_ptr(), cout, y.data_ptr(),
+                              cout + 2 * pad, pad, st)
+        assert rc == 0
+        want = ref + (0 if bias is None else bias.double())
+        if relu:
+            want = want.clamp(min=0)
+        if mask is not None:
+            want = torch.where(mask.double() > 0, want, torch.zeros_like(want))
+        got = y[:, pad:pad + cout].double()
+        slack = tol + 2.0 ** -8 * (0 if bias is None else bias.double().abs())
+        assert bool(((got - want).abs() <= slack).all()), float((got - want).abs().max())
+        # nothing beside the slice is written
+        assert bool((y[:, :pad] == 7).all()) and bool((y[:, pad + cout:] == 7).all())
+    assert surrogate.timeouts() == t0
