@@ -514,11 +514,11 @@ cudaError_t launch_conv_tc(const ConvArgs &a, cudaStream_t st) {
 // which ends the others.
 //
 // Measured (64 images; before with k_conv3x3_tc):
-//   32 -> 32, 160 x 400   467 -> 129 us, 4.1 TB/s; bound by the MMAs' reads of A from
-//                         shared memory (64 clocks a step, however few the channels)
-//   32 -> 96, 160 x 400   967 -> 194 us, 5.4 TB/s of HBM
-//   64 -> 64, 80 x 200    219 -> 68 us
-//   128 -> 384, 40 x 100  450 -> 131 us, 1725 TFLOP/s (0.91 of cuBLAS)
+//   8 -> 32, 160 x 400    318 -> 72 us, 4.6 TB/s
+//   32 -> 32, 160 x 400   467 -> 119 us, 4.4 TB/s
+//   32 -> 96, 160 x 400   967 -> 192 us, 5.5 TB/s of HBM
+//   64 -> 64, 80 x 200    219 -> 66 us
+//   128 -> 384, 40 x 100  450 -> 134 us, 1690 TFLOP/s (0.89 of cuBLAS)
 //   256 -> 256, 20 x 50   106 -> 52 us, 1460 TFLOP/s
 // One image, 256 -> 256, 20 x 50: 47 -> 12 us.
 constexpr int HB_THREADS = 352, HB_MAXW = 48, HB_MAXA = 8;
@@ -687,8 +687,11 @@ __device__ __forceinline__ int flat_first(const HaloArgs &a, int tile, int &row)
   return q - row * (a.W + 1);
 }
 
-// RB: bytes of a slot's row in a plane
-template <int RB, int MT, bool RES>
+// RB: bytes of a slot's row in a plane.  PL > 0: the stage's planes, known at
+// compile time with the tiling (TALL or WHOLE), and a tile's steps are
+// straight-line code with constant offsets; the issue of a step then costs about
+// 30 clocks, less than its MMA, against 65 with the offsets walked (PL = 0).
+template <int RB, int MT, bool RES, int PL, bool TALL>
 __global__ void __launch_bounds__(HB_THREADS, 1)
     k_conv3x3_halo(const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap xmap,
                    const HaloArgs a) {
@@ -741,46 +744,44 @@ __global__ void __launch_bounds__(HB_THREADS, 1)
   const uint32_t tmem = __shfl_sync(0xffffffffu, C.tmem, 0);
 
   if (warp == 10) {
-    // ---- input tiles
-    if (elect_one()) {
-      int s = 0, ph = 1, it = 0;
-      for (int g = g0; g < groups; g += step, ++it) {
-        if (!thread_wait(&C.a_empty[s], ph, &C.fail)) break;
-        mbar_expect(&C.a_full[s], (uint32_t)(MT * a.a_tx));
-        for (int m = 0; m < MT; ++m) {
-          const int tile = g * MT + m;  // one past the last: rows outside the images, all zeros
-          const uint32_t dst = smem_u32(sa) + (uint32_t)((s * MT + m) * a.a_bytes);
-          if (a.mode == TILE_FLAT) {
-            int row;
-            flat_first(a, tile, row);
-            for (int r = 0; r < a.nrows; ++r) {
-              const int T = row + r, b = T < 0 ? 0 : div_by(T, a.inv_h);
-              const int h = T < 0 ? -1 : T - b * (a.H + 1) - 1;
-              for (int p = 0; p < a.planes; ++p)
-                tma_load5(dst + p * a.ps + r * (a.W + 1) * RB, &xmap, 0, 0, h, b, p, &C.a_full[s]);
-            }
-          } else {
-            const int ty = a.tiles_x == 1 ? tile : div_by(tile, a.inv_x);
-            const int c = (tile - ty * a.tiles_x) * 8 - 1;
-            if (a.mode == TILE_WHOLE) {
-              const int b = a.tiles_y == 1 ? ty : div_by(ty, a.inv_y);
+    // ---- input tiles; the boxes of a tile are issued side by side, one per lane
+    int s = 0, ph = 1, it = 0;
+    for (int g = g0; g < groups; g += step, ++it) {
+      if (!warp_wait(&C.a_empty[s], ph, &C.fail)) break;
+      if (lane == 0) mbar_expect(&C.a_full[s], (uint32_t)(MT * a.a_tx));
+      __syncwarp();
+      for (int m = 0; m < MT; ++m) {
+        const int tile = g * MT + m;  // one past the last: rows outside the images, all zeros
+        const uint32_t dst = smem_u32(sa) + (uint32_t)((s * MT + m) * a.a_bytes);
+        if (a.mode == TILE_FLAT) {
+          int row;
+          flat_first(a, tile, row);
+          for (int q = lane; q < a.nrows * a.planes; q += 32) {
+            const int r = q / a.planes, p = q - r * a.planes;
+            const int T = row + r, b = T < 0 ? 0 : div_by(T, a.inv_h);
+            const int h = T < 0 ? -1 : T - b * (a.H + 1) - 1;
+            tma_load5(dst + p * a.ps + r * (a.W + 1) * RB, &xmap, 0, 0, h, b, p, &C.a_full[s]);
+          }
+        } else {
+          const int ty = a.tiles_x == 1 ? tile : div_by(tile, a.inv_x);
+          const int c = (tile - ty * a.tiles_x) * 8 - 1;
+          if (a.mode == TILE_WHOLE) {
+            const int b = a.tiles_y == 1 ? ty : div_by(ty, a.inv_y);
+            if (lane == 0)
               tma_load5(dst, &xmap, 0, c, (ty - b * a.tiles_y) * 16 - 1, b, 0, &C.a_full[s]);
-            } else {
-              for (int r = 0; r < 18; ++r) {
-                const int T = ty * 16 + r, b = div_by(T, a.inv_h);
-                tma_load5(dst + r * a.ky_st, &xmap, 0, c, T - b * (a.H + 1) - 1, b, 0, &C.a_full[s]);
-              }
-            }
+          } else if (lane < 18) {
+            const int T = ty * 16 + lane, b = div_by(T, a.inv_h);
+            tma_load5(dst + lane * a.ky_st, &xmap, 0, c, T - b * (a.H + 1) - 1, b, 0, &C.a_full[s]);
           }
         }
-        if (++s == a.na) {
-          s = 0;
-          ph ^= 1;
-        }
       }
-      // no copy outlives the CTA: wait for those of the last na tiles (bounded)
-      for (int q = max(0, it - a.na); q < it; ++q) mbar_wait(&C.a_full[q % a.na], (q / a.na) & 1);
+      if (++s == a.na) {
+        s = 0;
+        ph ^= 1;
+      }
     }
+    // no copy outlives the CTA: wait for those of the last na tiles (bounded)
+    for (int q = max(0, it - a.na); q < it; ++q) mbar_wait(&C.a_full[q % a.na], (q / a.na) & 1);
   } else if (warp == 9) {
     // ---- weights
     if (elect_one()) {
@@ -815,12 +816,13 @@ __global__ void __launch_bounds__(HB_THREADS, 1)
       const uint32_t whi = (uint32_t)(sw128_desc(0) >> 32), wlo0 = (uint32_t)sw128_desc(smem_u32(sw));
       const uint32_t sa0 = (smem_u32(sa) >> 4) | (RB == 16 ? 0u : 1u << 16), stage = (uint32_t)a.a_bytes >> 4;
       const uint32_t ps = (uint32_t)a.ps >> 4, wst = (uint32_t)a.nb * 8;  // in units of 16 bytes
-      constexpr int ROWS = RB == 16 ? 4 : 128 / RB;  // rows of a weight block
-      constexpr int PER = RB == 16 ? 1 : RB / 32;    // steps of a row
+      constexpr int ROWS = 128 / RB, PER = RB == 16 ? 1 : RB / 32;  // rows of a weight block, steps of a row
       const uint32_t ky_next = (uint32_t)((a.ky_st - 2 * RB) >> 4);  // from tap kx = 2 to the next row's 0
       int s = 0, sph = 0, ab = 0, abph = 1, ws = 0, wph = 0;
-      bool first = true;
-      for (int g = g0; g < groups; g += step) {
+      bool ok = true;
+      if (RES && g0 < groups)
+        for (int kb = 0; kb < a.kblocks && ok; ++kb) ok = thread_wait(&C.w_full[kb], 0, &C.fail);
+      for (int g = g0; g < groups && ok; g += step) {
         if (!thread_wait(&C.a_full[s], sph, &C.fail)) break;
         if (!thread_wait(&C.acc_empty[ab], abph, &C.fail)) break;
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
@@ -828,69 +830,91 @@ __global__ void __launch_bounds__(HB_THREADS, 1)
 #pragma unroll
         for (int m = 0; m < MT; ++m) {
           tap[m] = sa0 + (uint32_t)(s * MT + m) * stage;
-          if (a.mode == TILE_FLAT) {
+          if (PL == 0 && a.mode == TILE_FLAT) {
             int r;
             tap[m] += (uint32_t)(flat_first(a, g * MT + m, r) * (RB / 16));
           }
           row[m] = tap[m];
         }
         const uint32_t d0 = tmem + (uint32_t)(ab * MT * a.nbp);
-        int pl = 0, kx = 0, left = RB == 16 ? 5 : 9 * a.planes;
-        bool ok = true;
-        for (int kb = 0; kb < a.kblocks; ++kb) {
-          if (RES) {
-            if (first && !(ok = thread_wait(&C.w_full[kb], 0, &C.fail))) break;
-          } else if (!(ok = thread_wait(&C.w_full[ws], wph, &C.fail))) {
-            break;
+        auto w_next = [&]() {  // the ring's next block
+          tc_commit(&C.w_empty[ws]);
+          if (++ws == a.nw) {
+            ws = 0;
+            wph ^= 1;
           }
-          const uint32_t wd = wlo0 + (uint32_t)(RES ? kb : ws) * wst;
+        };
+        if constexpr (RB == 16) {
+          // 8 channels: taps 2 q and 2 q + 1 are the halves of step q (LBO apart), the
+          // zero plane the second half of the last
 #pragma unroll
-          for (int r = 0; r < ROWS; ++r) {
-            if constexpr (RB == 16) {
-              // 8 channels: taps 2 q and 2 q + 1 are the halves of step q (LBO apart), the
-              // zero plane the second half of the last
-              const int q = 4 * kb + r, t0 = 2 * q, t1 = t0 + 1;
-              if (q >= 5) continue;
-              const uint32_t o0 = (uint32_t)((t0 / 3) * 10 + t0 % 3);
-              const uint32_t o1 = t1 < 9 ? (uint32_t)((t1 / 3) * 10 + t1 % 3) : ps;
+          for (int q = 0; q < 5; ++q) {
+            const int t0 = 2 * q, t1 = t0 + 1;
+            const uint32_t o0 = (uint32_t)((t0 / 3) * 10 + t0 % 3);
+            const uint32_t o1 = t1 < 9 ? (uint32_t)((t1 / 3) * 10 + t1 % 3) : 180u;
+            if (!RES && (q & 3) == 0 && !(ok = thread_wait(&C.w_full[ws], wph, &C.fail))) break;
+            const uint32_t wd = wlo0 + (uint32_t)(RES ? q >> 2 : ws) * wst + 2 * (q & 3);
 #pragma unroll
-              for (int m = 0; m < MT; ++m)
-                tc_mma(d0 + m * a.nbp, (tap[m] + o0) | ((o1 - o0) << 16), ahi, wd + 2 * r, whi, idesc,
-                       r ? 1u : (uint32_t)(kb > 0));
-            } else if (ROWS == 1 || left > 0) {
+            for (int m = 0; m < MT; ++m)
+              tc_mma(d0 + m * a.nbp, (tap[m] + o0) | ((o1 - o0) << 16), ahi, wd, whi, idesc, q > 0);
+            if (!RES && ((q & 3) == 3 || q == 4)) w_next();
+          }
+        } else if constexpr (PL > 0) {
+          constexpr int PS = (TALL ? 10 : 180) * RB / 16, KY = (TALL ? PL * 10 : 10) * RB / 16;
+          constexpr int STEPS = 9 * PL * PER;
+          uint32_t wd = wlo0;
 #pragma unroll
-              for (int i = 0; i < PER; ++i)
+          for (int k = 0; k < STEPS; ++k) {
+            const int i = k % PER, r = k / PER, p = r % PL, t = r / PL;
+            const uint32_t o = (uint32_t)((t / 3) * KY + (t % 3) * (RB / 16) + p * PS + 2 * i);
+            if (k % 4 == 0) {
+              if (RES) {
+                if (k) wd += wst;
+              } else {
+                if (!(ok = thread_wait(&C.w_full[ws], wph, &C.fail))) break;
+                wd = wlo0 + (uint32_t)ws * wst;
+              }
+            }
 #pragma unroll
-                for (int m = 0; m < MT; ++m)
-                  tc_mma(d0 + m * a.nbp, row[m] + 2 * i, ahi, wd + 2 * (r * PER + i), whi, idesc,
-                         (r || i) ? 1u : (uint32_t)(kb > 0));
-              --left;
-              uint32_t adv = ps;
-              if (++pl == a.planes) {
-                pl = 0;
-                uint32_t t = RB / 16;
-                if (++kx == 3) {
-                  kx = 0;
-                  t = ky_next;
+            for (int m = 0; m < MT; ++m)
+              tc_mma(d0 + m * a.nbp, tap[m] + o, ahi, wd + 2 * (k % 4), whi, idesc, k > 0);
+            if (!RES && (k % 4 == 3 || k == STEPS - 1)) w_next();
+          }
+        } else {
+          int pl = 0, kx = 0, left = 9 * a.planes;
+          for (int kb = 0; kb < a.kblocks; ++kb) {
+            if (!RES && !(ok = thread_wait(&C.w_full[ws], wph, &C.fail))) break;
+            const uint32_t wd = wlo0 + (uint32_t)(RES ? kb : ws) * wst;
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) {
+              if (ROWS == 1 || left > 0) {
+#pragma unroll
+                for (int i = 0; i < PER; ++i)
+#pragma unroll
+                  for (int m = 0; m < MT; ++m)
+                    tc_mma(d0 + m * a.nbp, row[m] + 2 * i, ahi, wd + 2 * (r * PER + i), whi, idesc,
+                           (r || i) ? 1u : (uint32_t)(kb > 0));
+                --left;
+                uint32_t adv = ps;
+                if (++pl == a.planes) {
+                  pl = 0;
+                  uint32_t t = RB / 16;
+                  if (++kx == 3) {
+                    kx = 0;
+                    t = ky_next;
+                  }
+#pragma unroll
+                  for (int m = 0; m < MT; ++m) row[m] = tap[m] = tap[m] + t;
+                  adv = 0;
                 }
 #pragma unroll
-                for (int m = 0; m < MT; ++m) row[m] = tap[m] = tap[m] + t;
-                adv = 0;
+                for (int m = 0; m < MT; ++m) row[m] += adv;
               }
-#pragma unroll
-              for (int m = 0; m < MT; ++m) row[m] += adv;
             }
-          }
-          if (!RES) {
-            tc_commit(&C.w_empty[ws]);
-            if (++ws == a.nw) {
-              ws = 0;
-              wph ^= 1;
-            }
+            if (!RES) w_next();
           }
         }
         if (!ok) break;
-        first = false;
         tc_commit(&C.a_empty[s]);
         tc_commit(&C.acc_full[ab]);
         if (++s == a.na) {
@@ -1184,19 +1208,36 @@ cudaError_t allow_smem(K *kernel, std::atomic<unsigned long long> &done) {
   return e;
 }
 
-template <int RB, int MT, bool RES>
+template <int RB, int MT, bool RES, int PL, bool TALL>
 cudaError_t launch_halo(const HaloPlan &p, const CUtensorMap &wm, const CUtensorMap &xm, cudaStream_t st) {
   static std::atomic<unsigned long long> done{0};
-  cudaError_t e = allow_smem(k_conv3x3_halo<RB, MT, RES>, done);
+  cudaError_t e = allow_smem(k_conv3x3_halo<RB, MT, RES, PL, TALL>, done);
   if (e != cudaSuccess) return e;
-  k_conv3x3_halo<RB, MT, RES><<<p.grid, HB_THREADS, p.smem, st>>>(wm, xm, p.a);
+  k_conv3x3_halo<RB, MT, RES, PL, TALL><<<p.grid, HB_THREADS, p.smem, st>>>(wm, xm, p.a);
   return cudaGetLastError();
 }
-template <int RB>
-cudaError_t launch_halo_rb(const HaloPlan &p, const CUtensorMap &wm, const CUtensorMap &xm, cudaStream_t st) {
+template <int RB, int PL, bool TALL>
+cudaError_t launch_halo_pl(const HaloPlan &p, const CUtensorMap &wm, const CUtensorMap &xm, cudaStream_t st) {
   if (p.res)
-    return p.mt == 2 ? launch_halo<RB, 2, true>(p, wm, xm, st) : launch_halo<RB, 1, true>(p, wm, xm, st);
-  return p.mt == 2 ? launch_halo<RB, 2, false>(p, wm, xm, st) : launch_halo<RB, 1, false>(p, wm, xm, st);
+    return p.mt == 2 ? launch_halo<RB, 2, true, PL, TALL>(p, wm, xm, st)
+                     : launch_halo<RB, 1, true, PL, TALL>(p, wm, xm, st);
+  return p.mt == 2 ? launch_halo<RB, 2, false, PL, TALL>(p, wm, xm, st)
+                   : launch_halo<RB, 1, false, PL, TALL>(p, wm, xm, st);
+}
+cudaError_t launch_halo_plan(const HaloPlan &p, const CUtensorMap &wm, const CUtensorMap &xm, cudaStream_t st) {
+  const int m = p.a.mode, n = p.a.planes;
+  if (p.rb == 16) return launch_halo_pl<16, 0, false>(p, wm, xm, st);
+  if (p.rb == 32) return launch_halo_pl<32, 0, false>(p, wm, xm, st);
+  if (p.rb == 64) {
+    if (m == TILE_WHOLE && n == 1) return launch_halo_pl<64, 1, false>(p, wm, xm, st);
+    if (m == TILE_WHOLE && n == 3) return launch_halo_pl<64, 3, false>(p, wm, xm, st);
+    return launch_halo_pl<64, 0, false>(p, wm, xm, st);
+  }
+  if (m == TILE_WHOLE && n == 1) return launch_halo_pl<128, 1, false>(p, wm, xm, st);
+  if (m == TILE_WHOLE && n == 3) return launch_halo_pl<128, 3, false>(p, wm, xm, st);
+  if (m == TILE_TALL && n == 1) return launch_halo_pl<128, 1, true>(p, wm, xm, st);
+  if (m == TILE_TALL && n == 2) return launch_halo_pl<128, 2, true>(p, wm, xm, st);
+  return launch_halo_pl<128, 0, false>(p, wm, xm, st);
 }
 
 // true when the call was launched here (rc its status); false: not this kernel's
@@ -1220,9 +1261,7 @@ bool conv_halo(const ConvArgs &v, cudaStream_t st, cudaError_t &rc) {
   if (!encode_bf16(&wm, 2, v.w, wd, ws, wb, CU_TENSOR_MAP_SWIZZLE_128B) ||
       !encode_image(&xm, v.x, v.B, v.H, v.W, v.ldx, a.planes, p.rb, p.box_w, p.box_h, p.box_p))
     return false;
-  rc = p.rb == 128 ? launch_halo_rb<128>(p, wm, xm, st)
-     : p.rb == 64 ? launch_halo_rb<64>(p, wm, xm, st)
-     : p.rb == 32 ? launch_halo_rb<32>(p, wm, xm, st) : launch_halo_rb<16>(p, wm, xm, st);
+  rc = launch_halo_plan(p, wm, xm, st);
   return true;
 }
 
@@ -1617,6 +1656,552 @@ cudaError_t launch_wgrad_tc(const WgradArgs &a, int splits, cudaStream_t st) {
   dim3 grid((a.K + WTM - 1) / WTM, (a.N + BN - 1) / BN, splits);
   k_conv3x3_wgrad_tc<BN><<<grid, 128, tw_smem_bytes<BN>(), st>>>(a);
   return cudaGetLastError();
+}
+
+// --------------------------- weight gradient with the input tile resident
+// dW[o][tap][c] = sum_p dY[p][o] x[p + tap][c], K = pixels.  As in
+// k_conv3x3_halo a stage holds the halo of a 128-pixel tile of x, and beside it
+// the tile of dY; both are read MN-major (a pixel is a row of channels, the 8
+// pixels of a tile row a swizzle atom's 8 rows), so a tap is again a start
+// address shifted by whole slots.  The x side stacks taps: with 64-channel
+// planes two (the LBO is the distance of their slots), with 32-channel planes
+// the three of a tap row (a fourth atom is read and ignored), so that a block (plane,
+// taps) is one M = 128 operand and has its own accumulator of nb columns.
+// (Swapped sides, M = 64 outputs and N = 96, took 107 clocks a step for 32
+// outputs against 85.)  Blocks are dealt to the CTAs of grid x (512 columns of
+// TMEM hold 512 / nb of them), output-channel blocks to grid y, ranges of
+// tiles to grid z.  Every `flush` tiles (the 4096 to 8192 pixels of one chunk of
+// k_conv3x3_wgrad_tc, so that the tensor cores' FP32 sums stay as short) a
+// CTA adds its accumulators to its slot of the workspace; k_reduce_sums adds
+// the slots in order.  The CTAs of x = 0 also sum dY for the bias gradient
+// from the tiles they hold.
+// k_conv3x3_wgrad_tc fetches each x pixel nine times, in 16-byte copies, which
+// bound it, and needs the bias sums and two slow reductions beside it.  64
+// images, all of it, before and now: 32 -> 32 channels at 160 x 400 782 -> 150 us
+// (3.5 TB/s), 96 -> 32 1486 -> 389, 64 -> 64 at 80 x 200 413 -> 86, 128 -> 128 at
+// 40 x 100 281 -> 92, 768 -> 256 at 20 x 50 462 -> 198, 512 -> 512 at 10 x 25 255 ->
+// 111.  What remains is the MMAs' issue and, from 128 channels on, the tiles'
+// re-reading from L2 by the CTAs of grid x and y.
+// Roles: warps 0-7 bias sums and workspace (two groups of four, alternate
+// blocks), warp 8 MMAs, warp 9 tiles.
+constexpr int WH_THREADS = 320, WH_MAXA = 8;
+
+struct WgHaloArgs {
+  float *ws, *wsb;      // [slots][N][K], [slots][N] (null: no bias gradient)
+  int B, H, W, N, K, Cin;
+  int mode;             // TILE_*
+  int ky_st, sbo;       // x: strides of a tap row and 8 tile pixels (bytes)
+  int xps, yps, ysbo;   // plane strides of a stage's x and dY, 8 pixels of dY
+  int nrows;            // flat: image rows a stage holds
+  int tiles_x, tiles_y, tiles, range, flush;  // sub-tiles of 128 pixels; of a CTA; per flush
+  uint32_t inv_h, inv_w, inv_x, inv_y;
+  int blocks;           // x blocks in all
+  int xplanes, yplanes; // planes of a stage
+  int nb;               // output channels of a block, columns of an accumulator
+  int nacc;             // accumulator sets
+  int na, stage, y_at, cols, off_ctl;
+};
+
+struct WgHaloCtl {
+  uint64_t full[WH_MAXA], empty[WH_MAXA], acc_full[2], acc_empty[2], drain;
+  uint32_t tmem;
+  int fail;
+  float red[4][8][8][8];
+};
+
+// tensor maps of x and dY with boxes of 1, 2, 4 and 8 rows (a whole tile's rows in [0])
+struct WgMaps {
+  CUtensorMap x[4], y[4];
+};
+
+// Rows t0 .. t0 + n - 1 of the tall image in as few boxes as its images allow (a box may
+// take the zero rows above and below an image): issue(first row, h, image, log2 rows).
+// A box costs TMA about 75 clocks besides its bytes.
+template <class F>
+__device__ __forceinline__ void tall_rows(const WgHaloArgs &a, int t0, int n, F issue) {
+  for (int r = 0; r < n;) {
+    const int T = t0 + r, b = T < 0 ? 0 : div_by(T, a.inv_h), h = T < 0 ? -1 : T - b * (a.H + 1) - 1;
+    const int m = T < 0 ? 1 : min(n - r, a.H + 1 - h);
+    const int k = m >= 8 ? 3 : m >= 4 ? 2 : m >= 2 ? 1 : 0;
+    issue(r, h, b, k);
+    r += 1 << k;
+  }
+}
+
+template <int RBX, int RBY, int PER>
+__global__ void __launch_bounds__(WH_THREADS, 1)
+    k_wgrad_halo(const __grid_constant__ WgMaps maps, const WgHaloArgs a) {
+  extern __shared__ uint8_t wh_raw[];
+  uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(wh_raw) + 1023) &
+                                              ~(uintptr_t)1023);
+  WgHaloCtl &C = *reinterpret_cast<WgHaloCtl *>(base + a.off_ctl);
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  constexpr int TAPB = RBX == 128 ? 5 : 3;  // blocks of a plane
+  const int q0 = blockIdx.x * PER, nq = min(PER, a.blocks - q0), p0 = q0 / TAPB;
+  const int n0 = blockIdx.y * a.nb, z = blockIdx.z;
+  const int tbeg = z * a.range, tend = min(a.tiles, tbeg + a.range);
+  const bool bias = a.wsb && blockIdx.x == 0;
+
+  if (tid == 0) {
+    for (int s = 0; s < a.na; ++s) {
+      mbar_init(&C.full[s], 1);
+      mbar_init(&C.empty[s], bias ? 257 : 1);
+    }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&C.acc_full[s], 1);
+      mbar_init(&C.acc_empty[s], 256);
+    }
+    mbar_init(&C.drain, 1);
+    C.fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  if (warp == 8) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                     smem_u32(&C.tmem)),
+                 "r"(a.cols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+  const uint32_t tmem = __shfl_sync(0xffffffffu, C.tmem, 0);
+  const uint32_t sx = smem_u32(base), sy = sx + (uint32_t)a.y_at;
+
+  if (warp == 9) {
+    // ---- tiles of x (halo) and dY; lane = plane where a box holds one
+    const uint32_t bytes =
+        (uint32_t)(a.mode == TILE_FLAT ? a.nrows * (a.W + 1) * (a.xplanes * RBX + a.yplanes * RBY)
+                                       : a.xplanes * 180 * RBX + a.yplanes * 128 * RBY);
+    const int y0 = n0 / (RBY / 2);
+    int s = 0, ph = 1, it = 0;
+    for (int tile = tbeg; tile < tend; ++tile, ++it) {
+      if (!warp_wait(&C.empty[s], ph, &C.fail)) break;
+      uint64_t *bar = &C.full[s];
+      if (lane == 0) mbar_expect(bar, bytes);
+      __syncwarp();
+      const uint32_t dx = sx + (uint32_t)(s * a.stage), dy = sy + (uint32_t)(s * a.stage);
+      const int ty = a.tiles_x == 1 ? tile : div_by(tile, a.inv_x);
+      const int c = (tile - ty * a.tiles_x) * 8;
+      if (a.mode == TILE_WHOLE) {
+        const int b = a.tiles_y == 1 ? ty : div_by(ty, a.inv_y), h = (ty - b * a.tiles_y) * 16;
+        if (lane == 0) tma_load5(dx, &maps.x[0], 0, c - 1, h - 1, b, p0, bar);
+        if (lane == 1) tma_load5(dy, &maps.y[0], 0, c, h, b, y0, bar);
+      } else if (a.mode == TILE_TALL) {
+        tall_rows(a, ty * 16, 18, [&](int r, int h, int b, int k) {
+          if (lane < a.xplanes)
+            tma_load5(dx + lane * a.xps + r * a.ky_st, &maps.x[k], 0, c - 1, h, b, p0 + lane, bar);
+        });
+        tall_rows(a, ty * 16 + 1, 16, [&](int r, int h, int b, int k) {
+          if (lane < a.yplanes)
+            tma_load5(dy + lane * a.yps + r * a.ysbo, &maps.y[k], 0, c, h, b, y0 + lane, bar);
+        });
+      } else {
+        const int q = tile * 128 - 1;
+        tall_rows(a, q < 0 ? -1 : div_by(q, a.inv_w), a.nrows, [&](int r, int h, int b, int k) {
+          if (lane < a.xplanes)
+            tma_load5(dx + lane * a.xps + r * (a.W + 1) * RBX, &maps.x[k], 0, 0, h, b, p0 + lane, bar);
+          if (lane < a.yplanes)
+            tma_load5(dy + lane * a.yps + r * (a.W + 1) * RBY, &maps.y[k], 0, 0, h, b, y0 + lane, bar);
+        });
+      }
+      if (++s == a.na) {
+        s = 0;
+        ph ^= 1;
+      }
+    }
+    // no copy outlives the CTA
+    for (int q = max(0, it - a.na); q < it; ++q) mbar_wait(&C.full[q % a.na], (q / a.na) & 1);
+  } else if (warp == 8) {
+    // ---- MMAs
+    if (elect_one()) {
+      const uint32_t idesc = tc_idesc_mn(128, a.nb);
+      const uint32_t xhi = (uint32_t)(a.sbo >> 4) | (1u << 14) | ((RBX == 128 ? 2u : 4u) << 29);
+      const uint32_t yhi = (uint32_t)(a.ysbo >> 4) | (1u << 14) | ((RBY == 128 ? 2u : 4u) << 29);
+      const uint32_t ylbo = (uint32_t)(a.yps >> 4) << 16;
+      const uint32_t xst = (uint32_t)(2 * a.sbo) >> 4, yst = (uint32_t)(2 * a.ysbo) >> 4;
+      // x operand of each block, relative to the stage (units of 16 bytes), LBO in the high half
+      // (past the last block: the last again, into columns that nobody reads; the
+      // steps are straight-line code without tests, or their issue would bound them)
+      uint32_t off[PER];
+#pragma unroll
+      for (int j = 0; j < PER; ++j) {
+        const int q = q0 + min(j, nq - 1), pl = q / TAPB - p0, t = q % TAPB;
+        auto at = [&](int tap) { return (uint32_t)(((tap / 3) * a.ky_st + (tap % 3) * RBX) >> 4); };
+        uint32_t o, lbo;
+        if (RBX == 128) {
+          o = at(2 * t);
+          lbo = t < 4 ? at(2 * t + 1) - o : 0;  // the ninth tap stands alone
+        } else {
+          o = at(3 * t);
+          lbo = RBX >> 4;
+        }
+        off[j] = (o + (uint32_t)(pl * (a.xps >> 4))) | (lbo << 16);
+      }
+      int s = 0, ph = 0, ab = 0, abph = 1, left = 0;
+      bool ok = true;
+      for (int tile = tbeg; tile < tend; ++tile) {
+        uint32_t acc = 1;
+        if (left == 0) {  // a new set of sums
+          if (!(ok = thread_wait(&C.acc_empty[ab], abph, &C.fail))) break;
+          left = min(a.flush, tend - tile);
+          acc = 0;
+        }
+        if (!(ok = thread_wait(&C.full[s], ph, &C.fail))) break;
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        uint32_t ax = (sx + (uint32_t)(s * a.stage)) >> 4, by = ((sy + (uint32_t)(s * a.stage)) >> 4) | ylbo;
+        if (a.mode == TILE_FLAT) {
+          const int q = tile * 128 - 1, row = q < 0 ? -1 : div_by(q, a.inv_w);
+          const int f = q - row * (a.W + 1);
+          ax += (uint32_t)(f * (RBX >> 4));
+          by += (uint32_t)((f + a.W + 2) * (RBY >> 4));
+        }
+        const uint32_t d0 = tmem + (uint32_t)(ab * PER * a.nb);
+#pragma unroll
+        for (int i = 0; i < 8; ++i, ax += xst, by += yst) {
+#pragma unroll
+          for (int j = 0; j < PER; ++j)
+            tc_mma(d0 + (uint32_t)(j * a.nb), ax + off[j], xhi, by, yhi, idesc, i ? 1u : acc);
+        }
+        tc_commit(&C.empty[s]);
+        if (++s == a.na) {
+          s = 0;
+          ph ^= 1;
+        }
+        if (--left == 0) {
+          tc_commit(&C.acc_full[ab]);
+          if (++ab == a.nacc) {
+            ab = 0;
+            abph ^= 1;
+          }
+        }
+      }
+      tc_commit(&C.drain);
+      if (!mbar_wait(&C.drain, 0)) *(volatile int *)&C.fail = 2;
+    }
+  } else {
+    // ---- bias sums as the tiles pass, accumulators to the workspace as they fill
+    constexpr int CH = RBY / 16, RSTEP = 256 / CH;  // 16-byte chunks of a row; rows in a pass
+    const int e = warp >> 2, w4 = warp & 3, cc = tid % CH, r0 = tid / CH;
+    float sum[4][8];
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+      for (int k = 0; k < 8; ++k) sum[p][k] = 0.f;
+    float *out = a.ws + (size_t)z * a.N * a.K;
+    int s = 0, ph = 0, ab = 0, abph = 0;
+    bool ok = true;
+    for (int tile = tbeg; tile < tend && ok;) {
+      const int n = min(a.flush, tend - tile);
+      if (bias)
+        for (int k = 0; k < n && ok; ++k) {
+          if (!(ok = warp_wait(&C.full[s], ph, &C.fail))) break;
+          uint32_t yb = sy + (uint32_t)(s * a.stage);
+          if (a.mode == TILE_FLAT) {
+            const int q = (tile + k) * 128 - 1, row = q < 0 ? -1 : div_by(q, a.inv_w);
+            yb += (uint32_t)((q - row * (a.W + 1) + a.W + 2) * RBY);
+          }
+#pragma unroll
+          for (int p = 0; p < 4; ++p) {
+            if (p >= a.yplanes) break;
+#pragma unroll
+            for (int r = 0; r < 128 / RSTEP; ++r) {
+              const uint32_t ad = yb + (uint32_t)(p * a.yps + (r0 + r * RSTEP) * RBY);
+              const uint32_t x = RBY == 128 ? (ad >> 7) & 7 : (ad >> 7) & 3;  // swizzle, by address
+              uint32_t w[4];
+              asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];\n"
+                           : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
+                           : "r"(ad + ((cc ^ x) << 4)));
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                sum[p][2 * q] += bf2f((bf16_t)(w[q] & 0xffff));
+                sum[p][2 * q + 1] += bf2f((bf16_t)(w[q] >> 16));
+              }
+            }
+          }
+          mbar_arrive(&C.empty[s]);
+          if (++s == a.na) {
+            s = 0;
+            ph ^= 1;
+          }
+        }
+      // unit u: 32 columns of a block.  What the slot holds already is read a unit
+      // ahead (the first before the sums are in), so that its latency is hidden.
+      const bool add = tile > tbeg;
+      const int ncb = a.nb / 32, units = nq * ncb;
+      auto dest = [&](int u) -> float * {
+        const int j = u / ncb, cb = (u - j * ncb) * 32;
+        const int q = q0 + j, pl = q / TAPB, t = q - pl * TAPB;
+        const int tap = RBX == 128 ? 2 * t + (w4 >> 1) : 3 * t + w4;
+        const int c = RBX == 128 ? pl * 64 + (w4 & 1) * 32 + lane : pl * 32 + lane;
+        if (u >= units || (RBX == 128 ? tap >= 9 : w4 >= 3)) return nullptr;
+        return out + (size_t)(n0 + cb) * a.K + tap * a.Cin + c;
+      };
+      float old[32];
+      float *d = dest(e);
+      auto fetch = [&](const float *from) {
+#pragma unroll
+        for (int k = 0; k < 32; ++k) old[k] = add && from ? from[(size_t)k * a.K] : 0.f;
+      };
+      fetch(d);
+      if (!ok || !(ok = warp_wait(&C.acc_full[ab], abph, &C.fail))) break;
+      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+      const uint32_t t0 = tmem + ((uint32_t)(w4 * 32) << 16) + (uint32_t)(ab * PER * a.nb);
+      for (int u = e; u < units; u += 2) {
+        uint32_t r[32];
+        __syncwarp();
+        tmem_ld32(t0 + (uint32_t)(u * 32), r);
+        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+        float *now = d;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) r[k] = __float_as_uint(__uint_as_float(r[k]) + old[k]);
+        d = dest(u + 2);
+        fetch(d);
+        if (now) {
+#pragma unroll
+          for (int k = 0; k < 32; ++k) now[(size_t)k * a.K] = __uint_as_float(r[k]);
+        }
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+      __syncwarp();
+      mbar_arrive(&C.acc_empty[ab]);
+      if (++ab == a.nacc) {
+        ab = 0;
+        abph ^= 1;
+      }
+      tile += n;
+    }
+    if (bias) {
+      // over the pixel rows: lanes first, then the warps' sums in order
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        if (p >= a.yplanes) break;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          float v = sum[p][k];
+#pragma unroll
+          for (int o = CH; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          if (lane < CH) C.red[p][warp][lane][k] = v;
+        }
+      }
+      asm volatile("bar.sync 1, 256;\n" ::: "memory");
+      for (int n = tid; n < a.yplanes * (RBY / 2); n += 256) {
+        const int p = n / (RBY / 2), c = (n % (RBY / 2)) >> 3, k = n & 7;
+        float v = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) v += C.red[p][w][c][k];
+        a.wsb[(size_t)z * a.N + n0 + n] = v;
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+  __syncthreads();
+  if (tid == 0 && C.fail) atomicAdd(&g_tc_timeouts, 1);
+  if (warp == 8 && C.fail != 2)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(a.cols));
+}
+
+// Sums over chunks in a fixed order: out[i] = sum_z ws[z][i] for i < n, and out2[i] =
+// sum_z ws2[z][i] for i < n2.  G groups of 256 / G threads take every G-th chunk, and
+// their sums are added in order: eight groups of a warp for many chunks (one
+// thread per output walking up to 512 chunks left most of the GPU idle, 51 us for 9,216
+// outputs), one group for few.
+template <int G>
+__global__ void __launch_bounds__(256) k_reduce_sums(const float *ws, long n, float *out, const float *ws2,
+                                                     int n2, float *out2, int chunks) {
+  constexpr int L = 256 / G;
+  __shared__ float red[G][L];
+  const int l = threadIdx.x % L, g = threadIdx.x / L;
+  const long nb1 = (n + L - 1) / L, nb2 = (n2 + L - 1) / L;
+  for (long b = blockIdx.x; b < nb1 + nb2; b += gridDim.x) {
+    const bool second = b >= nb1;
+    const float *src = second ? ws2 : ws;
+    const long m = second ? n2 : n, i = (second ? b - nb1 : b) * L + l;
+    float s = 0.f;
+    if (i < m)
+      for (int z = g; z < chunks; z += G) s += src[(size_t)z * m + i];
+    if (G > 1) {
+      red[g][l] = s;
+      __syncthreads();
+      if (g == 0) {
+#pragma unroll
+        for (int k = 1; k < G; ++k) s += red[k][l];
+      }
+    }
+    if (g == 0 && i < m) (second ? out2 : out)[i] = s;
+    if (G > 1) __syncthreads();
+  }
+}
+
+struct WgHaloPlan {
+  WgHaloArgs a;
+  int rbx, rby, per, slots, gx, gy, box_w, box_h, box_p, ybox_w, ybox_h, ybox_p;
+  size_t smem;
+};
+
+// Chooses the tiling, the output-channel block (nb), the blocks of a CTA (per)
+// and the tile ranges, at most `most` of them (the workspace's slots), by an
+// estimate in clocks like halo_plan's.
+bool wgrad_halo_plan(const WgradArgs &v, int most, WgHaloPlan &best) {
+  if ((v.Cin & 31) || (v.N & 31)) return false;
+  const int rbx = v.Cin & 63 ? 64 : 128, rby = v.N & 63 ? 64 : 128;
+  auto up = [](long n, long d) { return (n + d - 1) / d; };
+  auto inv = [](long d) { return (uint32_t)(((1ull << 32) + d - 1) / d); };
+  const long rows = (long)v.B * (v.H + 1) - 1;
+  const int tapb = rbx == 128 ? 5 : 3, planes = v.Cin * 2 / rbx;
+  double best_c = 0.0;
+  bool found = false;
+  for (int mode : {TILE_WHOLE, TILE_TALL, TILE_FLAT}) {
+    WgHaloArgs a{};
+    a.mode = mode;
+    a.tiles_x = (int)up(v.W, 8);
+    a.tiles_y = (int)up(v.H, 16);
+    long tiles;
+    double boxes = 0.0;  // TMA boxes of a plane of x and one of dY
+    if (mode == TILE_FLAT) {
+      if (v.W > 30 || rbx != 128 || rby != 128) continue;
+      a.tiles_x = 1;
+      tiles = up(rows * (v.W + 1), 128);
+      a.nrows = (v.W + 128 + 2 * (v.W + 2) - 1) / (v.W + 1) + 1;
+      a.ky_st = (v.W + 1) * rbx;
+      a.sbo = 8 * rbx;
+      a.xps = a.yps = a.nrows * a.ky_st;
+      boxes = v.H >= 8 ? 8.0 : 2.0 * a.nrows;
+    } else {
+      tiles = (mode == TILE_WHOLE ? (long)v.B * a.tiles_y : up(rows, 16)) * a.tiles_x;
+      a.ky_st = a.sbo = 10 * rbx;
+      a.xps = 180 * rbx;
+      a.yps = 128 * rby;
+      if (mode == TILE_TALL) boxes = v.H >= 8 ? 11.0 : 34.0;
+    }
+    a.ysbo = 8 * rby;
+    a.tiles = (int)tiles;
+    if ((rows + 40) * (v.W + 1) + 256 >= (1L << 32) / (v.W + 1) || (rows + 40) * (v.H + 1) >= (1L << 32) ||
+        (tiles + 2) * a.tiles_x >= (1L << 32) || (tiles + 2) * a.tiles_y >= (1L << 32) || tiles > (1L << 30))
+      continue;
+    a.inv_h = inv(v.H + 1);
+    a.inv_w = inv(v.W + 1);
+    a.inv_x = inv(a.tiles_x);
+    a.inv_y = inv(a.tiles_y);
+    a.blocks = planes * tapb;
+    for (int nb : {32, 64, 128, 256}) {
+      if (nb > v.N || v.N % nb || nb % (rby / 2) || nb / (rby / 2) > 4) continue;
+      const int ny = v.N / nb;
+      for (int per : {9, 5, 4, 3, 2, 1}) {
+        if (per * nb > 512 || per > a.blocks) continue;
+        const int gx = (int)up(a.blocks, per);
+        if (gx * ny > 4 * kSms) continue;
+        int xpl = 1;  // planes that a CTA's blocks touch
+        for (int q = 0; q < a.blocks; q += per) {
+          const int last = q + per < a.blocks ? q + per - 1 : a.blocks - 1;
+          if (last / tapb - q / tapb + 1 > xpl) xpl = last / tapb - q / tapb + 1;
+        }
+        const int ypl = nb / (rby / 2);
+        const long y_at = ((long)xpl * a.xps + 1023) & ~1023L;
+        const long stage = (y_at + (long)ypl * a.yps + 1023) & ~1023L;
+        const int nacc = 2 * per * nb <= 512 ? 2 : 1;
+        int cols = 32;
+        while (cols < nacc * per * nb) cols <<= 1;
+        int na = WH_MAXA;
+        while (na && 1024 + 128 + (long)sizeof(WgHaloCtl) + na * stage > (long)kSmemMax) --na;
+        if (na < 2) continue;
+        long z = kSms / (gx * ny);
+        if (z < 1) z = 1;
+        if (z > most) z = most;
+        if (z > tiles) z = tiles;
+        const long range = up(tiles, z);
+        z = up(tiles, range);
+        const long nf = up(range, up(tiles, most));  // flushes of a range
+        const double mma = 8.0 * per * fmax(0.53 * nb, 32.0 + 0.25 * nb) + 300.0;
+        const double load = (double)(xpl * a.xps + ypl * a.yps) / 45.0 + 75.0 * boxes * 0.5 * (xpl + ypl);
+        const double flush = per * (nb / 32) * 400.0 + 2000.0;
+        const double c = (double)up(z * gx * ny, kSms) *
+                         (range * fmax(mma, load) + (nacc == 2 ? 1 : nf) * flush + 4000.0);
+        if (found && c >= best_c) continue;
+        found = true;
+        best_c = c;
+        best.a = a;
+        best.a.range = (int)range;
+        best.a.flush = (int)up(range, nf);
+        best.a.xplanes = xpl;
+        best.a.yplanes = ypl;
+        best.a.nb = nb;
+        best.a.nacc = nacc;
+        best.a.na = na;
+        best.a.stage = (int)stage;
+        best.a.y_at = (int)y_at;
+        best.a.cols = cols;
+        best.a.off_ctl = (int)((na * stage + 127) & ~127L);
+        best.smem = 1024 + best.a.off_ctl + sizeof(WgHaloCtl);
+        best.per = per;
+        best.slots = (int)z;
+        best.gx = gx;
+        best.gy = ny;
+      }
+    }
+  }
+  if (!found) return false;
+  best.rbx = rbx;
+  best.rby = rby;
+  const int m = best.a.mode;
+  best.box_w = m == TILE_FLAT ? v.W + 1 : 10;
+  best.ybox_w = m == TILE_FLAT ? v.W + 1 : 8;
+  best.box_h = m == TILE_WHOLE ? 18 : 1;
+  best.ybox_h = m == TILE_WHOLE ? 16 : 1;
+  best.box_p = m == TILE_WHOLE ? best.a.xplanes : 1;
+  best.ybox_p = m == TILE_WHOLE ? best.a.yplanes : 1;
+  return true;
+}
+
+template <int RBX, int RBY, int PER>
+cudaError_t launch_wgrad_per(const WgHaloPlan &p, const WgMaps &m, cudaStream_t st) {
+  static std::atomic<unsigned long long> done{0};
+  cudaError_t e = allow_smem(k_wgrad_halo<RBX, RBY, PER>, done);
+  if (e != cudaSuccess) return e;
+  k_wgrad_halo<RBX, RBY, PER><<<dim3(p.gx, p.gy, p.slots), WH_THREADS, p.smem, st>>>(m, p.a);
+  return cudaGetLastError();
+}
+template <int RBX, int RBY>
+cudaError_t launch_wgrad_halo(const WgHaloPlan &p, const WgMaps &m, cudaStream_t st) {
+  switch (p.per) {
+    case 9: return launch_wgrad_per<RBX, RBY, 9>(p, m, st);
+    case 5: return launch_wgrad_per<RBX, RBY, 5>(p, m, st);
+    case 4: return launch_wgrad_per<RBX, RBY, 4>(p, m, st);
+    case 3: return launch_wgrad_per<RBX, RBY, 3>(p, m, st);
+    case 2: return launch_wgrad_per<RBX, RBY, 2>(p, m, st);
+    default: return launch_wgrad_per<RBX, RBY, 1>(p, m, st);
+  }
+}
+
+// weight partials (and, when db, bias partials into wsb) of every tile range;
+// slots their number; with one slot the gradients themselves
+bool wgrad_halo(const WgradArgs &v, int most, float *wsb, float *dw, float *db, cudaStream_t st, int &slots,
+                cudaError_t &rc) {
+  WgHaloPlan p;
+  if (!wgrad_halo_plan(v, most, p)) return false;
+  WgMaps m;
+  for (int k = 0; k < 4; ++k) {
+    const int whole = p.a.mode == TILE_WHOLE;
+    if (whole && k) {
+      m.x[k] = m.x[0];
+      m.y[k] = m.y[0];
+    } else if (!encode_image(&m.x[k], v.x, v.B, v.H, v.W, v.ldx, v.Cin * 2 / p.rbx, p.rbx, p.box_w,
+                             whole ? p.box_h : 1 << k, p.box_p) ||
+               !encode_image(&m.y[k], v.dy, v.B, v.H, v.W, v.lddy, v.N * 2 / p.rby, p.rby, p.ybox_w,
+                             whole ? p.ybox_h : 1 << k, p.ybox_p)) {
+      return false;
+    }
+  }
+  WgHaloArgs &a = p.a;
+  a.ws = p.slots == 1 ? dw : v.ws;
+  a.wsb = !db ? nullptr : p.slots == 1 ? db : wsb;
+  a.B = v.B; a.H = v.H; a.W = v.W; a.N = v.N; a.K = v.K; a.Cin = v.Cin;
+  slots = p.slots;
+  rc = p.rbx == 128 ? (p.rby == 128 ? launch_wgrad_halo<128, 128>(p, m, st)
+                                    : launch_wgrad_halo<128, 64>(p, m, st))
+                    : (p.rby == 128 ? launch_wgrad_halo<64, 128>(p, m, st)
+                                    : launch_wgrad_halo<64, 64>(p, m, st));
+  return true;
 }
 
 // ------------------------------------------------------------- elementwise
@@ -2027,6 +2612,20 @@ int cem_sg_conv3x3_wgrad(const void *x, int ldx, const void *dy, int lddy, int B
   splits = (a.P + a.chunk - 1) / a.chunk;
   const long nw = (long)Cout * a.K;
   if (g_use_tc) {
+    cudaError_t he;
+    int hs;
+    // the bias partials lie behind the weight partials of `splits` chunks
+    float *wsb = a.ws + (size_t)splits * Cout * a.K;
+    if (wgrad_halo(a, splits, wsb, dw, db, st, hs, he)) {
+      if (he != cudaSuccess) return CEM_SG_ERR_CUDA;
+      if (hs == 1) return CEM_SG_OK;  // the kernel wrote dw and db
+      const int per = hs >= 16 ? 32 : 256;  // outputs of a block
+      const long nblk = (nw + per - 1) / per + (db ? (Cout + per - 1) / per : 0);
+      const int g = (int)(nblk < 8 * 1216 ? nblk : 8 * 1216), n2 = db ? Cout : 0;
+      if (hs >= 16) k_reduce_sums<8><<<g, 256, 0, st>>>(a.ws, nw, dw, wsb, n2, db, hs);
+      else k_reduce_sums<1><<<g, 256, 0, st>>>(a.ws, nw, dw, wsb, n2, db, hs);
+      return cudaGetLastError() == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
+    }
     // tcgen05: dW^T tiles of 128 k' x BN outputs; bias sums by a separate
     // coalesced reduction into the workspace after the weight partials
     a.wsb = nullptr;

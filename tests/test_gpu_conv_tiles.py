@@ -63,3 +63,48 @@ def test_conv_tilings(B, H, W, cin, cout):
         # nothing beside the slice is written
         assert bool((y[:, :pad] == 7).all()) and bool((y[:, pad + cout:] == 7).all())
     assert surrogate.timeouts() == t0
+
+
+# the same tilings for the weight gradient; 64 x 9 x 31 and 5 x 160 x 100 take several
+# tile ranges and workspace slots, 2 x 64 x 640 several flushes of a range
+@pytest.mark.parametrize("B,H,W", [(1, 16, 8), (2, 17, 33), (5, 20, 50), (7, 10, 25), (9, 3, 31), (3, 1, 1),
+                                   (2, 1, 64), (64, 9, 31), (5, 160, 100), (2, 64, 640)])
+@pytest.mark.parametrize("cin,cout", [(32, 32), (96, 32), (32, 64), (64, 64), (192, 96), (64, 128), (128, 256),
+                                      (512, 64), (24, 40)])
+@pytest.mark.parametrize("with_bias", [True, False])
+def test_wgrad_tilings(B, H, W, cin, cout, with_bias):
+    import torch
+    from paper_2509_01827_gb300 import build, surrogate
+    build.build()
+    L = surrogate.sg()
+    dev = "cuda"
+    g = torch.Generator(device=dev).manual_seed(B * 1000 + cin)
+    P, ld = B * H * W, cin + 16
+    x = torch.randn(P, ld, device=dev, generator=g).bfloat16()[:, 8:8 + cin]  # a channel slice
+    dy = torch.randn(P, cout, device=dev, generator=g).bfloat16()
+    need = L.cem_sg_wgrad_workspace(B, H, W, cin, cout)
+    ws = torch.full((need + 64,), 0xff, dtype=torch.uint8, device=dev)  # NaNs, and a guard behind
+    dw = torch.full((cout, 3, 3, cin), float("nan"), device=dev)
+    db = torch.full((cout,), float("nan"), device=dev)
+    t0 = surrogate.timeouts()
+    rc = L.cem_sg_conv3x3_wgrad(x.data_ptr(), ld, dy.data_ptr(), cout, B, H, W, cin, cout, dw.data_ptr(),
+                                db.data_ptr() if with_bias else None, ws.data_ptr(), need,
+                                torch.cuda.current_stream().cuda_stream)
+    assert rc == 0 and surrogate.timeouts() == t0
+    assert bool((ws[need:] == 0xff).all())
+    x64, y64 = x.double().view(B, H, W, cin), dy.double().view(B, H, W, cout)
+    p = torch.zeros(B, H + 2, W + 2, cin, dtype=torch.float64, device=dev)
+    p[:, 1:-1, 1:-1] = x64
+    yf = y64.reshape(P, cout)
+    for ky in range(3):
+        for kx in range(3):
+            w = p[:, ky:ky + H, kx:kx + W].reshape(P, cin)
+            # FP32 sums of at most 8192 pixels in steps of 16, each step at most 2^-23
+            # of the magnitudes off
+            tol = 512 * 2.0 ** -23 * (yf.abs().T @ w.abs()) + 1e-30
+            assert bool(((dw[:, ky, kx].double() - yf.T @ w).abs() <= tol).all()), (ky, kx)
+    if with_bias:
+        tol = 512 * 2.0 ** -23 * yf.abs().sum(0) + 1e-30
+        assert bool(((db.double() - yf.sum(0)).abs() <= tol).all())
+    else:
+        assert bool(torch.isnan(db).all())
