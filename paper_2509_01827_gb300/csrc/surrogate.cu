@@ -1378,16 +1378,6 @@ __global__ void __launch_bounds__(256) k_conv3x3_wgrad(WgradArgs a) {
     }
 }
 
-// out[i] = sum_z ws[z][i] in z order
-__global__ void k_reduce_splits(const float *ws, int splits, long n, float *out) {
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    float s = 0.f;
-    for (int z = 0; z < splits; ++z) s += ws[(size_t)z * n + i];
-    out[i] = s;
-  }
-}
-
-
 // ------------------------------------------- weight gradient on tcgen05
 // dW^T[k'][o] = sum_p A[p][k'] dY[p][o] with k' = (ky * 3 + kx) * Cin + c and
 // A the shifted input (zero outside the image): M = k' (128 per CTA), N = o
@@ -1665,8 +1655,9 @@ cudaError_t launch_wgrad_tc(const WgradArgs &a, int splits, cudaStream_t st) {
 // pixels of a tile row a swizzle atom's 8 rows), so a tap is again a start
 // address shifted by whole slots.  The x side stacks taps: with 64-channel
 // planes two (the LBO is the distance of their slots), with 32-channel planes
-// the three of a tap row (a fourth atom is read and ignored), so that a block (plane,
-// taps) is one M = 128 operand and has its own accumulator of nb columns.
+// the three of a tap row (a fourth atom is read and ignored; of 8 channels, unswizzled,
+// sixteen slots are), so that a block (plane, taps) is one M = 128 operand and has
+// its own accumulator of nb columns.
 // (Swapped sides, M = 64 outputs and N = 96, took 107 clocks a step for 32
 // outputs against 85.)  Blocks are dealt to the CTAs of grid x (512 columns of
 // TMEM hold 512 / nb of them), output-channel blocks to grid y, ranges of
@@ -1677,8 +1668,8 @@ cudaError_t launch_wgrad_tc(const WgradArgs &a, int splits, cudaStream_t st) {
 // from the tiles they hold.
 // k_conv3x3_wgrad_tc fetches each x pixel nine times, in 16-byte copies, which
 // bound it, and needs the bias sums and two slow reductions beside it.  64
-// images, all of it, before and now: 32 -> 32 channels at 160 x 400 782 -> 150 us
-// (3.5 TB/s), 96 -> 32 1486 -> 389, 64 -> 64 at 80 x 200 413 -> 86, 128 -> 128 at
+// images, all of it, before and now: 8 -> 32 channels at 160 x 400 387 -> 155 us, 32 -> 32
+// 782 -> 150 (3.5 TB/s), 96 -> 32 1486 -> 389, 64 -> 64 at 80 x 200 413 -> 86, 128 -> 128 at
 // 40 x 100 281 -> 92, 768 -> 256 at 20 x 50 462 -> 198, 512 -> 512 at 10 x 25 255 ->
 // 111.  What remains is the MMAs' issue and, from 128 channels on, the tiles'
 // re-reading from L2 by the CTAs of grid x and y.
@@ -1816,7 +1807,9 @@ __global__ void __launch_bounds__(WH_THREADS, 1)
     // ---- MMAs
     if (elect_one()) {
       const uint32_t idesc = tc_idesc_mn(128, a.nb);
-      const uint32_t xhi = (uint32_t)(a.sbo >> 4) | (1u << 14) | ((RBX == 128 ? 2u : 4u) << 29);
+      // 8 channels: unswizzled, SBO steps through M (a slot), LBO through K (a tile row)
+      const uint32_t xhi = RBX == 16 ? 1u | (1u << 14)
+                                     : (uint32_t)(a.sbo >> 4) | (1u << 14) | ((RBX == 128 ? 2u : 4u) << 29);
       const uint32_t yhi = (uint32_t)(a.ysbo >> 4) | (1u << 14) | ((RBY == 128 ? 2u : 4u) << 29);
       const uint32_t ylbo = (uint32_t)(a.yps >> 4) << 16;
       const uint32_t xst = (uint32_t)(2 * a.sbo) >> 4, yst = (uint32_t)(2 * a.ysbo) >> 4;
@@ -1834,7 +1827,7 @@ __global__ void __launch_bounds__(WH_THREADS, 1)
           lbo = t < 4 ? at(2 * t + 1) - o : 0;  // the ninth tap stands alone
         } else {
           o = at(3 * t);
-          lbo = RBX >> 4;
+          lbo = RBX == 64 ? RBX >> 4 : (uint32_t)a.sbo >> 4;
         }
         off[j] = (o + (uint32_t)(pl * (a.xps >> 4))) | (lbo << 16);
       }
@@ -1932,9 +1925,9 @@ __global__ void __launch_bounds__(WH_THREADS, 1)
       auto dest = [&](int u) -> float * {
         const int j = u / ncb, cb = (u - j * ncb) * 32;
         const int q = q0 + j, pl = q / TAPB, t = q - pl * TAPB;
-        const int tap = RBX == 128 ? 2 * t + (w4 >> 1) : 3 * t + w4;
-        const int c = RBX == 128 ? pl * 64 + (w4 & 1) * 32 + lane : pl * 32 + lane;
-        if (u >= units || (RBX == 128 ? tap >= 9 : w4 >= 3)) return nullptr;
+        const int tap = RBX == 128 ? 2 * t + (w4 >> 1) : RBX == 64 ? 3 * t + w4 : 3 * t + (lane >> 3);
+        const int c = RBX == 128 ? pl * 64 + (w4 & 1) * 32 + lane : RBX == 64 ? pl * 32 + lane : lane & 7;
+        if (u >= units || (RBX == 128 ? tap >= 9 : RBX == 64 ? w4 >= 3 : w4 > 0 || lane >= 24)) return nullptr;
         return out + (size_t)(n0 + cb) * a.K + tap * a.Cin + c;
       };
       float old[32];
@@ -2033,6 +2026,15 @@ __global__ void __launch_bounds__(256) k_reduce_sums(const float *ws, long n, fl
   }
 }
 
+void reduce_sums(const float *ws, long n, float *out, const float *ws2, int n2, float *out2, int chunks,
+                 cudaStream_t st) {
+  const int per = chunks >= 16 ? 32 : 256;  // outputs of a block
+  const long nblk = (n + per - 1) / per + (n2 + per - 1) / per;
+  const int g = (int)(nblk < 8 * 1216 ? nblk : 8 * 1216);
+  if (chunks >= 16) k_reduce_sums<8><<<g, 256, 0, st>>>(ws, n, out, ws2, n2, out2, chunks);
+  else k_reduce_sums<1><<<g, 256, 0, st>>>(ws, n, out, ws2, n2, out2, chunks);
+}
+
 struct WgHaloPlan {
   WgHaloArgs a;
   int rbx, rby, per, slots, gx, gy, box_w, box_h, box_p, ybox_w, ybox_h, ybox_p;
@@ -2043,8 +2045,8 @@ struct WgHaloPlan {
 // and the tile ranges, at most `most` of them (the workspace's slots), by an
 // estimate in clocks like halo_plan's.
 bool wgrad_halo_plan(const WgradArgs &v, int most, WgHaloPlan &best) {
-  if ((v.Cin & 31) || (v.N & 31)) return false;
-  const int rbx = v.Cin & 63 ? 64 : 128, rby = v.N & 63 ? 64 : 128;
+  if (((v.Cin & 31) && v.Cin != 8) || (v.N & 31)) return false;
+  const int rbx = v.Cin == 8 ? 16 : v.Cin & 63 ? 64 : 128, rby = v.N & 63 ? 64 : 128;
   auto up = [](long n, long d) { return (n + d - 1) / d; };
   auto inv = [](long d) { return (uint32_t)(((1ull << 32) + d - 1) / d); };
   const long rows = (long)v.B * (v.H + 1) - 1;
@@ -2068,6 +2070,7 @@ bool wgrad_halo_plan(const WgradArgs &v, int most, WgHaloPlan &best) {
       a.xps = a.yps = a.nrows * a.ky_st;
       boxes = v.H >= 8 ? 8.0 : 2.0 * a.nrows;
     } else {
+      if (mode == TILE_TALL && rbx == 16) continue;  // its rows do not start on 128 bytes
       tiles = (mode == TILE_WHOLE ? (long)v.B * a.tiles_y : up(rows, 16)) * a.tiles_x;
       a.ky_st = a.sbo = 10 * rbx;
       a.xps = 180 * rbx;
@@ -2088,7 +2091,7 @@ bool wgrad_halo_plan(const WgradArgs &v, int most, WgHaloPlan &best) {
       if (nb > v.N || v.N % nb || nb % (rby / 2) || nb / (rby / 2) > 4) continue;
       const int ny = v.N / nb;
       for (int per : {9, 5, 4, 3, 2, 1}) {
-        if (per * nb > 512 || per > a.blocks) continue;
+        if (per * nb > 512 || per > a.blocks || (rbx == 16 && per != 3 && per != 1)) continue;
         const int gx = (int)up(a.blocks, per);
         if (gx * ny > 4 * kSms) continue;
         int xpl = 1;  // planes that a CTA's blocks touch
@@ -2163,7 +2166,9 @@ cudaError_t launch_wgrad_per(const WgHaloPlan &p, const WgMaps &m, cudaStream_t 
 }
 template <int RBX, int RBY>
 cudaError_t launch_wgrad_halo(const WgHaloPlan &p, const WgMaps &m, cudaStream_t st) {
-  switch (p.per) {
+  if constexpr (RBX == 16)
+    return p.per == 3 ? launch_wgrad_per<16, RBY, 3>(p, m, st) : launch_wgrad_per<16, RBY, 1>(p, m, st);
+  else switch (p.per) {
     case 9: return launch_wgrad_per<RBX, RBY, 9>(p, m, st);
     case 5: return launch_wgrad_per<RBX, RBY, 5>(p, m, st);
     case 4: return launch_wgrad_per<RBX, RBY, 4>(p, m, st);
@@ -2199,8 +2204,10 @@ bool wgrad_halo(const WgradArgs &v, int most, float *wsb, float *dw, float *db, 
   slots = p.slots;
   rc = p.rbx == 128 ? (p.rby == 128 ? launch_wgrad_halo<128, 128>(p, m, st)
                                     : launch_wgrad_halo<128, 64>(p, m, st))
-                    : (p.rby == 128 ? launch_wgrad_halo<64, 128>(p, m, st)
-                                    : launch_wgrad_halo<64, 64>(p, m, st));
+     : p.rbx == 64 ? (p.rby == 128 ? launch_wgrad_halo<64, 128>(p, m, st)
+                                   : launch_wgrad_halo<64, 64>(p, m, st))
+                   : (p.rby == 128 ? launch_wgrad_halo<16, 128>(p, m, st)
+                                   : launch_wgrad_halo<16, 64>(p, m, st));
   return true;
 }
 
@@ -2234,130 +2241,164 @@ __device__ __forceinline__ uint4 pack8(const float f[8]) {
 __device__ __forceinline__ uint4 ld8(const bf16_t *p) { return *reinterpret_cast<const uint4 *>(p); }
 __device__ __forceinline__ void st8(bf16_t *p, uint4 v) { *reinterpret_cast<uint4 *>(p) = v; }
 
+// They are bound by HBM, so a thread's index work must stay small: a block row
+// (blockIdx.y, strided) is one image row, its threads walk (pixel, 8 channels) with one
+// 32-bit division.  (One flat 64-bit index and three 64-bit divisions took 299 us
+// for the level-0 pooling gradient of 64 images, this 210, 4 TB/s; upsampling 162 ->
+// 97.)
+
 // 2x2 max pooling: x [B, 2H, 2W] (pixel stride ldx) -> y [B, H, W, C] dense
-__global__ void k_maxpool2(const bf16_t *x, int ldx, int B, int H, int W, int C, bf16_t *y) {
-  const int C8 = C >> 3;
-  const long n = (long)B * H * W * C8;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const int c = (int)(i % C8) * 8;
-    const long pix = i / C8;
-    const int w = (int)(pix % W), h = (int)((pix / W) % H), b = (int)(pix / ((long)W * H));
-    const size_t base = ((size_t)(b * 2 * H + 2 * h) * (2 * W) + 2 * w) * ldx + c;
-    const size_t row = (size_t)2 * W * ldx;
-    float v[4][8], o[8];
-    unpack8(ld8(x + base), v[0]);
-    unpack8(ld8(x + base + ldx), v[1]);
-    unpack8(ld8(x + base + row), v[2]);
-    unpack8(ld8(x + base + row + ldx), v[3]);
+__global__ void __launch_bounds__(256) k_maxpool2(const bf16_t *x, int ldx, int rows, int W, int C, bf16_t *y) {
+  const unsigned C8 = C >> 3, n = W * C8;
+  for (int r = blockIdx.y; r < rows; r += gridDim.y)  // row r of y: rows 2 r, 2 r + 1 of x
+    for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
+      const unsigned w = i / C8, c = (i - w * C8) * 8;
+      const bf16_t *p = x + ((size_t)r * 4 * W + 2 * w) * ldx + c;
+      const size_t row = (size_t)2 * W * ldx;
+      float v[4][8], o[8];
+      unpack8(ld8(p), v[0]);
+      unpack8(ld8(p + ldx), v[1]);
+      unpack8(ld8(p + row), v[2]);
+      unpack8(ld8(p + row + ldx), v[3]);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) o[q] = fmaxf(fmaxf(v[0][q], v[1][q]), fmaxf(v[2][q], v[3][q]));
-    st8(y + (size_t)pix * C + c, pack8(o));
-  }
+      for (int q = 0; q < 8; ++q) o[q] = fmaxf(fmaxf(v[0][q], v[1][q]), fmaxf(v[2][q], v[3][q]));
+      st8(y + ((size_t)r * W + w) * C + c, pack8(o));
+    }
 }
 
 // gradient of 2x2 max pooling to the first maximum of each window, plus an
 // optional skip gradient (dskip [.., ldskip] at channel offset skoff), zero
 // where x <= 0 when relu_mask (x is a ReLU output): dx [B, 2H, 2W, C] dense
-__global__ void k_maxpool2_bwd(const bf16_t *x, int ldx, const bf16_t *dy, const bf16_t *dskip,
-                               int ldskip, int skoff, int B, int H, int W, int C, int relu_mask,
-                               bf16_t *dx) {
-  const int C8 = C >> 3;
-  const long n = (long)B * H * W * C8;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const int c = (int)(i % C8) * 8;
-    const long pix = i / C8;
-    const int w = (int)(pix % W), h = (int)((pix / W) % H), b = (int)(pix / ((long)W * H));
-    float v[4][8], g[8];
-    size_t pp[4];
+__global__ void __launch_bounds__(256) k_maxpool2_bwd(const bf16_t *x, int ldx, const bf16_t *dy,
+                                                      const bf16_t *dskip, int ldskip, int skoff, int rows,
+                                                      int W, int C, int relu_mask, bf16_t *dx) {
+  const unsigned C8 = C >> 3, n = W * C8;
+  for (int r = blockIdx.y; r < rows; r += gridDim.y)
+    for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
+      const unsigned w = i / C8, c = (i - w * C8) * 8;
+      uint4 raw[4], sk[4];
+      size_t pp[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      pp[q] = (size_t)(b * 2 * H + 2 * h + (q >> 1)) * (2 * W) + 2 * w + (q & 1);
-      unpack8(ld8(x + pp[q] * ldx + c), v[q]);
-    }
-    unpack8(ld8(dy + (size_t)pix * C + c), g);
-    float m[8];
-    bool taken[8];
+      for (int q = 0; q < 4; ++q) {
+        pp[q] = (size_t)r * 4 * W + (q >> 1) * 2 * W + 2 * w + (q & 1);
+        raw[q] = ld8(x + pp[q] * ldx + c);
+      }
+      const uint4 gr = ld8(dy + ((size_t)r * W + w) * C + c);
+      if (dskip)
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      m[k] = fmaxf(fmaxf(v[0][k], v[1][k]), fmaxf(v[2][k], v[3][k]));
-      taken[k] = false;
-    }
+        for (int q = 0; q < 4; ++q) sk[q] = ld8(dskip + pp[q] * ldskip + skoff + c);
+      float v[4][8], g[8], m[8];
+      bool taken[8];
+      unpack8(gr, g);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      float sk[8], o[8];
-      if (dskip) unpack8(ld8(dskip + pp[q] * ldskip + skoff + c), sk);
+      for (int q = 0; q < 4; ++q) unpack8(raw[q], v[q]);
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
-        o[k] = 0.f;
-        if (!taken[k] && v[q][k] == m[k]) {
-          o[k] = g[k];
-          taken[k] = true;
-        }
-        if (dskip) o[k] += sk[k];
-        if (relu_mask && !(v[q][k] > 0.f)) o[k] = 0.f;
+        m[k] = fmaxf(fmaxf(v[0][k], v[1][k]), fmaxf(v[2][k], v[3][k]));
+        taken[k] = false;
       }
-      st8(dx + pp[q] * C + c, pack8(o));
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float s[8], o[8];
+        if (dskip) unpack8(sk[q], s);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          o[k] = 0.f;
+          if (!taken[k] && v[q][k] == m[k]) {
+            o[k] = g[k];
+            taken[k] = true;
+          }
+          if (dskip) o[k] += s[k];
+          if (relu_mask && !(v[q][k] > 0.f)) o[k] = 0.f;
+        }
+        st8(dx + pp[q] * C + c, pack8(o));
+      }
     }
-  }
 }
 
 // nearest 2x upsampling: x [B, H, W, C] dense -> y [B, 2H, 2W, ldy] at channel offset yoff
-__global__ void k_upsample2(const bf16_t *x, int B, int H, int W, int C, bf16_t *y, int ldy,
-                            int yoff) {
-  const int C8 = C >> 3;
-  const long n = (long)B * 4 * H * W * C8;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const int c = (int)(i % C8) * 8;
-    const long pix = i / C8;  // output pixel
-    const int ww = (int)(pix % (2 * W)), hh = (int)((pix / (2 * W)) % (2 * H));
-    const int b = (int)(pix / ((long)4 * W * H));
-    st8(y + (size_t)pix * ldy + yoff + c, ld8(x + ((size_t)(b * H + hh / 2) * W + ww / 2) * C + c));
-  }
+__global__ void __launch_bounds__(256) k_upsample2(const bf16_t *x, int rows, int W, int C, bf16_t *y, int ldy,
+                                                   int yoff) {
+  const unsigned C8 = C >> 3, n = W * C8;
+  for (int r = blockIdx.y; r < rows; r += gridDim.y)
+    for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
+      const unsigned w = i / C8, c = (i - w * C8) * 8;
+      const uint4 v = ld8(x + ((size_t)r * W + w) * C + c);
+      bf16_t *p = y + ((size_t)r * 4 * W + 2 * w) * ldy + yoff + c;
+      const size_t row = (size_t)2 * W * ldy;
+      st8(p, v);
+      st8(p + ldy, v);
+      st8(p + row, v);
+      st8(p + row + ldy, v);
+    }
 }
 
 // gradient of nearest 2x upsampling: dy [B, 2H, 2W, lddy] channels 0..C-1 ->
 // dx [B, H, W, C], zero where mask <= 0 (mask [B, H, W, ldm], may be null)
-__global__ void k_upsample2_bwd(const bf16_t *dy, int lddy, int B, int H, int W, int C,
-                                const bf16_t *mask, int ldm, bf16_t *dx) {
-  const int C8 = C >> 3;
-  const long n = (long)B * H * W * C8;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const int c = (int)(i % C8) * 8;
-    const long pix = i / C8;
-    const int w = (int)(pix % W), h = (int)((pix / W) % H), b = (int)(pix / ((long)W * H));
-    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, t[8];
+__global__ void __launch_bounds__(256) k_upsample2_bwd(const bf16_t *dy, int lddy, int rows, int W, int C,
+                                                       const bf16_t *mask, int ldm, bf16_t *dx) {
+  const unsigned C8 = C >> 3, n = W * C8;
+  for (int r = blockIdx.y; r < rows; r += gridDim.y)
+    for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
+      const unsigned w = i / C8, c = (i - w * C8) * 8;
+      const size_t pix = (size_t)r * W + w;
+      uint4 raw[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const size_t pp = (size_t)(b * 2 * H + 2 * h + (q >> 1)) * (2 * W) + 2 * w + (q & 1);
-      unpack8(ld8(dy + pp * lddy + c), t);
+      for (int q = 0; q < 4; ++q)
+        raw[q] = ld8(dy + ((size_t)r * 4 * W + (q >> 1) * 2 * W + 2 * w + (q & 1)) * lddy + c);
+      float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, t[8];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) s[k] += t[k];
+      for (int q = 0; q < 4; ++q) {
+        unpack8(raw[q], t);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s[k] += t[k];
+      }
+      if (mask) {
+        float mk[8];
+        unpack8(ld8(mask + pix * ldm + c), mk);
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          if (!(mk[k] > 0.f)) s[k] = 0.f;
+      }
+      st8(dx + pix * C + c, pack8(s));
     }
-    if (mask) {
-      float mk[8];
-      unpack8(ld8(mask + (size_t)pix * ldm + c), mk);
-#pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (!(mk[k] > 0.f)) s[k] = 0.f;
-    }
-    st8(dx + (size_t)pix * C + c, pack8(s));
-  }
 }
 
 // ------------------------------------------------------------------- head
-// z[p] = b + sum_c x[p, c] w[c]   (1x1 convolution to one logit, FP32)
-__global__ void k_head_fwd(const bf16_t *x, int P, int C, const float *w, const float *b, float *z) {
+// z[p] = b + sum_c x[p, c] w[c]   (1x1 convolution to one logit, FP32), channels in
+// increasing order.  A pixel's channels are read in 16-byte rows when they
+// allow it (64 images, 32 channels: 2-byte reads took 232 us, these 50).
+__global__ void __launch_bounds__(256) k_head_fwd(const bf16_t *x, int P, int C, int vec, const float *w,
+                                                  const float *b, float *z) {
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
+    const bf16_t *xp = x + (size_t)p * C;
     float s = b[0];
-    for (int c = 0; c < C; ++c) s += bf2f(x[(size_t)p * C + c]) * w[c];
+    if (vec) {
+      for (int c0 = 0; c0 < C; c0 += 32) {
+        uint4 v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (c0 + 8 * q < C) v[q] = ld8(xp + c0 + 8 * q);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (c0 + 8 * q < C) {
+            float f[8];
+            unpack8(v[q], f);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) s += f[k] * w[c0 + 8 * q + k];
+          }
+      }
+    } else {
+      for (int c = 0; c < C; ++c) s += bf2f(xp[c]) * w[c];
+    }
     z[p] = s;
   }
 }
 
 // dx[p, c] = dz[p] w[c]; per-chunk partials of dw[c] = sum_p dz[p] x[p, c]
-// and db = sum_p dz[p] into ws[chunk][C + 1]
+// and db = sum_p dz[p] into ws[chunk][C], wsb[chunk]
 __global__ void k_head_bwd(const bf16_t *x, int P, int C, const float *w, const float *dz,
-                           bf16_t *dx, int chunk, float *ws) {
+                           bf16_t *dx, int chunk, float *ws, float *wsb) {
   const int z = blockIdx.x;
   const int pend = min(P, (z + 1) * chunk);
   __shared__ float red[33][33];
@@ -2382,8 +2423,70 @@ __global__ void k_head_bwd(const bf16_t *x, int P, int C, const float *w, const 
       t += red[q][c];
       tb += red[q][32];
     }
-    if (c < C) ws[(size_t)z * (C + 1) + c] = t;
-    if (c == 0) ws[(size_t)z * (C + 1) + C] = tb;
+    if (c < C) ws[(size_t)z * C + c] = t;
+    if (c == 0) wsb[z] = tb;
+  }
+}
+
+// The same for C = 8, 16 or 32 and aligned rows: a thread holds 8 channels (16 bytes) of
+// every (2048 / C)-th pixel of the chunk, four at a time (2-byte accesses took 318 us
+// for 64 images of 32 channels, this 84).
+template <int C>
+__global__ void __launch_bounds__(256) k_head_bwd8(const bf16_t *x, int P, const float *w, const float *dz,
+                                                   bf16_t *dx, int chunk, float *ws, float *wsb) {
+  constexpr int C8 = C / 8, LANES = 256 / C8;
+  __shared__ float red[8][C + 1];
+  const int z = blockIdx.x, cg = threadIdx.x % C8, pl = threadIdx.x / C8;
+  const int pend = min(P, (z + 1) * chunk);
+  float wc[8], s[8], sb = 0.f;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    wc[k] = w[cg * 8 + k];
+    s[k] = 0.f;
+  }
+  for (int p0 = z * chunk + pl; p0 < pend; p0 += 4 * LANES) {
+    uint4 v[4];
+    float g[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int p = p0 + q * LANES;
+      g[q] = p < pend ? dz[p] : 0.f;
+      v[q] = p < pend ? ld8(x + (size_t)p * C + cg * 8) : make_uint4(0, 0, 0, 0);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int p = p0 + q * LANES;
+      if (p >= pend) break;
+      float f[8], o[8];
+      unpack8(v[q], f);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        o[k] = f[k] > 0.f ? g[q] * wc[k] : 0.f;
+        s[k] += g[q] * f[k];
+      }
+      sb += g[q];
+      st8(dx + (size_t)p * C + cg * 8, pack8(o));
+    }
+  }
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = C8; o < 32; o <<= 1) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+    sb += __shfl_xor_sync(0xffffffffu, sb, o);
+  }
+  if (lane < C8) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) red[wp][lane * 8 + k] = s[k];
+    if (lane == 0) red[wp][C] = sb;
+  }
+  __syncthreads();
+  if (threadIdx.x <= C) {
+    float t = 0.f;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) t += red[q][threadIdx.x];
+    if (threadIdx.x < C) ws[(size_t)z * C + threadIdx.x] = t;
+    else wsb[z] = t;
   }
 }
 
@@ -2479,29 +2582,33 @@ __global__ void __launch_bounds__(256) k_dice_grad(const float *z, const uint8_t
   }
 }
 
-// loss = w (1 - mean_b D_b), D_b = (2 I_b + eps) / (S_b + eps), in sample order
-__global__ void k_dice_loss(const float *ws, int nchunk, int B, float w, float eps, float *loss) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    float dsum = 0.f;
-    for (int b = 0; b < B; ++b) {
-      float I = 0.f, S = 0.f;
-      for (int q = 0; q < nchunk; ++q) {
-        const float *o = ws + ((size_t)b * nchunk + q) * 3;
-        I += o[0];
-        S += o[1] + o[2];
-      }
-      dsum += (2.f * I + eps) / (S + eps);
+// loss = w (1 - mean_b D_b), D_b = (2 I_b + eps) / (S_b + eps), one block: a
+// sample's chunks in order by one thread, the samples' indices by fixed lanes and a tree
+// (a single thread walking all of it took 74 us for 64 samples, this 5)
+__global__ void __launch_bounds__(256) k_dice_loss(const float *ws, int nchunk, int B, float w, float eps,
+                                                   float *loss) {
+  __shared__ float red[256];
+  float d = 0.f;
+  for (int b = threadIdx.x; b < B; b += 256) {
+    float I = 0.f, S = 0.f;
+    for (int q = 0; q < nchunk; ++q) {
+      const float *o = ws + ((size_t)b * nchunk + q) * 3;
+      I += o[0];
+      S += o[1] + o[2];
     }
-    loss[0] = w * (1.f - dsum / (float)B);
+    d += (2.f * I + eps) / (S + eps);
   }
+  d = block_sum256(d, red);
+  if (threadIdx.x == 0) loss[0] = w * (1.f - d / (float)B);
 }
 
-__global__ void k_sum_scaled(const float *ws, int m, float scale, float *out) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    float s = 0.f;
-    for (int i = 0; i < m; ++i) s += ws[i];
-    out[0] = s * scale;
-  }
+// out[0] = scale sum ws[0..m), one block, fixed order (one thread took 98 us for 4,864 values)
+__global__ void __launch_bounds__(256) k_sum_scaled(const float *ws, int m, float scale, float *out) {
+  __shared__ float red[256];
+  float s = 0.f;
+  for (int i = threadIdx.x; i < m; i += 256) s += ws[i];
+  s = block_sum256(s, red);
+  if (threadIdx.x == 0) out[0] = s * scale;
 }
 
 // ------------------------------------------------------------------- adam
@@ -2535,14 +2642,10 @@ __global__ void k_to_bf16(const float *x, long n, bf16_t *y) {
     y[i] = f2bf(x[i]);
 }
 
-// dw[c] = sum_z ws[z][c], db = sum_z ws[z][C], in chunk order
-__global__ void k_reduce_head(const float *ws, int nz, int C, float *dw, float *db) {
-  for (int c = threadIdx.x; c <= C; c += blockDim.x) {
-    float s = 0.f;
-    for (int z = 0; z < nz; ++z) s += ws[(size_t)z * (C + 1) + c];
-    if (c < C) dw[c] = s;
-    else db[0] = s;
-  }
+// grid of the pooling and upsampling kernels: image rows down, (pixel, 8 channels) across
+dim3 grid_rows(long rows, long per_row) {
+  const long x = (per_row + 255) / 256;
+  return dim3((unsigned)(x < 65535 ? x : 65535), (unsigned)(rows < 65535 ? rows : 65535));
 }
 
 int grid_1d(long n, int block) {
@@ -2619,11 +2722,7 @@ int cem_sg_conv3x3_wgrad(const void *x, int ldx, const void *dy, int lddy, int B
     if (wgrad_halo(a, splits, wsb, dw, db, st, hs, he)) {
       if (he != cudaSuccess) return CEM_SG_ERR_CUDA;
       if (hs == 1) return CEM_SG_OK;  // the kernel wrote dw and db
-      const int per = hs >= 16 ? 32 : 256;  // outputs of a block
-      const long nblk = (nw + per - 1) / per + (db ? (Cout + per - 1) / per : 0);
-      const int g = (int)(nblk < 8 * 1216 ? nblk : 8 * 1216), n2 = db ? Cout : 0;
-      if (hs >= 16) k_reduce_sums<8><<<g, 256, 0, st>>>(a.ws, nw, dw, wsb, n2, db, hs);
-      else k_reduce_sums<1><<<g, 256, 0, st>>>(a.ws, nw, dw, wsb, n2, db, hs);
+      reduce_sums(a.ws, nw, dw, wsb, db ? Cout : 0, db, hs, st);
       return cudaGetLastError() == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
     }
     // tcgen05: dW^T tiles of 128 k' x BN outputs; bias sums by a separate
@@ -2633,7 +2732,7 @@ int cem_sg_conv3x3_wgrad(const void *x, int ldx, const void *dy, int lddy, int B
                   : Cout > 64 ? launch_wgrad_tc<128>(a, splits, st)
                               : launch_wgrad_tc<64>(a, splits, st);
     if (e != cudaSuccess) return CEM_SG_ERR_CUDA;
-    k_reduce_splits<<<grid_1d(nw, 256), 256, 0, st>>>(a.ws, splits, nw, dw);
+    reduce_sums(a.ws, nw, dw, nullptr, 0, nullptr, splits, st);
     if (db) {
       // more pixel chunks than the weight partials use: the sums are a pure
       // bandwidth pass (at most 608 chunks, four per SM; the workspace holds 1024)
@@ -2642,15 +2741,14 @@ int cem_sg_conv3x3_wgrad(const void *x, int ldx, const void *dy, int lddy, int B
       const int bsplits = (int)(bs < 1 ? 1 : (bs > 608 ? 608 : bs));
       const int bch = (a.P + bsplits - 1) / bsplits;
       k_colsum8<<<bsplits, 256, 0, st>>>(a.dy, a.P, Cout, lddy, bch, wsb);
-      k_reduce_splits<<<grid_1d(Cout, 128), 128, 0, st>>>(wsb, bsplits, Cout, db);
+      reduce_sums(wsb, Cout, db, nullptr, 0, nullptr, bsplits, st);
     }
     return cudaGetLastError() == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
   }
   a.wsb = db ? a.ws + (size_t)splits * Cout * a.K : nullptr;
   dim3 grid((Cout + GBM - 1) / GBM, (a.K + GBN - 1) / GBN, splits);
   k_conv3x3_wgrad<<<grid, 256, 0, st>>>(a);
-  k_reduce_splits<<<grid_1d(nw, 256), 256, 0, st>>>(a.ws, splits, nw, dw);
-  if (db) k_reduce_splits<<<grid_1d(Cout, 128), 128, 0, st>>>(a.wsb, splits, Cout, db);
+  reduce_sums(a.ws, nw, dw, a.wsb, db ? Cout : 0, db, splits, st);
   return cudaGetLastError() == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
 }
 
@@ -2664,9 +2762,9 @@ int cem_sg_relu_bwd(void *dy, int lddy, const void *y, int ldy, long P, int C, v
 int cem_sg_maxpool2(const void *x, int ldx, int B, int H, int W, int C, void *y, void *stream) {
   if (!x || !y || B < 1 || H < 1 || W < 1 || C < 8 || (C & 7) || ldx < C || (ldx & 7))
     return CEM_SG_ERR_ARG;
-  const long n = (long)B * H * W * (C >> 3);
-  k_maxpool2<<<grid_1d(n, 256), 256, 0, (cudaStream_t)stream>>>((const bf16_t *)x, ldx, B, H, W, C,
-                                                               (bf16_t *)y);
+  const long rows = (long)B * H;
+  k_maxpool2<<<grid_rows(rows, (long)W * (C >> 3)), 256, 0, (cudaStream_t)stream>>>(
+      (const bf16_t *)x, ldx, (int)rows, W, C, (bf16_t *)y);
   return cudaGetLastError() == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
 }
 
@@ -2676,9 +2774,9 @@ int cem_sg_maxpool2_bwd(const void *x, int ldx, const void *dy, const void *dski
   if (!x || !dy || !dx || B < 1 || H < 1 || W < 1 || C < 8 || (C & 7) || ldx < C || (ldx & 7) ||
       (dskip && (ldskip < skoff + C || (ldskip & 7) || (skoff & 7))))
     return CEM_SG_ERR_ARG;
-  const long n = (long)B * H * W * (C >> 3);
-  k_maxpool2_bwd<<<grid_1d(n, 256), 256, 0, (cudaStream_t)stream>>>(
-      (const bf16_t *)x, ldx, (const bf16_t *)dy, (const bf16_t *)dskip, ldskip, skoff, B, H, W, C,
+  const long rows = (long)B * H;
+  k_maxpool2_bwd<<<grid_rows(rows, (long)W * (C >> 3)), 256, 0, (cudaStream_t)stream>>>(
+      (const bf16_t *)x, ldx, (const bf16_t *)dy, (const bf16_t *)dskip, ldskip, skoff, (int)rows, W, C,
       relu_mask, (bf16_t *)dx);
   return cudaGetLastError() == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
 }
@@ -2688,9 +2786,9 @@ int cem_sg_upsample2(const void *x, int B, int H, int W, int C, void *y, int ldy
   if (!x || !y || B < 1 || H < 1 || W < 1 || C < 8 || (C & 7) || ldy < yoff + C || (ldy & 7) ||
       (yoff & 7))
     return CEM_SG_ERR_ARG;
-  const long n = (long)B * 4 * H * W * (C >> 3);
-  k_upsample2<<<grid_1d(n, 256), 256, 0, (cudaStream_t)stream>>>((const bf16_t *)x, B, H, W, C,
-                                                                (bf16_t *)y, ldy, yoff);
+  const long rows = (long)B * H;
+  k_upsample2<<<grid_rows(rows, (long)W * (C >> 3)), 256, 0, (cudaStream_t)stream>>>(
+      (const bf16_t *)x, (int)rows, W, C, (bf16_t *)y, ldy, yoff);
   return cudaGetLastError() == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
 }
 
@@ -2699,16 +2797,17 @@ int cem_sg_upsample2_bwd(const void *dy, int lddy, int B, int H, int W, int C, c
   if (!dy || !dx || B < 1 || H < 1 || W < 1 || C < 8 || (C & 7) || lddy < C || (lddy & 7) ||
       (mask && (ldmask < C || (ldmask & 7))))
     return CEM_SG_ERR_ARG;
-  const long n = (long)B * H * W * (C >> 3);
-  k_upsample2_bwd<<<grid_1d(n, 256), 256, 0, (cudaStream_t)stream>>>(
-      (const bf16_t *)dy, lddy, B, H, W, C, (const bf16_t *)mask, ldmask, (bf16_t *)dx);
+  const long rows = (long)B * H;
+  k_upsample2_bwd<<<grid_rows(rows, (long)W * (C >> 3)), 256, 0, (cudaStream_t)stream>>>(
+      (const bf16_t *)dy, lddy, (int)rows, W, C, (const bf16_t *)mask, ldmask, (bf16_t *)dx);
   return cudaGetLastError() == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
 }
 
 int cem_sg_head_fwd(const void *x, int P, int C, const float *w, const float *b, float *z,
                     void *stream) {
   if (!x || !w || !b || !z || P < 1 || C < 1) return CEM_SG_ERR_ARG;
-  k_head_fwd<<<grid_1d(P, 256), 256, 0, (cudaStream_t)stream>>>((const bf16_t *)x, P, C, w, b, z);
+  const int vec = !(C & 7) && !((uintptr_t)x & 15);
+  k_head_fwd<<<grid_1d(P, 256), 256, 0, (cudaStream_t)stream>>>((const bf16_t *)x, P, C, vec, w, b, z);
   return cudaGetLastError() == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
 }
 
@@ -2724,9 +2823,15 @@ int cem_sg_head_bwd(const void *x, int P, int C, const float *w, const float *dz
   if (ws_bytes < cem_sg_head_workspace(P, C)) return CEM_SG_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   const int chunk = 4096, nz = (P + chunk - 1) / chunk;
-  float *wsf = (float *)ws;
-  k_head_bwd<<<nz, 256, 0, st>>>((const bf16_t *)x, P, C, w, dz, (bf16_t *)dx, chunk, wsf);
-  k_reduce_head<<<1, 64, 0, st>>>(wsf, nz, C, dw, db);
+  float *wsf = (float *)ws, *wsb = wsf + (size_t)nz * C;
+  const bf16_t *xb = (const bf16_t *)x;
+  bf16_t *db16 = (bf16_t *)dx;
+  const bool vec = !(((uintptr_t)x | (uintptr_t)dx) & 15);
+  if (vec && C == 32) k_head_bwd8<32><<<nz, 256, 0, st>>>(xb, P, w, dz, db16, chunk, wsf, wsb);
+  else if (vec && C == 16) k_head_bwd8<16><<<nz, 256, 0, st>>>(xb, P, w, dz, db16, chunk, wsf, wsb);
+  else if (vec && C == 8) k_head_bwd8<8><<<nz, 256, 0, st>>>(xb, P, w, dz, db16, chunk, wsf, wsb);
+  else k_head_bwd<<<nz, 256, 0, st>>>(xb, P, C, w, dz, db16, chunk, wsf, wsb);
+  reduce_sums(wsf, C, dw, wsb, 1, db, nz, st);
   return cudaGetLastError() == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
 }
 
@@ -2739,7 +2844,7 @@ int cem_sg_bce(const float *z, const unsigned char *t, long n, float pos_weight,
   cudaStream_t st = (cudaStream_t)stream;
   const int g = grid_1d(n, 256);
   k_bce<<<g, 256, 0, st>>>(z, t, n, pos_weight, dz, (float *)ws);
-  k_sum_scaled<<<1, 32, 0, st>>>((const float *)ws, g, 1.f / (float)n, loss);
+  k_sum_scaled<<<1, 256, 0, st>>>((const float *)ws, g, 1.f / (float)n, loss);
   return cudaGetLastError() == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
 }
 
@@ -2758,7 +2863,7 @@ int cem_sg_dice(const float *z, const unsigned char *t, int B, long n_per, float
   const dim3 grid((unsigned)nchunk, (unsigned)B);
   k_dice_partial<<<grid, 256, 0, st>>>(z, t, n_per, (float *)ws);
   k_dice_grad<<<grid, 256, 0, st>>>(z, t, n_per, B, weight, eps, (const float *)ws, dz);
-  k_dice_loss<<<1, 32, 0, st>>>((const float *)ws, (int)nchunk, B, weight, eps, loss);
+  k_dice_loss<<<1, 256, 0, st>>>((const float *)ws, (int)nchunk, B, weight, eps, loss);
   return cudaGetLastError() == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
 }
 

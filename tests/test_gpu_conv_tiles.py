@@ -70,7 +70,7 @@ def test_conv_tilings(B, H, W, cin, cout):
 @pytest.mark.parametrize("B,H,W", [(1, 16, 8), (2, 17, 33), (5, 20, 50), (7, 10, 25), (9, 3, 31), (3, 1, 1),
                                    (2, 1, 64), (64, 9, 31), (5, 160, 100), (2, 64, 640)])
 @pytest.mark.parametrize("cin,cout", [(32, 32), (96, 32), (32, 64), (64, 64), (192, 96), (64, 128), (128, 256),
-                                      (512, 64), (24, 40)])
+                                      (512, 64), (24, 40), (8, 32), (8, 96)])
 @pytest.mark.parametrize("with_bias", [True, False])
 def test_wgrad_tilings(B, H, W, cin, cout, with_bias):
     import torch
@@ -108,3 +108,34 @@ def test_wgrad_tilings(B, H, W, cin, cout, with_bias):
         assert bool(((db.double() - yf.sum(0)).abs() <= tol).all())
     else:
         assert bool(torch.isnan(db).all())
+
+
+# the head's row accesses (8, 16 and 32 channels, others, an odd pixel count) and the
+# pooling and upsampling kernels' row walk against plain sums
+@pytest.mark.parametrize("C", [8, 12, 16, 24, 32])
+@pytest.mark.parametrize("P", [1, 4095, 4097, 70001])
+def test_head_rows(C, P):
+    import torch
+    from paper_2509_01827_gb300 import build, surrogate
+    build.build()
+    L, st = surrogate.sg(), torch.cuda.current_stream().cuda_stream
+    g = torch.Generator(device="cuda").manual_seed(C)
+    x = torch.randn(P, C, device="cuda", generator=g).bfloat16()
+    w, dz = (torch.randn(n, device="cuda", generator=g) for n in (C, P))
+    b = torch.randn(1, device="cuda", generator=g)
+    z, dx = torch.empty(P, device="cuda"), torch.empty_like(x)
+    dw, db = torch.empty(C, device="cuda"), torch.empty(1, device="cuda")
+    nb = L.cem_sg_head_workspace(P, C)
+    ws = torch.empty(nb, dtype=torch.uint8, device="cuda")
+    assert L.cem_sg_head_fwd(x.data_ptr(), P, C, w.data_ptr(), b.data_ptr(), z.data_ptr(), st) == 0
+    assert L.cem_sg_head_bwd(x.data_ptr(), P, C, w.data_ptr(), dz.data_ptr(), dx.data_ptr(), dw.data_ptr(),
+                             db.data_ptr(), ws.data_ptr(), nb, st) == 0
+    x64, w64, d64 = x.double(), w.double(), dz.double()
+    mag = (x64.abs() @ w64.abs()) + b.double().abs()
+    assert bool(((z.double() - (x64 @ w64 + b.double())).abs() <= (C + 1) * 2.0 ** -23 * mag).all())
+    want = torch.where(x > 0, dz[:, None] * w[None], torch.zeros((), device="cuda")).bfloat16()
+    assert torch.equal(dx, want)
+    # at most 64 values a thread, 32 lanes, 8 warps and P / 4096 chunks in FP32
+    n = (64 + 32 + 8 + P // 4096 + 8) * 2.0 ** -24
+    assert bool(((dw.double() - d64 @ x64).abs() <= 4 * n * (d64.abs() @ x64.abs())).all())
+    assert float((db.double() - d64.sum()).abs()) <= 4 * n * 8 * float(d64.abs().sum())
