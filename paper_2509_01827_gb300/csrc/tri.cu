@@ -281,8 +281,15 @@ __global__ void k_tri_edge32(TriDev d, int energy) {
   if (energy) block_sum_to(se, d.part);
 }
 
-__global__ void k_tri_node32(TriDev d, double lamN, double lamD, double dtd, double dtvd,
-                             int first, int energy, int part_off) {
+// Bound by the gather's loads (16 bytes of record and 16 of stress per
+// incidence, about 18 of them a node): one node per thread, eight incidences in
+// flight, and FP64 only where a node has a load or a prescribed velocity or the
+// step records energies (as a part of every node's update its conversions
+// alone took 7 us of the FP64 pipe for 0.5 M nodes).  ENERGY: the grid is the
+// one the partial sums are laid out for, its threads walk the nodes.
+template <bool ENERGY>
+__global__ void __launch_bounds__(kTB) k_tri_node32(TriDev d, double lamN, double lamD, double dtd, double dtvd,
+                                                    int first, int part_off) {
   double ke = 0.0, wn = 0.0, wd = 0.0;
   bool bad = false;
   const float dt = (float)dtd, dtv = (float)dtvd;
@@ -290,23 +297,37 @@ __global__ void k_tri_node32(TriDev d, double lamN, double lamD, double dtd, dou
     float fx = 0.f, fy = 0.f;
     const int deg = d.inc_deg[N];
     const TriInc32 *rec = d.inc32 + d.slice_off[N >> 5] + (N & 31);
-#pragma unroll 4
-    for (int k = 0; k < deg; ++k) {
+    const int loaded = d.lflag[N], dm = d.dmask[N];
+    const float mi = d.minvf[N];
+    const float2 vo = d.v2[N];
+    float4 U = d.u4[N];
+    int k = 0;
+    for (; k + 8 <= deg; k += 8) {
+      TriInc32 r[8];
+      float4 s[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) r[q] = rec[32L * (k + q)];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) s[q] = d.sig32[r[q].g];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        fx = fx + (r[q].b * s[q].x + r[q].c * s[q].z) * r[q].q3;
+        fy = fy + (r[q].c * s[q].y + r[q].b * s[q].z) * r[q].q3;
+      }
+    }
+#pragma unroll 2
+    for (; k < deg; ++k) {
       const TriInc32 r = rec[32L * k];
       const float4 s = d.sig32[r.g];
       fx = fx + (r.b * s.x + r.c * s.z) * r.q3;
       fy = fy + (r.c * s.y + r.b * s.z) * r.q3;
     }
-    const int loaded = d.lflag[N];
-    const int dm = d.dmask[N];
     float fex = 0.f, fey = 0.f;
     if (loaded) {
       const double2 F = d.F[N];
       fex = (float)(lamN * F.x);
       fey = (float)(lamN * F.y);
     }
-    const float mi = d.minvf[N];
-    const float2 vo = d.v2[N];
     float vxn = vo.x + dtv * ((fex - fx) * mi);
     float vyn = vo.y + dtv * ((fey - fy) * mi);
     if (dm) {
@@ -314,35 +335,54 @@ __global__ void k_tri_node32(TriDev d, double lamN, double lamD, double dtd, dou
       if (dm & 1) vxn = (float)(lamD * V.x);
       if (dm & 2) vyn = (float)(lamD * V.y);
     }
-    const double vbx = first ? (double)vo.x : 0.5 * ((double)vo.x + (double)vxn);
-    const double vby = first ? (double)vo.y : 0.5 * ((double)vo.y + (double)vyn);
-    if (energy) {
+    if (ENERGY) {
       wn += d.Wn[N];
       wd += d.Wd[N];
     }
-    if (loaded) d.Wn[N] = d.Wn[N] + dtd * ((double)fex * vbx + (double)fey * vby);
-    if (dm) {
-      const double m = d.m[N], dv = dtvd;
-      const double Rx = m * (((double)vxn - (double)vo.x) / dv) - ((double)fex - (double)fx);
-      const double Ry = m * (((double)vyn - (double)vo.y) / dv) - ((double)fey - (double)fy);
-      double w = 0.0;
-      if (dm & 1) w = w + Rx * vbx;
-      if (dm & 2) w = w + Ry * vby;
-      d.Wd[N] = d.Wd[N] + dtd * w;
+    if (ENERGY || loaded || dm) {
+      const double vbx = first ? (double)vo.x : 0.5 * ((double)vo.x + (double)vxn);
+      const double vby = first ? (double)vo.y : 0.5 * ((double)vo.y + (double)vyn);
+      if (loaded) d.Wn[N] = d.Wn[N] + dtd * ((double)fex * vbx + (double)fey * vby);
+      if (dm) {
+        const double m = d.m[N], dv = dtvd;
+        const double Rx = m * (((double)vxn - (double)vo.x) / dv) - ((double)fex - (double)fx);
+        const double Ry = m * (((double)vyn - (double)vo.y) / dv) - ((double)fey - (double)fy);
+        double w = 0.0;
+        if (dm & 1) w = w + Rx * vbx;
+        if (dm & 2) w = w + Ry * vby;
+        d.Wd[N] = d.Wd[N] + dtd * w;
+      }
+      if (ENERGY) ke += 0.5 * (d.m[N] * (vbx * vbx + vby * vby));
     }
-    if (energy) ke += 0.5 * (d.m[N] * (vbx * vbx + vby * vby));
     d.v2[N] = make_float2(vxn, vyn);
-    float4 U = d.u4[N];
     two_sum_acc(U.x, U.y, dt * vxn);
     two_sum_acc(U.z, U.w, dt * vyn);
     d.u4[N] = U;
     bad |= !(fabsf(vxn) <= FLT_MAX) || !(fabsf(vyn) <= FLT_MAX);
   }
   if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(d.status, 1);
-  if (energy) {
+  if (ENERGY) {
     block_sum_to(ke, d.part + part_off);
     block_sum_to(wn, d.part + part_off + gridDim.x);
     block_sum_to(wd, d.part + part_off + 2 * gridDim.x);
+  }
+}
+
+// node fields as the x block then the y block, FP64
+__global__ void k_tri_fields(TriDev d, int which_v, double *out) {
+  for (int N = blockIdx.x * blockDim.x + threadIdx.x; N < d.nn; N += gridDim.x * blockDim.x) {
+    double2 f;
+    if (d.precision != CEM_FP32_MIXED) {
+      f = which_v ? d.v[N] : d.u[N];
+    } else if (which_v) {
+      const float2 v = d.v2[N];
+      f = make_double2((double)v.x, (double)v.y);
+    } else {
+      const float4 U = d.u4[N];
+      f = make_double2((double)U.x + (double)U.y, (double)U.z + (double)U.w);
+    }
+    out[N] = f.x;
+    out[d.nn + N] = f.y;
   }
 }
 
@@ -485,6 +525,7 @@ struct TriMesh {
   cem_free_fn free_fn = nullptr;
   void *ctx = nullptr;
   std::vector<void *> blocks;
+  double *field = nullptr;  // [2 nn] node field laid out for the getters, where the edges' memory is too small
   // host geometry
   std::vector<double> X;
   std::vector<int> conn;
@@ -1008,7 +1049,10 @@ cem_status tri_step(TriMesh *t, int n, std::string &err) {
     if (t->precision == CEM_FP32_MIXED) {
       k_tri_strain32<<<gs, kTB, 0, t->st>>>(t->d);
       k_tri_edge32<<<ge, kTB, 0, t->st>>>(t->d, energy ? 1 : 0);
-      k_tri_node32<<<gn, kTB, 0, t->st>>>(t->d, lamN, lamD, dt, dtv, s == 0 ? 1 : 0, energy ? 1 : 0, ge);
+      if (energy) k_tri_node32<true><<<gn, kTB, 0, t->st>>>(t->d, lamN, lamD, dt, dtv, s == 0 ? 1 : 0, ge);
+      else
+        k_tri_node32<false><<<(t->nn + kTB - 1) / kTB, kTB, 0, t->st>>>(t->d, lamN, lamD, dt, dtv,
+                                                                          s == 0 ? 1 : 0, ge);
     } else {
       k_tri_strain<<<gs, kTB, 0, t->st>>>(t->d);
       k_tri_edge<<<ge, kTB, 0, t->st>>>(t->d, energy ? 1 : 0);
@@ -1048,32 +1092,30 @@ cem_status tri_get_fields(TriMesh *t, int which, void *out, long n_bytes, int on
   std::vector<double> h;
   if (which == CEM_FIELD_U || which == CEM_FIELD_V) {
     if (n_bytes < 16 * n) { err = "buffer too small"; return CEM_ERR_ARG; }
-    std::vector<double> il(2 * n);
-    cudaError_t ce;
-    if (t->precision == CEM_FP32_MIXED && which == CEM_FIELD_U) {
-      std::vector<float4> u4(n);
-      ce = cudaMemcpyAsync(u4.data(), t->d.u4, 16 * n, cudaMemcpyDeviceToHost, t->st);
-      if (ce == cudaSuccess) ce = cudaStreamSynchronize(t->st);
-      for (long N = 0; N < n; ++N) {
-        il[2 * N] = (double)u4[N].x + (double)u4[N].y;
-        il[2 * N + 1] = (double)u4[N].z + (double)u4[N].w;
-      }
-    } else if (t->precision == CEM_FP32_MIXED) {
-      std::vector<float2> v2(n);
-      ce = cudaMemcpyAsync(v2.data(), t->d.v2, 8 * n, cudaMemcpyDeviceToHost, t->st);
-      if (ce == cudaSuccess) ce = cudaStreamSynchronize(t->st);
-      for (long N = 0; N < n; ++N) { il[2 * N] = v2[N].x; il[2 * N + 1] = v2[N].y; }
-    } else {
-      ce = cudaMemcpyAsync(il.data(), which == CEM_FIELD_U ? t->d.u : t->d.v, 16 * n,
-                           cudaMemcpyDeviceToHost, t->st);
-      if (ce == cudaSuccess) ce = cudaStreamSynchronize(t->st);
+    // laid out on the device (copying the records out and splitting them on the
+    // host took 1.6 ms for 0.5 M nodes), in the edge stresses' memory, which no call
+    // leaves a value in: 32 bytes an edge, and only a mesh in which most nodes are in
+    // no triangle has fewer than one edge for two nodes.  The caller's device memory
+    // is written in the order of the legacy stream, as a plain cudaMemcpy would.
+    double *field = reinterpret_cast<double *>(t->d.sig);
+    if (2 * (long)t->ned < n) {
+      if (!t->field && !tri_alloc_n(t, t->field, 2 * (size_t)n)) { err = "field allocation failed"; return CEM_ERR_CUDA; }
+      field = t->field;
+    }
+    k_tri_fields<<<(int)((n + kTB - 1) / kTB), kTB, 0, t->st>>>(t->d, which == CEM_FIELD_V ? 1 : 0, field);
+    cudaError_t ce = cudaGetLastError();
+    if (ce == cudaSuccess && !on_device)
+      ce = cudaMemcpyAsync(out, field, 16 * n, cudaMemcpyDeviceToHost, t->st);
+    if (ce == cudaSuccess) ce = cudaStreamSynchronize(t->st);
+    if (ce == cudaSuccess && on_device) {
+      ce = cudaMemcpyAsync(out, field, 16 * n, cudaMemcpyDeviceToDevice, cudaStreamLegacy);
+      if (ce == cudaSuccess) ce = cudaStreamSynchronize(cudaStreamLegacy);
     }
     if (ce != cudaSuccess) {
       err = "copy failed";
       return CEM_ERR_CUDA;
     }
-    h.resize(2 * n);
-    for (long N = 0; N < n; ++N) { h[N] = il[2 * N]; h[n + N] = il[2 * N + 1]; }
+    return CEM_OK;
   } else if (which == CEM_FIELD_MASS) {
     if (n_bytes < 8 * n) { err = "buffer too small"; return CEM_ERR_ARG; }
     h.resize(n);

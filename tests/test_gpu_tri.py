@@ -176,3 +176,53 @@ def test_crack_evaluation_against_the_oracle(precision):
         gce = p.gc[elem].astype(np.float64)[:, None]
         near = np.any(np.abs(Go / gce - 1.0) < 1e-3, axis=1)
         np.testing.assert_array_equal(cg[~near], co[~near])
+
+
+def _fans(spokes):
+    """One fan of triangles per entry: a hub with that many spokes around it
+    (closed), so that the hub's gather list has 5 entries a triangle."""
+    X, conn = [], []
+    for q, n in enumerate(spokes):
+        hub = len(X)
+        X.append([3.0e-3 * q, 0.0])
+        for k in range(n):
+            t = 2.0 * np.pi * (k + 0.2 * np.sin(k)) / n
+            X.append([3.0e-3 * q + 1e-3 * np.cos(t), 1e-3 * np.sin(t)])
+        for k in range(n):
+            conn.append([hub, hub + 1 + k, hub + 1 + (k + 1) % n])
+    return inputs.TriProblem(name="fans", X=np.array(X), conn=np.array(conn, np.int32))
+
+
+def test_fp32_gather_lists_of_every_length():
+    """Gather lists of 9 to 60 entries (remainders of every size after the
+    groups of eight), with energy recorded each step and never: the two
+    kernels give identical fields, and both agree with the FP64 oracle to the
+    FP32-mixed mode's 1e-5; a device destination gets what a host one gets."""
+    import torch
+
+    from oracle.cst_oracle import from_problem
+    from paper_2509_01827_gb300 import cem
+    p = _fans([3, 4, 5, 6, 7, 8, 9, 12])
+    rng = np.random.default_rng(5)
+    n = p.n_nodes
+    p.init = (rng.standard_normal(n) * 1e-7, rng.standard_normal(n) * 1e-7,
+              rng.standard_normal(n) * 0.1, rng.standard_normal(n) * 0.1)
+    got = []
+    for every in (0, 1):
+        p.energy_every = every
+        g = cem.TriSolver(p, precision=cem.CEM_FP32_MIXED)
+        g.step(40)
+        got.append(g.nodes())
+    o = from_problem(p)
+    o.step(40)
+    want = o.nodes()
+    for k in ("ux", "uy", "vx", "vy"):
+        np.testing.assert_array_equal(got[0][k], got[1][k], err_msg=k)
+    for k in ("ux", "uy"):
+        assert np.max(np.abs(got[0][k] - want[k])) < 1e-5 * np.max(np.abs(want[k])), k
+    t = torch.empty(2 * n, dtype=torch.float64, device="cuda")
+    for which, k in ((cem.CEM_FIELD_U, "u"), (cem.CEM_FIELD_V, "v")):
+        assert cem.lib().cem_get_fields(g.h, which, t.data_ptr(), t.numel() * 8, 1) == 0
+        h = t.cpu().numpy()
+        np.testing.assert_array_equal(h[:n], got[1][k + "x"])
+        np.testing.assert_array_equal(h[n:], got[1][k + "y"])
