@@ -731,9 +731,8 @@ __device__ __forceinline__ void march32_tile(const DevState &d, int tile_x, int 
 // Neighbouring warps share their halo columns through L1.  Each tile writes
 // its own energy partial pair, tiles past the last write zeros.
 constexpr int kMarchWarps = 4;
-// tile heights: at least 8 node rows (the energy partials are sized for
-// that), at most 64 (one bit per owned row; cem_batch_set_config checks it)
-constexpr int kMarchRowsMin = 8;
+// tile heights: at most 64 node rows (one bit per owned row;
+// cem_batch_set_config checks it)
 
 __host__ __device__ inline int march_tiles_x(int nx) { return (nx + 1 + WX - 1) / WX; }
 __host__ __device__ inline int march_tiles_y(int ny, int ty) { return (ny + 1 + ty - 1) / ty; }
@@ -908,10 +907,28 @@ cudaError_t set_all_smem_attrs() {
 cudaError_t launch_eval32(const DevState &d, int cur, cudaStream_t st);
 cudaError_t launch_eval32_batch(const BatchDev &b, cudaStream_t st);
 
-// Tile height of a mesh stepped alone: 8 node rows.  Many short tiles (3-4
-// waves of resident warps on the 2048 x 2048 plate) measured faster than
-// one wave of tall ones (2048^2 step: 65 us at 8 rows, 73 at 16, 96 at 32).
-int march_rows_solo(const DevState &) { return kMarchRowsMin; }
+// Tile height of a mesh stepped alone.  A tile marches its rows and three more one
+// after another, 1.6 us each whatever else runs, and 2432 resident warps (four CTAs of
+// four on each of 152 SMs) get through one row each in another 0.9 us when they share
+// the SMs' issue slots, so the height r with the least (r + 3) (1.6 + 0.9 tiles / 2432)
+// is taken.  The node update of an elastic n x n plate, us, at 8 / 6 / 4 / 2 / 1 rows:
+// n = 128 22.0 / 20.5 / 17.4 / 12.7 / 10.9, 512 25.3 / 22.7 / 18.6 / 16.6 / 16.7,
+// 1024 30.9 / 27.9 / 24.9 / 25.4 / -, 2048 58.2 / 59.8 / 66.7 / 88 / 131.
+int march_rows_solo(const DevState &d) {
+  constexpr int kRows[] = {8, 6, 4, 3, 2, 1};
+  constexpr long kWarps = 16 * 152;
+  int best = 0;
+  long best_c = 0;
+  for (int r : kRows) {
+    const long tiles = (long)march_tiles_x(d.g.nx) * march_tiles_y(d.g.ny, r);
+    const long c = (r + 3) * (16 * kWarps + 9 * tiles);
+    if (best == 0 || c < best_c) {
+      best = r;
+      best_c = c;
+    }
+  }
+  return best;
+}
 
 namespace {
 // one thread per (node row, tile column) entry of the row flags
@@ -947,10 +964,12 @@ int groups_fp32(const DevState &d, int tile_rows) {
   return march_groups(d.g.nx, d.g.ny, tile_rows);
 }
 
-// energy partials: tiles of the smallest tile height first, then the piece
-// blocks (at most 1216), then the phantom update's warps (at most 1216
-// blocks of kPhWarps)
-int energy_parts_fp32(const DevState &d) { return tiles_fp32(d, 8) + kPhWarps * 1216 + 1216 + 8; }
+// energy partials: tiles of the smallest tile height first (8 node rows in a
+// batch), then the piece blocks (at most 1216), then the phantom update's warps
+// (at most 1216 blocks of kPhWarps)
+int energy_parts_fp32(const DevState &d) {
+  return std::max(tiles_fp32(d, 8), tiles_fp32(d, march_rows_solo(d))) + kPhWarps * 1216 + 1216 + 8;
+}
 
 // piece-force blocks: one thread per split element in FP32, per piece in FP64
 int grid_pieces(const DevState &d) {

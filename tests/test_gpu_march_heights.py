@@ -1,0 +1,47 @@
+"""FP32-mixed node update: a mesh stepped alone picks its tile height from its
+size (1 to 8 node rows), a batch marches tiles of 8 rows or more.  The height
+decides which warp marches a node, not the node's arithmetic, so the fields
+and cracks of both are identical, bit for bit (needs a GPU)."""
+import numpy as np
+import pytest
+
+from paper_2509_01827_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2509_01827_gb300 import build
+    build.build()
+
+
+# the heights these sizes take alone: 1, 1, 2, 3, 4 and 6 rows
+@pytest.mark.parametrize("nx,ny,steps", [(59, 23, 260), (100, 40, 260), (512, 512, 40),
+                                         (770, 767, 20), (1030, 1021, 12), (1440, 1450, 8)])
+def test_solo_heights_equal_batch(nx, ny, steps):
+    from paper_2509_01827_gb300.cem import CEM_FP32_MIXED, Batch, Solver
+    p = inputs.notched_plate(nx, ny, traction=1e6 if nx == 100 else 2.5e6, phantom_cap=8000, crack_cap=4000)
+    p.energy_every = 7
+    a, c = Solver(p, precision=CEM_FP32_MIXED), Solver(p, precision=CEM_FP32_MIXED)
+    rng = np.random.default_rng(nx)
+    n = a.nodes()["vx"].size
+    v = dict(vx=rng.standard_normal(n) * 0.05, vy=rng.standard_normal(n) * 0.05)
+    for s in (a, c):
+        s.set_state(**v)
+    a.step(steps)
+    b = Batch([c])
+    b.set_config(16, 152)
+    b.step(steps)
+    na, nc = a.nodes(), c.nodes()
+    for k in ("ux", "uy", "vx", "vy", "m"):
+        np.testing.assert_array_equal(na[k], nc[k], err_msg=k)
+    ca, cc = a.cracks(), c.cracks()
+    for k in ("elem", "ka", "kb", "step", "nodes"):
+        np.testing.assert_array_equal(ca[k], cc[k], err_msg=k)
+    # the records differ by the grouping of FP32 partial sums at most: sums of
+    # non-negative terms, each partial of a few thousand terms rounded once a term
+    ea, ec = a.energy(), c.energy()
+    for k in ("KE", "SE"):
+        np.testing.assert_allclose(ea[k], ec[k], rtol=4096 * 2.0 ** -24, err_msg=k)
+    b.close()
