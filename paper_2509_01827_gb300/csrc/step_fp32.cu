@@ -459,6 +459,7 @@ __device__ __forceinline__ void march32_tile(const DevState &d, int tile_x, int 
   // terms this lane adds for the column right of its last (ua) and left of
   // its first (da), rows t-2 and t-1
   float2 ua0 = z2, ua1 = z2, da0 = z2, da1 = z2;
+  bool pieces_in = false;  // this step's piece forces are visible
   unsigned pk_on = 0;  // bit k: element (c_k, t-2) is split; its piece forces come this row
   bool bad = false;    // some updated velocity is not finite
   float se = 0.f;      // A/4 eps.sigma of owned edges
@@ -621,6 +622,13 @@ __device__ __forceinline__ void march32_tile(const DevState &d, int tile_x, int 
     // ---- pieces of split elements (c_k, t-2), prefetched into L1 one row ago:
     // local nodes 0 (c_k, t-2), 1 (c_k+1, t-2), 2 (c_k+1, t-1), 3 (c_k, t-1)
     if (!CLEAN && __any_sync(FULL, pk_on != 0)) {
+      if (!pieces_in) {
+        // the piece forces come from the kernel before this one (when launched as
+        // its programmatic dependent): wait until it has completed and its writes
+        // are visible.  Rows before the first split element did not need it.
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        pieces_in = true;
+      }
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         if ((pk_on >> k) & 1) {
@@ -640,7 +648,7 @@ __device__ __forceinline__ void march32_tile(const DevState &d, int tile_x, int 
     for (int k = 0; k < K; ++k)
       if (es0[k] == ST_CRACKED) {
         pk_on |= 1u << k;
-        prefetch_l1(d.pfe + (size_t)((t - 1) * g.nx + c0 + k) * 8);
+        if (pieces_in) prefetch_l1(d.pfe + (size_t)((t - 1) * g.nx + c0 + k) * 8);
       }
     // ---- nodes (c_k, t-2): every edge and piece touching them is in
     {
@@ -700,6 +708,8 @@ __device__ __forceinline__ void march32_tile(const DevState &d, int tile_x, int 
     da0 = da1; da1 = da2;
   }
   cp_async_wait<0>();  // no copy into the ring outlives the tile
+  // this kernel completes only after the one before it, whichever tiles met a piece
+  if (!CLEAN && !pieces_in) asm volatile("griddepcontrol.wait;" ::: "memory");
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     while (spmask[k]) {
@@ -767,10 +777,6 @@ __device__ __forceinline__ void march32_group(const DevState &d, int group, int 
     if (tile_clean(d, tile_x, tile_y * ty, ty)) {
       march32_tile<ENERGY, true>(d, tile_x, tile_y, ty, cur, first, part, rings[w]);
     } else {
-      // the other tiles read the piece forces of the kernel before this one
-      // (when launched as its programmatic dependent): wait until it has
-      // completed and its writes are visible
-      asm volatile("griddepcontrol.wait;" ::: "memory");
       march32_tile<ENERGY, false>(d, tile_x, tile_y, ty, cur, first, part, rings[w]);
     }
   } else if (ENERGY && lane == 0) {
@@ -783,9 +789,9 @@ template <bool ENERGY>
 __global__ void __launch_bounds__(32 * kMarchWarps, 4) k_march32(DevState d, int cur, int first,
                                                                   int ty) {
   // launched as a programmatic dependent of the kernel before it (the piece
-  // forces), which writes only the piece forces and its energy partials: a
-  // clean tile reads neither and starts at once, the others wait for that
-  // kernel (march32_group).  Everything else the tiles read was written by
+  // forces), which writes only the piece forces and its energy partials: every
+  // tile starts at once, and waits for that kernel when it first reads a
+  // piece force (a clean tile never).  Everything else the tiles read was written by
   // kernels that completed before the piece forces started.  The kernels
   // that follow may be placed once every CTA of this kernel has started
   // (they wait for it themselves).
