@@ -325,8 +325,11 @@ def cem_save_state(h) -> bytes:
 
 
 def cem_load_state(h, blob: bytes):
-    buf = C.create_string_buffer(blob, len(blob))
-    _chk(h, lib().cem_load_state(h, buf, len(blob)))
+    # the bytes object's own memory: a copy of it (fresh pages each call) took
+    # as long as the transfer
+    if not isinstance(blob, bytes):
+        raise TypeError(blob)
+    _chk(h, lib().cem_load_state(h, blob, len(blob)))
 
 
 def cem_mesh_destroy(h):
