@@ -347,10 +347,14 @@ constexpr int kHalo = (2 + kCols - 1) / kCols;
 constexpr int WX = (32 - 2 * kHalo) * kCols;  // owned columns of a tile
 static_assert(WX == kMarchWX && kHalo * kCols == kMarchLeft && 32 * kCols == kMarchSpan,
               "the row flags describe these tiles");
+struct MarchRow {
+  float4 u[kCols][32];
+  float2 v[kCols][32];
+  float mi[kCols][32];
+};
 struct MarchRing {
-  float4 u[kRing][kCols][32];
-  float2 v[kRing][kCols][32];
-  float mi[kRing][kCols][32];
+  MarchRow row[kRing];
+  __device__ __forceinline__ MarchRow &of(int r) { return row[(r + 4 * kRing) & (kRing - 1)]; }
 };
 
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem, int valid) {
@@ -404,21 +408,37 @@ __device__ __forceinline__ void march32_tile(const DevState &d, int tile_x, int 
   const float dt = d.mat.dtf;
   const float dtv = first ? 0.5f * dt : dt;
 
-  // stage node row r into ring slot r mod kRing (zeros outside the mesh; v
-  // and 1/m only for the owned nodes), one commit group per row
+  // stage node row r into its ring slot, one commit group per row.  v and 1/m
+  // are staged for the owned nodes only; u outside the mesh is zero (a clean
+  // tile's columns are all inside it).  Rows past j0 + TY + 1 are not read.
   auto stage = [&](int r) {
-    const int q = (r + 4 * kRing) & (kRing - 1);
-    const bool rin = r >= 0 && r <= g.ny;
-    const bool rown = own_lane && r >= j0 && r < j0 + TY;
+    if (r <= j0 + TY + 1) {
+      MarchRow &w = ring.of(r);
+      const bool rown = r >= j0 && r < j0 + TY && own_lane;
+      if (CLEAN) {
+        const int N = r * stride + c0;
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-      const int c = c0 + k;
-      const bool in = rin && c >= 0 && c <= g.nx;
-      const int N = in ? r * stride + c : 0;
-      cp_async16(&ring.u[q][k][lane], u4 + N, in ? 16 : 0);
-      const bool mine = in && rown;
-      cp_async8(&ring.v[q][k][lane], d.v2 + N, mine ? 8 : 0);
-      cp_async4(&ring.mi[q][k][lane], d.minvf + N, mine ? 4 : 0);
+        for (int k = 0; k < K; ++k) cp_async16(&w.u[k][lane], u4 + N + k, 16);
+        if (rown) {
+#pragma unroll
+          for (int k = 0; k < K; ++k) {
+            cp_async8(&w.v[k][lane], d.v2 + N + k, 8);
+            cp_async4(&w.mi[k][lane], d.minvf + N + k, 4);
+          }
+        }
+      } else {
+        const bool rin = r >= 0 && r <= g.ny;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          const int c = c0 + k;
+          const bool in = rin && c >= 0 && c <= g.nx;
+          const int N = in ? r * stride + c : 0;
+          cp_async16(&w.u[k][lane], u4 + N, in ? 16 : 0);
+          const bool mine = in && rown;
+          cp_async8(&w.v[k][lane], d.v2 + N, mine ? 8 : 0);
+          cp_async4(&w.mi[k][lane], d.minvf + N, mine ? 4 : 0);
+        }
+      }
     }
     cp_async_commit();
   };
@@ -448,7 +468,7 @@ __device__ __forceinline__ void march32_tile(const DevState &d, int tile_x, int 
   unsigned long long spmask[K];  // owned rows whose node has a load or prescribed velocity
 #pragma unroll
   for (int k = 0; k < K; ++k) {
-    U1[k] = ring.u[(j0 - 2 + 4 * kRing) & (kRing - 1)][k][lane];
+    U1[k] = ring.of(j0 - 2).u[k][lane];
     es1[k] = load_es(j0 - 3, k);
     esn[k] = load_es(j0 - 2, k);
     nf1[k] = nf2[k] = 0;
@@ -469,12 +489,12 @@ __device__ __forceinline__ void march32_tile(const DevState &d, int tile_x, int 
 #pragma unroll 1
   for (int t = j0 - 1; t <= j0 + TY + 1; ++t) {
     cp_async_wait<kAhead - 1>();  // rows up to t are in
-    const int sl = (t + 4 * kRing) & (kRing - 1);
+    const MarchRow &row = ring.of(t);
     float4 U0[K];
     int es0[K], nf0[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-      U0[k] = ring.u[sl][k][lane];
+      U0[k] = row.u[k][lane];
       es0[k] = esn[k];  // element (c_k, t-1)
       esn[k] = load_es(t, k);
       nf0[k] = load_nf(t, k);
@@ -658,36 +678,48 @@ __device__ __forceinline__ void march32_tile(const DevState &d, int tile_x, int 
       own0[K - 1] = padd(own0[K - 1], make_float2(dx, dy));
     }
     const int r = t - 2;
-    if (own_lane && r >= j0 && r <= g.ny) {
-      const int s2 = (r + 4 * kRing) & (kRing - 1);
+    if (r >= j0 && (CLEAN || r <= g.ny)) {
+      // both columns' updates side by side, without a branch between them
+      // (one after the other their latencies add up: 380 of a row's 870 clocks);
+      // the lanes and nodes they do not belong to store nothing
+      const MarchRow &old = ring.of(r);
+      const int N = r * stride + c0;
+      float4 U[K];
+      float2 vo[K], vn[K];
+      float mio[K];
+      bool mine[K];
 #pragma unroll
       for (int k = 0; k < K; ++k) {
-        const int c = c0 + k;
-        if (c > g.nx) continue;
-        const int N = r * stride + c;
-        const float fx = own0[k].x, fy = own0[k].y;
-        if (nf2[k]) {
-          // nodes with loads or prescribed velocities are updated after the
-          // march (FP64 work, out of the loop's registers)
-          d.fsp[N] = make_float2(fx, fy);
+        U[k] = old.u[k][lane];
+        vo[k] = old.v[k][lane];
+        mio[k] = old.mi[k][lane];
+        mine[k] = own_lane && (CLEAN || c0 + k <= g.nx);
+      }
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        vn[k].x = fmaf(dtv, -own0[k].x * mio[k], vo[k].x);
+        vn[k].y = fmaf(dtv, -own0[k].y * mio[k], vo[k].y);
+        df_add(U[k].x, U[k].y, dt * vn[k].x);
+        df_add(U[k].z, U[k].w, dt * vn[k].y);
+      }
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        if (!CLEAN && nf2[k]) {
+          // nodes with loads or prescribed velocities (owned ones) are updated
+          // after the march (FP64 work, out of the loop's registers)
+          d.fsp[N + k] = own0[k];
           spmask[k] |= 1ull << (r - j0);
-        } else {
-          const float4 Uo = ring.u[s2][k][lane];
-          const float2 vo = ring.v[s2][k][lane];
-          const float mio = ring.mi[s2][k][lane];
-          const float vxn = fmaf(dtv, -fx * mio, vo.x);
-          const float vyn = fmaf(dtv, -fy * mio, vo.y);
-          d.v2[N] = make_float2(vxn, vyn);
-          bad |= !(fabsf(vxn + vyn) <= FLT_MAX);  // NaN or Inf in either
-          float4 U = Uo;
-          df_add(U.x, U.y, dt * vxn);
-          df_add(U.z, U.w, dt * vyn);
-          d.u4[cur ^ 1][N] = U;
-          if (ENERGY && mio > 0.f) {
-            const float bx = first ? vo.x : 0.5f * (vo.x + vxn);
-            const float by = first ? vo.y : 0.5f * (vo.y + vyn);
-            ke2 += __fdividef(fmaf(bx, bx, by * by), mio);
-          }
+          mine[k] = false;
+        }
+        if (mine[k]) {
+          d.v2[N + k] = vn[k];
+          d.u4[cur ^ 1][N + k] = U[k];
+        }
+        bad |= mine[k] && !(fabsf(vn[k].x + vn[k].y) <= FLT_MAX);  // NaN or Inf in either
+        if (ENERGY && mine[k] && mio[k] > 0.f) {
+          const float bx = first ? vo[k].x : 0.5f * (vo[k].x + vn[k].x);
+          const float by = first ? vo[k].y : 0.5f * (vo[k].y + vn[k].y);
+          ke2 += __fdividef(fmaf(bx, bx, by * by), mio[k]);
         }
       }
     }
@@ -710,15 +742,57 @@ __device__ __forceinline__ void march32_tile(const DevState &d, int tile_x, int 
   cp_async_wait<0>();  // no copy into the ring outlives the tile
   // this kernel completes only after the one before it, whichever tiles met a piece
   if (!CLEAN && !pieces_in) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (!CLEAN) {
+    // nodes with loads or prescribed velocities, listed in the ring's memory
+    // and shared out over the warp's lanes: a lane that worked through its own
+    // columns' nodes took 1,000 clocks for each, and a loaded edge that runs up
+    // a tile gives all of its rows to one lane (16,400 clocks for 16 rows, with
+    // the whole grid waiting for the tiles beside the hole of a plate)
+    int *list = reinterpret_cast<int *>(&ring);
+    constexpr int kPush = 16;  // entries a lane adds for each column at a time
+    static_assert(32 * K * kPush * sizeof(int) <= sizeof(MarchRing), "list fits the ring");
+    unsigned long long left = 0;
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    while (spmask[k]) {
-      const int r = j0 + __ffsll((long long)spmask[k]) - 1;
-      spmask[k] &= spmask[k] - 1;
-      const int N = r * stride + c0 + k;
+    for (int k = 0; k < K; ++k) left |= spmask[k];
+    auto special = [&](int N) {
       const float2 F = d.fsp[N];
       ke += update_special(d, N, cur, first, F.x, F.y, u4[N], d.v2[N], d.minvf[N],
                            (int)d.nflag[N], ENERGY ? 1 : 0);
+    };
+    // a loaded row gives each lane one node a column: no list for that
+    bool few = true;
+#pragma unroll
+    for (int k = 0; k < K; ++k) few = few && (spmask[k] & (spmask[k] - 1)) == 0;
+    if (__all_sync(FULL, few)) {
+#pragma unroll
+      for (int k = 0; k < K; ++k)
+        if (spmask[k]) special((j0 + __ffsll((long long)spmask[k]) - 1) * stride + c0 + k);
+      left = 0;
+    }
+    while (__any_sync(FULL, left != 0)) {
+      int mine = 0;
+#pragma unroll
+      for (int k = 0; k < K; ++k) mine += min(__popcll(spmask[k]), kPush);
+      int at = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(FULL, at, o);
+        if (lane >= o) at += v;
+      }
+      const int total = __shfl_sync(FULL, at, 31);
+      at -= mine;
+      left = 0;
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        for (int q = 0; q < kPush && spmask[k]; ++q) {
+          list[at++] = (j0 + __ffsll((long long)spmask[k]) - 1) * stride + c0 + k;
+          spmask[k] &= spmask[k] - 1;
+        }
+        left |= spmask[k];
+      }
+      __syncwarp();  // the list, and the forces left by the lanes of the march
+      for (int q = lane; q < total; q += 32) special(list[q]);
+      __syncwarp();  // the list is read before it is written again
     }
   }
   // a non-finite velocity (NaN or Inf) is reported through the status word
@@ -914,20 +988,20 @@ cudaError_t launch_eval32(const DevState &d, int cur, cudaStream_t st);
 cudaError_t launch_eval32_batch(const BatchDev &b, cudaStream_t st);
 
 // Tile height of a mesh stepped alone.  A tile marches its rows and three more one
-// after another, 1.6 us each whatever else runs, and 2432 resident warps (four CTAs of
-// four on each of 152 SMs) get through one row each in another 0.9 us when they share
-// the SMs' issue slots, so the height r with the least (r + 3) (1.6 + 0.9 tiles / 2432)
-// is taken.  The node update of an elastic n x n plate, us, at 8 / 6 / 4 / 2 / 1 rows:
-// n = 128 22.0 / 20.5 / 17.4 / 12.7 / 10.9, 512 25.3 / 22.7 / 18.6 / 16.6 / 16.7,
-// 1024 30.9 / 27.9 / 24.9 / 25.4 / -, 2048 58.2 / 59.8 / 66.7 / 88 / 131.
+// after another, 0.6 us each whatever else runs, and 2432 resident warps (four CTAs of
+// four on each of 152 SMs) get through one row each in another 1 us when they share
+// the SMs' issue slots, so the height r with the least (r + 3) (0.6 + tiles / 2432) is
+// taken.  The node update of an elastic n x n plate, us, at 16 / 8 / 4 / 2 / 1 rows:
+// n = 128 19.4 / 14.4 / 12.4 / 10.6 / 10.6, 512 22.6 / 17.0 / 14.3 / 14.3 / 14.8,
+// 1024 26.8 / 23.3 / 22.9 / 25.5 / 35.1, 2048 52.5 / 55.4 / 62.0 / 80.0 / 115.
 int march_rows_solo(const DevState &d) {
-  constexpr int kRows[] = {8, 6, 4, 3, 2, 1};
+  constexpr int kRows[] = {16, 8, 6, 4, 3, 2, 1};
   constexpr long kWarps = 16 * 152;
   int best = 0;
   long best_c = 0;
   for (int r : kRows) {
     const long tiles = (long)march_tiles_x(d.g.nx) * march_tiles_y(d.g.ny, r);
-    const long c = (r + 3) * (16 * kWarps + 9 * tiles);
+    const long c = (r + 3) * (3 * kWarps + 5 * tiles);
     if (best == 0 || c < best_c) {
       best = r;
       best_c = c;

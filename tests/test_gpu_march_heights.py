@@ -1,5 +1,5 @@
 """FP32-mixed node update: a mesh stepped alone picks its tile height from its
-size (1 to 8 node rows), a batch marches tiles of 8 rows or more.  The height
+size (1 to 16 node rows), a batch marches tiles of 8 rows or more.  The height
 decides which warp marches a node, not the node's arithmetic, so the fields
 and cracks of both are identical, bit for bit (needs a GPU)."""
 import numpy as np
@@ -16,7 +16,7 @@ def _built():
     build.build()
 
 
-# the heights these sizes take alone: 1, 1, 2, 3, 4 and 6 rows
+# the heights these sizes take alone: 1, 1, 3, 4, 6 and 8 rows, 16 above
 @pytest.mark.parametrize("nx,ny,steps", [(59, 23, 260), (100, 40, 260), (512, 512, 40),
                                          (770, 767, 20), (1030, 1021, 12), (1440, 1450, 8)])
 def test_solo_heights_equal_batch(nx, ny, steps):
