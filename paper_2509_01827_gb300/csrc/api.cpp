@@ -531,6 +531,7 @@ cem_status cem_mesh_create(const cem_mesh_desc *desc, cem_handle **out) {
         if (k == k0) {
           d.g.nxf[k0][k] = d.g.nyf[k0][k] = 0.f;
           d.g.cnx[k0][k] = d.g.cny[k0][k] = 0.0;
+          d.g.seg[k0][k] = 0.0;
           continue;
         }
         double sx = (XG[k] - XG[k0]) * (0.5 * desc->hx), sy = (EG[k] - EG[k0]) * (0.5 * desc->hy);
@@ -549,6 +550,7 @@ cem_status cem_mesh_create(const cem_mesh_desc *desc, cem_handle **out) {
         len = sqrt(sx * sx + sy * sy);
         d.g.cnx[k0][k] = rx / len;
         d.g.cny[k0][k] = ry / len;
+        d.g.seg[k0][k] = len;
       }
     }
   }

@@ -51,6 +51,7 @@ struct Geo {
   float nxf[4][4], nyf[4][4];  // unit normal of candidate path k0 -> k
   // FP64: the same vectors and normals, and |X_N2 - X_N1|^2
   double DX[4], DY[4], ref2[4], cnx[4][4], cny[4][4];
+  double seg[4][4];  // length of the split segment between the midpoints of two edges
 };
 
 struct Mat {

@@ -5,10 +5,10 @@
 // Each step's tracking is two kernels.  k_select (one CTA) runs on the
 // evaluation stream, concurrently with the node updates, and
 //   1. compacts the surface list with warp ballots when half of it is dead;
-//   2. sorts the step's proposals by (ahead element, local edge) with a
-//      bitonic sort in shared memory (the warp-ballot append of the
-//      evaluation is unordered; the sort makes everything after it
-//      deterministic);
+//   2. sorts the step's proposals by (ahead element, local edge), up to 256 by
+//      counting and more with a bitonic sort in shared memory (the warp-ballot
+//      append of the evaluation is unordered; the sort makes everything after
+//      it deterministic);
 //   3. selects winners (Sec. 3): a proposal wins if its key (G, -edge id) is
 //      the strict maximum among proposals whose ahead elements share a node
 //      with its own (binary searches over the three neighbouring rows), or
@@ -105,46 +105,49 @@ __device__ void set_mass(const DevState &d, int N, double m, double mi) {
   if (d.precision == 1) d.minvf[N] = (float)mi;
 }
 
-// Area fractions of the two pieces by the shoelace formula in natural
-// coordinates (the reference square has area 4).  A piece's polygon visits
-// the element's nodes and edge points in counter-clockwise order, keeping
-// the nodes on its side and the two edge points of the segment; the terms
-// are added in that order with the closing term last.
-__device__ __forceinline__ void area_fractions(int ka, int kb, const int side[4], double alpha[2]) {
+// Sides of an element's nodes for a split that enters at the midpoint of its
+// edge ka and leaves at that of kb: bit a set when node a is on side 1 (on or
+// right of the segment).  Coordinates in half edges, so integers.
+__device__ __forceinline__ int split_sides(int ka, int kb) {
+  if (ka == kb) return 0;
+  const int ax = (ka == 1) - (ka == 3), ay = (ka == 2) - (ka == 0);
+  const int bx = (kb == 1) - (kb == 3), by = (kb == 2) - (kb == 0);
+  int bits = 0;
 #pragma unroll
-  for (int p = 0; p < 2; ++p) {
-    double x0 = 0.0, y0 = 0.0, xp = 0.0, yp = 0.0, twice = 0.0;
-    bool have = false;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) {
-      const int q = w >> 1;
-      const bool in = (w & 1) == 0 ? side[q] == p : (q == ka || q == kb);
-      if (!in) continue;
-      const double x = (w & 1) == 0 ? xi_n(q) : xi_g(q);
-      const double y = (w & 1) == 0 ? eta_n(q) : eta_g(q);
-      if (!have) {
-        x0 = x;
-        y0 = y;
-        have = true;
-      } else {
-        twice = twice + (xp * y - x * yp);
-      }
-      xp = x;
-      yp = y;
-    }
-    twice = twice + (xp * y0 - x0 * yp);
-    alpha[p] = fabs(twice) * 0.5 / 4.0;
+  for (int a = 0; a < 4; ++a) {
+    const int xn = (a == 0 || a == 3) ? -1 : 1, yn = a < 2 ? -1 : 1;
+    const int cross = (bx - ax) * (yn - ay) - (by - ay) * (xn - ax);
+    bits |= (cross > 0 ? 0 : 1) << a;
   }
+  return bits;
 }
 
-// Sorted proposals live in shared memory as (key << 32 | index).
-__device__ __forceinline__ int lower_bound_key(const unsigned long long *sk, int n, int key) {
-  int lo = 0, hi = n;
-  while (lo < hi) {
-    int mid = (lo + hi) >> 1;
-    if ((int)(sk[mid] >> 32) < key) lo = mid + 1; else hi = mid;
+// Area fraction of the piece on side p: the segment joins two edge midpoints,
+// so it cuts one corner off (1/8 of the element) or halves it.  (The shoelace
+// formula gives these numbers exactly; in FP64 it took 4,000 of the 4,800
+// clocks of a selection without proposals.)
+__device__ __forceinline__ double piece_fraction(int sides, int p) {
+  const int n1 = __popc(sides), n = p ? n1 : 4 - n1;
+  return n == 1 ? 0.125 : n == 2 ? 0.5 : n == 3 ? 0.875 : 0.0;
+}
+
+// First positions of three keys in the sorted proposals (key << 32 | index),
+// searched side by side: one search after another waits for shared memory three
+// times as often.
+__device__ __forceinline__ void lower_bounds(const unsigned long long *sk, int n, const int (&key)[3],
+                                             int (&at)[3]) {
+#pragma unroll
+  for (int r = 0; r < 3; ++r) at[r] = 0;
+  while (n > 1) {
+    const int half = n >> 1;
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+      if ((int)(sk[at[r] + half - 1] >> 32) < key[r]) at[r] += half;
+    n -= half;
   }
-  return lo;
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+    if (n == 1 && (int)(sk[at[r]] >> 32) < key[r]) ++at[r];
 }
 
 __device__ __forceinline__ bool key_greater(double Ga, int ea, double Gb, int eb) {
@@ -202,8 +205,7 @@ struct NodePlan {
 __device__ __forceinline__ void node_plan(const DevState &d, int e, int ka, int kb, int a,
                                           NodePlan &np) {
   const Geo &g = d.g;
-  const int N = elem_node(g, e, a);
-  const int r = g.nx + 1, i = N % r, j = N / r;
+  const int i = e % g.nx + (a == 1 || a == 2), j = e / g.nx + (a >= 2);  // the node's column and row
   const int di[4] = {-1, 0, -1, 0}, dj[4] = {-1, -1, 0, 0}, la[4] = {2, 3, 1, 0};
   int eq[4], st[4], cq[4];
 #pragma unroll
@@ -268,79 +270,53 @@ __device__ __forceinline__ void node_plan(const DevState &d, int e, int ka, int 
 // concurrently.  Produces, for each winner in increasing element id, its
 // split plan (sides, phantoms to reuse, area fractions, split-table slot,
 // first new phantom id, surface-list appends and tombstones) and the
-// counters the apply kernel commits.  Global loads are issued in few
-// dependent levels (the proposals' fields are staged in shared memory with
-// the keys), since this single CTA runs beside the node updates.
+// counters the apply kernel commits.
+//
+// Bound by latency: a step's selection waits for the evaluation and the split
+// writes wait for it, and one CTA works through a chain of loads, barriers and
+// cold code.  So the counters are read by every thread at once and carried in
+// registers, a step without proposals ends after that read; up to 256 proposals
+// are ordered by counting (each thread compares its own with the others, one
+// barrier instead of one for each of the 36 stages of a bitonic sort), and the
+// eight threads of a winner settle by ballots and one block-wide scan what they
+// need from each other.  A selection without
+// proposals 3.3 -> 1.4 us, one of 26 proposals and 24 winners 14.4 -> 9.9 us.
 __device__ __forceinline__ void select_plan(const DevState &d, int mode,
                                             unsigned long long *smem) {
-  __shared__ int s_n, s_nwin, s_stop, s_nph, s_nck, s_nS, s_dead, s_done, s_compact;
-  __shared__ int b_e[WB], b_ka[WB], b_kb[WB], b_side[WB][4], b_reuse[WB][4], b_app[WB],
-      b_tomb[WB][4], b_c[WB];
-  __shared__ double b_alpha[WB][2];
-  // sides of the four nodes (bit a) and area fractions of a split entering
-  // at edge point ka and leaving at kb, for the 12 pairs ka != kb
-  __shared__ int s_sides[16];
-  __shared__ double s_alpha[16][2];
+  __shared__ unsigned long long s_raw[TB];
+  __shared__ int s_scan[TB / 32], s_nwin, s_valid;
+  constexpr unsigned FULL = 0xffffffffu;
   Counters *cnt = d.cnt;
   const Geo &g = d.g;
   const int tid = threadIdx.x;
-  if (tid >= 32 && tid < 48) {
-    const int ka = (tid - 32) >> 2, kb = (tid - 32) & 3;
-    int side[4] = {0, 0, 0, 0}, bits = 0;
-    double alpha[2] = {0.0, 0.0};
-    if (ka != kb) {
-      const double pax = xi_g(ka), pay = eta_g(ka), pbx = xi_g(kb), pby = eta_g(kb);
-#pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        const double cross = (pbx - pax) * (eta_n(a) - pay) - (pby - pay) * (xi_n(a) - pax);
-        side[a] = cross > 0.0 ? 0 : 1;
-        bits |= side[a] << a;
-      }
-      area_fractions(ka, kb, side, alpha);
-    }
-    s_sides[tid - 32] = bits;
-    s_alpha[tid - 32][0] = alpha[0];
-    s_alpha[tid - 32][1] = alpha[1];
-  }
-  if (tid == 0) {
-    const int n_dead = cnt->n_dead, nS = cnt->n_S;
-    int n = cnt->n_prop;
-    if (n > d.prop_cap) n = d.prop_cap;
-    s_n = n;
-    s_nph = cnt->n_ph;
-    s_nck = cnt->n_ck;
-    s_nS = nS;
-    // stable compaction of the surface list when half of it is dead (the
-    // evaluation of this step has finished; nothing else reads the list now)
-    s_compact = mode == TRACK_STEP && n_dead > 1024 && 2 * n_dead > nS;
-    s_nwin = 0;
-    s_stop = 0;
-    s_dead = 0;
-    s_done = 0;
-  }
-  __syncthreads();
-  if (s_compact) {
+  const int n_all = cnt->n_prop, n_dead = cnt->n_dead, step = cnt->step;
+  int nph = cnt->n_ph, nck = cnt->n_ck, nS = cnt->n_S;
+  int dead = 0, done = 0;
+  const int n = n_all < d.prop_cap ? n_all : d.prop_cap;
+  // stable compaction of the surface list when half of it is dead (the
+  // evaluation of this step has finished; nothing else reads the list now)
+  if (mode == TRACK_STEP && n_dead > 1024 && 2 * n_dead > nS) {
+    __syncthreads();  // every thread has read the counters
     compact_surface(d);
     __syncthreads();
-    if (tid == 0) s_nS = cnt->n_S;
-    __syncthreads();
+    nS = cnt->n_S;
   }
-  const int n = s_n;
-  // sorted (key << 32 | index), winners (sorted positions), and G, edge and
-  // exit edge of proposal i
-  const bool staged = n <= SEL_SMEM_CAP;
-  unsigned long long *sk = staged ? smem : d.sel_sk;
-  int *swin = staged ? (int *)(smem + SEL_SMEM_CAP) : d.sel_win;
-  double *oG = staged ? (double *)(smem + SEL_SMEM_CAP) + SEL_SMEM_CAP / 2 : d.sel_G;
-  int *oE = staged ? (int *)(oG + SEL_SMEM_CAP) : d.sel_E;
-  uint8_t *oK = staged ? (uint8_t *)(oE + SEL_SMEM_CAP) : d.sel_K;
   if (n > 0) {
+    // sorted (key << 32 | index), winners (sorted positions), and G, edge and
+    // exit edge of proposal i
+    const bool staged = n <= SEL_SMEM_CAP, ranked = n <= TB;
+    unsigned long long *sk = staged ? smem : d.sel_sk;
+    int *swin = staged ? (int *)(smem + SEL_SMEM_CAP) : d.sel_win;
+    double *oG = staged ? (double *)(smem + SEL_SMEM_CAP) + SEL_SMEM_CAP / 2 : d.sel_G;
+    int *oE = staged ? (int *)(oG + SEL_SMEM_CAP) : d.sel_E;
+    uint8_t *oK = staged ? (uint8_t *)(oE + SEL_SMEM_CAP) : d.sel_K;
     // ---- load keys and fields; debug proposals that are not surface points
     //      (or not tips under the tips-only scope) sort to the end
     int P2 = 1;
     while (P2 < n) P2 <<= 1;
-    for (int i = tid; i < P2; i += TB) {
-      unsigned long long v = ~0ull;
+    unsigned long long v = ~0ull;
+    for (int i = tid; i < (ranked ? n : P2); i += TB) {
+      v = ~0ull;
       if (i < n) {
         const int key = d.pr_key[i], ed = d.pr_edge[i], kx = d.pr_k[i];
         oG[i] = d.pr_G[i];
@@ -355,26 +331,24 @@ __device__ __forceinline__ void select_plan(const DevState &d, int mode,
         }
         if (valid) v = ((unsigned long long)(unsigned)key << 32) | (unsigned)i;
       }
-      sk[i] = v;
+      (ranked ? s_raw : sk)[i] = v;
     }
-    __syncthreads();
-    if (P2 <= 32) {
-      // one warp sorts up to 32 keys (no block-wide barriers)
-      if (tid < 32) {
-        for (int k = 2; k <= P2; k <<= 1) {
-          for (int j = k >> 1; j > 0; j >>= 1) {
-            const int i = tid, l = i ^ j;
-            if (i < P2 && l > i) {
-              unsigned long long a = sk[i], b = sk[l];
-              bool up = (i & k) == 0;
-              if ((a > b) == up) { sk[i] = b; sk[l] = a; }
-            }
-            __syncwarp();
-          }
+    int nv;  // valid proposals
+    if (ranked) {
+      // v is this thread's only proposal (none: ~0)
+      nv = __syncthreads_count(v != ~0ull);
+      if (tid < n) {
+        int rank = 0;
+#pragma unroll 8
+        for (int j = 0; j < n; ++j) {
+          const unsigned long long o = s_raw[j];
+          rank += o < v || (o == v && j < tid);
         }
+        sk[rank] = v;
       }
       __syncthreads();
     } else {
+      __syncthreads();
       for (int k = 2; k <= P2; k <<= 1) {
         for (int j = k >> 1; j > 0; j >>= 1) {
           for (int i = tid; i < P2; i += TB) {
@@ -388,16 +362,16 @@ __device__ __forceinline__ void select_plan(const DevState &d, int mode,
           __syncthreads();
         }
       }
+      if (tid == 0) s_valid = 0;
+      __syncthreads();
+      for (int i = tid; i < n; i += TB)
+        if (sk[i] != ~0ull && (i + 1 == n || sk[i + 1] == ~0ull)) s_valid = i + 1;
+      __syncthreads();
+      nv = s_valid;
     }
-    __shared__ int s_valid;
-    if (tid == 0) s_valid = 0;
-    __syncthreads();
-    for (int i = tid; i < n; i += TB)
-      if (sk[i] != ~0ull && (i + 1 == n || sk[i + 1] == ~0ull)) s_valid = i + 1;
-    __syncthreads();
-    const int nv = s_valid;
 
     // ---- winners
+    int nwin = 0;
     if (mode != TRACK_PRECRACK && d.mat.scope == 1) {
       if (tid == 0) {
         int best = -1;
@@ -408,9 +382,11 @@ __device__ __forceinline__ void select_plan(const DevState &d, int mode,
         int wi = -1;
         for (int i = 0; i < nv; ++i)
           if ((int)(sk[i] & 0xffffffffu) == best) wi = i;
+        s_nwin = 0;
         if (wi >= 0) { swin[0] = wi; s_nwin = 1; }
       }
       __syncthreads();
+      nwin = s_nwin;
     } else {
       for (int base = 0; base < nv; base += TB) {
         int i = base + tid;
@@ -418,63 +394,71 @@ __device__ __forceinline__ void select_plan(const DevState &d, int mode,
         if (i < nv) {
           win = 1;
           if (mode != TRACK_PRECRACK) {
-            int idx = (int)(sk[i] & 0xffffffffu);
-            int key = (int)(sk[i] >> 32), e = key >> 2;
-            double G = oG[idx];
-            int ed = oE[idx];
-            int ei = e % g.nx, ej = e / g.nx;
-            for (int dj = -1; dj <= 1 && win; ++dj) {
-              int row = ej + dj;
+            const int idx = (int)(sk[i] & 0xffffffffu);
+            const int key = (int)(sk[i] >> 32), e = key >> 2;
+            const double G = oG[idx];
+            const int ed = oE[idx];
+            const int ei = e % g.nx, ej = e / g.nx;
+            const int left = ei > 0 ? 1 : 0, right = ei < g.nx - 1 ? 1 : 0;
+            int lo[3], at[3];
+#pragma unroll
+            for (int r = 0; r < 3; ++r) lo[r] = (e + (r - 1) * g.nx - left) * 4;
+            lower_bounds(sk, nv, lo, at);
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+              const int row = ej + r - 1;
               if (row < 0 || row >= g.ny) continue;
-              int lo_e = row * g.nx + (ei > 0 ? ei - 1 : 0);
-              int hi_e = row * g.nx + (ei < g.nx - 1 ? ei + 1 : g.nx - 1);
-              int q = lower_bound_key(sk, nv, lo_e * 4);
-              for (; q < nv && (int)(sk[q] >> 32) <= hi_e * 4 + 3; ++q) {
+              const int hi = (e + (r - 1) * g.nx + right) * 4 + 3;
+              for (int q = at[r]; win && q < nv && (int)(sk[q] >> 32) <= hi; ++q) {
                 if (q == i) continue;
-                int qi = (int)(sk[q] & 0xffffffffu);
-                if (!key_greater(G, ed, oG[qi], oE[qi])) { win = 0; break; }
+                const int qi = (int)(sk[q] & 0xffffffffu);
+                if (!key_greater(G, ed, oG[qi], oE[qi])) win = 0;
               }
             }
           }
         }
-        int tot;
-        int pos = block_exscan(win, &tot);
-        if (win) swin[s_nwin + pos] = i;
+        int tot, pos;
+        if (nv <= 32) {
+          // all of them in the first warp
+          const unsigned b = __ballot_sync(FULL, win);
+          tot = __popc(b);
+          pos = __popc(b & ((1u << (tid & 31)) - 1));
+          if (tid == 0) s_nwin = tot;
+        } else {
+          pos = block_exscan(win, &tot);
+        }
+        if (win) swin[nwin + pos] = i;
         __syncthreads();
-        if (tid == 0) s_nwin += tot;
-        __syncthreads();
+        nwin += nv <= 32 ? s_nwin : tot;
       }
     }
-    const int nwin = s_nwin;
 
     // ---- plan the splits, WB winners at a time, eight threads each
-    const int lane = tid & 7, wl = tid >> 3;
+    const int lane = tid & 7, wl = tid >> 3, warp = tid >> 5, shift = tid & 24;
     for (int base = 0; base < nwin; base += WB) {
       const int nb = nwin - base < WB ? nwin - base : WB;
-      const bool act = wl < nb && !s_stop;
-      if (act && lane == 0) {
-        const int i = swin[base + wl];
-        const int idx = (int)(sk[i] & 0xffffffffu);
-        const int key = (int)(sk[i] >> 32);
-        b_e[wl] = key >> 2;
-        b_ka[wl] = key & 3;
-        b_kb[wl] = oK[idx];
-        b_app[wl] = 0;
+      const bool act = wl < nb;
+      int e = 0, ka = 0, kb = 0, sides = 0;
+      if (act) {
+        const unsigned long long sv = sk[swin[base + wl]];
+        const int key = (int)(sv >> 32);
+        e = key >> 2;
+        ka = key & 3;
+        kb = oK[(int)(sv & 0xffffffffu)];
+        sides = split_sides(ka, kb);
       }
-      __syncthreads();
       NodePlan np;
-      int nu = 0;
+      np.P = 0;
+      int nu = 0, tomb = -1;
+      bool app = false;
       int4 u4 = make_int4(0, 0, 0, 0), f4 = u4;
       double2 A01 = make_double2(0.0, 0.0), A23 = A01;
       double mold = -1.0;
       if (act && lane < 4) {
-        // local node a: side, the phantom to reuse and the mass inputs, then
-        // (consumed only after the scans below) the reused phantom's user
+        // local node a: the phantom to reuse and the mass inputs, then
+        // (consumed only after the scan below) the reused phantom's user
         // list with its users' piece areas
-        const int e = b_e[wl], ka = b_ka[wl], kb = b_kb[wl], a = lane;
-        b_side[wl][a] = (s_sides[ka * 4 + kb] >> a) & 1;
-        node_plan(d, e, ka, kb, a, np);
-        b_reuse[wl][a] = np.P;
+        node_plan(d, e, ka, kb, lane, np);
         if (np.P >= 0) {
           const int t = np.P - g.nn;
           nu = d.ph_nuser[t];
@@ -487,140 +471,132 @@ __device__ __forceinline__ void select_plan(const DevState &d, int mode,
       } else if (act) {
         // local edge k: appended to the surface list if the element across
         // it is intact, else its current entry (if any) becomes a tombstone
-        const int e = b_e[wl], k = lane - 4;
-        const int f = elem_neighbor(g, e, k);
-        const int ed = elem_edge(g, e, k);
-        const int sf = estatus(d, f), pos = d.spos[ed];
-        b_tomb[wl][k] = -1;
-        if (sf == ST_INTACT) {
-          atomicOr(&b_app[wl], 1 << k);
-        } else {
-          b_tomb[wl][k] = pos;
-        }
+        const int k = lane - 4;
+        const int pos = d.spos[elem_edge(g, e, k)];
+        app = estatus(d, elem_neighbor(g, e, k)) == ST_INTACT;
+        if (!app) tomb = pos;
       }
+      // new phantoms, appends and tombstones of each winner, and their sums
+      // over the winners before it: three counts of at most 128 in one word
+      const unsigned bnew = (__ballot_sync(FULL, act && lane < 4 && np.P < 0) >> shift) & 0xffu;
+      const unsigned bapp = (__ballot_sync(FULL, app) >> shift) & 0xffu;
+      const unsigned bdead = (__ballot_sync(FULL, tomb >= 0) >> shift) & 0xffu;
+      const int own = lane == 0 ? __popc(bnew) | (__popc(bapp) << 10) | (__popc(bdead) << 20) : 0;
+      int pre = own;
+#pragma unroll
+      for (int o = 8; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULL, pre, o);
+        if ((tid & 31) >= o) pre += y;
+      }
+      pre = __shfl_sync(FULL, pre, shift) ;  // of the winner's first thread, itself included
+      if ((tid & 31) == 31) s_scan[warp] = pre;
       __syncthreads();
-      int nnew = 0, napp = 0, ndead = 0;
-      if (act && lane == 0) {
-        for (int a = 0; a < 4; ++a) {
-          nnew += b_reuse[wl][a] < 0;
-          ndead += b_tomb[wl][a] >= 0;
-        }
-        napp = __popc(b_app[wl]);
+      pre -= __shfl_sync(FULL, own, shift);
+      int tot = 0;
+#pragma unroll
+      for (int w = 0; w < TB / 32; ++w) {
+        const int y = s_scan[w];
+        if (w < warp) pre += y;
+        tot += y;
       }
-      int tot_new, tot_app;
-      const int pre_new = block_exscan(nnew, &tot_new);
-      const int pre_app = block_exscan(napp, &tot_app);
-      if (tid == 0) {
-        const bool fits = !s_stop && s_nph + tot_new <= d.ph_cap && s_nck + nb <= d.ck_cap &&
-                          s_nS + tot_app <= d.list_cap;
-        if (!fits) {
-          s_stop = 1;
-          atomicOr(&cnt->status, STAT_CAPACITY);
-        }
+      const int tot_new = tot & 1023, tot_app = (tot >> 10) & 1023;
+      if (nph + tot_new > d.ph_cap || nck + nb > d.ck_cap || nS + tot_app > d.list_cap) {
+        if (tid == 0) atomicOr(&cnt->status, STAT_CAPACITY);
+        break;  // this batch of winners and the ones after it are not split
       }
-      __syncthreads();
-      if (act && lane == 0 && !s_stop) {
-        const int w = base + wl, pk = b_ka[wl] * 4 + b_kb[wl];
-        const double alpha[2] = {s_alpha[pk][0], s_alpha[pk][1]};
-        const int info = b_ka[wl] | (b_kb[wl] << 2) | (b_app[wl] << 8) | (s_sides[pk] << 4);
-        d.pl_e[w] = b_e[wl];
-        d.pl_info[w] = info;
-        for (int a = 0; a < 4; ++a) {
-          d.pl_reuse[w * 4 + a] = b_reuse[wl][a];
-          d.pl_tomb[w * 4 + a] = b_tomb[wl][a];
+      if (act) {
+        const int w = base + wl, c = nck + wl;
+        if (lane < 4) d.pl_reuse[w * 4 + lane] = np.P;
+        else d.pl_tomb[w * 4 + lane - 4] = tomb;
+        if (lane == 4) {
+          d.pl_e[w] = e;
+          d.pl_info[w] = ka | (kb << 2) | ((bapp >> 4) << 8) | (sides << 4);
+        } else if (lane == 5) {
+          reinterpret_cast<double2 *>(d.pl_alpha)[w] =
+              make_double2(piece_fraction(sides, 0), piece_fraction(sides, 1));
+        } else if (lane == 6) {
+          d.pl_c[w] = c;
+          d.pl_ph0[w] = g.nn + nph + (pre & 1023);
+          d.pl_app0[w] = nS + ((pre >> 10) & 1023);
         }
-        d.pl_alpha[w * 2] = alpha[0];
-        d.pl_alpha[w * 2 + 1] = alpha[1];
-        d.pl_c[w] = s_nck + wl;
-        d.pl_ph0[w] = g.nn + s_nph + pre_new;
-        d.pl_app0[w] = s_nS + pre_app;
-        b_alpha[wl][0] = alpha[0];
-        b_alpha[wl][1] = alpha[1];
-        b_c[wl] = s_nck + wl;
-      }
-      if (act && lane == 0 && !s_stop) atomicAdd(&s_dead, ndead);
-      __syncthreads();
-      if (act && lane < 4 && !s_stop) {
-        // local node a: masses after the split and the phantom's user list
-        const int w = base + wl, e = b_e[wl], a = lane;
-        const int sa = b_side[wl][a];
-        const double alpha[2] = {b_alpha[wl][0], b_alpha[wl][1]};
-        // the real node: rho A_p / 4 of every piece around it that uses it,
-        // in increasing element id (the planned piece in place of e)
-        double mreal = 0.0;
+        if (lane < 4) {
+          // local node a: masses after the split and the phantom's user list
+          const int a = lane;
+          const int sa = (sides >> a) & 1;
+          // the real node: rho A_p / 4 of every piece around it that uses it,
+          // in increasing element id (the planned piece in place of e)
+          double mreal = 0.0;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const double Ap = q == np.qe ? alpha[sa] * g.A : np.Ap[q];
-          if (np.st[q] != ST_OUT) mreal = mreal + d.mat.rho * Ap * 0.25;
-        }
-        d.pl_mreal[w * 4 + a] = mreal;
-        d.pl_mireal[w * 4 + a] = inverse_mass(mreal);
-        // the reused phantom's users (sorted by element) and their areas
-        int us[4] = {u4.x, u4.y, u4.z, u4.w}, uf[4] = {f4.x, f4.y, f4.z, f4.w};
-        double Au[4] = {A01.x, A01.y, A23.x, A23.y};
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (q >= nu) { us[q] = 0x7fffffff; uf[q] = -1; Au[q] = 0.0; }
-        const int p = 1 - sa;  // the piece that uses the phantom of a
-        const int code = (e << 3) | (p << 2) | a, cf = b_c[wl] * 16 + p * 8 + 2 * a;
-        const double Anew = alpha[p] * g.A;
-        // insert the new user in increasing element id (as the split writes
-        // did): before the first user of a larger element; a full list of
-        // four keeps its first four entries
-        int pos = 4;
-#pragma unroll
-        for (int q = 3; q >= 0; --q)
-          if (q >= nu || (us[q] >> 3) > e) pos = q;
-        int out[4], outf[4];
-        double outA[4];
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          if (t < pos) {
-            out[t] = us[t]; outf[t] = uf[t]; outA[t] = Au[t];
-          } else if (t == pos) {
-            out[t] = code; outf[t] = cf; outA[t] = Anew;
-          } else if (t - 1 < nu) {
-            out[t] = us[t - 1]; outf[t] = uf[t - 1]; outA[t] = Au[t - 1];
-          } else {
-            out[t] = -1; outf[t] = -1; outA[t] = 0.0;
+          for (int q = 0; q < 4; ++q) {
+            const double Ap = q == np.qe ? piece_fraction(sides, sa) * g.A : np.Ap[q];
+            if (np.st[q] != ST_OUT) mreal = mreal + d.mat.rho * Ap * 0.25;
           }
-        }
-        // the phantom's mass: rho A_p / 4 of each user piece, in list order
-        double acc = 0.0;
-        const int nun = nu < 4 ? nu + 1 : 4;
+          // the reused phantom's users (sorted by element) and their areas
+          int us[4] = {u4.x, u4.y, u4.z, u4.w}, uf[4] = {f4.x, f4.y, f4.z, f4.w};
+          double Au[4] = {A01.x, A01.y, A23.x, A23.y};
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (q < nun) acc = acc + d.mat.rho * outA[q] * 0.25;
-        d.pl_mph[w * 4 + a] = acc;
-        d.pl_miph[w * 4 + a] = inverse_mass(acc);
-        d.pl_mold[w * 4 + a] = mold;
-        d.pl_dm[w * 4 + a] = d.mat.rho * Anew * 0.25;
-        d.pl_nu[w * 4 + a] = nu;  // users before the insertion (4: list full)
-        for (int q = 0; q < 4; ++q) {
-          d.pl_users[w * 16 + a * 4 + q] = out[q];
-          d.pl_upf[w * 16 + a * 4 + q] = outf[q];
-          d.pl_uap[w * 16 + a * 4 + q] = outA[q];
+          for (int q = 0; q < 4; ++q)
+            if (q >= nu) { us[q] = 0x7fffffff; uf[q] = -1; Au[q] = 0.0; }
+          const int p = 1 - sa;  // the piece that uses the phantom of a
+          const int code = (e << 3) | (p << 2) | a, cf = c * 16 + p * 8 + 2 * a;
+          const double Anew = piece_fraction(sides, p) * g.A;
+          // insert the new user in increasing element id (as the split writes
+          // did): before the first user of a larger element; a full list of
+          // four keeps its first four entries
+          int pos = 4;
+#pragma unroll
+          for (int q = 3; q >= 0; --q)
+            if (q >= nu || (us[q] >> 3) > e) pos = q;
+          int out[4], outf[4];
+          double outA[4];
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            if (t < pos) {
+              out[t] = us[t]; outf[t] = uf[t]; outA[t] = Au[t];
+            } else if (t == pos) {
+              out[t] = code; outf[t] = cf; outA[t] = Anew;
+            } else if (t - 1 < nu) {
+              out[t] = us[t - 1]; outf[t] = uf[t - 1]; outA[t] = Au[t - 1];
+            } else {
+              out[t] = -1; outf[t] = -1; outA[t] = 0.0;
+            }
+          }
+          // the phantom's mass: rho A_p / 4 of each user piece, in list order
+          double acc = 0.0;
+          const int nun = nu < 4 ? nu + 1 : 4;
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (q < nun) acc = acc + d.mat.rho * outA[q] * 0.25;
+          const int o = w * 4 + a;
+          d.pl_mreal[o] = mreal;
+          d.pl_mireal[o] = inverse_mass(mreal);
+          d.pl_mph[o] = acc;
+          d.pl_miph[o] = inverse_mass(acc);
+          d.pl_mold[o] = mold;
+          d.pl_dm[o] = d.mat.rho * Anew * 0.25;
+          d.pl_nu[o] = nu;  // users before the insertion (4: list full)
+          reinterpret_cast<int4 *>(d.pl_users)[o] = make_int4(out[0], out[1], out[2], out[3]);
+          reinterpret_cast<int4 *>(d.pl_upf)[o] = make_int4(outf[0], outf[1], outf[2], outf[3]);
+          reinterpret_cast<double2 *>(d.pl_uap)[2 * o] = make_double2(outA[0], outA[1]);
+          reinterpret_cast<double2 *>(d.pl_uap)[2 * o + 1] = make_double2(outA[2], outA[3]);
         }
       }
-      __syncthreads();
-      if (tid == 0 && !s_stop) {
-        s_nph += tot_new;
-        s_nck += nb;
-        s_nS += tot_app;
-        s_done = base + nb;
-      }
-      __syncthreads();
+      nph += tot_new;
+      nck += nb;
+      nS += tot_app;
+      dead += tot >> 20;
+      done = base + nb;
+      if (done < nwin) __syncthreads();  // the sums are read before they are written again
     }
   }
-  __syncthreads();
   if (tid == 0) {
-    cnt->pend_nwin = s_done;
-    cnt->pend_nph = s_nph;
-    cnt->pend_nck = s_nck;
-    cnt->pend_nS = s_nS;
-    cnt->pend_dead = s_dead;
-    cnt->pend_step = cnt->step;
-    cnt->n_prop_last = cnt->n_prop;
+    cnt->pend_nwin = done;
+    cnt->pend_nph = nph;
+    cnt->pend_nck = nck;
+    cnt->pend_nS = nS;
+    cnt->pend_dead = dead;
+    cnt->pend_step = step;
+    cnt->n_prop_last = n_all;
     cnt->n_prop = 0;
   }
 }
@@ -675,16 +651,22 @@ __device__ __forceinline__ void apply_tables(const DevState &d, VBlk vb, int mod
   const int nwarps = (vb.gx * blockDim.x) >> 5;
   for (int wb = warp * 4; wb < nw; wb += nwarps * 4) {
     const int w = wb + grp;
-    const bool act = w < nw;
-    const int a = lane & 3;
-    if (act && lane < 4) {
+    if (w >= nw) continue;
+    // the plan's fields are all read before the first write (the compiler
+    // keeps loads behind stores it cannot tell apart: one wait each)
+    const int a = lane & 3, o = w * 4 + a;
+    const int e = d.pl_e[w], info = d.pl_info[w], c = d.pl_c[w];
+    if (lane < 4) {
       // local node a: its phantom (new or shared), node lists, user list
-      const int e = d.pl_e[w], info = d.pl_info[w], c = d.pl_c[w];
+      const int reuse = d.pl_reuse[o], P = apply_phantom(d, w, a), nu = d.pl_nu[o];
+      const int4 us = reinterpret_cast<const int4 *>(d.pl_users)[o];
+      const int4 uf = reinterpret_cast<const int4 *>(d.pl_upf)[o];
+      const double2 A01 = reinterpret_cast<const double2 *>(d.pl_uap)[2 * o];
+      const double2 A23 = reinterpret_cast<const double2 *>(d.pl_uap)[2 * o + 1];
       const int sd = (info >> (4 + a)) & 1;
       const int N = elem_node(g, e, a);
-      const int P = apply_phantom(d, w, a);
       const int t = P - g.nn;
-      if (d.pl_reuse[w * 4 + a] < 0) {
+      if (reuse < 0) {
         d.ph_owner[t] = N;
         d.ph_creator[t] = e * 4 + a;
         d.Wn[P] = 0.0;
@@ -692,55 +674,41 @@ __device__ __forceinline__ void apply_tables(const DevState &d, VBlk vb, int mod
       }
       d.ck_node[c * 8 + sd * 4 + a] = N;
       d.ck_node[c * 8 + (1 - sd) * 4 + a] = P;
-      const int nu = d.pl_nu[w * 4 + a];
       if (nu >= 4) {
         atomicOr(&cnt->status, STAT_CAPACITY);
       } else {
-        reinterpret_cast<int4 *>(d.ph_users)[t] = reinterpret_cast<const int4 *>(d.pl_users)[w * 4 + a];
-        reinterpret_cast<int4 *>(d.ph_upf)[t] = reinterpret_cast<const int4 *>(d.pl_upf)[w * 4 + a];
-        const double2 *ua = reinterpret_cast<const double2 *>(d.pl_uap + w * 16 + a * 4);
-        reinterpret_cast<double2 *>(d.ph_uap)[2 * t] = ua[0];
-        reinterpret_cast<double2 *>(d.ph_uap)[2 * t + 1] = ua[1];
+        reinterpret_cast<int4 *>(d.ph_users)[t] = us;
+        reinterpret_cast<int4 *>(d.ph_upf)[t] = uf;
+        reinterpret_cast<double2 *>(d.ph_uap)[2 * t] = A01;
+        reinterpret_cast<double2 *>(d.ph_uap)[2 * t + 1] = A23;
         d.ph_nuser[t] = nu + 1;
       }
-    } else if (act) {
+    } else {
       // lanes 4-7: surface list at local edge k = lane - 4; lane 4 also
       // writes the split record
-      const int e = d.pl_e[w], info = d.pl_info[w];
       const int k = lane - 4;
+      const int app = (info >> 8) & 15, app0 = d.pl_app0[w], pos = d.pl_tomb[o];
       const int ed = elem_edge(g, e, k);
-      const int app = (info >> 8) & 15;
+      const double2 al = reinterpret_cast<const double2 *>(d.pl_alpha)[w];
+      const float gc = lane == 4 ? d.gc[e] : 0.f;
       if ((app >> k) & 1) {
-        const int dst = d.pl_app0[w] + __popc(app & ((1 << k) - 1));
+        const int dst = app0 + __popc(app & ((1 << k) - 1));
         const int f = elem_neighbor(g, e, k);
         d.S[dst] = ed;
         d.S_info[dst] = f * 4 + ((k + 2) & 3);
         d.S_G[dst] = 0.0;
         d.spos[ed] = dst;
-      } else {
-        const int pos = d.pl_tomb[w * 4 + k];
-        if (pos >= 0) {
-          d.S[pos] = -1;
-          d.spos[ed] = -1;
-        }
+      } else if (pos >= 0) {
+        d.S[pos] = -1;
+        d.spos[ed] = -1;
       }
       if (lane == 4) {
-        const int c = d.pl_c[w];
-        const int ka = info & 3, kb = (info >> 2) & 3;
         d.ck_elem[c] = e;
         d.ck_info[c] = info & 0xff;
-        d.ck_Ap[c * 2] = d.pl_alpha[w * 2] * g.A;
-        d.ck_Ap[c * 2 + 1] = d.pl_alpha[w * 2 + 1] * g.A;
+        reinterpret_cast<double2 *>(d.ck_Ap)[c] = make_double2(al.x * g.A, al.y * g.A);
         d.ck_step[c] = mode == TRACK_PRECRACK ? -1 : step;
-        if (mode == TRACK_PRECRACK) {
-          d.ck_ud[c] = 0.0;
-        } else {
-          const double xa = (xi_g(ka) + 1.0) * (0.5 * g.hx), ya = (eta_g(ka) + 1.0) * (0.5 * g.hy);
-          const double xb = (xi_g(kb) + 1.0) * (0.5 * g.hx), yb = (eta_g(kb) + 1.0) * (0.5 * g.hy);
-          const double sx = xb - xa, sy = yb - ya;
-          const double L = sqrt(sx * sx + sy * sy);
-          d.ck_ud[c] = (double)d.gc[e] * L;
-        }
+        // U_d = G_c times the segment's length
+        d.ck_ud[c] = mode == TRACK_PRECRACK ? 0.0 : (double)gc * g.seg[info & 3][(info >> 2) & 3];
         d.crack_of[e] = c;
       }
     }
@@ -862,7 +830,6 @@ __device__ __forceinline__ void ring_status(const DevState &d, Counters *ring) {
 // until the node update has completed and its writes are visible.
 __global__ void __launch_bounds__(256) k_apply(DevState d, int cur_next, int mode, Counters *ring) {
   const VBlk vb = hw_vblk();
-  apply_tables(d, vb, mode);
   // with at most four winners per warp each thread has at most one node
   // write (or the element's): its plan is read before the wait, so that
   // only the node update's own outputs are read after it
@@ -876,6 +843,7 @@ __global__ void __launch_bounds__(256) k_apply(DevState d, int cur_next, int mod
     if (lane < 4) q = split_node(d, w, lane);
     else if (lane == 4) es = d.pl_e[w];
   }
+  apply_tables(d, vb, mode);
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;");
   if (!one_pass) {
