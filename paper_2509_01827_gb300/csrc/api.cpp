@@ -1641,7 +1641,7 @@ cem_status batch_upload(cem_handle *b) {
     for (int q = 0; q < gph; ++q) wph.push_back(make_int4(s, q, tiles + gp, gph));
     // the evaluation has no energy partials: a few virtual blocks per member
     // walk its list (its length, not its capacity, sets the work)
-    const int ge = mixed ? std::min(grid_eval(d), 8) : std::min(grid_eval64(d), 32);
+    const int ge = std::min(mixed ? grid_eval(d) : grid_eval64(d), 32);
     for (int q = 0; q < ge; ++q) we.push_back(make_int4(s, q, 0, ge));
     // FP32 phantom blocks write one energy partial per warp
     nparts[s] = tiles + gp + (p->precision == CEM_FP32_MIXED ? kPhWarps : 1) * gph;
