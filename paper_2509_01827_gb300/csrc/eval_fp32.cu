@@ -178,7 +178,11 @@ __device__ __forceinline__ void eval32(const DevState &d, VBlk vb, int cur) {
   }
 }
 
-__global__ void __launch_bounds__(kEvalTB) k_eval32(DevState d, int cur) { eval32(d, hw_vblk(), cur); }
+__global__ void __launch_bounds__(kEvalTB) k_eval32(DevState d, int cur) {
+  wait_for_predecessors();
+  release_dependents();
+  eval32(d, hw_vblk(), cur);
+}
 
 __global__ void __launch_bounds__(kEvalTB) k_eval32_batch(BatchDev b) {
   __shared__ DevState sd;
@@ -214,8 +218,7 @@ cudaError_t eval32_carveouts() {
 cudaError_t launch_eval32(const DevState &d, int cur, cudaStream_t st) {
   cudaError_t e = eval32_carveouts();
   if (e != cudaSuccess) return e;
-  k_eval32<<<grid_eval(d), kEvalTB, 0, st>>>(d, cur);
-  return cudaGetLastError();
+  return launch_dependent(k_eval32, grid_eval(d), kEvalTB, 0, st, d, cur);
 }
 
 cudaError_t launch_eval32_batch(const BatchDev &b, cudaStream_t st) {

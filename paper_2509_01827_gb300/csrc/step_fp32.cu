@@ -262,9 +262,7 @@ __device__ __forceinline__ void pieces32(const DevState &d, VBlk vb, int cur, in
 }
 
 __global__ void k_pieces32(DevState d, int cur, int energy, int part_off) {
-  // a programmatic dependent of the previous step's split writes (see k_march32)
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;");
+  release_dependents();  // the node update waits where it first reads a piece force
   pieces32(d, hw_vblk(), cur, energy, part_off);
 }
 
@@ -646,7 +644,7 @@ __device__ __forceinline__ void march32_tile(const DevState &d, int tile_x, int 
         // the piece forces come from the kernel before this one (when launched as
         // its programmatic dependent): wait until it has completed and its writes
         // are visible.  Rows before the first split element did not need it.
-        asm volatile("griddepcontrol.wait;" ::: "memory");
+        wait_for_predecessors();
         pieces_in = true;
       }
 #pragma unroll
@@ -741,7 +739,7 @@ __device__ __forceinline__ void march32_tile(const DevState &d, int tile_x, int 
   }
   cp_async_wait<0>();  // no copy into the ring outlives the tile
   // this kernel completes only after the one before it, whichever tiles met a piece
-  if (!CLEAN && !pieces_in) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (!CLEAN && !pieces_in) wait_for_predecessors();
   if (!CLEAN) {
     // nodes with loads or prescribed velocities, listed in the ring's memory
     // and shared out over the warp's lanes: a lane that worked through its own
@@ -869,7 +867,7 @@ __global__ void __launch_bounds__(32 * kMarchWarps, 4) k_march32(DevState d, int
   // kernels that completed before the piece forces started.  The kernels
   // that follow may be placed once every CTA of this kernel has started
   // (they wait for it themselves).
-  asm volatile("griddepcontrol.launch_dependents;");
+  release_dependents();
   __shared__ MarchRing rings[kMarchWarps];
   march32_group<ENERGY>(d, blockIdx.x, ty, cur, first, rings);
 }
@@ -1053,7 +1051,7 @@ int energy_parts_fp32(const DevState &d) {
 
 // piece-force blocks: one thread per split element in FP32, per piece in FP64
 int grid_pieces(const DevState &d) {
-  return grid_for(d.precision == 1 ? d.ck_cap : 2 * d.ck_cap, 256, 1216);
+  return grid_for(d.precision == 1 ? d.ck_cap : 2 * d.ck_cap, 256, 304);
 }
 // side-branch grids: two phantom blocks and one evaluation block per SM, so that
 // they start together with the node update and share the SMs with it
@@ -1077,17 +1075,8 @@ cudaError_t launch_step_fp32(const DevState &d, int cur, bool first, bool energy
   cudaStream_t st = ss.main;
   auto node_update = [&]() {
     // a programmatic dependent of the piece forces before it on the main stream
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(groups);
-    cfg.blockDim = dim3(32 * kMarchWarps);
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (energy) cudaLaunchKernelEx(&cfg, k_march32<true>, d, cur, f, ty);
-    else cudaLaunchKernelEx(&cfg, k_march32<false>, d, cur, f, ty);
+    if (energy) launch_dependent(k_march32<true>, groups, 32 * kMarchWarps, 0, st, d, cur, f, ty);
+    else launch_dependent(k_march32<false>, groups, 32 * kMarchWarps, 0, st, d, cur, f, ty);
   };
   if (marks) {
     // the step's kernels one after another

@@ -147,6 +147,8 @@ __device__ __forceinline__ void pieces64(const DevState &d, VBlk vb, int cur, in
 }
 
 __global__ void k_pieces64(DevState d, int cur, int energy, int part_off) {
+  wait_for_predecessors();
+  release_dependents();  // the node update waits where it first reads a piece force
   pieces64(d, hw_vblk(), cur, energy, part_off);
 }
 
@@ -359,6 +361,9 @@ __device__ __forceinline__ void main64_tile(const DevState &d, VBlk vb, int cur,
   }
   __syncthreads();
 
+  // only the node sums read what the kernel before this one (the piece forces)
+  // writes: the strains and stresses above run beside it
+  wait_for_predecessors();
   double ke = 0.0, se = 0.0;
   const double qA = g.A * 0.25;
   for (int q = tid; q < T.tx * T.ty; q += NT) {
@@ -420,6 +425,10 @@ __device__ __forceinline__ void main64_tile(const DevState &d, VBlk vb, int cur,
 }
 
 __global__ void __launch_bounds__(NT) k_main64(DevState d, int cur, int first, int energy) {
+  // a programmatic dependent of the piece forces (7 us, most of it latency), which
+  // start after the previous step's split writes have completed: it runs beside
+  // them and waits where main64_tile first needs them
+  release_dependents();
   extern __shared__ double sm64[];
   main64_tile(d, hw_vblk(), cur, first, energy, sm64);
 }
@@ -492,7 +501,11 @@ __device__ __forceinline__ void eval64(const DevState &d, VBlk vb, int cur) {
   }
 }
 
-__global__ void __launch_bounds__(kEvalTB) k_eval64(DevState d, int cur) { eval64(d, hw_vblk(), cur); }
+__global__ void __launch_bounds__(kEvalTB) k_eval64(DevState d, int cur) {
+  wait_for_predecessors();
+  release_dependents();
+  eval64(d, hw_vblk(), cur);
+}
 
 // ---------------------------------------------------------------- batched
 // One launch per kernel kind for every member of a batch (persistent grids
@@ -514,6 +527,7 @@ __global__ void __launch_bounds__(NT) k_main64_batch(BatchDev b, int first, int 
 }
 
 __global__ void k_pieces64_batch(BatchDev b, int energy) {
+  release_dependents();
   __shared__ DevState sd;
   int held = -1, w0, w1;
   const int n = *b.bstep;
@@ -690,13 +704,13 @@ cudaError_t launch_step_fp64(const DevState &d, int cur, bool first, bool energy
   }
   cudaEventRecord(ss.fork, st);
   cudaStreamWaitEvent(ss.aux2, ss.fork, 0);
-  k_eval64<<<ge, kEvalTB, 0, ss.aux2>>>(d, cur);
+  launch_dependent(k_eval64, ge, kEvalTB, 0, ss.aux2, d, cur);
   launch_select(d, TRACK_STEP, ss.aux2);
-  k_pieces64<<<gp, kPieceTB, 0, st>>>(d, cur, energy ? 1 : 0, tiles);
+  launch_dependent(k_pieces64, gp, kPieceTB, 0, st, d, cur, energy ? 1 : 0, tiles);
   cudaEventRecord(ss.fork, st);
   cudaStreamWaitEvent(ss.aux1, ss.fork, 0);
   k_phantom64<<<gph, 256, 0, ss.aux1>>>(d, cur, first ? 1 : 0, energy ? 1 : 0, tiles + gp);
-  k_main64<<<grid, NT, smem, st>>>(d, cur, first ? 1 : 0, energy ? 1 : 0);
+  launch_dependent(k_main64, grid, NT, smem, st, d, cur, first ? 1 : 0, energy ? 1 : 0);
   cudaEventRecord(ss.join1, ss.aux1);
   cudaEventRecord(ss.join2, ss.aux2);
   cudaStreamWaitEvent(st, ss.join1, 0);
@@ -723,7 +737,7 @@ cudaError_t launch_step_fp64_batch(const BatchDev &b, bool first, bool energy, i
   cudaEventRecord(ss.fork, st);
   cudaStreamWaitEvent(ss.aux1, ss.fork, 0);
   k_phantom64_batch<<<gph, 256, 0, ss.aux1>>>(b, first ? 1 : 0, energy ? 1 : 0);
-  k_main64_batch<<<gm, NT, Tile64(32, 12).bytes(energy), st>>>(b, first ? 1 : 0, energy ? 1 : 0);
+  launch_dependent(k_main64_batch, gm, NT, Tile64(32, 12).bytes(energy), st, b, first ? 1 : 0, energy ? 1 : 0);
   cudaEventRecord(ss.join1, ss.aux1);
   cudaEventRecord(ss.join2, ss.aux2);
   cudaStreamWaitEvent(st, ss.join1, 0);

@@ -603,6 +603,7 @@ __device__ __forceinline__ void select_plan(const DevState &d, int mode,
 
 __global__ void __launch_bounds__(TB, 4) k_select(DevState d, int mode) {
   extern __shared__ unsigned long long smem[];
+  wait_for_predecessors();
   select_plan(d, mode, smem);
 }
 
@@ -844,8 +845,8 @@ __global__ void __launch_bounds__(256) k_apply(DevState d, int cur_next, int mod
     else if (lane == 4) es = d.pl_e[w];
   }
   apply_tables(d, vb, mode);
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;");
+  wait_for_predecessors();
+  release_dependents();
   if (!one_pass) {
     apply_nodes(d, vb, cur_next, mode);
   } else {
@@ -977,8 +978,7 @@ cudaError_t launch_select(const DevState &d, int mode, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  k_select<<<1, TB, sm, st>>>(d, mode);
-  return cudaGetLastError();
+  return launch_dependent(k_select, 1, TB, sm, st, d, mode);
 }
 
 cudaError_t launch_apply(const DevState &d, int cur_next, int mode, cudaStream_t st,
