@@ -352,7 +352,7 @@ cem_status cem_batch_create(cem_handle *const *members, int n, const long *step_
  * fixed at 32 x 8), grid_main the persistent grid of the node update
  * (1 .. 64 x SMs).  Nodal results do not depend on it; in FP32 the energy
  * records group their partial sums by tile (last-bit differences).
- * Default: chosen from the members' sizes (FP64 grid: 3 x SMs). */
+ * Default: chosen from the members' sizes (FP64 grid: 16 x SMs). */
 cem_status cem_batch_set_config(cem_handle *batch, int tile_rows, int grid_main);
 
 /* Autotuner: times steps_per_candidate real steps (after one untimed step)
