@@ -501,7 +501,13 @@ cudaError_t launch_conv_tc(const ConvArgs &a, cudaStream_t st) {
 //          instead of 2);
 //   flat   narrow images (W <= 30) as one long row with a zero after each
 //          image row, 128 consecutive pixels to a tile, one TMA box per image
-//          row and plane: 25 x 10 images fill 87% of the rows instead of 71%.
+//          row and plane: 25 x 10 images fill 87% of the rows instead of 71%;
+//   box    for more channels than a stage can hold beside a weight ring: tiles
+//          bw x bh x bb pixels (wide, tall, images; at most 128, whatever covers the
+//          images best), and a stage is the 64 channels of one tap, fetched anew for
+//          each tap by one shifted TMA box: nine times the input's bytes, but any
+//          number of channels, two tiles to a weight block and no slots beside the
+//          tile (25 x 10 images fill 98% of the rows).
 // The weights stay in shared memory for the whole (persistent) CTA when they
 // fit, else they stream by TMA through a ring, each block serving MT tiles.
 //
@@ -520,10 +526,13 @@ cudaError_t launch_conv_tc(const ConvArgs &a, cudaStream_t st) {
 //   64 -> 64, 80 x 200    219 -> 66 us
 //   128 -> 384, 40 x 100  450 -> 134 us, 1690 TFLOP/s (0.89 of cuBLAS)
 //   256 -> 256, 20 x 50   106 -> 52 us, 1460 TFLOP/s
-// One image, 256 -> 256, 20 x 50: 47 -> 12 us.
+//   768 -> 256, 20 x 50   316 -> 151 us (box)
+//   512 -> 512, 10 x 25   94 -> 54 us, 1390 TFLOP/s (box; 113 with whole stages)
+//   512 -> 256, 10 x 25   78 -> 33 us (box)
+// One image, 256 -> 256, 20 x 50: 47 -> 12 us; 768 -> 256: 105 -> 37 us (box).
 constexpr int HB_THREADS = 352, HB_MAXW = 48, HB_MAXA = 8;
 
-enum : int { TILE_WHOLE = 0, TILE_TALL = 1, TILE_FLAT = 2 };
+enum : int { TILE_WHOLE = 0, TILE_TALL = 1, TILE_FLAT = 2, TILE_BOX = 3 };
 
 struct HaloArgs {
   const float *bias;
@@ -531,7 +540,10 @@ struct HaloArgs {
   const bf16_t *mask;
   int B, H, W, N, relu, ldy, yoff, ldm;
   int mode;             // TILE_*
-  int planes;           // of a stage
+  int planes;           // of a stage (box: of the input)
+  int cps;              // stages of a tile (box: one for each 64 of k)
+  int bw, bh, bb;       // box: pixels of a tile
+  uint32_t inv_bw, inv_bp;  // ceil(2^32 / bw), / (bw bh)
   int ky_st, ps, sbo;   // strides of a tap row, a plane and 8 tile rows (bytes)
   int a_bytes, a_tx;    // a stage's size; the bytes its copies bring in
   int nrows;            // flat: image rows a stage holds
@@ -661,7 +673,17 @@ __device__ __forceinline__ int div_by(int n, uint32_t inv) { return (int)__umulh
 // output pixel of row m of a sub-tile, or -1 outside the images
 __device__ __forceinline__ int halo_pixel(const HaloArgs &a, int tile, int m) {
   int b, h, c;
-  if (a.mode == TILE_FLAT) {
+  if (a.mode == TILE_BOX) {
+    // divisors of 1 have no reciprocal
+    const int n = a.bw * a.bh, i = n == 1 ? m : div_by(m, a.inv_bp), k = m - i * n;
+    const int r = a.bw == 1 ? k : div_by(k, a.inv_bw);
+    const int ty = a.tiles_x == 1 ? tile : div_by(tile, a.inv_x);
+    const int tb = a.tiles_y == 1 ? ty : div_by(ty, a.inv_y);
+    c = (tile - ty * a.tiles_x) * a.bw + k - r * a.bw;
+    h = (ty - tb * a.tiles_y) * a.bh + r;
+    b = tb * a.bb + i;
+    if (i >= a.bb) return -1;
+  } else if (a.mode == TILE_FLAT) {
     const int q = a.W + 1 + tile * 128 + m, T = div_by(q, a.inv_w);
     c = q - T * (a.W + 1);
     b = div_by(T, a.inv_h);
@@ -688,10 +710,10 @@ __device__ __forceinline__ int flat_first(const HaloArgs &a, int tile, int &row)
 }
 
 // RB: bytes of a slot's row in a plane.  PL > 0: the stage's planes, known at
-// compile time with the tiling (TALL or WHOLE), and a tile's steps are
+// compile time with the tiling (MODE: WHOLE or TALL), and a tile's steps are
 // straight-line code with constant offsets; the issue of a step then costs about
 // 30 clocks, less than its MMA, against 65 with the offsets walked (PL = 0).
-template <int RB, int MT, bool RES, int PL, bool TALL>
+template <int RB, int MT, bool RES, int PL, int MODE>
 __global__ void __launch_bounds__(HB_THREADS, 1)
     k_conv3x3_halo(const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap xmap,
                    const HaloArgs a) {
@@ -746,41 +768,56 @@ __global__ void __launch_bounds__(HB_THREADS, 1)
   if (warp == 10) {
     // ---- input tiles; the boxes of a tile are issued side by side, one per lane
     int s = 0, ph = 1, it = 0;
-    for (int g = g0; g < groups; g += step, ++it) {
-      if (!warp_wait(&C.a_empty[s], ph, &C.fail)) break;
-      if (lane == 0) mbar_expect(&C.a_full[s], (uint32_t)(MT * a.a_tx));
-      __syncwarp();
-      for (int m = 0; m < MT; ++m) {
-        const int tile = g * MT + m;  // one past the last: rows outside the images, all zeros
-        const uint32_t dst = smem_u32(sa) + (uint32_t)((s * MT + m) * a.a_bytes);
-        if (a.mode == TILE_FLAT) {
-          int row;
-          flat_first(a, tile, row);
-          for (int q = lane; q < a.nrows * a.planes; q += 32) {
-            const int r = q / a.planes, p = q - r * a.planes;
-            const int T = row + r, b = T < 0 ? 0 : div_by(T, a.inv_h);
-            const int h = T < 0 ? -1 : T - b * (a.H + 1) - 1;
-            tma_load5(dst + p * a.ps + r * (a.W + 1) * RB, &xmap, 0, 0, h, b, p, &C.a_full[s]);
-          }
-        } else {
-          const int ty = a.tiles_x == 1 ? tile : div_by(tile, a.inv_x);
-          const int c = (tile - ty * a.tiles_x) * 8 - 1;
-          if (a.mode == TILE_WHOLE) {
-            const int b = a.tiles_y == 1 ? ty : div_by(ty, a.inv_y);
+    bool ok = true;
+    for (int g = g0; g < groups && ok; g += step) {
+      int tap = 0, pl = 0;  // of the stage (box)
+      for (int cp = 0; cp < a.cps; ++cp, ++it) {
+        ok = warp_wait(&C.a_empty[s], ph, &C.fail);
+        if (!ok) break;
+        if (lane == 0) mbar_expect(&C.a_full[s], (uint32_t)(MT * a.a_tx));
+        __syncwarp();
+        for (int m = 0; m < MT; ++m) {
+          const int tile = g * MT + m;  // one past the last: rows outside the images, all zeros
+          const uint32_t dst = smem_u32(sa) + (uint32_t)((s * MT + m) * a.a_bytes);
+          if (MODE == TILE_BOX) {
+            const int ty = a.tiles_x == 1 ? tile : div_by(tile, a.inv_x);
+            const int tb = a.tiles_y == 1 ? ty : div_by(ty, a.inv_y);
             if (lane == 0)
-              tma_load5(dst, &xmap, 0, c, (ty - b * a.tiles_y) * 16 - 1, b, 0, &C.a_full[s]);
-          } else if (lane < 18) {
-            const int T = ty * 16 + lane, b = div_by(T, a.inv_h);
-            tma_load5(dst + lane * a.ky_st, &xmap, 0, c, T - b * (a.H + 1) - 1, b, 0, &C.a_full[s]);
+              tma_load5(dst, &xmap, 0, (tile - ty * a.tiles_x) * a.bw + tap % 3 - 1,
+                        (ty - tb * a.tiles_y) * a.bh + tap / 3 - 1, tb * a.bb, pl, &C.a_full[s]);
+          } else if (a.mode == TILE_FLAT) {
+            int row;
+            flat_first(a, tile, row);
+            for (int q = lane; q < a.nrows * a.planes; q += 32) {
+              const int r = q / a.planes, p = q - r * a.planes;
+              const int T = row + r, b = T < 0 ? 0 : div_by(T, a.inv_h);
+              const int h = T < 0 ? -1 : T - b * (a.H + 1) - 1;
+              tma_load5(dst + p * a.ps + r * (a.W + 1) * RB, &xmap, 0, 0, h, b, p, &C.a_full[s]);
+            }
+          } else {
+            const int ty = a.tiles_x == 1 ? tile : div_by(tile, a.inv_x);
+            const int c = (tile - ty * a.tiles_x) * 8 - 1;
+            if (a.mode == TILE_WHOLE) {
+              const int b = a.tiles_y == 1 ? ty : div_by(ty, a.inv_y);
+              if (lane == 0)
+                tma_load5(dst, &xmap, 0, c, (ty - b * a.tiles_y) * 16 - 1, b, 0, &C.a_full[s]);
+            } else if (lane < 18) {
+              const int T = ty * 16 + lane, b = div_by(T, a.inv_h);
+              tma_load5(dst + lane * a.ky_st, &xmap, 0, c, T - b * (a.H + 1) - 1, b, 0, &C.a_full[s]);
+            }
           }
         }
-      }
-      if (++s == a.na) {
-        s = 0;
-        ph ^= 1;
+        if (++pl == a.planes) {
+          pl = 0;
+          ++tap;
+        }
+        if (++s == a.na) {
+          s = 0;
+          ph ^= 1;
+        }
       }
     }
-    // no copy outlives the CTA: wait for those of the last na tiles (bounded)
+    // no copy outlives the CTA: wait for those of the last na stages (bounded)
     for (int q = max(0, it - a.na); q < it; ++q) mbar_wait(&C.a_full[q % a.na], (q / a.na) & 1);
   } else if (warp == 9) {
     // ---- weights
@@ -823,8 +860,40 @@ __global__ void __launch_bounds__(HB_THREADS, 1)
       if (RES && g0 < groups)
         for (int kb = 0; kb < a.kblocks && ok; ++kb) ok = thread_wait(&C.w_full[kb], 0, &C.fail);
       for (int g = g0; g < groups && ok; g += step) {
-        if (!thread_wait(&C.a_full[s], sph, &C.fail)) break;
         if (!thread_wait(&C.acc_empty[ab], abph, &C.fail)) break;
+        if constexpr (MODE == TILE_BOX) {
+          // a stage and a weight block for each 64 of k
+          const uint32_t d0 = tmem + (uint32_t)(ab * MT * a.nbp);
+          for (int kb = 0; kb < a.kblocks; ++kb) {
+            ok = thread_wait(&C.a_full[s], sph, &C.fail) && thread_wait(&C.w_full[ws], wph, &C.fail);
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            const uint32_t wd = wlo0 + (uint32_t)ws * wst, ad = sa0 + (uint32_t)(s * MT) * stage;
+#pragma unroll
+            for (int i = 0; i < PER; ++i)
+#pragma unroll
+              for (int m = 0; m < MT; ++m)
+                tc_mma(d0 + m * a.nbp, ad + m * stage + 2 * i, ahi, wd + 2 * i, whi, idesc, i ? 1u : (uint32_t)(kb > 0));
+            tc_commit(&C.w_empty[ws]);
+            tc_commit(&C.a_empty[s]);
+            if (++ws == a.nw) {
+              ws = 0;
+              wph ^= 1;
+            }
+            if (++s == a.na) {
+              s = 0;
+              sph ^= 1;
+            }
+          }
+          if (!ok) break;
+          tc_commit(&C.acc_full[ab]);
+          if (++ab == a.nacc) {
+            ab = 0;
+            abph ^= 1;
+          }
+          continue;
+        }
+        if (!thread_wait(&C.a_full[s], sph, &C.fail)) break;
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         uint32_t tap[MT], row[MT];
 #pragma unroll
@@ -860,7 +929,7 @@ __global__ void __launch_bounds__(HB_THREADS, 1)
             if (!RES && ((q & 3) == 3 || q == 4)) w_next();
           }
         } else if constexpr (PL > 0) {
-          constexpr int PS = (TALL ? 10 : 180) * RB / 16, KY = (TALL ? PL * 10 : 10) * RB / 16;
+          constexpr int PS = (MODE == TILE_TALL ? 10 : 180) * RB / 16, KY = (MODE == TILE_TALL ? PL * 10 : 10) * RB / 16;
           constexpr int STEPS = 9 * PL * PER;
           uint32_t wd = wlo0;
 #pragma unroll
@@ -1031,7 +1100,7 @@ constexpr size_t kSmemMax = 232448;  // 227 KB a CTA
 
 struct HaloPlan {
   HaloArgs a;
-  int rb, mt, res, grid, box_w, box_h, box_p;
+  int rb, mt, res, grid, box_w, box_h, box_b, box_p;
   size_t smem;
 };
 
@@ -1042,8 +1111,8 @@ struct HaloPlan {
 // about 45 bytes per clock from L2, a ring no more than it holds in 2000 clocks
 // (the latency under load).  Few tiles (a single image's deep levels) come out with
 // many narrow channel blocks, so that the K loop runs on more SMs.  False when
-// no plan fits (an input stage of more than about 560 channels, channels that
-// are neither 8 nor a multiple of 16): k_conv3x3_tc takes those.
+// no plan fits (channels that are neither 8 nor a multiple of 16, or more than a
+// stage holds and no multiple of 64): k_conv3x3_tc takes those.
 bool halo_plan(const ConvArgs &v, HaloPlan &best) {
   if ((v.Cin & 15) && v.Cin != 8) return false;
   const int rb = !(v.Cin & 63) ? 128 : !(v.Cin & 31) ? 64 : !(v.Cin & 15) ? 32 : 16;
@@ -1054,15 +1123,36 @@ bool halo_plan(const ConvArgs &v, HaloPlan &best) {
   const size_t fixed = 1024 + 128 + sizeof(HaloCtl);
   double best_c = 0.0;
   bool found = false;
-  for (int mode : {TILE_WHOLE, TILE_TALL, TILE_FLAT}) {
+  for (int mode : {TILE_WHOLE, TILE_TALL, TILE_FLAT, TILE_BOX}) {
     HaloArgs a{};
     a.mode = mode;
     a.planes = v.Cin * 2 / rb;
     a.kblocks = kblocks;
+    a.cps = 1;
     a.tiles_x = (int)up(v.W, 8);
     a.tiles_y = (int)up(v.H, 16);
     long tiles;
-    if (mode == TILE_FLAT) {
+    if (mode == TILE_BOX) {
+      if (rb != 128) continue;
+      // the widths' best cover of the images by at most 128 pixels
+      tiles = 0;
+      for (int bw = 1; bw <= std::min(v.W, 128); ++bw) {
+        const int bh = std::min(v.H, 128 / bw), bb = bw == v.W && bh == v.H ? std::min(v.B, 128 / (bw * bh)) : 1;
+        const long n = up(v.W, bw) * up(v.H, bh) * up(v.B, bb);
+        if (tiles && n >= tiles) continue;
+        tiles = n;
+        a.bw = bw;
+        a.bh = bh;
+        a.bb = bb;
+      }
+      a.tiles_x = (int)up(v.W, a.bw);
+      a.tiles_y = (int)up(v.H, a.bh);
+      a.inv_bw = inv(a.bw);
+      a.inv_bp = inv(a.bw * a.bh);
+      a.cps = kblocks;
+      a.sbo = 8 * rb;
+      a.a_tx = a.bw * a.bh * a.bb * rb;
+    } else if (mode == TILE_FLAT) {
       if (v.W > 30 || rb != 128) continue;
       a.tiles_x = 1;
       tiles = up(rows * (v.W + 1), 128);
@@ -1078,7 +1168,7 @@ bool halo_plan(const ConvArgs &v, HaloPlan &best) {
       a.ky_st = a.sbo = mode == TILE_WHOLE ? 10 * rb : a.planes * a.ps;
       a.a_tx = 180 * a.planes * rb;
     }
-    a.a_bytes = ((rb == 16 ? 2 * a.a_tx : a.a_tx) + 1023) & ~1023;
+    a.a_bytes = mode == TILE_BOX ? 128 * rb : ((rb == 16 ? 2 * a.a_tx : a.a_tx) + 1023) & ~1023;
     a.tiles = (int)tiles;
     // limits of the kernel's divisions by reciprocals
     if ((rows + 40) * (v.W + 1) + 256 >= (1L << 32) / (v.W + 1) || (rows + 40) * (v.H + 1) >= (1L << 32) ||
@@ -1097,7 +1187,7 @@ bool halo_plan(const ConvArgs &v, HaloPlan &best) {
         if (mt * nbp > 512) continue;
         const int nacc = 2 * mt * nbp <= 512 ? 2 : 1;
         const size_t ast = (size_t)mt * a.a_bytes;
-        for (int res = 1; res >= 0; --res) {
+        for (int res = mode == TILE_BOX ? 0 : 1; res >= 0; --res) {
           if (res && kblocks > HB_MAXW) continue;
           int na = HB_MAXA;
           while (na && fixed + (res ? kblocks : 2) * wst + na * ast > kSmemMax) --na;
@@ -1106,20 +1196,30 @@ bool halo_plan(const ConvArgs &v, HaloPlan &best) {
           int per = kSms / nblk;
           if (per > groups) per = groups;
           const double mma = ((v.K + 15) / 16) * mt * fmax(0.53 * nb, 58.0 + 0.2 * nb) + 350.0;
-          const double la = mt * (double)a.a_tx / 45.0;
+          // box: a box's start besides, for each stage and its weights
+          const double la = a.cps * mt * (double)a.a_tx / 45.0 + (mode == TILE_BOX ? a.cps * (mt + 1) * 75.0 : 0.0);
           const double epi = mt * (nbp / 32) * 300.0;
+          if (mode == TILE_BOX) {
+            // as many stages as weight blocks
+            na = 0;
+            while (na < HB_MAXA && fixed + (na + 1) * (wst + ast) <= kSmemMax) ++na;
+            if (na < 2) continue;
+          }
           // with a ring: one or two input stages, the rest of the memory for the ring
-          for (int ns = res ? na : na < 2 ? na : 2; ns; ns = res ? 0 : ns - 1) {
+          for (int ns = res || mode == TILE_BOX ? na : na < 2 ? na : 2; ns; ns = res || mode == TILE_BOX ? 0 : ns - 1) {
             int nw = kblocks;
-            if (!res) {
+            if (mode == TILE_BOX) {
+              nw = ns;
+            } else if (!res) {
               nw = 2;
               while (nw < 12 && nw < kblocks && fixed + (nw + 1) * wst + ns * ast <= kSmemMax) ++nw;
             }
-            const double lw = kblocks * (double)wst / (res ? 45.0 : fmin(45.0, nw * (double)wst / 2000.0));
+            const double fl = nw * (double)wst + (mode == TILE_BOX ? ns * (double)ast : 0.0);  // bytes in flight
+            const double lw = kblocks * (double)wst / (res ? 45.0 : fmin(45.0, fl / 2000.0));
             double t = fmax(mma, fmax(la + (res ? 0.0 : lw), epi));
             if (ns == 1) t += la + 1000.0;
             if (nacc == 1) t += epi;
-            const double c = ((groups + per - 1) / per) * t + la + 2500.0 + (res ? lw : 0.0);
+            const double c = ((groups + per - 1) / per) * t + la / a.cps + 2500.0 + (res ? lw : 0.0);
             if (found && c >= best_c) continue;
             found = true;
             best_c = c;
@@ -1145,15 +1245,16 @@ bool halo_plan(const ConvArgs &v, HaloPlan &best) {
     }
   }
   // k_conv3x3_tc keeps calls it does faster: 256-channel blocks of deep layers
-  // (1700 clocks per tile and 64 of k), where too little memory is left
-  // beside the input stage for a weight ring (512 -> 512 channels, 64 images
-  // of 10 x 25: 94 us there, 113 here)
+  // (1700 clocks per tile and 64 of k) whose channels are no multiple of 64, where
+  // too little memory is left beside the input stage for a weight ring
   const double old_c = (double)up((long)v.B * v.H * v.W, 128) * up(v.N, 256) / kSms * kblocks * 1700.0;
   if (!found || (v.N > 128 && v.B * (long)v.H * v.W >= 128L * kSms / 2 && best_c > old_c)) return false;
   best.rb = rb;
-  best.box_w = best.a.mode == TILE_FLAT ? v.W + 1 : 10;
-  best.box_h = best.a.mode == TILE_WHOLE ? 18 : 1;
-  best.box_p = best.a.mode == TILE_FLAT ? 1 : best.a.planes;
+  const int m = best.a.mode;
+  best.box_w = m == TILE_BOX ? best.a.bw : m == TILE_FLAT ? v.W + 1 : 10;
+  best.box_h = m == TILE_BOX ? best.a.bh : m == TILE_WHOLE ? 18 : 1;
+  best.box_b = m == TILE_BOX ? best.a.bb : 1;
+  best.box_p = m == TILE_FLAT || m == TILE_BOX ? 1 : best.a.planes;
   return true;
 }
 
@@ -1183,12 +1284,13 @@ bool encode_bf16(CUtensorMap *map, int rank, const void *p, const cuuint64_t *di
 }
 // NHWC images as (channel in plane, w, h, image, plane) of planes of rb bytes
 bool encode_image(CUtensorMap *map, const void *x, int B, int H, int W, int ld, int planes, int rb,
-                  int box_w, int box_h, int box_p) {
+                  int box_w, int box_h, int box_p, int box_b = 1) {
   const cuuint64_t px = (cuuint64_t)ld * 2;
   const cuuint64_t dims[5] = {(cuuint64_t)rb / 2, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B,
                               (cuuint64_t)planes};
   const cuuint64_t st[4] = {px, px * W, px * W * H, (cuuint64_t)rb};
-  const cuuint32_t box[5] = {(cuuint32_t)rb / 2, (cuuint32_t)box_w, (cuuint32_t)box_h, 1, (cuuint32_t)box_p};
+  const cuuint32_t box[5] = {(cuuint32_t)rb / 2, (cuuint32_t)box_w, (cuuint32_t)box_h, (cuuint32_t)box_b,
+                             (cuuint32_t)box_p};
   return encode_bf16(map, 5, x, dims, st, box,
                      rb == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
                      : rb == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
@@ -1208,36 +1310,39 @@ cudaError_t allow_smem(K *kernel, std::atomic<unsigned long long> &done) {
   return e;
 }
 
-template <int RB, int MT, bool RES, int PL, bool TALL>
+template <int RB, int MT, bool RES, int PL, int MODE>
 cudaError_t launch_halo(const HaloPlan &p, const CUtensorMap &wm, const CUtensorMap &xm, cudaStream_t st) {
   static std::atomic<unsigned long long> done{0};
-  cudaError_t e = allow_smem(k_conv3x3_halo<RB, MT, RES, PL, TALL>, done);
+  cudaError_t e = allow_smem(k_conv3x3_halo<RB, MT, RES, PL, MODE>, done);
   if (e != cudaSuccess) return e;
-  k_conv3x3_halo<RB, MT, RES, PL, TALL><<<p.grid, HB_THREADS, p.smem, st>>>(wm, xm, p.a);
+  k_conv3x3_halo<RB, MT, RES, PL, MODE><<<p.grid, HB_THREADS, p.smem, st>>>(wm, xm, p.a);
   return cudaGetLastError();
 }
-template <int RB, int PL, bool TALL>
+template <int RB, int PL, int MODE>
 cudaError_t launch_halo_pl(const HaloPlan &p, const CUtensorMap &wm, const CUtensorMap &xm, cudaStream_t st) {
   if (p.res)
-    return p.mt == 2 ? launch_halo<RB, 2, true, PL, TALL>(p, wm, xm, st)
-                     : launch_halo<RB, 1, true, PL, TALL>(p, wm, xm, st);
-  return p.mt == 2 ? launch_halo<RB, 2, false, PL, TALL>(p, wm, xm, st)
-                   : launch_halo<RB, 1, false, PL, TALL>(p, wm, xm, st);
+    return p.mt == 2 ? launch_halo<RB, 2, true, PL, MODE>(p, wm, xm, st)
+                     : launch_halo<RB, 1, true, PL, MODE>(p, wm, xm, st);
+  return p.mt == 2 ? launch_halo<RB, 2, false, PL, MODE>(p, wm, xm, st)
+                   : launch_halo<RB, 1, false, PL, MODE>(p, wm, xm, st);
 }
 cudaError_t launch_halo_plan(const HaloPlan &p, const CUtensorMap &wm, const CUtensorMap &xm, cudaStream_t st) {
   const int m = p.a.mode, n = p.a.planes;
-  if (p.rb == 16) return launch_halo_pl<16, 0, false>(p, wm, xm, st);
-  if (p.rb == 32) return launch_halo_pl<32, 0, false>(p, wm, xm, st);
+  if (m == TILE_BOX)
+    return p.mt == 2 ? launch_halo<128, 2, false, 0, TILE_BOX>(p, wm, xm, st)
+                     : launch_halo<128, 1, false, 0, TILE_BOX>(p, wm, xm, st);
+  if (p.rb == 16) return launch_halo_pl<16, 0, TILE_WHOLE>(p, wm, xm, st);
+  if (p.rb == 32) return launch_halo_pl<32, 0, TILE_WHOLE>(p, wm, xm, st);
   if (p.rb == 64) {
-    if (m == TILE_WHOLE && n == 1) return launch_halo_pl<64, 1, false>(p, wm, xm, st);
-    if (m == TILE_WHOLE && n == 3) return launch_halo_pl<64, 3, false>(p, wm, xm, st);
-    return launch_halo_pl<64, 0, false>(p, wm, xm, st);
+    if (m == TILE_WHOLE && n == 1) return launch_halo_pl<64, 1, TILE_WHOLE>(p, wm, xm, st);
+    if (m == TILE_WHOLE && n == 3) return launch_halo_pl<64, 3, TILE_WHOLE>(p, wm, xm, st);
+    return launch_halo_pl<64, 0, TILE_WHOLE>(p, wm, xm, st);
   }
-  if (m == TILE_WHOLE && n == 1) return launch_halo_pl<128, 1, false>(p, wm, xm, st);
-  if (m == TILE_WHOLE && n == 3) return launch_halo_pl<128, 3, false>(p, wm, xm, st);
-  if (m == TILE_TALL && n == 1) return launch_halo_pl<128, 1, true>(p, wm, xm, st);
-  if (m == TILE_TALL && n == 2) return launch_halo_pl<128, 2, true>(p, wm, xm, st);
-  return launch_halo_pl<128, 0, false>(p, wm, xm, st);
+  if (m == TILE_WHOLE && n == 1) return launch_halo_pl<128, 1, TILE_WHOLE>(p, wm, xm, st);
+  if (m == TILE_WHOLE && n == 3) return launch_halo_pl<128, 3, TILE_WHOLE>(p, wm, xm, st);
+  if (m == TILE_TALL && n == 1) return launch_halo_pl<128, 1, TILE_TALL>(p, wm, xm, st);
+  if (m == TILE_TALL && n == 2) return launch_halo_pl<128, 2, TILE_TALL>(p, wm, xm, st);
+  return launch_halo_pl<128, 0, TILE_WHOLE>(p, wm, xm, st);  // walked: any tiling but box
 }
 
 // true when the call was launched here (rc its status); false: not this kernel's
@@ -1259,7 +1364,7 @@ bool conv_halo(const ConvArgs &v, cudaStream_t st, cudaError_t &rc) {
   const cuuint64_t wd[2] = {(cuuint64_t)v.K, (cuuint64_t)v.N}, ws[1] = {(cuuint64_t)v.K * 2};
   const cuuint32_t wb[2] = {64, (cuuint32_t)a.nb};
   if (!encode_bf16(&wm, 2, v.w, wd, ws, wb, CU_TENSOR_MAP_SWIZZLE_128B) ||
-      !encode_image(&xm, v.x, v.B, v.H, v.W, v.ldx, a.planes, p.rb, p.box_w, p.box_h, p.box_p))
+      !encode_image(&xm, v.x, v.B, v.H, v.W, v.ldx, a.planes, p.rb, p.box_w, p.box_h, p.box_p, p.box_b))
     return false;
   rc = launch_halo_plan(p, wm, xm, st);
   return true;

@@ -22,9 +22,10 @@ def conv64(x, w):
 # whose tiles span two of them, narrow images as one row, single pixels
 @pytest.mark.parametrize("B,H,W", [(1, 16, 8), (2, 17, 33), (3, 15, 7), (5, 20, 50), (7, 10, 25), (4, 5, 30),
                                    (9, 3, 31), (3, 1, 1), (2, 1, 64), (2, 64, 1), (70, 16, 40)])
-# one to many channel planes of every width; channel blocks of odd sizes
+# one to many channel planes of every width (the last two: a tap's channels at a
+# time); channel blocks of odd sizes
 @pytest.mark.parametrize("cin,cout", [(8, 32), (16, 2), (32, 96), (48, 24), (64, 10), (96, 40), (192, 64),
-                                      (128, 264), (512, 48)])
+                                      (128, 264), (512, 48), (768, 256), (1024, 24)])
 def test_conv_tilings(B, H, W, cin, cout):
     import torch
     from paper_2509_01827_gb300 import build, surrogate
