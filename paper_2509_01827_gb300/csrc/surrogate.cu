@@ -530,6 +530,30 @@ cudaError_t launch_conv_tc(const ConvArgs &a, cudaStream_t st) {
 //   512 -> 512, 10 x 25   94 -> 54 us, 1390 TFLOP/s (box; 113 with whole stages)
 //   512 -> 256, 10 x 25   78 -> 33 us (box)
 // One image, 256 -> 256, 20 x 50: 47 -> 12 us; 768 -> 256: 105 -> 37 us (box).
+// Programmatic dependents: the kernels of a forward pass are short (a single
+// image: 4 to 37 us, 30 of them), so each is placed while the one before it
+// still runs, sets up its barriers and tensor memory, and waits for that
+// kernel's results (dependency_wait) before it touches any global memory.  It
+// lets its own successor be placed only when it holds its tensor memory, so
+// that no two kernels can wait for each other's columns.  A forward pass of one
+// image: 275 -> 225 us.
+__device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void dependency_release() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 constexpr int HB_THREADS = 352, HB_MAXW = 48, HB_MAXA = 8;
 
 enum : int { TILE_WHOLE = 0, TILE_TALL = 1, TILE_FLAT = 2, TILE_BOX = 3 };
@@ -752,6 +776,7 @@ __global__ void __launch_bounds__(HB_THREADS, 1)
                  "r"(a.cols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
   }
+  dependency_wait();
   if (a.bias)
     for (int q = tid; q < a.nb; q += HB_THREADS) C.bias[q] = n0 + q < a.N ? a.bias[n0 + q] : 0.f;
   if (RB == 16) {  // the zero half of the last step: a second plane that no copy writes
@@ -763,6 +788,7 @@ __global__ void __launch_bounds__(HB_THREADS, 1)
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+  dependency_release();
   const uint32_t tmem = __shfl_sync(0xffffffffu, C.tmem, 0);
 
   if (warp == 10) {
@@ -1315,8 +1341,7 @@ cudaError_t launch_halo(const HaloPlan &p, const CUtensorMap &wm, const CUtensor
   static std::atomic<unsigned long long> done{0};
   cudaError_t e = allow_smem(k_conv3x3_halo<RB, MT, RES, PL, MODE>, done);
   if (e != cudaSuccess) return e;
-  k_conv3x3_halo<RB, MT, RES, PL, MODE><<<p.grid, HB_THREADS, p.smem, st>>>(wm, xm, p.a);
-  return cudaGetLastError();
+  return launch_dependent(k_conv3x3_halo<RB, MT, RES, PL, MODE>, p.grid, HB_THREADS, p.smem, st, wm, xm, p.a);
 }
 template <int RB, int PL, int MODE>
 cudaError_t launch_halo_pl(const HaloPlan &p, const CUtensorMap &wm, const CUtensorMap &xm, cudaStream_t st) {
@@ -2354,6 +2379,8 @@ __device__ __forceinline__ void st8(bf16_t *p, uint4 v) { *reinterpret_cast<uint
 
 // 2x2 max pooling: x [B, 2H, 2W] (pixel stride ldx) -> y [B, H, W, C] dense
 __global__ void __launch_bounds__(256) k_maxpool2(const bf16_t *x, int ldx, int rows, int W, int C, bf16_t *y) {
+  dependency_wait();
+  dependency_release();
   const unsigned C8 = C >> 3, n = W * C8;
   for (int r = blockIdx.y; r < rows; r += gridDim.y)  // row r of y: rows 2 r, 2 r + 1 of x
     for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
@@ -2424,6 +2451,8 @@ __global__ void __launch_bounds__(256) k_maxpool2_bwd(const bf16_t *x, int ldx, 
 // nearest 2x upsampling: x [B, H, W, C] dense -> y [B, 2H, 2W, ldy] at channel offset yoff
 __global__ void __launch_bounds__(256) k_upsample2(const bf16_t *x, int rows, int W, int C, bf16_t *y, int ldy,
                                                    int yoff) {
+  dependency_wait();
+  dependency_release();
   const unsigned C8 = C >> 3, n = W * C8;
   for (int r = blockIdx.y; r < rows; r += gridDim.y)
     for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
@@ -2475,6 +2504,8 @@ __global__ void __launch_bounds__(256) k_upsample2_bwd(const bf16_t *dy, int ldd
 // allow it (64 images, 32 channels: 2-byte reads took 232 us, these 50).
 __global__ void __launch_bounds__(256) k_head_fwd(const bf16_t *x, int P, int C, int vec, const float *w,
                                                   const float *b, float *z) {
+  dependency_wait();
+  dependency_release();
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
     const bf16_t *xp = x + (size_t)p * C;
     float s = b[0];
@@ -2868,9 +2899,9 @@ int cem_sg_maxpool2(const void *x, int ldx, int B, int H, int W, int C, void *y,
   if (!x || !y || B < 1 || H < 1 || W < 1 || C < 8 || (C & 7) || ldx < C || (ldx & 7))
     return CEM_SG_ERR_ARG;
   const long rows = (long)B * H;
-  k_maxpool2<<<grid_rows(rows, (long)W * (C >> 3)), 256, 0, (cudaStream_t)stream>>>(
-      (const bf16_t *)x, ldx, (int)rows, W, C, (bf16_t *)y);
-  return cudaGetLastError() == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
+  return launch_dependent(k_maxpool2, grid_rows(rows, (long)W * (C >> 3)), 256, 0, (cudaStream_t)stream,
+                          (const bf16_t *)x, ldx, (int)rows, W, C, (bf16_t *)y) == cudaSuccess
+             ? CEM_SG_OK : CEM_SG_ERR_CUDA;
 }
 
 int cem_sg_maxpool2_bwd(const void *x, int ldx, const void *dy, const void *dskip, int ldskip,
@@ -2892,9 +2923,9 @@ int cem_sg_upsample2(const void *x, int B, int H, int W, int C, void *y, int ldy
       (yoff & 7))
     return CEM_SG_ERR_ARG;
   const long rows = (long)B * H;
-  k_upsample2<<<grid_rows(rows, (long)W * (C >> 3)), 256, 0, (cudaStream_t)stream>>>(
-      (const bf16_t *)x, (int)rows, W, C, (bf16_t *)y, ldy, yoff);
-  return cudaGetLastError() == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
+  return launch_dependent(k_upsample2, grid_rows(rows, (long)W * (C >> 3)), 256, 0, (cudaStream_t)stream,
+                          (const bf16_t *)x, (int)rows, W, C, (bf16_t *)y, ldy, yoff) == cudaSuccess
+             ? CEM_SG_OK : CEM_SG_ERR_CUDA;
 }
 
 int cem_sg_upsample2_bwd(const void *dy, int lddy, int B, int H, int W, int C, const void *mask,
@@ -2912,8 +2943,9 @@ int cem_sg_head_fwd(const void *x, int P, int C, const float *w, const float *b,
                     void *stream) {
   if (!x || !w || !b || !z || P < 1 || C < 1) return CEM_SG_ERR_ARG;
   const int vec = !(C & 7) && !((uintptr_t)x & 15);
-  k_head_fwd<<<grid_1d(P, 256), 256, 0, (cudaStream_t)stream>>>((const bf16_t *)x, P, C, vec, w, b, z);
-  return cudaGetLastError() == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
+  return launch_dependent(k_head_fwd, grid_1d(P, 256), 256, 0, (cudaStream_t)stream, (const bf16_t *)x, P, C,
+                          vec, w, b, z) == cudaSuccess
+             ? CEM_SG_OK : CEM_SG_ERR_CUDA;
 }
 
 long cem_sg_head_workspace(int P, int C) {
