@@ -94,15 +94,20 @@ __device__ __forceinline__ Stress3 stress32(const Mat &m, float exx, float eyy, 
 }
 
 
+// load factors of the current step (Neumann, Dirichlet)
+__device__ __forceinline__ double2 load_factors(const DevState &d) {
+  const int idx = d.cnt->step - d.cnt->lam_base;
+  return make_double2(d.lamN[idx], d.lamD[idx]);
+}
+
 // Central-difference update of a node that carries a load, a prescribed
 // velocity, or whose kinetic energy is recorded this step.  Kept out of line:
 // if it were inlined, the compiler could predicate its FP64 instructions into
 // the update of every node, and on this GPU the FP64 pipe is 1/64 of FP32.
-__device__ __noinline__ double update_special(const DevState &d, int N, int cur, int first,
+__device__ __noinline__ double update_special(const DevState &d, int N, int cur, int first, double2 lam,
                                               float fx, float fy, float4 U, float2 vo, float minv,
                                               int nf, int energy) {
-  const int idx = d.cnt->step - d.cnt->lam_base;
-  const double lamN = d.lamN[idx], lamD = d.lamD[idx];
+  const double lamN = lam.x, lamD = lam.y;
   const float dt = d.mat.dtf;
   const float dtv = first ? 0.5f * dt : dt;
   float fex = 0.f, fey = 0.f;
@@ -453,6 +458,9 @@ __device__ __forceinline__ void march32_tile(const DevState &d, int tile_x, int 
                ? (int)d.nflag[r * stride + c] : 0;
   };
 
+  // read beside the first rows: two loads one after another at the tile's end otherwise
+  double2 lam = make_double2(0.0, 0.0);
+  if (!CLEAN) lam = load_factors(d);
 #pragma unroll
   for (int q = 0; q <= kAhead; ++q) stage(j0 - 2 + q);  // rows j0-2 .. j0+kAhead-2
   cp_async_wait<kAhead>();  // row j0 - 2 is in
@@ -754,7 +762,7 @@ __device__ __forceinline__ void march32_tile(const DevState &d, int tile_x, int 
     for (int k = 0; k < K; ++k) left |= spmask[k];
     auto special = [&](int N) {
       const float2 F = d.fsp[N];
-      ke += update_special(d, N, cur, first, F.x, F.y, u4[N], d.v2[N], d.minvf[N],
+      ke += update_special(d, N, cur, first, lam, F.x, F.y, u4[N], d.v2[N], d.minvf[N],
                            (int)d.nflag[N], ENERGY ? 1 : 0);
     };
     // a loaded row gives each lane one node a column: no list for that
@@ -895,7 +903,7 @@ __device__ __forceinline__ void phantom32(const DevState &d, VBlk vb, int cur, i
       }
     }
     if (energy)
-      ke += update_special(d, N, cur, first, fx, fy, d.u4[cur][N], d.v2[N], d.minvf[N], 0, 1);
+      ke += update_special(d, N, cur, first, make_double2(0.0, 0.0), fx, fy, d.u4[cur][N], d.v2[N], d.minvf[N], 0, 1);
     else
       update_plain(d, N, cur, dtv, dt, fx, fy, d.u4[cur][N], d.v2[N], d.minvf[N]);
   }

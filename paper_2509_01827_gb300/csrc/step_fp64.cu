@@ -198,6 +198,10 @@ inline double tile64_cost(const Tile64 &t) {
          52 * w(t.tx * t.ty);
 }
 
+__device__ __forceinline__ void prefetch_l1(const void *p) {
+  asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
+}
+
 // x / 2 and 2 x of a normal number or zero, by its exponent field
 __device__ __forceinline__ double half64(double x) {
   const int h = __double2hiint(x);
@@ -258,6 +262,16 @@ __device__ __forceinline__ void main64_tile(const DevState &d, VBlk vb, int cur,
     uint8_t s = ST_OUT;
     if (i >= 0 && j >= 0 && i < g.nx && j < g.ny) s = d.estate[j * g.nx + i];
     sst[q] = s;
+  }
+  // what the node updates at the end read besides, on its way into L1
+  for (int q = tid; q < T.tx * T.ty; q += NT) {
+    const int i = i0 + q % T.tx, j = j0 + q / T.tx;
+    if (i > g.nx || j > g.ny) continue;
+    const int N = j * (g.nx + 1) + i;
+    prefetch_l1(d.vx + N);
+    prefetch_l1(d.vy + N);
+    prefetch_l1(d.minv + N);
+    prefetch_l1(d.nflag + N);
   }
   ok = __syncthreads_and(ok);
 
