@@ -2723,27 +2723,54 @@ __global__ void __launch_bounds__(256) k_dice_grad(const float *z, const uint8_t
 // (a single thread walking all of it took 74 us for 64 samples, this 5)
 __global__ void __launch_bounds__(256) k_dice_loss(const float *ws, int nchunk, int B, float w, float eps,
                                                    float *loss) {
-  __shared__ float red[256];
+  // each image's sums by a thread, the images' terms added in their order
+  __shared__ float term[256];
   float d = 0.f;
-  for (int b = threadIdx.x; b < B; b += 256) {
-    float I = 0.f, S = 0.f;
-    for (int q = 0; q < nchunk; ++q) {
-      const float *o = ws + ((size_t)b * nchunk + q) * 3;
-      I += o[0];
-      S += o[1] + o[2];
+  for (int b0 = 0; b0 < B; b0 += 256) {
+    const int b = b0 + threadIdx.x;
+    if (b < B) {
+      float I = 0.f, S = 0.f;
+      for (int q = 0; q < nchunk; ++q) {
+        const float *o = ws + ((size_t)b * nchunk + q) * 3;
+        I += o[0];
+        S += o[1] + o[2];
+      }
+      term[threadIdx.x] = (2.f * I + eps) / (S + eps);
     }
-    d += (2.f * I + eps) / (S + eps);
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int q = 0; q < min(256, B - b0); ++q) d += term[q];
+    __syncthreads();
   }
-  d = block_sum256(d, red);
   if (threadIdx.x == 0) loss[0] = w * (1.f - d / (float)B);
 }
-
-// out[0] = scale sum ws[0..m), one block, fixed order (one thread took 98 us for 4,864 values)
 __global__ void __launch_bounds__(256) k_sum_scaled(const float *ws, int m, float scale, float *out) {
-  __shared__ float red[256];
+  // added one after another in a fixed order, from shared memory (from global
+  // memory the two sums of a loss took 230 us, nearly all of it waiting)
+  __shared__ __align__(16) float v[4096];
   float s = 0.f;
-  for (int i = threadIdx.x; i < m; i += 256) s += ws[i];
-  s = block_sum256(s, red);
+  for (int i0 = 0; i0 < m; i0 += 4096) {
+    const int k = min(4096, m - i0);
+    for (int i = threadIdx.x; i < k; i += 256) v[i] = ws[i0 + i];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      int i = 0;
+      for (; i + 16 <= k; i += 16) {
+        float4 a[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) a[q] = *reinterpret_cast<const float4 *>(v + i + 4 * q);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          s += a[q].x;
+          s += a[q].y;
+          s += a[q].z;
+          s += a[q].w;
+        }
+      }
+      for (; i < k; ++i) s += v[i];
+    }
+    __syncthreads();
+  }
   if (threadIdx.x == 0) out[0] = s * scale;
 }
 

@@ -45,3 +45,28 @@ def test_solo_heights_equal_batch(nx, ny, steps):
     for k in ("KE", "SE"):
         np.testing.assert_allclose(ea[k], ec[k], rtol=4096 * 2.0 ** -24, err_msg=k)
     b.close()
+
+
+@pytest.mark.parametrize("mode", ["neumann", "dirichlet"])
+def test_loaded_edges_up_a_tile(mode):
+    """A plate with a loaded hole (or driven outer edges): columns of loaded
+    nodes run up the tiles, up to 64 to a tile column and so more than a lane
+    lists at a time.  Every tile height gives the same fields."""
+    from paper_2509_01827_gb300.cem import CEM_FP32_MIXED, Batch, Solver
+    p = inputs.fragmentation(n=130, r=0.02, mode=mode, phantom_cap=8000, crack_cap=4000)
+    want = None
+    for rows in (0, 8, 32, 64):
+        s = Solver(p, precision=CEM_FP32_MIXED)
+        if rows:
+            b = Batch([s])
+            b.set_config(rows, 152)
+            b.step(60)
+        else:
+            s.step(60)
+        got = s.nodes()
+        assert np.max(np.abs(got["vx"])) > 0
+        want = want or got
+        for k in ("ux", "uy", "vx", "vy", "m"):
+            np.testing.assert_array_equal(got[k], want[k], err_msg=k)
+        if rows:
+            b.close()
