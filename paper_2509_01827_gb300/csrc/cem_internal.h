@@ -262,20 +262,28 @@ inline cudaError_t match_tile_carveout(K *kernel) {
 // and selection: 31.5 -> 29.0 us on a breaking 1024 x 1024 plate in FP32).  It
 // does not for the FP32 piece forces, whose waiting CTAs hold the slots the
 // evaluation wants (13.1 -> 13.7 us, 400 x 160), nor in a batch (70 -> 74 us).
+// carveout: the shared-memory split asked for, in percent of the most (0: the kernel's own).
 template <class... P, class... A>
-inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
-                                    cudaStream_t st, A... args) {
-  cudaLaunchAttribute attr[1];
+inline cudaError_t launch_dependent_carveout(int carveout, void (*kernel)(P...), dim3 grid, dim3 block,
+                                             size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  attr[1].val.sharedMemCarveout = (unsigned)carveout;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = carveout ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+template <class... P, class... A>
+inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                                    cudaStream_t st, A... args) {
+  return launch_dependent_carveout(0, kernel, grid, block, smem, st, args...);
 }
 #ifdef __CUDACC__
 // waits for the kernels this one was launched as a programmatic dependent of

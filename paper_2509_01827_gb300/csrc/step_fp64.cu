@@ -166,7 +166,7 @@ __global__ void k_pieces64(DevState d, int cur, int energy, int part_off) {
 //     takes the plain formulas instead (a CTA-wide vote);
 //   - the bracketed pairs of Eq. 6's sum are formed per edge, up to a sign,
 //     not per element and node.
-// About 120 instead of 309 FP64 instructions per node: 2683 -> 1156 us on the
+// About 120 instead of 309 FP64 instructions per node: 2683 -> 1095 us on the
 // 2048 x 2048 plate, 58 -> 26 us on 400 x 160, 36 -> 10 us on 100 x 40.
 // The tile shape follows the mesh (tile64_shape): a small mesh is cut finer so
 // that every SM gets a share.
@@ -183,10 +183,10 @@ struct Tile64 {
   __host__ __device__ int elems() const { return ew * eh; }
   __host__ __device__ int hedges() const { return hw * hh; }
   __host__ __device__ int vedges() const { return vw * vh; }
-  // node products (4), element sums (4), edge terms (6) and, on record steps,
-  // eps.sigma; then the element states
-  __host__ __device__ size_t bytes(bool energy) const {
-    return 8 * (4 * (size_t)nodes() + 4 * (size_t)elems() +
+  // node products (4, or 2 of square elements), element sums (4), edge terms (6)
+  // and, on record steps, eps.sigma; then the element states
+  __host__ __device__ size_t bytes(bool energy, bool square) const {
+    return 8 * ((square ? 2 : 4) * (size_t)nodes() + 4 * (size_t)elems() +
                 (energy ? 7 : 6) * (size_t)(hedges() + vedges())) + elems();
   }
 };
@@ -231,7 +231,7 @@ __device__ __forceinline__ void main64_tile(const DevState &d, VBlk vb, int cur,
   double *pc = square ? pa : pb + nn, *pd = square ? pb : pc + nn;
   // element sums: half the normal derivatives that enter exx (vertical edges)
   // and eyy (horizontal edges), and the whole ones that enter gxy
-  double *eX = sm + 4 * nn, *eN = eX + ne, *eXv = eN + ne, *eNu = eXv + ne;
+  double *eX = pd + nn, *eN = eX + ne, *eXv = eN + ne, *eNu = eXv + ne;
   // edge terms, planes of nhe (nve) values: see edge_terms
   const int planes = energy ? 7 : 6;
   double *H = eNu + ne, *V = H + planes * nhe;
@@ -658,7 +658,7 @@ namespace {
 cudaError_t fp64_attrs() {
   static bool done = false;
   if (done) return cudaSuccess;
-  const int most = (int)Tile64(32, 12).bytes(true);
+  const int most = (int)Tile64(32, 12).bytes(true, false);
   cudaError_t e = cudaFuncSetAttribute(k_main64, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_main64_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
@@ -700,8 +700,15 @@ cudaError_t launch_step_fp64(const DevState &d, int cur, bool first, bool energy
   int gx, gy;
   grid_main64(d, gx, gy);
   const dim3 grid(gx, gy);
-  const size_t smem = Tile64(d.t64x, d.t64y).bytes(energy);
   int tiles = gx * gy;
+  // Three CTAs of 32 x 12 square elements (70 KB each) feed the FP64 pipe better than
+  // two (2048 x 2048: 1136 -> 1097 us, the pipe 80% busy with two; 1000 x 1000: 295 ->
+  // 281), if the SM gives them all of its memory.  Meshes of few waves keep the side
+  // kernels' split, as an SM changes it only when it is empty (100 x 40: 18.7 us a
+  // step, 19.7 otherwise), and two CTAs, as a third on some SMs leaves others idle
+  // (400 x 160: 32.7 and 37.9).
+  const bool large = tiles >= 3 * 3 * 152;
+  const size_t smem = Tile64(d.t64x, d.t64y).bytes(energy, large && d.g.rxh == d.g.ryh);
   int gp = grid_pieces64(d);
   int gph = grid_phantoms(d);
   const int ge = grid_eval64(d);
@@ -724,7 +731,7 @@ cudaError_t launch_step_fp64(const DevState &d, int cur, bool first, bool energy
   cudaEventRecord(ss.fork, st);
   cudaStreamWaitEvent(ss.aux1, ss.fork, 0);
   k_phantom64<<<gph, 256, 0, ss.aux1>>>(d, cur, first ? 1 : 0, energy ? 1 : 0, tiles + gp);
-  launch_dependent(k_main64, grid, NT, smem, st, d, cur, first ? 1 : 0, energy ? 1 : 0);
+  launch_dependent_carveout(large ? 100 : 0, k_main64, grid, NT, smem, st, d, cur, first ? 1 : 0, energy ? 1 : 0);
   cudaEventRecord(ss.join1, ss.aux1);
   cudaEventRecord(ss.join2, ss.aux2);
   cudaStreamWaitEvent(st, ss.join1, 0);
@@ -751,7 +758,7 @@ cudaError_t launch_step_fp64_batch(const BatchDev &b, bool first, bool energy, i
   cudaEventRecord(ss.fork, st);
   cudaStreamWaitEvent(ss.aux1, ss.fork, 0);
   k_phantom64_batch<<<gph, 256, 0, ss.aux1>>>(b, first ? 1 : 0, energy ? 1 : 0);
-  launch_dependent(k_main64_batch, gm, NT, Tile64(32, 12).bytes(energy), st, b, first ? 1 : 0, energy ? 1 : 0);
+  launch_dependent(k_main64_batch, gm, NT, Tile64(32, 12).bytes(energy, false), st, b, first ? 1 : 0, energy ? 1 : 0);
   cudaEventRecord(ss.join1, ss.aux1);
   cudaEventRecord(ss.join2, ss.aux2);
   cudaStreamWaitEvent(st, ss.join1, 0);
