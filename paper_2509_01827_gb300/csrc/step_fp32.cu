@@ -1000,8 +1000,10 @@ cudaError_t launch_eval32_batch(const BatchDev &b, cudaStream_t st);
 // taken.  The node update of an elastic n x n plate, us, at 16 / 8 / 4 / 2 / 1 rows:
 // n = 128 19.4 / 14.4 / 12.4 / 10.6 / 10.6, 512 22.6 / 17.0 / 14.3 / 14.3 / 14.8,
 // 1024 26.8 / 23.3 / 22.9 / 25.5 / 35.1, 2048 52.5 / 55.4 / 62.0 / 80.0 / 115.
+// Not 16, although an intact 2048 x 2048 plate would gain by it: once it cracks, the
+// tiles of the general kind set the time (59.3 us at 16 rows after 400 steps, 55.7 at 8).
 int march_rows_solo(const DevState &d) {
-  constexpr int kRows[] = {16, 8, 6, 4, 3, 2, 1};
+  constexpr int kRows[] = {8, 6, 4, 3, 2, 1};
   constexpr long kWarps = 16 * 152;
   int best = 0;
   long best_c = 0;
