@@ -184,6 +184,145 @@ __global__ void __launch_bounds__(kEvalTB) k_eval32(DevState d, int cur) {
   eval32(d, hw_vblk(), cur);
 }
 
+// Everything the FP32 evaluation of surface point (e, k0) reads, loaded in
+// one level: the displacement pairs of e's nodes, the states of its four
+// neighbours, the two far nodes of each neighbour inside the mesh (across
+// the edges other than k0) and G_c of e.
+struct EvalPatch {
+  float4 ue[4];     // e's nodes, local order
+  float4 far[4][2]; // neighbour across edge k: its two nodes not on edge k
+  int st[4];        // neighbour states (ST_OUT outside the mesh)
+  float gc;
+};
+
+__device__ __forceinline__ void load_patch(const DevState &d, const U32x2 &U, int e, int k0,
+                                           EvalPatch &P) {
+  const Geo &g = d.g;
+  const int i = e % g.nx, j = e / g.nx, r = g.nx + 1;
+  const int n0 = j * r + i, n1 = n0 + 1, n2 = n0 + r + 1, n3 = n0 + r;
+  const int nd[4] = {n0, n1, n2, n3};
+  // far nodes of the neighbour below, right, above, left
+  const int fa[4][2] = {{n0 - r, n1 - r}, {n1 + 1, n2 + 1}, {n2 + r, n3 + r}, {n0 - 1, n3 - 1}};
+#pragma unroll
+  for (int a = 0; a < 4; ++a) P.ue[a] = U.u[nd[a]];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int f = elem_neighbor(g, e, k);
+    P.st[k] = estatus(d, f);
+    const bool use = f >= 0 && k != k0;
+    P.far[k][0] = use ? U.u[fa[k][0]] : make_float4(0.f, 0.f, 0.f, 0.f);
+    P.far[k][1] = use ? U.u[fa[k][1]] : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  P.gc = d.gc[e];
+}
+
+// The neighbour across edge k in its own local node order.
+__device__ __forceinline__ void neighbour_nodes(const EvalPatch &P, int k, float4 (&q)[4]) {
+  switch (k) {
+    case 0: q[0] = P.far[0][0]; q[1] = P.far[0][1]; q[2] = P.ue[1]; q[3] = P.ue[0]; break;
+    case 1: q[0] = P.ue[1]; q[1] = P.far[1][0]; q[2] = P.far[1][1]; q[3] = P.ue[2]; break;
+    case 2: q[0] = P.ue[3]; q[1] = P.ue[2]; q[2] = P.far[2][0]; q[3] = P.far[2][1]; break;
+    default: q[0] = P.far[3][0]; q[1] = P.ue[0]; q[2] = P.ue[3]; q[3] = P.far[3][1]; break;
+  }
+}
+
+__device__ __forceinline__ void used_stress32(const DevState &d, const EvalPatch &P, int k,
+                                              float s[3]) {
+  float e1[3];
+  own_strain32(d.g, P.ue, k, e1);
+  if (P.st[k] == ST_INTACT) {
+    float4 q[4];
+    neighbour_nodes(P, k, q);
+    float e2[3];
+    own_strain32(d.g, q, (k + 2) & 3, e2);
+    for (int c = 0; c < 3; ++c) e1[c] = 0.5f * (e1[c] + e2[c]);
+  }
+  const Mat &m = d.mat;
+  s[0] = m.D11f * e1[0] + m.D12f * e1[1];
+  s[1] = m.D12f * e1[0] + m.D11f * e1[1];
+  s[2] = m.D33f * e1[2];
+}
+
+__device__ __forceinline__ void eval_G32(const DevState &d, const EvalPatch &P, int k0,
+                                         float G[4]) {
+  const Geo &g = d.g;
+  const float DX = g.DXf[k0], DY = g.DYf[k0];
+  float4 P1 = P.ue[0], P2 = P.ue[1];
+#pragma unroll
+  for (int a = 1; a < 4; ++a)
+    if (a == k0) { P1 = P.ue[a]; P2 = P.ue[(a + 1) & 3]; }
+  float dux = df_diff(P1.x, P1.y, P2.x, P2.y);
+  float duy = df_diff(P1.z, P1.w, P2.z, P2.w);
+  // |x_N2 - x_N1|^2 - |X_N2 - X_N1|^2 without cancellation
+  float stretch = 2.f * (DX * dux + DY * duy) + (dux * dux + duy * duy);
+  float H = stretch > 0.f ? 1.f : 0.f;
+  float ddx = dux * H, ddy = duy * H;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    if (k == k0) { G[k] = -1.f; continue; }
+    const float nx = g.nxf[k0][k], ny = g.nyf[k0][k];
+    float s[3];
+    used_stress32(d, P, k, s);
+    float tx = s[0] * nx + s[2] * ny;
+    float ty = s[2] * nx + s[1] * ny;
+    G[k] = 0.5f * (ddx * tx + ddy * ty);
+  }
+}
+
+// Large meshes: a thread per point, its candidates one after another, one
+// block of 256 threads per SM.  There the piece forces and the node update set
+// the step, and this form takes less from them: a breaking 2048 x 2048 plate's
+// step 61.5 / 67.9 / 84.7 us after 400 / 4000 / 9000 steps, 62.8 / 73.4 / 94.4 with the
+// split above, which alone is done sooner (12.7 / 14.5 / 17.8 against 19.0 / 13.7 /
+// 22.9 us) and on a 1024 x 1024 plate, whose step is the chain of evaluation,
+// selection and split writes, the better one (with it 31.5 us, 36 before).
+constexpr int kLargeMesh = 1 << 21;  // nodes
+__device__ __forceinline__ void eval32_points(const DevState &d, VBlk vb, int cur) {
+  const int n = d.cnt->n_S;
+  const U32x2 U{d.u4[cur]};
+  for (int base = vb.x * blockDim.x; base < n; base += vb.gx * blockDim.x) {
+    int i = base + threadIdx.x;
+    bool has = false;
+    int key = 0, edge = 0, kk = -1;
+    double Gk = 0.0;
+    if (i < n) {
+      edge = d.S[i];
+      const int info = d.S_info[i];
+      if (edge >= 0) {
+        key = info;
+        int e = key >> 2, k0 = key & 3;
+        if (d.mat.scope != 2 || is_tip_edge(d, e, k0)) {
+          EvalPatch P;
+          load_patch(d, U, e, k0, P);
+          float G32[4];
+          eval_G32(d, P, k0, G32);
+          float gc = P.gc;
+          bool near = false;
+          for (int k = 0; k < 4; ++k)
+            if (k != k0 && fabsf(G32[k] / gc - 1.f) < 1e-3f) near = true;
+          double G[4];
+          if (near) {
+            // FP64 re-check near the threshold
+            for (int k = 0; k < 4; ++k) G[k] = recheck64(d, d.u4[cur], e, k0, k);
+          } else {
+            for (int k = 0; k < 4; ++k) G[k] = (double)G32[k];
+          }
+          double gm = -1.0;
+          for (int k = 0; k < 4; ++k) gm = fmax(gm, G[k]);
+          d.S_G[i] = gm;
+          kk = rule64(d, e, k0, G);
+          if (kk >= 0) { has = true; Gk = G[kk]; }
+        }
+      }
+    }
+    append_proposal(d, has, key, edge, kk, Gk);
+  }
+}
+
+__global__ void __launch_bounds__(256, 4) k_eval32_points(DevState d, int cur) {
+  eval32_points(d, hw_vblk(), cur);
+}
+
 __global__ void __launch_bounds__(kEvalTB) k_eval32_batch(BatchDev b) {
   __shared__ DevState sd;
   int held = -1, w0, w1;
@@ -211,6 +350,7 @@ cudaError_t eval32_carveouts() {
   if (done) return cudaSuccess;
   cudaError_t e = match_tile_carveout(k_eval32);
   if (e == cudaSuccess) e = match_tile_carveout(k_eval32_batch);
+  if (e == cudaSuccess) e = match_tile_carveout(k_eval32_points);
   if (e == cudaSuccess) done = true;
   return e;
 }
@@ -218,6 +358,10 @@ cudaError_t eval32_carveouts() {
 cudaError_t launch_eval32(const DevState &d, int cur, cudaStream_t st) {
   cudaError_t e = eval32_carveouts();
   if (e != cudaSuccess) return e;
+  if (d.g.nn > kLargeMesh) {
+    k_eval32_points<<<grid_for(d.list_cap, 256, 152), 256, 0, st>>>(d, cur);
+    return cudaGetLastError();
+  }
   return launch_dependent(k_eval32, grid_eval(d), kEvalTB, 0, st, d, cur);
 }
 

@@ -1,5 +1,5 @@
 """FP32-mixed node update: a mesh stepped alone picks its tile height from its
-size (1 to 16 node rows), a batch marches tiles of 8 rows or more.  The height
+size (1 to 8 node rows), a batch marches tiles of 8 rows or more.  The height
 decides which warp marches a node, not the node's arithmetic, so the fields
 and cracks of both are identical, bit for bit (needs a GPU)."""
 import numpy as np
@@ -16,7 +16,7 @@ def _built():
     build.build()
 
 
-# the heights these sizes take alone: 1, 1, 3, 4, 6 and 8 rows, 16 above
+# the heights these sizes take alone: 1, 1, 3, 4, 6 and 8 rows
 @pytest.mark.parametrize("nx,ny,steps", [(59, 23, 260), (100, 40, 260), (512, 512, 40),
                                          (770, 767, 20), (1030, 1021, 12), (1440, 1450, 8)])
 def test_solo_heights_equal_batch(nx, ny, steps):
@@ -70,3 +70,23 @@ def test_loaded_edges_up_a_tile(mode):
             np.testing.assert_array_equal(got[k], want[k], err_msg=k)
         if rows:
             b.close()
+
+
+def test_large_mesh_evaluation_equals_batch():
+    """Above two million nodes a plate stepped alone evaluates a thread per
+    surface point, a batch always a warp per candidate path: cracks and fields
+    of a breaking plate are the same."""
+    from paper_2509_01827_gb300.cem import CEM_FP32_MIXED, Batch, Solver
+    p = inputs.fragmentation(n=1500, p0=80e6, phantom_cap=40000, crack_cap=20000)
+    a, c = Solver(p, precision=CEM_FP32_MIXED), Solver(p, precision=CEM_FP32_MIXED)
+    a.step(330)
+    b = Batch([c])
+    b.step(330)
+    assert a.counts()["n_cracked"] > 0
+    na, nc = a.nodes(), c.nodes()
+    for k in ("ux", "uy", "vx", "vy", "m"):
+        np.testing.assert_array_equal(na[k], nc[k], err_msg=k)
+    ca, cc = a.cracks(), c.cracks()
+    for k in ("elem", "ka", "kb", "step"):
+        np.testing.assert_array_equal(ca[k], cc[k], err_msg=k)
+    b.close()
