@@ -333,6 +333,7 @@ __global__ void __launch_bounds__(kEvalTB) k_eval32_batch(BatchDev b) {
     stage_member(b.ds, it.x, sd, held);
     if (!member_active(sd, n)) continue;
     eval32(sd, VBlk{it.y, 0, it.w, 1}, member_cur(sd, n));
+    __syncthreads();  // this item's shared values are read before the next one's (39 members on: two a block)
   }
 }
 

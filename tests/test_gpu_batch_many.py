@@ -1,0 +1,37 @@
+"""A batch of so many FP32 members that a block of the evaluation takes several
+work items of one member (from 39 members on): every member ends where it ends
+when stepped alone, bit for bit (needs a GPU)."""
+import numpy as np
+import pytest
+
+from paper_2509_01827_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("count", [39, 64])
+def test_many_members_equal_solo_runs(count):
+    from paper_2509_01827_gb300 import build
+    from paper_2509_01827_gb300.cem import CEM_FP32_MIXED, Batch, Solver
+    build.build()
+    probs = [inputs.notched_plate(50 + s % 11, 20 + s % 7, notch_len=0.02 + 2e-4 * s,
+                                  traction=(2.0 + 0.02 * s) * 1e6, phantom_cap=8000, crack_cap=2000)
+             for s in range(count)]
+    members = [Solver(p, precision=CEM_FP32_MIXED) for p in probs]
+    b = Batch(members)
+    b.step(280)
+    grown = 0
+    for p, m in zip(probs, members):
+        s = Solver(p, precision=CEM_FP32_MIXED)
+        pre = s.counts()["n_cracked"]
+        s.step(280)
+        grown += s.counts()["n_cracked"] > pre
+        got, want = m.nodes(), s.nodes()
+        for k in ("ux", "uy", "vx", "vy", "m"):
+            np.testing.assert_array_equal(got[k], want[k], err_msg=k)
+        got, want = m.cracks(), s.cracks()
+        for k in ("elem", "ka", "kb", "step", "nodes"):
+            np.testing.assert_array_equal(got[k], want[k], err_msg=k)
+        s.close()
+    assert grown > count // 2
+    b.close()
