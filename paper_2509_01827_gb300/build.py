@@ -30,7 +30,7 @@ UNITS = [
     ("tri.cu", ["-fmad=false"]),
     ("api.cpp", []),
 ]
-HEADERS = ["cem_internal.h", "q4_fp64.cuh", "eval_common.cuh", "tri_internal.h"]
+HEADERS = ["cem_internal.h", "q4_fp64.cuh", "eval_common.cuh", "tri_internal.h", "per_device.h"]
 
 
 def _stale(obj, deps):

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "per_device.h"
+
 namespace cem {
 
 enum : int { ST_INTACT = 0, ST_CRACKED = 1, ST_OUT = 2 };

@@ -270,14 +270,14 @@ cudaError_t launch_element_stress(const DevState &d, int cur, double *out4, cuda
 }
 
 cudaError_t energy_carveouts() {
-  static bool done = false;
-  if (done) return cudaSuccess;
-  cudaError_t e = match_tile_carveout(k_energy_pre);
-  if (e == cudaSuccess) e = match_tile_carveout(k_energy_post);
-  if (e == cudaSuccess) e = match_tile_carveout(k_energy_pre_batch);
-  if (e == cudaSuccess) e = match_tile_carveout(k_energy_post_batch);
-  if (e == cudaSuccess) done = true;
-  return e;
+  static PerDevice attrs;
+  return attrs.once([] {
+    cudaError_t e = match_tile_carveout(k_energy_pre);
+    if (e == cudaSuccess) e = match_tile_carveout(k_energy_post);
+    if (e == cudaSuccess) e = match_tile_carveout(k_energy_pre_batch);
+    if (e == cudaSuccess) e = match_tile_carveout(k_energy_post_batch);
+    return e;
+  });
 }
 
 cudaError_t launch_energy_pre(const DevState &d, cudaStream_t st) {

@@ -347,13 +347,13 @@ int grid_for(int n, int block, int maxb) {
 int grid_eval(const DevState &d) { return grid_for(d.list_cap, kEvalPts, 608); }
 
 cudaError_t eval32_carveouts() {
-  static bool done = false;
-  if (done) return cudaSuccess;
-  cudaError_t e = match_tile_carveout(k_eval32);
-  if (e == cudaSuccess) e = match_tile_carveout(k_eval32_batch);
-  if (e == cudaSuccess) e = match_tile_carveout(k_eval32_points);
-  if (e == cudaSuccess) done = true;
-  return e;
+  static PerDevice attrs;
+  return attrs.once([] {
+    cudaError_t e = match_tile_carveout(k_eval32);
+    if (e == cudaSuccess) e = match_tile_carveout(k_eval32_batch);
+    if (e == cudaSuccess) e = match_tile_carveout(k_eval32_points);
+    return e;
+  });
 }
 
 cudaError_t launch_eval32(const DevState &d, int cur, cudaStream_t st) {

@@ -970,8 +970,8 @@ int grid_for(int n, int block, int maxb) {
 }
 
 cudaError_t set_all_smem_attrs() {
-  static bool done = false;
-  if (!done) {
+  static PerDevice attrs;
+  return attrs.once([] {
     // every kernel of the step asks for one shared-memory split, so that the
     // side branches can share SMs with the node update
     cudaError_t e = match_tile_carveout(k_phantom32);
@@ -982,10 +982,8 @@ cudaError_t set_all_smem_attrs() {
     if (e == cudaSuccess) e = match_tile_carveout(k_march32<false>);
     if (e == cudaSuccess) e = match_tile_carveout(k_march32_batch<true>);
     if (e == cudaSuccess) e = match_tile_carveout(k_march32_batch<false>);
-    if (e != cudaSuccess) return e;
-    done = true;
-  }
-  return cudaSuccess;
+    return e;
+  });
 }
 
 }  // namespace

@@ -656,22 +656,22 @@ namespace {
 // match_tile_carveout), so that the surface evaluation's blocks do not keep
 // the node update off their SMs.
 cudaError_t fp64_attrs() {
-  static bool done = false;
-  if (done) return cudaSuccess;
-  const int most = (int)Tile64(32, 12).bytes(true, false);
-  cudaError_t e = cudaFuncSetAttribute(k_main64, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_main64_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  if (e == cudaSuccess) e = match_tile_carveout(k_main64);
-  if (e == cudaSuccess) e = match_tile_carveout(k_main64_batch);
-  if (e == cudaSuccess) e = match_tile_carveout(k_pieces64);
-  if (e == cudaSuccess) e = match_tile_carveout(k_pieces64_batch);
-  if (e == cudaSuccess) e = match_tile_carveout(k_phantom64);
-  if (e == cudaSuccess) e = match_tile_carveout(k_phantom64_batch);
-  if (e == cudaSuccess) e = match_tile_carveout(k_eval64);
-  if (e == cudaSuccess) e = match_tile_carveout(k_eval64_batch);
-  done = e == cudaSuccess;
-  return e;
+  static PerDevice attrs;
+  return attrs.once([] {
+    const int most = (int)Tile64(32, 12).bytes(true, false);
+    cudaError_t e = cudaFuncSetAttribute(k_main64, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_main64_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess) e = match_tile_carveout(k_main64);
+    if (e == cudaSuccess) e = match_tile_carveout(k_main64_batch);
+    if (e == cudaSuccess) e = match_tile_carveout(k_pieces64);
+    if (e == cudaSuccess) e = match_tile_carveout(k_pieces64_batch);
+    if (e == cudaSuccess) e = match_tile_carveout(k_phantom64);
+    if (e == cudaSuccess) e = match_tile_carveout(k_phantom64_batch);
+    if (e == cudaSuccess) e = match_tile_carveout(k_eval64);
+    if (e == cudaSuccess) e = match_tile_carveout(k_eval64_batch);
+    return e;
+  });
 }
 }  // namespace
 

@@ -20,9 +20,8 @@
 #include <math.h>
 #include <stdint.h>
 
-#include <atomic>
-
 #include "../../include/cem_surrogate.h"
+#include "per_device.h"
 
 namespace {
 
@@ -461,6 +460,14 @@ __global__ void __launch_bounds__(128, 1) k_conv3x3_tc(ConvArgs a) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(BN));
 }
 
+// raises a kernel's dynamic shared-memory limit, once per device
+template <class K>
+cudaError_t allow_smem(K *kernel, size_t bytes, PerDevice &attrs) {
+  return attrs.once([=] {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  });
+}
+
 template <int BN>
 size_t tc_smem_bytes() {
   return sizeof(TcSmem<BN>) + 1024;
@@ -468,14 +475,9 @@ size_t tc_smem_bytes() {
 
 template <int BN>
 cudaError_t launch_conv_tc(const ConvArgs &a, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(k_conv3x3_tc<BN>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)tc_smem_bytes<BN>());
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static PerDevice attrs;
+  const cudaError_t ae = allow_smem(k_conv3x3_tc<BN>, tc_smem_bytes<BN>(), attrs);
+  if (ae != cudaSuccess) return ae;
   dim3 grid((a.P + TCM - 1) / TCM, (a.N + BN - 1) / BN);
   k_conv3x3_tc<BN><<<grid, 128, tc_smem_bytes<BN>(), st>>>(a);
   return cudaGetLastError();
@@ -1323,23 +1325,10 @@ bool encode_image(CUtensorMap *map, const void *x, int B, int H, int W, int ld, 
                      : rb == 32 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
-// raises a kernel's dynamic shared-memory limit, once per device
-template <class K>
-cudaError_t allow_smem(K *kernel, std::atomic<unsigned long long> &done) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const unsigned long long bit = 1ull << (dev & 63);
-  if (done.load() & bit) return cudaSuccess;
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
-  if (e == cudaSuccess) done.fetch_or(bit);
-  return e;
-}
-
 template <int RB, int MT, bool RES, int PL, int MODE>
 cudaError_t launch_halo(const HaloPlan &p, const CUtensorMap &wm, const CUtensorMap &xm, cudaStream_t st) {
-  static std::atomic<unsigned long long> done{0};
-  cudaError_t e = allow_smem(k_conv3x3_halo<RB, MT, RES, PL, MODE>, done);
+  static PerDevice attrs;
+  cudaError_t e = allow_smem(k_conv3x3_halo<RB, MT, RES, PL, MODE>, kSmemMax, attrs);
   if (e != cudaSuccess) return e;
   return launch_dependent(k_conv3x3_halo<RB, MT, RES, PL, MODE>, p.grid, HB_THREADS, p.smem, st, wm, xm, p.a);
 }
@@ -1765,14 +1754,9 @@ size_t tw_smem_bytes() {
 
 template <int BN>
 cudaError_t launch_wgrad_tc(const WgradArgs &a, int splits, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(k_conv3x3_wgrad_tc<BN>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)tw_smem_bytes<BN>());
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static PerDevice attrs;
+  const cudaError_t ae = allow_smem(k_conv3x3_wgrad_tc<BN>, tw_smem_bytes<BN>(), attrs);
+  if (ae != cudaSuccess) return ae;
   dim3 grid((a.K + WTM - 1) / WTM, (a.N + BN - 1) / BN, splits);
   k_conv3x3_wgrad_tc<BN><<<grid, 128, tw_smem_bytes<BN>(), st>>>(a);
   return cudaGetLastError();
@@ -2288,8 +2272,8 @@ bool wgrad_halo_plan(const WgradArgs &v, int most, WgHaloPlan &best) {
 
 template <int RBX, int RBY, int PER>
 cudaError_t launch_wgrad_per(const WgHaloPlan &p, const WgMaps &m, cudaStream_t st) {
-  static std::atomic<unsigned long long> done{0};
-  cudaError_t e = allow_smem(k_wgrad_halo<RBX, RBY, PER>, done);
+  static PerDevice attrs;
+  cudaError_t e = allow_smem(k_wgrad_halo<RBX, RBY, PER>, kSmemMax, attrs);
   if (e != cudaSuccess) return e;
   k_wgrad_halo<RBX, RBY, PER><<<dim3(p.gx, p.gy, p.slots), WH_THREADS, p.smem, st>>>(m, p.a);
   return cudaGetLastError();

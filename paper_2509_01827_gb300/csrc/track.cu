@@ -968,16 +968,16 @@ __global__ void k_status_copy(const Counters *cnt, Counters *out) {
 }  // namespace
 
 cudaError_t launch_select(const DevState &d, int mode, cudaStream_t st) {
-  size_t sm = select_smem_bytes();
-  static bool attr = false;
-  if (!attr) {
+  constexpr size_t sm = select_smem_bytes();
+  static PerDevice attrs;
+  const cudaError_t ae = attrs.once([] {
     cudaError_t e = cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sm);
     if (e == cudaSuccess) e = match_tile_carveout(k_select);
     if (e == cudaSuccess) e = match_tile_carveout(k_apply);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+    return e;
+  });
+  if (ae != cudaSuccess) return ae;
   return launch_dependent(k_select, 1, TB, sm, st, d, mode);
 }
 
@@ -1017,16 +1017,16 @@ cudaError_t launch_surface_info(const DevState &d, int *out3, cudaStream_t st) {
 }
 
 cudaError_t launch_select_batch(const BatchDev &b, cudaStream_t st) {
-  size_t sm = select_smem_bytes();
-  static bool attr = false;
-  if (!attr) {
+  constexpr size_t sm = select_smem_bytes();
+  static PerDevice attrs;
+  const cudaError_t ae = attrs.once([] {
     cudaError_t e = cudaFuncSetAttribute(k_select_batch,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e == cudaSuccess) e = match_tile_carveout(k_select_batch);
     if (e == cudaSuccess) e = match_tile_carveout(k_apply_batch);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+    return e;
+  });
+  if (ae != cudaSuccess) return ae;
   k_select_batch<<<b.n < 304 ? b.n : 304, TB, sm, st>>>(b);
   return cudaGetLastError();
 }
