@@ -775,6 +775,7 @@ __device__ __forceinline__ void march32_tile(const DevState &d, int tile_x, int 
         if (spmask[k]) special((j0 + __ffsll((long long)spmask[k]) - 1) * stride + c0 + k);
       left = 0;
     }
+    __syncwarp();  // every lane has read its rows of the ring, and its copies into it are done
     while (__any_sync(FULL, left != 0)) {
       int mine = 0;
 #pragma unroll

@@ -68,3 +68,12 @@ def test_a_barrier_between_items(kernel, fns):
     if any(_shares(c, fns) for c in calls):
         last = max(loop.rindex(c + "(") if c + "(" in loop else loop.rindex(c + "<") for c in calls)
         assert "__syncthreads();" in loop[last:]
+
+
+def test_loaded_node_list_waits_for_the_ring():
+    """The march lists a tile's loaded nodes in the memory of its row ring, at
+    positions that other lanes' rows held: votes and shuffles order no memory, so a
+    warp barrier stands between the ring's last use and the list's first write."""
+    body = _functions(_sources()["step_fp32.cu"])["march32_tile"]
+    last_use = max(body.rindex("ring.of("), body.rindex("cp_async_wait<0>"))
+    assert "__syncwarp();" in body[last_use:body.index("list[at++]")]
