@@ -53,8 +53,7 @@ long cem_sg_wgrad_workspace(int B, int H, int W, int Cin, int Cout);
  * sum_p dy[p, o] x[p + (ky-1, kx-1), c] (FP32), db[o] = sum_p dy[p, o]
  * (db may be NULL).  The data gradient is cem_sg_conv3x3 applied to dy with
  * the transposed, flipped weights that cem_sg_adam writes.  Cin, Cout, ldx,
- * lddy multiples of 8.  A non-finite x may make dw non-finite for all nine
- * taps of its channel, the taps that would use it outside the image too. */
+ * lddy multiples of 8. */
 int cem_sg_conv3x3_wgrad(const void *x, int ldx, const void *dy, int lddy, int B, int H, int W,
                          int Cin, int Cout, float *dw, float *db, void *ws, long ws_bytes,
                          void *stream);

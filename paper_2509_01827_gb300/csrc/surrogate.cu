@@ -1762,6 +1762,70 @@ cudaError_t launch_wgrad_tc(const WgradArgs &a, int splits, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+// Non-finite inputs.  Tiles that reach past an image (or across the zero rows and
+// columns between two) multiply the image's border pixels with the zero dY outside it:
+// nothing is added unless such a pixel is not finite, when 0 x Inf or 0 x NaN would make
+// the weight gradients of the taps that look from outside NaN.  Whatever finishes dw
+// (k_reduce_sums, or k_wgrad_halo where a range has all of an entry) forms those again from
+// the pixels inside, one warp each; it looks for them at entries that are not finite, so
+// finite gradients cost a comparison (64 images, 512 -> 512 channels at 10 x 25: 111 us
+// with it as without; one infinity at a corner 0.4 ms, all of x NaN 1.3 ms).
+struct DwInputs {
+  const bf16_t *x, *dy;
+  int B, H, W, Cin, ldx, lddy, K;
+};
+inline DwInputs dw_inputs(const WgradArgs &v) {
+  return DwInputs{v.x, v.dy, v.B, v.H, v.W, v.Cin, v.ldx, v.lddy, v.K};
+}
+__device__ __forceinline__ bool finite_bf(bf16_t v) { return (v & 0x7f80) != 0x7f80; }
+
+// dw entry i = (o, tap, c), whose sum over the tiles is s; whole warps call it
+__device__ __noinline__ float dw_inside(const DwInputs &v, long i, float s) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int o = (int)(i / v.K), k = (int)(i - (long)o * v.K), tap = k / v.Cin;
+  const int dh = tap / 3 - 1, dw = tap % 3 - 1;
+  const bf16_t *x = v.x + (k - tap * v.Cin), *dy = v.dy + o;
+  // is one of the border pixels that this tap would read for a pixel outside not finite?
+  bool bad = false;
+  for (int side = 0; side < 2 && !bad; ++side) {
+    // the image's last row (column) for the taps above (left), its first for those below (right)
+    const int d = side ? dw : dh, n = d == 0 ? 0 : v.B * (side ? v.H : v.W);
+    for (int q0 = 0, steps = 1; q0 < n && !bad; q0 += 32 * steps, steps = 8) {  // the first 32, 256 at a time then
+      bool odd = false;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        if (j >= steps) break;
+        const int q = min(q0 + j * 32 + lane, n - 1), b = q / v.W;
+        const size_t p = side ? (size_t)q * v.W + (d < 0 ? v.W - 1 : 0)
+                              : ((size_t)b * v.H + (d < 0 ? v.H - 1 : 0)) * v.W + (q - b * v.W);
+        odd |= !finite_bf(x[p * v.ldx]);
+      }
+      bad = __any_sync(FULL, odd);
+    }
+  }
+  if (!bad) return s;
+  const int P = v.B * v.H * v.W;
+  double sum = 0.0;
+  for (int p0 = 0, steps = 1; p0 < P; p0 += 32 * steps, steps = 8) {
+    float t = 0.f;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int p = p0 + q * 32 + lane;
+      if (q >= steps || p >= P) continue;
+      const int r = p / v.W, w = p - r * v.W + dw, h = r % v.H + dh;
+      const bool in = h >= 0 && h < v.H && w >= 0 && w < v.W;
+      const float xv = in ? bf2f(x[((long)p + dh * v.W + dw) * v.ldx]) : 0.f;
+      t += xv * bf2f(dy[(size_t)p * v.lddy]);
+    }
+    sum += (double)t;
+    if (__any_sync(FULL, isnan(sum))) return __int_as_float(0x7fc00000);  // whatever follows
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(FULL, sum, off);
+  return (float)sum;
+}
+
 // --------------------------- weight gradient with the input tile resident
 // dW[o][tap][c] = sum_p dY[p][o] x[p + tap][c], K = pixels.  As in
 // k_conv3x3_halo a stage holds the halo of a 128-pixel tile of x, and beside it
@@ -1805,6 +1869,8 @@ struct WgHaloArgs {
   int nb;               // output channels of a block, columns of an accumulator
   int nacc;             // accumulator sets
   int na, stage, y_at, cols, off_ctl;
+  int inside;           // the range has all of dw's sums, from tiles that reach past the images
+  DwInputs in;
 };
 
 struct WgHaloCtl {
@@ -1835,7 +1901,7 @@ __device__ __forceinline__ void tall_rows(const WgHaloArgs &a, int t0, int n, F 
 
 template <int RBX, int RBY, int PER>
 __global__ void __launch_bounds__(WH_THREADS, 1)
-    k_wgrad_halo(const __grid_constant__ WgMaps maps, const WgHaloArgs a) {
+    k_wgrad_halo(const __grid_constant__ WgMaps maps, const __grid_constant__ WgHaloArgs a) {
   extern __shared__ uint8_t wh_raw[];
   uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(wh_raw) + 1023) &
                                               ~(uintptr_t)1023);
@@ -1996,6 +2062,17 @@ __global__ void __launch_bounds__(WH_THREADS, 1)
 #pragma unroll
       for (int k = 0; k < 8; ++k) sum[p][k] = 0.f;
     float *out = a.ws + (size_t)z * a.N * a.K;
+    // where this lane's row of a unit's 32 columns goes (null: nowhere)
+    const int ncb = a.nb / 32, units = nq * ncb;
+    auto dest = [&](int u) -> float * {
+      const int j = u / ncb, cb = (u - j * ncb) * 32;
+      const int q = q0 + j, pl = q / TAPB, t = q - pl * TAPB;
+      const int tap = RBX == 128 ? 2 * t + (w4 >> 1) : RBX == 64 ? 3 * t + w4 : 3 * t + (lane >> 3);
+      const int c = RBX == 128 ? pl * 64 + (w4 & 1) * 32 + lane : RBX == 64 ? pl * 32 + lane : lane & 7;
+      if (u >= units || (RBX == 128 ? tap >= 9 : RBX == 64 ? w4 >= 3 : w4 > 0 || lane >= 24)) return nullptr;
+      return out + (size_t)(n0 + cb) * a.K + tap * a.Cin + c;
+    };
+    float odd = 0.f;  // NaN once a sum of the range is not finite
     int s = 0, ph = 0, ab = 0, abph = 0;
     bool ok = true;
     for (int tile = tbeg; tile < tend && ok;) {
@@ -2035,15 +2112,6 @@ __global__ void __launch_bounds__(WH_THREADS, 1)
       // unit u: 32 columns of a block.  What the slot holds already is read a unit
       // ahead (the first before the sums are in), so that its latency is hidden.
       const bool add = tile > tbeg;
-      const int ncb = a.nb / 32, units = nq * ncb;
-      auto dest = [&](int u) -> float * {
-        const int j = u / ncb, cb = (u - j * ncb) * 32;
-        const int q = q0 + j, pl = q / TAPB, t = q - pl * TAPB;
-        const int tap = RBX == 128 ? 2 * t + (w4 >> 1) : RBX == 64 ? 3 * t + w4 : 3 * t + (lane >> 3);
-        const int c = RBX == 128 ? pl * 64 + (w4 & 1) * 32 + lane : RBX == 64 ? pl * 32 + lane : lane & 7;
-        if (u >= units || (RBX == 128 ? tap >= 9 : RBX == 64 ? w4 >= 3 : w4 > 0 || lane >= 24)) return nullptr;
-        return out + (size_t)(n0 + cb) * a.K + tap * a.Cin + c;
-      };
       float old[32];
       float *d = dest(e);
       auto fetch = [&](const float *from) {
@@ -2066,7 +2134,10 @@ __global__ void __launch_bounds__(WH_THREADS, 1)
         fetch(d);
         if (now) {
 #pragma unroll
-          for (int k = 0; k < 32; ++k) now[(size_t)k * a.K] = __uint_as_float(r[k]);
+          for (int k = 0; k < 32; ++k) {
+            now[(size_t)k * a.K] = __uint_as_float(r[k]);
+            if (a.inside) odd = fmaf(__uint_as_float(r[k]), 0.f, odd);
+          }
         }
       }
       asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -2077,6 +2148,24 @@ __global__ void __launch_bounds__(WH_THREADS, 1)
         abph ^= 1;
       }
       tile += n;
+    }
+    if (ok && a.inside && __any_sync(0xffffffffu, isnan(odd))) {
+#pragma unroll 1
+      for (int u = e; u < units; u += 2) {
+        float *d = dest(u);
+#pragma unroll 1
+        for (int k = 0; k < 32; ++k) {
+          const float was = d ? d[(size_t)k * a.K] : 0.f;
+          unsigned again = __ballot_sync(0xffffffffu, !isfinite(was));
+          while (again) {
+            const int q = __ffs(again) - 1;
+            again &= again - 1;
+            const long at = (long)__shfl_sync(0xffffffffu, (long long)(d - out) + (long long)k * a.K, q);
+            const float t = dw_inside(a.in, at, __shfl_sync(0xffffffffu, was, q));
+            if (lane == q) d[(size_t)k * a.K] = t;
+          }
+        }
+      }
     }
     if (bias) {
       // over the pixel rows: lanes first, then the warps' sums in order
@@ -2112,14 +2201,17 @@ __global__ void __launch_bounds__(WH_THREADS, 1)
 // sum_z ws2[z][i] for i < n2.  G groups of 256 / G threads take every G-th chunk, and
 // their sums are added in order: eight groups of a warp for many chunks (one
 // thread per output walking up to 512 chunks left most of the GPU idle, 51 us for 9,216
-// outputs), one group for few.
-template <int G>
-__global__ void __launch_bounds__(256) k_reduce_sums(const float *ws, long n, float *out, const float *ws2,
-                                                     int n2, float *out2, int chunks) {
+// outputs), one group for few.  INSIDE: out is a weight gradient from tiles that reach
+// past the images (see dw_inside).
+template <int G, bool INSIDE>
+__global__ void __launch_bounds__(256, 8) k_reduce_sums(const float *ws, long n, float *out, const float *ws2,
+                                                        int n2, float *out2, int chunks,
+                                                        const __grid_constant__ DwInputs v) {
   constexpr int L = 256 / G;
   __shared__ float red[G][L];
   const int l = threadIdx.x % L, g = threadIdx.x / L;
   const long nb1 = (n + L - 1) / L, nb2 = (n2 + L - 1) / L;
+  float odd = 0.f;  // NaN once an entry of out is not finite
   for (long b = blockIdx.x; b < nb1 + nb2; b += gridDim.x) {
     const bool second = b >= nb1;
     const float *src = second ? ws2 : ws;
@@ -2135,18 +2227,37 @@ __global__ void __launch_bounds__(256) k_reduce_sums(const float *ws, long n, fl
         for (int k = 1; k < G; ++k) s += red[k][l];
       }
     }
-    if (g == 0 && i < m) (second ? out2 : out)[i] = s;
+    if (g == 0 && i < m) {
+      (second ? out2 : out)[i] = s;
+      if (INSIDE && !second) odd = fmaf(s, 0.f, odd);
+    }
     if (G > 1) __syncthreads();
+  }
+  if (INSIDE && g == 0 && __any_sync(0xffffffffu, isnan(odd))) {  // whole warps
+    for (long b = blockIdx.x; b < nb1; b += gridDim.x) {
+      const long i = b * L + l;
+      const float s = i < n ? out[i] : 0.f;
+      unsigned again = __ballot_sync(0xffffffffu, !isfinite(s));
+      while (again) {
+        const int q = __ffs(again) - 1;
+        again &= again - 1;
+        const float t = dw_inside(v, i - (threadIdx.x & 31) + q, __shfl_sync(0xffffffffu, s, q));
+        if ((threadIdx.x & 31) == q) out[i] = t;
+      }
+    }
   }
 }
 
 void reduce_sums(const float *ws, long n, float *out, const float *ws2, int n2, float *out2, int chunks,
-                 cudaStream_t st) {
+                 cudaStream_t st, const DwInputs *v = nullptr) {
   const int per = chunks >= 16 ? 32 : 256;  // outputs of a block
   const long nblk = (n + per - 1) / per + (n2 + per - 1) / per;
   const int g = (int)(nblk < 8 * 1216 ? nblk : 8 * 1216);
-  if (chunks >= 16) k_reduce_sums<8><<<g, 256, 0, st>>>(ws, n, out, ws2, n2, out2, chunks);
-  else k_reduce_sums<1><<<g, 256, 0, st>>>(ws, n, out, ws2, n2, out2, chunks);
+  auto launch = [&](auto kernel) {
+    kernel<<<g, 256, 0, st>>>(ws, n, out, ws2, n2, out2, chunks, v ? *v : DwInputs{});
+  };
+  if (chunks >= 16) v ? launch(k_reduce_sums<8, true>) : launch(k_reduce_sums<8, false>);
+  else v ? launch(k_reduce_sums<1, true>) : launch(k_reduce_sums<1, false>);
 }
 
 struct WgHaloPlan {
@@ -2293,9 +2404,10 @@ cudaError_t launch_wgrad_halo(const WgHaloPlan &p, const WgMaps &m, cudaStream_t
 }
 
 // weight partials (and, when db, bias partials into wsb) of every tile range;
-// slots their number; with one slot the gradients themselves
+// slots their number; with one slot the gradients themselves; outside: tiles reach past
+// the images, the sums still need dw_inside
 bool wgrad_halo(const WgradArgs &v, int most, float *wsb, float *dw, float *db, cudaStream_t st, int &slots,
-                cudaError_t &rc) {
+                bool &outside, cudaError_t &rc) {
   WgHaloPlan p;
   if (!wgrad_halo_plan(v, most, p)) return false;
   WgMaps m;
@@ -2315,7 +2427,10 @@ bool wgrad_halo(const WgradArgs &v, int most, float *wsb, float *dw, float *db, 
   a.ws = p.slots == 1 ? dw : v.ws;
   a.wsb = !db ? nullptr : p.slots == 1 ? db : wsb;
   a.B = v.B; a.H = v.H; a.W = v.W; a.N = v.N; a.K = v.K; a.Cin = v.Cin;
+  a.in = dw_inputs(v);
   slots = p.slots;
+  outside = a.mode != TILE_WHOLE || v.W % 8 || v.H % 16;
+  a.inside = outside && slots == 1;
   rc = p.rbx == 128 ? (p.rby == 128 ? launch_wgrad_halo<128, 128>(p, m, st)
                                     : launch_wgrad_halo<128, 64>(p, m, st))
      : p.rbx == 64 ? (p.rby == 128 ? launch_wgrad_halo<64, 128>(p, m, st)
@@ -2864,12 +2979,14 @@ int cem_sg_conv3x3_wgrad(const void *x, int ldx, const void *dy, int lddy, int B
   if (g_use_tc) {
     cudaError_t he;
     int hs;
+    bool outside;
     // the bias partials lie behind the weight partials of `splits` chunks
     float *wsb = a.ws + (size_t)splits * Cout * a.K;
-    if (wgrad_halo(a, splits, wsb, dw, db, st, hs, he)) {
+    if (wgrad_halo(a, splits, wsb, dw, db, st, hs, outside, he)) {
       if (he != cudaSuccess) return CEM_SG_ERR_CUDA;
       if (hs == 1) return CEM_SG_OK;  // the kernel wrote dw and db
-      reduce_sums(a.ws, nw, dw, wsb, db ? Cout : 0, db, hs, st);
+      const DwInputs in = dw_inputs(a);
+      reduce_sums(a.ws, nw, dw, wsb, db ? Cout : 0, db, hs, st, outside ? &in : nullptr);
       return cudaGetLastError() == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
     }
     // tcgen05: dW^T tiles of 128 k' x BN outputs; bias sums by a separate
