@@ -2470,131 +2470,140 @@ __device__ __forceinline__ uint4 pack8(const float f[8]) {
 __device__ __forceinline__ uint4 ld8(const bf16_t *p) { return *reinterpret_cast<const uint4 *>(p); }
 __device__ __forceinline__ void st8(bf16_t *p, uint4 v) { *reinterpret_cast<uint4 *>(p) = v; }
 
-// They are bound by HBM, so a thread's index work must stay small: a block row
-// (blockIdx.y, strided) is one image row, its threads walk (pixel, 8 channels) with one
-// 32-bit division.  (One flat 64-bit index and three 64-bit divisions took 299 us
-// for the level-0 pooling gradient of 64 images, this 210, 4 TB/s; upsampling 162 ->
-// 97.)
+// They are bound by HBM, so a thread's index work must stay small: one 32-bit index over
+// (image row, pixel, 8 channels) and two divisions.  (A 64-bit index and three 64-bit
+// divisions took 286 us for the level-0 pooling gradient of 64 images, this 176, 4.9 TB/s;
+// upsampling 94 -> 83.  A block to an image row, with one division, took 197 and 83, and
+// left most of its threads idle on narrow images: 4096 of 4 x 4, 8 channels, 90 us
+// against 6.)
+struct Piece {
+  unsigned r, w, c;  // image row, pixel, first channel
+  __device__ __forceinline__ Piece(unsigned t, unsigned n, unsigned C8) : r(t / n) {
+    const unsigned i = t - r * n;
+    w = i / C8;
+    c = (i - w * C8) * 8;
+  }
+};
 
 // 2x2 max pooling: x [B, 2H, 2W] (pixel stride ldx) -> y [B, H, W, C] dense
-__global__ void __launch_bounds__(256) k_maxpool2(const bf16_t *x, int ldx, int rows, int W, int C, bf16_t *y) {
+__global__ void __launch_bounds__(256) k_maxpool2(const bf16_t *x, int ldx, unsigned rows, int W, int C, bf16_t *y) {
   dependency_wait();
   dependency_release();
-  const unsigned C8 = C >> 3, n = W * C8;
-  for (int r = blockIdx.y; r < rows; r += gridDim.y)  // row r of y: rows 2 r, 2 r + 1 of x
-    for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
-      const unsigned w = i / C8, c = (i - w * C8) * 8;
-      const bf16_t *p = x + ((size_t)r * 4 * W + 2 * w) * ldx + c;
-      const size_t row = (size_t)2 * W * ldx;
-      float v[4][8], o[8];
-      unpack8(ld8(p), v[0]);
-      unpack8(ld8(p + ldx), v[1]);
-      unpack8(ld8(p + row), v[2]);
-      unpack8(ld8(p + row + ldx), v[3]);
+  const unsigned C8 = C >> 3, n = W * C8, total = rows * n;
+  for (unsigned t = blockIdx.x * 256 + threadIdx.x; t < total; t += gridDim.x * 256) {
+    const Piece q0(t, n, C8);
+    const unsigned r = q0.r, w = q0.w, c = q0.c;
+    const bf16_t *p = x + ((size_t)r * 4 * W + 2 * w) * ldx + c;
+    const size_t row = (size_t)2 * W * ldx;
+    float v[4][8], o[8];
+    unpack8(ld8(p), v[0]);
+    unpack8(ld8(p + ldx), v[1]);
+    unpack8(ld8(p + row), v[2]);
+    unpack8(ld8(p + row + ldx), v[3]);
 #pragma unroll
-      for (int q = 0; q < 8; ++q) o[q] = fmaxf(fmaxf(v[0][q], v[1][q]), fmaxf(v[2][q], v[3][q]));
-      st8(y + ((size_t)r * W + w) * C + c, pack8(o));
-    }
+    for (int q = 0; q < 8; ++q) o[q] = fmaxf(fmaxf(v[0][q], v[1][q]), fmaxf(v[2][q], v[3][q]));
+    st8(y + ((size_t)r * W + w) * C + c, pack8(o));
+  }
 }
 
 // gradient of 2x2 max pooling to the first maximum of each window, plus an
 // optional skip gradient (dskip [.., ldskip] at channel offset skoff), zero
 // where x <= 0 when relu_mask (x is a ReLU output): dx [B, 2H, 2W, C] dense
 __global__ void __launch_bounds__(256) k_maxpool2_bwd(const bf16_t *x, int ldx, const bf16_t *dy,
-                                                      const bf16_t *dskip, int ldskip, int skoff, int rows,
+                                                      const bf16_t *dskip, int ldskip, int skoff, unsigned rows,
                                                       int W, int C, int relu_mask, bf16_t *dx) {
-  const unsigned C8 = C >> 3, n = W * C8;
-  for (int r = blockIdx.y; r < rows; r += gridDim.y)
-    for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
-      const unsigned w = i / C8, c = (i - w * C8) * 8;
-      uint4 raw[4], sk[4];
-      size_t pp[4];
+  const unsigned C8 = C >> 3, n = W * C8, total = rows * n;
+  for (unsigned t = blockIdx.x * 256 + threadIdx.x; t < total; t += gridDim.x * 256) {
+    const Piece q0(t, n, C8);
+    const unsigned r = q0.r, w = q0.w, c = q0.c;
+    uint4 raw[4], sk[4];
+    size_t pp[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        pp[q] = (size_t)r * 4 * W + (q >> 1) * 2 * W + 2 * w + (q & 1);
-        raw[q] = ld8(x + pp[q] * ldx + c);
-      }
-      const uint4 gr = ld8(dy + ((size_t)r * W + w) * C + c);
-      if (dskip)
+    for (int q = 0; q < 4; ++q) {
+      pp[q] = (size_t)r * 4 * W + (q >> 1) * 2 * W + 2 * w + (q & 1);
+      raw[q] = ld8(x + pp[q] * ldx + c);
+    }
+    const uint4 gr = ld8(dy + ((size_t)r * W + w) * C + c);
+    if (dskip)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) sk[q] = ld8(dskip + pp[q] * ldskip + skoff + c);
-      float v[4][8], g[8], m[8];
-      bool taken[8];
-      unpack8(gr, g);
+      for (int q = 0; q < 4; ++q) sk[q] = ld8(dskip + pp[q] * ldskip + skoff + c);
+    float v[4][8], g[8], m[8];
+    bool taken[8];
+    unpack8(gr, g);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) unpack8(raw[q], v[q]);
+    for (int q = 0; q < 4; ++q) unpack8(raw[q], v[q]);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      m[k] = fmaxf(fmaxf(v[0][k], v[1][k]), fmaxf(v[2][k], v[3][k]));
+      taken[k] = false;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float s[8], o[8];
+      if (dskip) unpack8(sk[q], s);
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
-        m[k] = fmaxf(fmaxf(v[0][k], v[1][k]), fmaxf(v[2][k], v[3][k]));
-        taken[k] = false;
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        float s[8], o[8];
-        if (dskip) unpack8(sk[q], s);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          o[k] = 0.f;
-          if (!taken[k] && v[q][k] == m[k]) {
-            o[k] = g[k];
-            taken[k] = true;
-          }
-          if (dskip) o[k] += s[k];
-          if (relu_mask && !(v[q][k] > 0.f)) o[k] = 0.f;
+        o[k] = 0.f;
+        if (!taken[k] && v[q][k] == m[k]) {
+          o[k] = g[k];
+          taken[k] = true;
         }
-        st8(dx + pp[q] * C + c, pack8(o));
+        if (dskip) o[k] += s[k];
+        if (relu_mask && !(v[q][k] > 0.f)) o[k] = 0.f;
       }
+      st8(dx + pp[q] * C + c, pack8(o));
     }
+  }
 }
 
 // nearest 2x upsampling: x [B, H, W, C] dense -> y [B, 2H, 2W, ldy] at channel offset yoff
-__global__ void __launch_bounds__(256) k_upsample2(const bf16_t *x, int rows, int W, int C, bf16_t *y, int ldy,
+__global__ void __launch_bounds__(256) k_upsample2(const bf16_t *x, unsigned rows, int W, int C, bf16_t *y, int ldy,
                                                    int yoff) {
   dependency_wait();
   dependency_release();
-  const unsigned C8 = C >> 3, n = W * C8;
-  for (int r = blockIdx.y; r < rows; r += gridDim.y)
-    for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
-      const unsigned w = i / C8, c = (i - w * C8) * 8;
-      const uint4 v = ld8(x + ((size_t)r * W + w) * C + c);
-      bf16_t *p = y + ((size_t)r * 4 * W + 2 * w) * ldy + yoff + c;
-      const size_t row = (size_t)2 * W * ldy;
-      st8(p, v);
-      st8(p + ldy, v);
-      st8(p + row, v);
-      st8(p + row + ldy, v);
-    }
+  const unsigned C8 = C >> 3, n = W * C8, total = rows * n;
+  for (unsigned t = blockIdx.x * 256 + threadIdx.x; t < total; t += gridDim.x * 256) {
+    const Piece q0(t, n, C8);
+    const unsigned r = q0.r, w = q0.w, c = q0.c;
+    const uint4 v = ld8(x + ((size_t)r * W + w) * C + c);
+    bf16_t *p = y + ((size_t)r * 4 * W + 2 * w) * ldy + yoff + c;
+    const size_t row = (size_t)2 * W * ldy;
+    st8(p, v);
+    st8(p + ldy, v);
+    st8(p + row, v);
+    st8(p + row + ldy, v);
+  }
 }
 
 // gradient of nearest 2x upsampling: dy [B, 2H, 2W, lddy] channels 0..C-1 ->
 // dx [B, H, W, C], zero where mask <= 0 (mask [B, H, W, ldm], may be null)
-__global__ void __launch_bounds__(256) k_upsample2_bwd(const bf16_t *dy, int lddy, int rows, int W, int C,
+__global__ void __launch_bounds__(256) k_upsample2_bwd(const bf16_t *dy, int lddy, unsigned rows, int W, int C,
                                                        const bf16_t *mask, int ldm, bf16_t *dx) {
-  const unsigned C8 = C >> 3, n = W * C8;
-  for (int r = blockIdx.y; r < rows; r += gridDim.y)
-    for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
-      const unsigned w = i / C8, c = (i - w * C8) * 8;
-      const size_t pix = (size_t)r * W + w;
-      uint4 raw[4];
+  const unsigned C8 = C >> 3, n = W * C8, total = rows * n;
+  for (unsigned t = blockIdx.x * 256 + threadIdx.x; t < total; t += gridDim.x * 256) {
+    const Piece q0(t, n, C8);
+    const unsigned r = q0.r, w = q0.w, c = q0.c;
+    const size_t pix = (size_t)r * W + w;
+    uint4 raw[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        raw[q] = ld8(dy + ((size_t)r * 4 * W + (q >> 1) * 2 * W + 2 * w + (q & 1)) * lddy + c);
-      float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, t[8];
+    for (int q = 0; q < 4; ++q)
+      raw[q] = ld8(dy + ((size_t)r * 4 * W + (q >> 1) * 2 * W + 2 * w + (q & 1)) * lddy + c);
+    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, d[8];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        unpack8(raw[q], t);
+    for (int q = 0; q < 4; ++q) {
+      unpack8(raw[q], d);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) s[k] += t[k];
-      }
-      if (mask) {
-        float mk[8];
-        unpack8(ld8(mask + pix * ldm + c), mk);
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-          if (!(mk[k] > 0.f)) s[k] = 0.f;
-      }
-      st8(dx + pix * C + c, pack8(s));
+      for (int k = 0; k < 8; ++k) s[k] += d[k];
     }
+    if (mask) {
+      float mk[8];
+      unpack8(ld8(mask + pix * ldm + c), mk);
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (!(mk[k] > 0.f)) s[k] = 0.f;
+    }
+    st8(dx + pix * C + c, pack8(s));
+  }
 }
 
 // ------------------------------------------------------------------- head
@@ -2904,10 +2913,17 @@ __global__ void k_to_bf16(const float *x, long n, bf16_t *y) {
     y[i] = f2bf(x[i]);
 }
 
-// grid of the pooling and upsampling kernels: image rows down, (pixel, 8 channels) across
-dim3 grid_rows(long rows, long per_row) {
-  const long x = (per_row + 255) / 256;
-  return dim3((unsigned)(x < 65535 ? x : 65535), (unsigned)(rows < 65535 ? rows : 65535));
+// Launches of the pooling and upsampling kernels: launch(first image row, rows, blocks), one
+// unless the pieces (a pixel's 8 channels) need more than 31 bits
+template <class F>
+cudaError_t for_pieces(long rows, long per_row, F launch) {
+  const long most = per_row < (1L << 31) ? ((1L << 31) - 1) / per_row : 1;
+  for (long r = 0; r < rows; r += most) {
+    const long k = rows - r < most ? rows - r : most, blocks = (k * per_row + 255) / 256;
+    const cudaError_t e = launch(r, (unsigned)k, (unsigned)(blocks < (1 << 22) ? blocks : 1 << 22));
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 int grid_1d(long n, int block) {
@@ -3026,10 +3042,11 @@ int cem_sg_relu_bwd(void *dy, int lddy, const void *y, int ldy, long P, int C, v
 int cem_sg_maxpool2(const void *x, int ldx, int B, int H, int W, int C, void *y, void *stream) {
   if (!x || !y || B < 1 || H < 1 || W < 1 || C < 8 || (C & 7) || ldx < C || (ldx & 7))
     return CEM_SG_ERR_ARG;
-  const long rows = (long)B * H;
-  return launch_dependent(k_maxpool2, grid_rows(rows, (long)W * (C >> 3)), 256, 0, (cudaStream_t)stream,
-                          (const bf16_t *)x, ldx, (int)rows, W, C, (bf16_t *)y) == cudaSuccess
-             ? CEM_SG_OK : CEM_SG_ERR_CUDA;
+  const cudaError_t e = for_pieces((long)B * H, (long)W * (C >> 3), [&](long r, unsigned rows, unsigned blocks) {
+    return launch_dependent(k_maxpool2, blocks, 256, 0, (cudaStream_t)stream,
+                            (const bf16_t *)x + r * 4 * W * ldx, ldx, rows, W, C, (bf16_t *)y + r * W * C);
+  });
+  return e == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
 }
 
 int cem_sg_maxpool2_bwd(const void *x, int ldx, const void *dy, const void *dskip, int ldskip,
@@ -3038,11 +3055,14 @@ int cem_sg_maxpool2_bwd(const void *x, int ldx, const void *dy, const void *dski
   if (!x || !dy || !dx || B < 1 || H < 1 || W < 1 || C < 8 || (C & 7) || ldx < C || (ldx & 7) ||
       (dskip && (ldskip < skoff + C || (ldskip & 7) || (skoff & 7))))
     return CEM_SG_ERR_ARG;
-  const long rows = (long)B * H;
-  k_maxpool2_bwd<<<grid_rows(rows, (long)W * (C >> 3)), 256, 0, (cudaStream_t)stream>>>(
-      (const bf16_t *)x, ldx, (const bf16_t *)dy, (const bf16_t *)dskip, ldskip, skoff, (int)rows, W, C,
-      relu_mask, (bf16_t *)dx);
-  return cudaGetLastError() == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
+  const cudaError_t e = for_pieces((long)B * H, (long)W * (C >> 3), [&](long r, unsigned rows, unsigned blocks) {
+    k_maxpool2_bwd<<<blocks, 256, 0, (cudaStream_t)stream>>>(
+        (const bf16_t *)x + r * 4 * W * ldx, ldx, (const bf16_t *)dy + r * W * C,
+        dskip ? (const bf16_t *)dskip + r * 4 * W * ldskip : nullptr, ldskip, skoff, rows, W, C, relu_mask,
+        (bf16_t *)dx + r * 4 * W * C);
+    return cudaGetLastError();
+  });
+  return e == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
 }
 
 int cem_sg_upsample2(const void *x, int B, int H, int W, int C, void *y, int ldy, int yoff,
@@ -3050,10 +3070,11 @@ int cem_sg_upsample2(const void *x, int B, int H, int W, int C, void *y, int ldy
   if (!x || !y || B < 1 || H < 1 || W < 1 || C < 8 || (C & 7) || ldy < yoff + C || (ldy & 7) ||
       (yoff & 7))
     return CEM_SG_ERR_ARG;
-  const long rows = (long)B * H;
-  return launch_dependent(k_upsample2, grid_rows(rows, (long)W * (C >> 3)), 256, 0, (cudaStream_t)stream,
-                          (const bf16_t *)x, (int)rows, W, C, (bf16_t *)y, ldy, yoff) == cudaSuccess
-             ? CEM_SG_OK : CEM_SG_ERR_CUDA;
+  const cudaError_t e = for_pieces((long)B * H, (long)W * (C >> 3), [&](long r, unsigned rows, unsigned blocks) {
+    return launch_dependent(k_upsample2, blocks, 256, 0, (cudaStream_t)stream, (const bf16_t *)x + r * W * C, rows,
+                            W, C, (bf16_t *)y + r * 4 * W * ldy, ldy, yoff);
+  });
+  return e == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
 }
 
 int cem_sg_upsample2_bwd(const void *dy, int lddy, int B, int H, int W, int C, const void *mask,
@@ -3061,10 +3082,13 @@ int cem_sg_upsample2_bwd(const void *dy, int lddy, int B, int H, int W, int C, c
   if (!dy || !dx || B < 1 || H < 1 || W < 1 || C < 8 || (C & 7) || lddy < C || (lddy & 7) ||
       (mask && (ldmask < C || (ldmask & 7))))
     return CEM_SG_ERR_ARG;
-  const long rows = (long)B * H;
-  k_upsample2_bwd<<<grid_rows(rows, (long)W * (C >> 3)), 256, 0, (cudaStream_t)stream>>>(
-      (const bf16_t *)dy, lddy, (int)rows, W, C, (const bf16_t *)mask, ldmask, (bf16_t *)dx);
-  return cudaGetLastError() == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
+  const cudaError_t e = for_pieces((long)B * H, (long)W * (C >> 3), [&](long r, unsigned rows, unsigned blocks) {
+    k_upsample2_bwd<<<blocks, 256, 0, (cudaStream_t)stream>>>(
+        (const bf16_t *)dy + r * 4 * W * lddy, lddy, rows, W, C,
+        mask ? (const bf16_t *)mask + r * W * ldmask : nullptr, ldmask, (bf16_t *)dx + r * W * C);
+    return cudaGetLastError();
+  });
+  return e == cudaSuccess ? CEM_SG_OK : CEM_SG_ERR_CUDA;
 }
 
 int cem_sg_head_fwd(const void *x, int P, int C, const float *w, const float *b, float *z,
