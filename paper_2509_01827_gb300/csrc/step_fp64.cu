@@ -746,7 +746,9 @@ cudaError_t launch_step_fp64_batch(const BatchDev &b, bool first, bool energy, i
   cudaError_t e = fp64_attrs();
   if (e != cudaSuccess) return e;
   const int gm = grid_main < 1 ? 1 : grid_main;
-  const int gp = grid_for(b.n_pieces, 1, 1216), gph = grid_for(b.n_ph, 1, 1216);
+  // four times the piece blocks of 256 threads that the SMs hold, as these have 64: 64 specimens
+  // of 50 x 20 to 100 x 40 elements, most of them split, 409 us a step with 1216, 318 so
+  const int gp = grid_for(b.n_pieces, 1, 4 * 1216), gph = grid_for(b.n_ph, 1, 1216);
   const int ge = grid_for(b.n_eval, 1, 1216);
   cudaStream_t st = ss.main;
   cudaEventRecord(ss.fork, st);
