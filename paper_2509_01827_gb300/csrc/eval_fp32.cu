@@ -346,11 +346,14 @@ int grid_for(int n, int block, int maxb) {
 
 int grid_eval(const DevState &d) { return grid_for(d.list_cap, kEvalPts, 608); }
 
+// k_eval32 asks for no shared-memory split.  With the node update's (164 KB) an SM that
+// runs it keeps little L1 for the piece forces beside it, which gather nodes: a
+// 1024 x 1024 plate with 590,000 split elements took 141 us a step so, 116 without; with
+// 59,000 of them 40 and 37, and as long with few.
 cudaError_t eval32_carveouts() {
   static PerDevice attrs;
   return attrs.once([] {
-    cudaError_t e = match_tile_carveout(k_eval32);
-    if (e == cudaSuccess) e = match_tile_carveout(k_eval32_batch);
+    cudaError_t e = match_tile_carveout(k_eval32_batch);
     if (e == cudaSuccess) e = match_tile_carveout(k_eval32_points);
     return e;
   });

@@ -1058,12 +1058,16 @@ int energy_parts_fp32(const DevState &d) {
   return std::max(tiles_fp32(d, 8), tiles_fp32(d, march_rows_solo(d))) + kPhWarps * 1216 + 1216 + 8;
 }
 
-// piece-force blocks: one thread per split element in FP32, per piece in FP64
-int grid_pieces(const DevState &d) {
-  return grid_for(d.precision == 1 ? d.ck_cap : 2 * d.ck_cap, 256, 304);
-}
-// side-branch grids: two phantom blocks and one evaluation block per SM, so that
-// they start together with the node update and share the SMs with it
+// piece-force blocks: one thread per split element.  As many as the SMs hold at
+// once, so that hundreds of thousands of split elements are shared out evenly
+// whatever else runs (1024 x 1024, 590,000 of them: 140 us a step with 304 blocks, 116 with
+// 1216).  Meshes of more than two million nodes keep 304: their node update sets
+// the step and its CTAs are placed after the piece blocks' (an intact 2048 x 2048 plate:
+// 55.2 and 56.1 us; with 1.1 million split elements 245 and 247).
+constexpr int kLargeMesh = 1 << 21;  // nodes
+int grid_pieces(const DevState &d) { return grid_for(d.ck_cap, 256, d.g.nn > kLargeMesh ? 304 : 1216); }
+// side-branch grid: two phantom blocks per SM, so that they start together with
+// the node update and share the SMs with it
 int grid_phantoms(const DevState &d) { return grid_for(d.ph_cap, 256, 304); }
 
 // energy partials one FP32 step writes with the given tile height

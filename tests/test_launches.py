@@ -53,6 +53,18 @@ def test_batch_grids_fill_the_gpu(native):
             assert grid >= 1216
 
 
+@pytest.mark.parametrize("side,blocks", [(1024, 1216), (1440, 1216), (2048, 304)])
+def test_piece_blocks_and_evaluation_split(native, monkeypatch, side, blocks):
+    """Plates with hundreds of thousands of split elements: the piece forces have as
+    many blocks as the SMs hold (meshes whose node update sets the step: two an SM),
+    and the evaluation beside them leaves the SMs their L1."""
+    monkeypatch.setenv("MESH_SIDE", str(side))
+    lines = native("step_grids").splitlines()
+    assert lines[0] == "0" or side == 2048
+    launches = [tuple(int(v) for v in line.split()) for line in lines[1:]]
+    assert max(grid for block, grid in launches if block == 256 and grid > 1) == blocks
+
+
 @pytest.mark.gpu
 def test_two_devices_in_one_process():
     import torch
