@@ -282,11 +282,12 @@ __global__ void k_tri_edge32(TriDev d, int energy) {
 }
 
 // Bound by the gather's loads (16 bytes of record and 16 of stress per
-// incidence, about 18 of them a node): one node per thread, eight incidences in
-// flight, and FP64 only where a node has a load or a prescribed velocity or the
-// step records energies (as a part of every node's update its conversions
-// alone took 7 us of the FP64 pipe for 0.5 M nodes).  ENERGY: the grid is the
-// one the partial sums are laid out for, its threads walk the nodes.
+// incidence, about 18 of them a node): one node per thread, four incidences in
+// flight (eight took 81.0 us a step for 0.5 M nodes, four 78.0; 16.4 and 14.4 us on
+// the smallest meshes), and FP64 only where a node has a load or a prescribed
+// velocity or the step records energies (as a part of every node's update its
+// conversions alone took 7 us of the FP64 pipe for 0.5 M nodes).  ENERGY: the grid
+// is the one the partial sums are laid out for, its threads walk the nodes.
 template <bool ENERGY>
 __global__ void __launch_bounds__(kTB) k_tri_node32(TriDev d, double lamN, double lamD, double dtd, double dtvd,
                                                     int first, int part_off) {
@@ -297,31 +298,17 @@ __global__ void __launch_bounds__(kTB) k_tri_node32(TriDev d, double lamN, doubl
     float fx = 0.f, fy = 0.f;
     const int deg = d.inc_deg[N];
     const TriInc32 *rec = d.inc32 + d.slice_off[N >> 5] + (N & 31);
-    const int loaded = d.lflag[N], dm = d.dmask[N];
-    const float mi = d.minvf[N];
-    const float2 vo = d.v2[N];
-    float4 U = d.u4[N];
-    int k = 0;
-    for (; k + 8 <= deg; k += 8) {
-      TriInc32 r[8];
-      float4 s[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) r[q] = rec[32L * (k + q)];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) s[q] = d.sig32[r[q].g];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        fx = fx + (r[q].b * s[q].x + r[q].c * s[q].z) * r[q].q3;
-        fy = fy + (r[q].c * s[q].y + r[q].b * s[q].z) * r[q].q3;
-      }
-    }
-#pragma unroll 2
-    for (; k < deg; ++k) {
+#pragma unroll 4
+    for (int k = 0; k < deg; ++k) {
       const TriInc32 r = rec[32L * k];
       const float4 s = d.sig32[r.g];
       fx = fx + (r.b * s.x + r.c * s.z) * r.q3;
       fy = fy + (r.c * s.y + r.b * s.z) * r.q3;
     }
+    const int loaded = d.lflag[N], dm = d.dmask[N];
+    const float mi = d.minvf[N];
+    const float2 vo = d.v2[N];
+    float4 U = d.u4[N];
     float fex = 0.f, fey = 0.f;
     if (loaded) {
       const double2 F = d.F[N];
