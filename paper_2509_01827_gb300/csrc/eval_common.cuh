@@ -68,10 +68,9 @@ __device__ __forceinline__ bool is_tip_edge(const DevState &d, int e, int k0) {
   return (info & 3) == kf || ((info >> 2) & 3) == kf;
 }
 
-// G of the three candidate paths of surface point (e, k0); G[k0] = -1.
+// G of the candidate path of local edge k of surface point (e, k0), -1 for k = k0:
 // delta_d = (u_N2 - u_N1) H(|x_N2 - x_N1| > |X_N2 - X_N1|), G = delta_d.(sigma n)/2.
-// eval_G64_k: the candidate of local edge k alone (-1 for k = k0).  The
-// reference vectors and unit normals are the mesh's (Geo: formed once, their
+// The reference vectors and unit normals are the mesh's (Geo: formed once, their
 // square root and divisions with it).
 template <class UA>
 __device__ __forceinline__ double eval_G64_k(const DevState &d, const UA &U, int e, int k0, int k) {
@@ -90,11 +89,6 @@ __device__ __forceinline__ double eval_G64_k(const DevState &d, const UA &U, int
   double tx = s[0] * nx + s[2] * ny;
   double ty = s[2] * nx + s[1] * ny;
   return 0.5 * (ddx * tx + ddy * ty);
-}
-
-template <class UA>
-__device__ void eval_G64(const DevState &d, const UA &U, int e, int k0, double G[4]) {
-  for (int k = 0; k < 4; ++k) G[k] = eval_G64_k(d, U, e, k0, k);
 }
 
 // Q4 cracking conditions with the split ratio gamma (Sec. 2.2).

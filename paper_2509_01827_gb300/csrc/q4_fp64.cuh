@@ -110,16 +110,6 @@ __device__ __forceinline__ void node_force64(const Geo &g, const double s[4][3],
   fy = sy * qA;
 }
 
-__device__ __forceinline__ void node_force64_rt(const Geo &g, int a, const double s[4][3],
-                                                double qA, double &fx, double &fy) {
-  switch (a) {
-    case 0: node_force64<0>(g, s, qA, fx, fy); break;
-    case 1: node_force64<1>(g, s, qA, fx, fy); break;
-    case 2: node_force64<2>(g, s, qA, fx, fy); break;
-    default: node_force64<3>(g, s, qA, fx, fy); break;
-  }
-}
-
 // ----------------------------------------------------------------- geometry
 __device__ __forceinline__ int elem_node(const Geo &g, int e, int a) {
   int i = e % g.nx, j = e / g.nx, r = g.nx + 1;
@@ -164,11 +154,5 @@ __device__ __forceinline__ void edge_sides(const Geo &g, int gid, int &lo, int &
 __device__ __forceinline__ int estatus(const DevState &d, int e) {
   return e < 0 ? ST_OUT : (int)d.estate[e];
 }
-
-// Natural coordinates of nodes and edge midpoints.
-__host__ __device__ constexpr double xi_n(int a) { return (a == 0 || a == 3) ? -1.0 : 1.0; }
-__host__ __device__ constexpr double eta_n(int a) { return a < 2 ? -1.0 : 1.0; }
-__host__ __device__ constexpr double xi_g(int k) { return k == 1 ? 1.0 : k == 3 ? -1.0 : 0.0; }
-__host__ __device__ constexpr double eta_g(int k) { return k == 0 ? -1.0 : k == 2 ? 1.0 : 0.0; }
 
 }  // namespace cem
