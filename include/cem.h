@@ -356,9 +356,9 @@ cem_status cem_batch_create(cem_handle *const *members, int n, const long *step_
 cem_status cem_batch_set_config(cem_handle *batch, int tile_rows, int grid_main);
 
 /* Autotuner: times steps_per_candidate real steps (after one untimed step)
- * for each candidate configuration -- tile heights {16, 8, 32, 64} (FP32
- * only) x grids {1, 2, 3, 4} x SMs -- keeps the fastest and returns it.  The timed
- * steps advance the simulation like cem_step. */
+ * for each candidate configuration -- FP32: tile heights {16, 8, 32, 64} x
+ * grids {1, 2, 3, 4} x SMs; FP64: grids {2, 4, 8, 16} x SMs -- keeps the fastest
+ * and returns it.  The timed steps advance the simulation like cem_step. */
 cem_status cem_batch_autotune(cem_handle *batch, int steps_per_candidate, int *tile_rows,
                               int *grid_main);
 

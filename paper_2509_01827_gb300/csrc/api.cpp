@@ -1973,9 +1973,11 @@ cem_status cem_batch_autotune(cem_handle *b, int steps_per_candidate, int *tile_
   if (steps_per_candidate < 1) return fail(b, CEM_ERR_ARG, "steps_per_candidate >= 1");
   CUDA_TRY(b, cudaSetDevice(b->device));
   std::vector<std::pair<int, int>> cand;
+  // FP64 has one tile height, and its update gains up to 16 CTAs per SM (cem_batch_create)
+  const bool mixed = p->precision == CEM_FP32_MIXED;
   const int rows[4] = {16, 8, 32, 64};
-  for (int r = 0; r < (p->precision == CEM_FP32_MIXED ? 4 : 1); ++r)
-    for (int k = 1; k <= 4; ++k) cand.push_back({rows[r], k * p->sms});
+  for (int r = 0; r < (mixed ? 4 : 1); ++r)
+    for (int k = 1; k <= 4; ++k) cand.push_back({rows[r], (mixed ? k : 1 << k) * p->sms});
   cudaEvent_t e0, e1;
   CUDA_TRY(b, cudaEventCreate(&e0));
   CUDA_TRY(b, cudaEventCreate(&e1));
