@@ -348,8 +348,8 @@ cem_status cem_batch_create(cem_handle *const *members, int n, const long *step_
                             void *cuda_stream, cem_handle **out);
 
 /* Launch configuration of a batch: tile_rows (8 .. 64) is the height of the
- * FP32 node update's tiles (28 nodes wide, one warp each; the FP64 tiles are
- * fixed at 32 x 8), grid_main the persistent grid of the node update
+ * FP32 node update's tiles (60 nodes wide, one warp each; the FP64 tiles
+ * follow each member's size, up to 32 x 12), grid_main the persistent grid of the node update
  * (1 .. 64 x SMs).  Nodal results do not depend on it; in FP32 the energy
  * records group their partial sums by tile (last-bit differences).
  * Default: chosen from the members' sizes (FP64 grid: 16 x SMs). */

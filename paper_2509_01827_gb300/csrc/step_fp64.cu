@@ -614,7 +614,8 @@ int energy_parts_fp32(const DevState &d);
 // the 152 SMs, plus a constant for a tile's load and barrier latency (about
 // 60 warp instructions' time; it matters for small meshes only).  On the 100 x
 // 40 plate that is 16 x 2 nodes (10 us; 32 x 8 takes 36), on 400 x 160 32 x 8,
-// on large meshes 32 x 12, of which two CTAs share an SM.
+// on large meshes 32 x 12, of which three CTAs share an SM where the elements are
+// square, two elsewhere (launch_step_fp64).
 void tile64_shape(int nx, int ny, int &tx, int &ty) {
   constexpr int kTx[] = {32, 16}, kTy[] = {12, 8, 6, 4, 3, 2, 1}, kSms = 152;
   double best = 0.0;

@@ -2827,11 +2827,11 @@ __global__ void __launch_bounds__(256) k_dice_grad(const float *z, const uint8_t
 }
 
 // loss = w (1 - mean_b D_b), D_b = (2 I_b + eps) / (S_b + eps), one block: a
-// sample's chunks in order by one thread, the samples' indices by fixed lanes and a tree
-// (a single thread walking all of it took 74 us for 64 samples, this 5)
+// sample's chunks in order by one thread, the samples' terms one after another by
+// thread 0 (the Dice term of 64 images of 64,000 pixels, all three kernels: 84 us
+// when a single thread walked all of it, 34 so)
 __global__ void __launch_bounds__(256) k_dice_loss(const float *ws, int nchunk, int B, float w, float eps,
                                                    float *loss) {
-  // each image's sums by a thread, the images' terms added in their order
   __shared__ float term[256];
   float d = 0.f;
   for (int b0 = 0; b0 < B; b0 += 256) {
