@@ -270,12 +270,13 @@ __device__ __forceinline__ void eval_G32(const DevState &d, const EvalPatch &P, 
 }
 
 // Large meshes: a thread per point, its candidates one after another, one
-// block of 256 threads per SM.  There the piece forces and the node update set
-// the step, and this form takes less from them: a breaking 2048 x 2048 plate's
-// step 61.5 / 67.9 / 84.7 us after 400 / 4000 / 9000 steps, 62.8 / 73.4 / 94.4 with the
-// split above, which alone is done sooner (12.7 / 14.5 / 17.8 against 19.0 / 13.7 /
-// 22.9 us) and on a 1024 x 1024 plate, whose step is the chain of evaluation,
-// selection and split writes, the better one (with it 31.5 us, 36 before).
+// block of 256 threads per SM.  There the node update sets the step, or the piece
+// forces once much is broken, and this form takes less from them: an intact
+// 2048 x 2048 plate's step is 55.0 us, 57.5 with the split above, one with 1.1
+// million split elements 245 and 322 us (between, after 400 to 9000 steps of a breaking
+// plate, both take as long within 2%).  On a 1024 x 1024 plate, whose step is the chain
+// of evaluation, selection and split writes, the split is the better one (40 us
+// while it breaks, 45 with this form).
 constexpr int kLargeMesh = 1 << 21;  // nodes
 __device__ __forceinline__ void eval32_points(const DevState &d, VBlk vb, int cur) {
   const int n = d.cnt->n_S;
