@@ -2133,11 +2133,13 @@ __global__ void __launch_bounds__(WH_THREADS, 1)
         d = dest(u + 2);
         fetch(d);
         if (now) {
+          float z[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
           for (int k = 0; k < 32; ++k) {
             now[(size_t)k * a.K] = __uint_as_float(r[k]);
-            if (a.inside) odd = fmaf(__uint_as_float(r[k]), 0.f, odd);
+            z[k & 3] = fmaf(__uint_as_float(r[k]), 0.f, z[k & 3]);
           }
+          odd += (z[0] + z[1]) + (z[2] + z[3]);
         }
       }
       asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
